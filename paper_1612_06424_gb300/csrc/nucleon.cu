@@ -184,60 +184,97 @@ __global__ void __launch_bounds__(256, 2) k_nucleon_block(int n, long long nsite
   }
 }
 
-// W[ix][iy] = (W1, W2) for slices ix of B_xi and iy of B_eta; one block per
-// (ix, iy), FP64.  g5 P_- = g5 (1 - g0)/2 in the chiral basis: rows
-// (1/2)[[1,0,1,0],[0,1,0,1],[1,0,1,0],[0,1,0,1]] times diag(1,1,-1,-1) on the
-// left: M = (1/2)[[1,0,1,0],[0,1,0,1],[-1,0,-1,0],[0,-1,0,-1]].
-__global__ void __launch_bounds__(256) k_nucleon_contract(int n, int ny, const double2* Bx, const double2* By,
-                                                          double2* W) {
-  const int ix = blockIdx.x / ny, iy = blockIdx.x % ny;
+// Wick contractions of every pair (ix of B_xi, iy of B_eta), FP64.  g5 P_- = g5 (1 - g0)/2 in the
+// chiral basis is (1/2)[[1,0,1,0],[0,1,0,1],[-1,0,-1,0],[0,-1,0,-1]], so with
+// u_h = B_eta_h + B_eta_{h+2} and d_h = B_xi_h - B_xi_{h+2} (h = 0, 1)
+//   W1 = -(1/2) sum_ijk sum_h d_h[j][i][k] u_h[i][j][k],
+//   W2 = -(1/2) sum_ijk sum_h d_h[k][i][j] u_h[i][j][k].
+//
+// Bound by the FP64 pipe (20 instructions per (i,j,k) and pair of slices, the GB300 issues about 2
+// per clock and SM) just above the read of the blocks.  The sum over (i,j,k) is therefore cut into
+// enough parts for every SM: a block takes 16 x 16 (j, k) tiles of one i (one thread an element, so
+// that the transposed rows B_xi[k][i][j0..] are read as runs of 1 KB too), and one read of B_xi serves
+// CT_NY sink slices.  Part p of pair (ix, iy) goes to part[((ix ny + iy) nsplit + p) 4]; k_contract_sum
+// adds the parts in a fixed order.  120 factors, 8 sink slices: 38.7 ms with one block per pair of
+// slices, 0.61 ms so.
+constexpr int CT = 16;     // edge of a (j, k) tile
+constexpr int CT_NY = 4;   // sink slices per block
+
+__global__ void __launch_bounds__(CT * CT) k_nucleon_contract(int n, int ny, int nsplit, const double2* Bx,
+                                                              const double2* By, double* part) {
+  // grid: ((ix, group of sink slices), part), the part fastest
+  const int sp = (int)(blockIdx.x % (unsigned)nsplit), pr = (int)(blockIdx.x / (unsigned)nsplit);
+  const int ngy = (ny + CT_NY - 1) / CT_NY;
+  const int ix = pr / ngy, iy0 = (pr - ix * ngy) * CT_NY;
   const long long n3 = (long long)n * n * n;
   const double2* bx = Bx + (long long)ix * n3 * 4;
-  const double2* by = By + (long long)iy * n3 * 4;
-  const double M[4][4] = {{0.5, 0, 0.5, 0}, {0, 0.5, 0, 0.5}, {-0.5, 0, -0.5, 0}, {0, -0.5, 0, -0.5}};
-  double w1r = 0, w1i = 0, w2r = 0, w2i = 0;
-  for (long long e = threadIdx.x; e < n3; e += blockDim.x) {
-    const int k = (int)(e % n), j = (int)((e / n) % n), i = (int)(e / ((long long)n * n));
-    const double2* yv = by + e * 4;                                      // B_eta[i][j][k]
-    const double2* x1 = bx + ((((long long)j * n + i) * n) + k) * 4;   // B_xi[j][i][k]
-    const double2* x2 = bx + ((((long long)k * n + i) * n) + j) * 4;   // B_xi[k][i][j]
-    double2 my[4];
+  const int nt = (n + CT - 1) / CT;
+  const int tj = threadIdx.x / CT, tk = threadIdx.x % CT;
+  double acc[CT_NY][4];
 #pragma unroll
-    for (int g = 0; g < 4; g++) {
-      double re = 0, im = 0;
+  for (int y = 0; y < CT_NY; y++)
 #pragma unroll
-      for (int d = 0; d < 4; d++) {
-        re += M[g][d] * yv[d].x;
-        im += M[g][d] * yv[d].y;
+    for (int q = 0; q < 4; q++) acc[y][q] = 0.0;
+  const long long tiles = (long long)n * nt * nt;
+  for (long long tile = sp; tile < tiles; tile += nsplit) {
+    const int i = (int)(tile / (nt * nt)), r = (int)(tile - (long long)i * nt * nt);
+    const int j = (r / nt) * CT + tj, k = (r % nt) * CT + tk;
+    if (j >= n || k >= n) continue;
+    const double2* x1 = bx + ((((long long)j * n + i) * n) + k) * 4;  // B_xi[j][i][k]
+    const double2* x2 = bx + ((((long long)k * n + i) * n) + j) * 4;  // B_xi[k][i][j]
+    double2 d1[2], d2[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const double2 a = __ldg(x1 + h), b = __ldg(x1 + h + 2), c = __ldg(x2 + h), e = __ldg(x2 + h + 2);
+      d1[h] = make_double2(a.x - b.x, a.y - b.y);
+      d2[h] = make_double2(c.x - e.x, c.y - e.y);
+    }
+    const double2* yv = By + ((long long)iy0 * n3 + (((long long)i * n + j) * n) + k) * 4;  // B_eta[i][j][k]
+#pragma unroll
+    for (int y = 0; y < CT_NY; y++) {
+      if (iy0 + y >= ny) break;
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        const double2 a = __ldg(yv + (long long)y * n3 * 4 + h), b = __ldg(yv + (long long)y * n3 * 4 + h + 2);
+        const double2 u = make_double2(a.x + b.x, a.y + b.y);
+        acc[y][0] = fma(d1[h].x, u.x, fma(-d1[h].y, u.y, acc[y][0]));
+        acc[y][1] = fma(d1[h].x, u.y, fma(d1[h].y, u.x, acc[y][1]));
+        acc[y][2] = fma(d2[h].x, u.x, fma(-d2[h].y, u.y, acc[y][2]));
+        acc[y][3] = fma(d2[h].x, u.y, fma(d2[h].y, u.x, acc[y][3]));
       }
-      my[g] = make_double2(re, im);
-    }
-#pragma unroll
-    for (int g = 0; g < 4; g++) {
-      const double2 a = x1[g], b = x2[g];
-      w1r += a.x * my[g].x - a.y * my[g].y;
-      w1i += a.x * my[g].y + a.y * my[g].x;
-      w2r += b.x * my[g].x - b.y * my[g].y;
-      w2i += b.x * my[g].y + b.y * my[g].x;
     }
   }
-  __shared__ double sh[4][8];
-  double v[4] = {w1r, w1i, w2r, w2i};
+  __shared__ double sh[CT_NY * 4][CT * CT / 32];
 #pragma unroll
-  for (int q = 0; q < 4; q++)
+  for (int y = 0; y < CT_NY; y++)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-  if ((threadIdx.x & 31) == 0)
+    for (int q = 0; q < 4; q++) {
+      double v = acc[y][q];
 #pragma unroll
-    for (int q = 0; q < 4; q++) sh[q][threadIdx.x >> 5] = v[q];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if ((threadIdx.x & 31) == 0) sh[y * 4 + q][threadIdx.x >> 5] = v;
+    }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double r[4] = {0, 0, 0, 0};
-    for (int q = 0; q < 4; q++)
-      for (int w = 0; w < 8; w++) r[q] += sh[q][w];
-    W[(long long)blockIdx.x * 2] = make_double2(-r[0], -r[1]);
-    W[(long long)blockIdx.x * 2 + 1] = make_double2(-r[2], -r[3]);
+  if (threadIdx.x < CT_NY * 4) {
+    const int iy = iy0 + threadIdx.x / 4;
+    if (iy < ny) {
+      double r = 0.0;
+      for (int w = 0; w < CT * CT / 32; w++) r += sh[threadIdx.x][w];
+      part[(((long long)ix * ny + iy) * nsplit + sp) * 4 + threadIdx.x % 4] = r;
+    }
   }
+}
+
+// W[pair] = -(1/2) sum of the pair's nsplit parts, one warp per value, lanes then shuffles in a fixed
+// order.  part may be W itself when nsplit is 1.
+__global__ void __launch_bounds__(128) k_contract_sum(int nsplit, const double* part, double* W) {
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* p = part + (long long)blockIdx.x * nsplit * 4 + q;
+  double r = 0.0;
+  for (int k = lane; k < nsplit; k += 32) r += p[4LL * k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  if (lane == 0) W[(long long)blockIdx.x * 4 + q] = -0.5 * r;
 }
 
 // out[e] = (1/count) sum_j in[j * size + e], summed in j order (FP64).
@@ -479,7 +516,25 @@ extern "C" int lqcd_nucleon_contract(int n, int n_x, const double* B_xi, int n_y
     lq_set_error("nucleon_contract: bad arguments");
     return LQCD_EBADARG;
   }
-  k_nucleon_contract<<<(unsigned)(n_x * n_y), 256, 0, (cudaStream_t)stream>>>(n, n_y, (const double2*)B_xi,
-                                                                              (const double2*)B_eta, (double2*)W);
-  return launched_here();
+  cudaStream_t st = (cudaStream_t)stream;
+  // parts: about four blocks per SM over all pairs, no more than there are tiles
+  const long long ngy = (n_y + CT_NY - 1) / CT_NY, nt = (n + CT - 1) / CT;
+  long long nsplit = (152 * 4 + n_x * ngy - 1) / (n_x * ngy);
+  nsplit = std::max(1LL, std::min(nsplit, (long long)n * nt * nt));
+  void* scratch = nullptr;
+  if (nsplit > 1 && cudaMallocAsync(&scratch, sizeof(double) * 4 * (size_t)(n_x * (long long)n_y * nsplit), st) != cudaSuccess) {
+    cudaGetLastError();
+    scratch = nullptr;
+    nsplit = 1;  // no scratch to be had: one part per pair, summed in place
+  }
+  double* part = scratch ? (double*)scratch : W;
+  k_nucleon_contract<<<(unsigned)(n_x * ngy * nsplit), CT * CT, 0, st>>>(n, n_y, (int)nsplit, (const double2*)B_xi,
+                                                                         (const double2*)B_eta, part);
+  int rc = launched_here();
+  if (!rc) {
+    k_contract_sum<<<(unsigned)((long long)n_x * n_y), 128, 0, st>>>((int)nsplit, part, W);
+    rc = launched_here();
+  }
+  if (scratch) cudaFreeAsync(scratch, st);
+  return rc;
 }
