@@ -54,24 +54,26 @@ LQ_DI su3<double> mmd(const su3<double>& a, const su3<double>& b) {
     for (int j = 0; j < 3; j++) {
       cd t = {0, 0};
 #pragma unroll
-      for (int k = 0; k < 3; k++) t = t + a.m[i][k] * conj(b.m[j][k]);
+      for (int k = 0; k < 3; k++) fma_cc(t, b.m[j][k], a.m[i][k]);
       r.m[i][j] = t;
     }
   return r;
 }
 
-// a^dag * b
-LQ_DI su3<double> mdm(const su3<double>& a, const su3<double>& b) {
-  su3<double> r;
+// r - a^dag * b
+LQ_DI su3<double> sub_mdm(su3<double> r, const su3<double>& a, const su3<double>& b) {
 #pragma unroll
   for (int i = 0; i < 3; i++)
 #pragma unroll
-    for (int j = 0; j < 3; j++) {
-      cd t = {0, 0};
+    for (int j = 0; j < 3; j++)
 #pragma unroll
-      for (int k = 0; k < 3; k++) t = t + conj(a.m[k][i]) * b.m[k][j];
-      r.m[i][j] = t;
-    }
+      for (int k = 0; k < 3; k++) {  // r -= conj(a_ki) b_kj
+        cd& t = r.m[i][j];
+        t.re = fma(-a.m[k][i].re, b.m[k][j].re, t.re);
+        t.re = fma(-a.m[k][i].im, b.m[k][j].im, t.re);
+        t.im = fma(-a.m[k][i].re, b.m[k][j].im, t.im);
+        t.im = fma(a.m[k][i].im, b.m[k][j].re, t.im);
+      }
   return r;
 }
 
@@ -88,6 +90,9 @@ LQ_DI void nat_coords(const Geom& g, long long i, int x[4]) {
   x[0] = (int)(i / g.L[1]);
 }
 
+// max(a, b) that keeps a NaN of either
+LQ_DI double max_nan(double a, double b) { return a >= b ? a : (a == a ? b : a); }
+
 // ------------------------------------------------------------- link packing
 __global__ void k_pack_links(Geom g, const double2* U, double2* U64, float4* U32, uint2* U16,
                              unsigned long long* maxdev) {
@@ -100,21 +105,25 @@ __global__ void k_pack_links(Geom g, const double2* U, double2* U64, float4* U32
   double dev = 0.0;
   for (int mu = 0; mu < 4; mu++) {
     su3<double> u = ld_nat(U, i, mu);
-    // unitarity: |U U^dag - 1|, |det U - 1|
-    su3<double> uu = mmd(u, u);
+    // unitarity: |U U^dag - 1| (Hermitian: the upper triangle), |det U - 1|; the largest of the
+    // squares, one root at the end
 #pragma unroll
     for (int a = 0; a < 3; a++)
 #pragma unroll
-      for (int b = 0; b < 3; b++) {
-        cd e = uu.m[a][b];
-        if (a == b) e.re -= 1.0;
-        dev = fmax(dev, sqrt(norm2(e)));
+      for (int b = a; b < 3; b++) {
+        cd e = {a == b ? -1.0 : 0.0, 0.0};
+#pragma unroll
+        for (int k = 0; k < 3; k++) fma_cc(e, u.m[b][k], u.m[a][k]);
+        dev = max_nan(dev, norm2(e));
       }
-    cd det = u.m[0][0] * (u.m[1][1] * u.m[2][2] - u.m[1][2] * u.m[2][1]) -
-             u.m[0][1] * (u.m[1][0] * u.m[2][2] - u.m[1][2] * u.m[2][0]) +
-             u.m[0][2] * (u.m[1][0] * u.m[2][1] - u.m[1][1] * u.m[2][0]);
-    det.re -= 1.0;
-    dev = fmax(dev, sqrt(norm2(det)));
+    cd det = {-1.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+      const cd minor = u.m[1][k1] * u.m[2][k2] - u.m[1][k2] * u.m[2][k1];
+      fma_c(det, u.m[0][k], minor);
+    }
+    dev = max_nan(dev, norm2(det));
     const long long base = (long long)(p * 4 + mu);
 #pragma unroll
     for (int k = 0; k < 9; k++) U64[(base * 9 + k) * g.Vh + cb] = make_double2(u.m[k / 3][k % 3].re, u.m[k / 3][k % 3].im);
@@ -132,6 +141,7 @@ __global__ void k_pack_links(Geom g, const double2* U, double2* U64, float4* U32
       U16[(base * 3 + k) * g.Vh + cb] = make_uint2(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1));
     }
   }
+  dev = sqrt(dev);
   if (!(dev == dev)) dev = 1e300;  // NaN counts as non-unitary
   atomicMax(maxdev, (unsigned long long)__double_as_longlong(dev));
 }
@@ -151,13 +161,23 @@ LQ_DI su3<double> link_bc(const Geom& g, const double2* U, const int x[4], int m
 
 LQ_DI void shift(const Geom& g, const int x[4], int mu, int d, int y[4]) {
 #pragma unroll
-  for (int k = 0; k < 4; k++) y[k] = x[k];
-  y[mu] += d;
-  if (y[mu] < 0) y[mu] += g.L[mu];
-  if (y[mu] >= g.L[mu]) y[mu] -= g.L[mu];
+  for (int k = 0; k < 4; k++) {  // (no indexing by mu: the coordinates stay in registers)
+    int v = x[k] + (k == mu ? d : 0);
+    if (v < 0) v += g.L[k];
+    if (v >= g.L[k]) v -= g.L[k];
+    y[k] = v;
+  }
 }
 
-// Fhat_mu_nu(x) = (Q - Q^dag)/8, Q = sum of the 4 leaves at x (mu -> nu).
+// Fhat_mu_nu(x) = (Q - Q^dag)/8, Q = sum of the 4 leaves at x (mu -> nu):
+//   L1 = U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag,
+//   L2 = U_nu(x) U_mu(x+nu-mu)^dag U_nu(x-mu)^dag U_mu(x-mu),
+//   L3 = U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_nu(x-nu),
+//   L4 = U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu) U_mu(x)^dag.
+// Q - Q^dag = M - M^dag with L3, L4 replaced by -L3^dag, -L4^dag, which pairs the leaves on a
+// common outer link: ten products a plane instead of twelve.
+//   M = U_mu(x) { U_nu(x+mu) [U_nu(x) U_mu(x+nu)]^dag - [U_mu(x-nu) U_nu(x-nu+mu)]^dag U_nu(x-nu) }
+//     + { U_nu(x) [U_nu(x-mu) U_mu(x-mu+nu)]^dag - [U_mu(x-mu-nu) U_nu(x-nu)]^dag U_nu(x-mu-nu) } U_mu(x-mu)
 LQ_DI su3<double> fhat(const Geom& g, const double2* U, const int x[4], int mu, int nu) {
   int xpm[4], xpn[4], xmm[4], xmn[4], xmmpn[4], xmmmn[4], xmnpm[4];
   shift(g, x, mu, 1, xpm);
@@ -167,36 +187,39 @@ LQ_DI su3<double> fhat(const Geom& g, const double2* U, const int x[4], int mu, 
   shift(g, xmm, nu, 1, xmmpn);
   shift(g, xmm, nu, -1, xmmmn);
   shift(g, xmn, mu, 1, xmnpm);
-  // leaf 1: U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-  su3<double> q = mmd(mmd(mm(link_bc(g, U, x, mu), link_bc(g, U, xpm, nu)), link_bc(g, U, xpn, mu)), link_bc(g, U, x, nu));
-  // leaf 2: U_nu(x) U_mu(x+nu-mu)^dag U_nu(x-mu)^dag U_mu(x-mu)
-  su3<double> l2 =
-      mm(mmd(mmd(link_bc(g, U, x, nu), link_bc(g, U, xmmpn, mu)), link_bc(g, U, xmm, nu)), link_bc(g, U, xmm, mu));
-  // leaf 3: U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_nu(x-nu)
-  //        = [U_nu(x-mu-nu) U_mu(x-mu)]^dag U_mu(x-mu-nu) U_nu(x-nu)
-  su3<double> l3 = mm(mdm(mm(link_bc(g, U, xmmmn, nu), link_bc(g, U, xmm, mu)), link_bc(g, U, xmmmn, mu)),
-                      link_bc(g, U, xmn, nu));
-  // leaf 4: U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu) U_mu(x)^dag
-  su3<double> l4 = mmd(mm(mdm(link_bc(g, U, xmn, nu), link_bc(g, U, xmn, mu)), link_bc(g, U, xmnpm, nu)), link_bc(g, U, x, mu));
+  su3<double> q;
+  {
+    const su3<double> un = link_bc(g, U, xmn, nu);
+    su3<double> t = mmd(link_bc(g, U, xpm, nu), mm(link_bc(g, U, x, nu), link_bc(g, U, xpn, mu)));
+    t = sub_mdm(t, mm(link_bc(g, U, xmn, mu), link_bc(g, U, xmnpm, nu)), un);
+    q = mm(link_bc(g, U, x, mu), t);
+    t = mmd(link_bc(g, U, x, nu), mm(link_bc(g, U, xmm, nu), link_bc(g, U, xmmpn, mu)));
+    t = sub_mdm(t, mm(link_bc(g, U, xmmmn, mu), un), link_bc(g, U, xmmmn, nu));
+    const su3<double> um = link_bc(g, U, xmm, mu);
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+      for (int b = 0; b < 3; b++)
+#pragma unroll
+        for (int k = 0; k < 3; k++) fma_c(q.m[a][b], t.m[a][k], um.m[k][b]);
+  }
   su3<double> f;
 #pragma unroll
   for (int a = 0; a < 3; a++)
 #pragma unroll
-    for (int b = 0; b < 3; b++) {
-      cd t = q.m[a][b] + l2.m[a][b] + l3.m[a][b] + l4.m[a][b];
-      cd tt = q.m[b][a] + l2.m[b][a] + l3.m[b][a] + l4.m[b][a];
-      f.m[a][b] = 0.125 * (t - conj(tt));
-    }
+    for (int b = 0; b < 3; b++) f.m[a][b] = 0.125 * (q.m[a][b] - conj(q.m[b][a]));
   return f;
 }
-
 
 // Pack the 6x6 Hermitian block B into 36 reals: 6 diagonal, then the 15
 // entries below the diagonal row by row.
 LQ_DI void pack_herm6(const cd B[6][6], double out[36]) {
+#pragma unroll
   for (int r = 0; r < 6; r++) out[r] = B[r][r].re;
   int q = 6;
+#pragma unroll
   for (int r = 1; r < 6; r++)
+#pragma unroll
     for (int c = 0; c < r; c++) {
       // Hermitian part of the pair (r,c), (c,r)
       out[q] = 0.5 * (B[r][c].re + B[c][r].re);
@@ -205,107 +228,164 @@ LQ_DI void pack_herm6(const cd B[6][6], double out[36]) {
     }
 }
 
-// Gauss-Jordan inversion with partial pivoting (6x6 complex).  Returns
-// false for a singular block.
-LQ_DI bool invert6(const cd B[6][6], cd R[6][6]) {
-  cd M[6][12];
-  for (int r = 0; r < 6; r++)
-    for (int c = 0; c < 6; c++) {
-      M[r][c] = B[r][c];
-      M[r][6 + c] = {r == c ? 1.0 : 0.0, 0.0};
-    }
+// In-place Gauss-Jordan inversion with partial pivoting (6x6 complex), all indices static so that
+// the block stays in registers (row swaps are selects).  Returns false for a singular block.
+LQ_DI bool invert6(cd (&M)[6][6]) {
+  int piv[6];
+  bool ok = true;
+#pragma unroll
   for (int col = 0; col < 6; col++) {
-    int piv = col;
+    int p = col;
     double best = norm2(M[col][col]);
+#pragma unroll
     for (int r = col + 1; r < 6; r++) {
-      double v = norm2(M[r][col]);
+      const double v = norm2(M[r][col]);
       if (v > best) {
         best = v;
-        piv = r;
+        p = r;
       }
     }
-    if (!(best > 0.0)) return false;
-    if (piv != col)
-      for (int c = 0; c < 12; c++) {
-        cd t = M[col][c];
-        M[col][c] = M[piv][c];
-        M[piv][c] = t;
+    piv[col] = p;
+    if (!(best > 0.0)) ok = false;
+#pragma unroll
+    for (int r = col + 1; r < 6; r++) {
+      const bool sw = r == p;
+#pragma unroll
+      for (int c = 0; c < 6; c++) {
+        const cd a = M[col][c], b = M[r][c];
+        M[col][c] = {sw ? b.re : a.re, sw ? b.im : a.im};
+        M[r][c] = {sw ? a.re : b.re, sw ? a.im : b.im};
       }
-    cd d = M[col][col];
-    double dn = norm2(d);
-    cd inv = {d.re / dn, -d.im / dn};
-    for (int c = 0; c < 12; c++) M[col][c] = M[col][c] * inv;
+    }
+    const cd d = M[col][col];
+    const double dn = norm2(d);
+    const cd inv = {d.re / dn, -d.im / dn};
+    M[col][col] = {1.0, 0.0};
+#pragma unroll
+    for (int c = 0; c < 6; c++) M[col][c] = M[col][c] * inv;
+#pragma unroll
     for (int r = 0; r < 6; r++) {
       if (r == col) continue;
-      cd f = M[r][col];
-      if (f.re == 0.0 && f.im == 0.0) continue;
-      for (int c = 0; c < 12; c++) M[r][c] = M[r][c] - f * M[col][c];
+      const cd mf = {-M[r][col].re, -M[r][col].im};
+      M[r][col] = {0.0, 0.0};
+#pragma unroll
+      for (int c = 0; c < 6; c++) fma_c(M[r][c], mf, M[col][c]);
     }
   }
-  for (int r = 0; r < 6; r++)
-    for (int c = 0; c < 6; c++) R[r][c] = M[r][6 + c];
-  return true;
+  // undo the row swaps on the columns, last first
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    const int col = 5 - k;
+#pragma unroll
+    for (int c = col + 1; c < 6; c++) {
+      const bool sw = c == piv[col];
+#pragma unroll
+      for (int r = 0; r < 6; r++) {
+        const cd a = M[r][col], b = M[r][c];
+        M[r][col] = {sw ? b.re : a.re, sw ? b.im : a.im};
+        M[r][c] = {sw ? a.re : b.re, sw ? a.im : b.im};
+      }
+    }
+  }
+  return ok;
 }
 
-__global__ void k_clover(Geom g, const double2* U, double kappa, double csw, double2* A64, double2* Ai64, float4* A32,
-                         float4* Ai32, int* fail) {
+// i Fhat of one plane per thread (Hermitian: 3 real diagonal entries, then the entries (1,0), (2,0),
+// (2,1)), planes 0-2 = (0,1) (0,2) (0,3), 3-5 = (2,3) (3,1) (1,2), into G[plane * 9 + k][site].
+//
+// Bound by the FP64 pipe (10 products a plane, 6480 multiply-adds a site); a thread a plane keeps the
+// matrices in registers, where one thread for the whole site spilled 1.7 KB.  24^3 x 48, with
+// k_clover_blocks: 20.6 ms with twelve products a plane, products without fused multiply-adds, an
+// augmented elimination and all in one thread; 8.9 ms so.
+__global__ void __launch_bounds__(128) k_fhat(Geom g, const double2* U, double* G) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2 * g.Vh) return;
+  const long long V = 2LL * g.Vh;
+  if (i >= V) return;
   int x[4];
   nat_coords(g, i, x);
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-  const long long cb = i >> 1;
-  const long long Vh = g.Vh;
-  const double d = 1.0 / (2.0 * kappa);
-  su3<double> E[3], M[3];
-  if (csw != 0.0) {
-    for (int l = 0; l < 3; l++) E[l] = fhat(g, U, x, 0, l + 1);
-    M[0] = fhat(g, U, x, 2, 3);
-    M[1] = fhat(g, U, x, 3, 1);
-    M[2] = fhat(g, U, x, 1, 2);
+  const int pl = blockIdx.y;
+  const int mu = pl < 3 ? 0 : (pl == 3 ? 2 : pl == 4 ? 3 : 1);
+  const int nu = pl < 3 ? pl + 1 : (pl == 3 ? 3 : pl == 4 ? 1 : 2);
+  const su3<double> f = fhat(g, U, x, mu, nu);
+  double* out = G + (long long)pl * 9 * V + (long long)p * g.Vh + (i >> 1);
+#pragma unroll
+  for (int a = 0; a < 3; a++) out[a * V] = -f.m[a][a].im;
+  const int ra[3] = {1, 2, 2}, rb[3] = {0, 0, 1};
+#pragma unroll
+  for (int k = 0; k < 3; k++) {  // i f
+    out[(3 + 2 * k) * V] = -f.m[ra[k]][rb[k]].im;
+    out[(4 + 2 * k) * V] = f.m[ra[k]][rb[k]].re;
   }
-  for (int blk = 0; blk < 2; blk++) {
-    const double sg = blk == 0 ? 1.0 : -1.0;
-    cd H[3][3][3];
-    for (int l = 0; l < 3; l++)
-      for (int a = 0; a < 3; a++)
-        for (int b = 0; b < 3; b++) {
-          if (csw == 0.0) {
-            H[l][a][b] = {0.0, 0.0};
-          } else {
-            cd t = sg * E[l].m[a][b] - M[l].m[a][b];
-            H[l][a][b] = (0.5 * csw) * ti(t);  // c_sw (i/2) (+-E_l - M_l)
-          }
-        }
-    cd B[6][6];
-    for (int a = 0; a < 3; a++)
-      for (int b = 0; b < 3; b++) {
-        cd dd = {a == b ? d : 0.0, 0.0};
-        B[a][b] = dd + H[2][a][b];
-        B[3 + a][3 + b] = dd - H[2][a][b];
-        B[a][3 + b] = H[0][a][b] - ti(H[1][a][b]);
-        B[3 + a][b] = H[0][a][b] + ti(H[1][a][b]);
+}
+
+// The two clover blocks B+- = 1/(2 kappa) + sum_l s_l (x) H+-_l, H+-_l = (c_sw/2)(+-i E_l - i M_l), from G,
+// and their inverses on even sites; one thread per (site, block).
+__global__ void __launch_bounds__(128) k_clover_blocks(Geom g, const double* G, double kappa, double csw, double2* A64,
+                                                       double2* Ai64, float4* A32, float4* Ai32, int* fail) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long Vh = g.Vh, V = 2 * Vh;
+  if (q >= V) return;
+  const int p = q >= Vh;
+  const long long cb = q - p * Vh;
+  const int blk = blockIdx.y;
+  const double d = 1.0 / (2.0 * kappa);
+  cd H[3][3][3];
+#pragma unroll
+  for (int l = 0; l < 3; l++) {
+    double h[9];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+      if (csw == 0.0) {
+        h[k] = 0.0;
+      } else {
+        const double e = G[(l * 9 + k) * V + q], m = G[((3 + l) * 9 + k) * V + q];
+        h[k] = (0.5 * csw) * (blk == 0 ? e - m : -e - m);
       }
-    double pk[36];
-    pack_herm6(B, pk);
-    for (int k = 0; k < 18; k++) A64[((long long)p * 36 + blk * 18 + k) * Vh + cb] = make_double2(pk[2 * k], pk[2 * k + 1]);
-    for (int k = 0; k < 9; k++)
-      A32[((long long)p * 18 + blk * 9 + k) * Vh + cb] =
-          make_float4((float)pk[4 * k], (float)pk[4 * k + 1], (float)pk[4 * k + 2], (float)pk[4 * k + 3]);
-    if (p == 0) {
-      cd R[6][6];
-      if (!invert6(B, R)) {
-        atomicExch(fail, 1);
-        for (int r = 0; r < 6; r++)
-          for (int c = 0; c < 6; c++) R[r][c] = {0.0, 0.0};
-      }
-      pack_herm6(R, pk);
-      for (int k = 0; k < 18; k++) Ai64[((long long)blk * 18 + k) * Vh + cb] = make_double2(pk[2 * k], pk[2 * k + 1]);
-      for (int k = 0; k < 9; k++)
-        Ai32[((long long)blk * 9 + k) * Vh + cb] =
-            make_float4((float)pk[4 * k], (float)pk[4 * k + 1], (float)pk[4 * k + 2], (float)pk[4 * k + 3]);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++) H[l][a][a] = {h[a], 0.0};
+    const int ra[3] = {1, 2, 2}, rb[3] = {0, 0, 1};
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      H[l][ra[k]][rb[k]] = {h[3 + 2 * k], h[4 + 2 * k]};
+      H[l][rb[k]][ra[k]] = {h[3 + 2 * k], -h[4 + 2 * k]};
     }
   }
+  cd B[6][6];
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int b = 0; b < 3; b++) {
+      const cd dd = {a == b ? d : 0.0, 0.0};
+      B[a][b] = dd + H[2][a][b];
+      B[3 + a][3 + b] = dd - H[2][a][b];
+      B[a][3 + b] = H[0][a][b] - ti(H[1][a][b]);
+      B[3 + a][b] = H[0][a][b] + ti(H[1][a][b]);
+    }
+  double pk[36];
+  pack_herm6(B, pk);
+#pragma unroll
+  for (int k = 0; k < 18; k++) A64[((long long)p * 36 + blk * 18 + k) * Vh + cb] = make_double2(pk[2 * k], pk[2 * k + 1]);
+#pragma unroll
+  for (int k = 0; k < 9; k++)
+    A32[((long long)p * 18 + blk * 9 + k) * Vh + cb] =
+        make_float4((float)pk[4 * k], (float)pk[4 * k + 1], (float)pk[4 * k + 2], (float)pk[4 * k + 3]);
+  if (p != 0) return;
+  if (!invert6(B)) {
+    atomicExch(fail, 1);
+#pragma unroll
+    for (int r = 0; r < 6; r++)
+#pragma unroll
+      for (int c = 0; c < 6; c++) B[r][c] = {0.0, 0.0};
+  }
+  pack_herm6(B, pk);
+#pragma unroll
+  for (int k = 0; k < 18; k++) Ai64[((long long)blk * 18 + k) * Vh + cb] = make_double2(pk[2 * k], pk[2 * k + 1]);
+#pragma unroll
+  for (int k = 0; k < 9; k++)
+    Ai32[((long long)blk * 9 + k) * Vh + cb] =
+        make_float4((float)pk[4 * k], (float)pk[4 * k + 1], (float)pk[4 * k + 2], (float)pk[4 * k + 3]);
 }
 
 }  // namespace lq
@@ -322,7 +402,19 @@ int lq_launch_pack_links(const lq::Geom& g, const double2* U, double2* U64, floa
 int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, double2* A64, double2* Ai64,
                      float4* A32, float4* Ai32, int* fail, cudaStream_t st) {
   const long long V = 2 * g.Vh;
-  lq::k_clover<<<(unsigned)((V + 63) / 64), 64, 0, st>>>(g, U, kappa, csw, A64, Ai64, A32, Ai32, fail);
+  double* G = nullptr;
+  if (csw != 0.0) {
+    if (cudaMallocAsync((void**)&G, sizeof(double) * 54 * V, st) != cudaSuccess) {
+      cudaGetLastError();
+      lq_set_error("set_gauge: device allocation of the clover scratch failed");
+      return LQCD_ENOMEM;
+    }
+    lq::k_fhat<<<dim3((unsigned)((V + 127) / 128), 6), 128, 0, st>>>(g, U, G);
+    lq_count_launch();
+  }
+  lq::k_clover_blocks<<<dim3((unsigned)((V + 127) / 128), 2), 128, 0, st>>>(g, G, kappa, csw, A64, Ai64, A32, Ai32,
+                                                                          fail);
   lq_count_launch();
+  if (G) cudaFreeAsync(G, st);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
