@@ -75,9 +75,8 @@ METRIC = "s per 12-source factorized propagator @ res 1e-10 (Dslash HBM GB/s vs 
 UNIT = "s/propagator"
 # kernels of one BiCGStab iteration as lqcd_stencil_bench numbers them, with their launches per iteration
 HOP_KERNELS = {1: ("k_hop_clinv (A_ee^-1 D_hop, first half of D^)", 2), 2: ("k_hop_lin + <r0,v>", 1),
-               3: ("k_hop_lin + <t,s>, |t|^2", 1)}
-BLAS_KERNELS = {4: ("k_bicg_s_w (s = r - alpha v)", 1), 5: ("k_bicg_xr_w (x, r update + 2 dots)", 1),
-                6: ("k_bicg_p_w (p update)", 1)}
+               3: ("k_hop_lin + <t,s>, |t|^2, <r0,t>, <r0,s>", 1)}
+BLAS_KERNELS = {4: ("k_bicg_s_w (s = r - alpha v)", 1), 5: ("k_bicg_xrp_w (x, r, p update + |r|^2)", 1)}
 DTYPE = {64: "f64", 32: "f32+f64", 16: "f16+f32+f64"}
 
 

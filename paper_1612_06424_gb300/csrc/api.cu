@@ -102,7 +102,7 @@ int check_lat(const lqcd_lattice* L) {
 // A batch with its own descriptor / flag / scalar / partial storage.
 struct BatchStore {
   Batch b;
-  DBuf sys, active, sc, partial;
+  DBuf sys, active, sc, partial, count;
   std::vector<lq::SysDesc> h_sys;
   std::vector<lq::SolverScal> h_sc;
   std::vector<int> h_active;
@@ -140,7 +140,8 @@ struct BatchStore {
     for (int k = 0; k < n; k++)
       if ((doms[k].t1 - doms[k].t0 + 1) % 4 != 0) b.tblk_ok = 0;
     b.nby = (int)((maxn + LQ_BLOCK - 1) / LQ_BLOCK);
-    b.pstride = (int)((12 * maxn + LQ_BLOCK - 1) / LQ_BLOCK);
+    // four doubles per block of the vector kernels, eight per 64-site block of the stencil's RED_TSW
+    b.pstride = (int)std::max((12 * maxn + LQ_BLOCK - 1) / LQ_BLOCK, 2 * ((maxn + 63) / 64));
     if ((long long)n * b.pstride >= (1LL << 31)) {
       lq_set_error("batch too large for one grid (systems x blocks per system >= 2^31)");
       return LQCD_EBADARG;
@@ -149,11 +150,14 @@ struct BatchStore {
     RC(active.alloc(sizeof(int) * n, st));
     RC(sc.alloc(sizeof(lq::SolverScal) * n, st));
     RC(partial.alloc(sizeof(double) * 4 * (size_t)n * b.pstride, st));
+    RC(count.alloc(sizeof(unsigned) * n, st));
+    CK(cudaMemsetAsync(count.p, 0, sizeof(unsigned) * n, st));
     CK(cudaMemcpyAsync(sys.p, h_sys.data(), sizeof(lq::SysDesc) * n, cudaMemcpyHostToDevice, st));
     b.sys = sys.as<lq::SysDesc>();
     b.active = active.as<int>();
     b.sc = sc.as<lq::SolverScal>();
     b.partial = partial.as<double>();
+    b.count = count.as<unsigned>();
     h_sc.assign(n, lq::SolverScal{});
     h_active.assign(n, 1);
     CK(cudaMemcpyAsync(sc.p, h_sc.data(), sizeof(lq::SolverScal) * n, cudaMemcpyHostToDevice, st));
@@ -385,18 +389,14 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
       // check that follows decides (0.5 tol measured 2.8% faster than 0.3 tol on the 48^3 x 96
       // factorized propagator, worst final residual 8.5e-11)
       RC(lq_finalize(lq::FIN_INIT, b, tau * tau, 0.25 * tol * tol, lq_words_per_site(P), st));
-      // one BiCGStab iteration: 10 kernels, all scalars and flags on the device
+      // one BiCGStab iteration: 6 kernels, all scalars and flags on the device
       auto iteration = [&](cudaStream_t s_) -> int {
         RC(lq_hop_clinv(P, dag, clov, L, b, p, none, te, 1.0, 0.0, s_));
-        RC(lq_hop_lin(P, dag, clov, lq::RED_DOT_W, L, b, 1, te, p, none, r0, v, -0.25, 1.0, 0.0, s_));
-        RC(lq_finalize(lq::FIN_ALPHA, b, 0, 0, lq_hop_wps(P, b), s_));
+        RC(lq_hop_lin(P, dag, clov, lq::RED_DOT_W, L, b, 1, te, p, none, r0, v, -0.25, 1.0, 0.0, s_, lq::FIN_ALPHA));
         RC(lq_bicg_s(P, b, r, v, s, s_));
         RC(lq_hop_clinv(P, dag, clov, L, b, s, none, te, 1.0, 0.0, s_));
-        RC(lq_hop_lin(P, dag, clov, lq::RED_TS, L, b, 1, te, s, none, none, t, -0.25, 1.0, 0.0, s_));
-        RC(lq_finalize(lq::FIN_OMEGA, b, 0, 0, lq_hop_wps(P, b), s_));
-        RC(lq_bicg_xr(P, b, xs, p, s, t, r, r0, s_));
-        RC(lq_finalize(lq::FIN_BETA, b, 0, 0, lq_words_per_site(P), s_));
-        RC(lq_bicg_p(P, b, p, r, v, s_));
+        RC(lq_hop_lin(P, dag, clov, lq::RED_TSW, L, b, 1, te, s, none, r0, t, -0.25, 1.0, 0.0, s_, lq::FIN_OMEGA_BETA));
+        RC(lq_bicg_xrp(P, b, xs, p, s, t, v, r, s_, lq::FIN_STOP));
         return 0;
       };
       if (use_graph && budget >= 2 * check_every) {
@@ -1825,15 +1825,13 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
       case 2:  // v = A_oo p - 1/4 D_hop te, with <r0, v>
         return lq_hop_lin(precision, false, clov, lq::RED_DOT_W, L, b, 1, q.v(0), q.v(1), none, q.v(3), q.v(2),
                           -0.25, 1.0, 0.0, st);
-      case 3:  // t = A_oo s - 1/4 D_hop te, with <t, s> and |t|^2
-        return lq_hop_lin(precision, false, clov, lq::RED_TS, L, b, 1, q.v(0), q.v(1), none, none, q.v(2), -0.25,
+      case 3:  // t = A_oo s - 1/4 D_hop te, with <t, s>, |t|^2, <r0, t> and <r0, s>
+        return lq_hop_lin(precision, false, clov, lq::RED_TSW, L, b, 1, q.v(0), q.v(1), none, q.v(3), q.v(2), -0.25,
                           1.0, 0.0, st);
       case 4:  // s = r - alpha v
         return lq_bicg_s(precision, b, q.v(0), q.v(1), q.v(2), st);
-      case 5:  // x += alpha p + omega s, r = s - omega t, <r0, r>, |r|^2
-        return lq_bicg_xr(precision, b, q.v(2), q.v(0), q.v(1), q.v(4), q.v(5), q.v(3), st);
-      default:  // p = r + beta (p - omega v)
-        return lq_bicg_p(precision, b, q.v(2), q.v(0), q.v(1), st);
+      default:  // x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2
+        return lq_bicg_xrp(precision, b, q.v(2), q.v(0), q.v(1), q.v(4), q.v(3), q.v(5), st);
     }
   };
   for (int w = 0; w < 3; w++) RC(launch());
@@ -1854,7 +1852,7 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
   const double S = precision == 64 ? 192.0 : precision == 32 ? 96.0 : 52.0;
   const double Lk = precision == 64 ? 144.0 : precision == 32 ? 48.0 : 24.0;
   const double C = clov ? (precision == 64 ? 576.0 : 288.0) : 0.0;
-  static const double passes[7] = {3, 2, 4, 3, 3, 7, 4};
+  static const double passes[7] = {3, 2, 4, 4, 3, 8, 8};
   double bytes = 0.0, sites = 0.0;
   std::vector<std::vector<char>> used(L->fields.size(), std::vector<char>(L->dims[0], 0));
   for (int k = 0; k < n_sys; k++) {
@@ -1869,7 +1867,7 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
   // flop per system site: hop 1320, site-diagonal block 504 (clover) or 24, epilogue and reductions
   const double diag = clov ? 504.0 : 24.0;
   const double flop[7] = {1320.0 + diag + 72.0, 1320.0 + diag + 24.0, 1320.0 + diag + 72.0 + 96.0,
-                          1320.0 + diag + 72.0 + 144.0, 96.0, 432.0, 192.0};
+                          1320.0 + diag + 72.0 + 336.0, 96.0, 528.0, 528.0};
   const double fl = sites * flop[kernel];
   if (ms_per_launch) *ms_per_launch = ms / reps;
   if (bytes_per_launch) *bytes_per_launch = bytes;

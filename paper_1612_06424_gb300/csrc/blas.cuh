@@ -12,9 +12,8 @@
 // Inner products accumulate per thread and per warp in the kernel's own
 // precision (FP32 for the FP32 / FP16 solver: FP64 arithmetic is a small
 // fraction of the FP32 rate on this GPU), then in FP64 across the warps of a
-// block and across blocks; `k_finalize` sums a system's block partials in a
-// fixed order, so every result is deterministic for a given launch shape.  `wps` (words per site) tells the finalize how many blocks the
-// producing kernel used per system.
+// block and across blocks; a system's block partials are summed in a fixed order
+// (finalize.cuh), so every result is deterministic for a given launch shape.
 #pragma once
 
 #include "dslash.cuh"
@@ -119,99 +118,89 @@ __global__ void __launch_bounds__(128) k_bicg_s_h(VecArgs va, const void* r, con
   Prec<16>::store(sys_ptr_w<16>(so, sd.off), nrm_ptr_w(son, sd.off), sd.n, j, a);
 }
 
-// ------------------- x += alpha p + omega s ; r = s - omega t ; <r0,r>, |r|^2
+// ------- x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v) ; |r|^2
+// One pass over the five vectors: beta is known beforehand (FIN_OMEGA_BETA takes <r0, r> from <r0, s>
+// and <r0, t>).  8 vector passes against 11 for an x, r update followed by a p update, for one more
+// (r0) in the stencil before it.
+//
+// Words per thread: two independent words keep more loads in flight and halve the partials.
+constexpr int XRP_WPT = 2;
+
 template <int P>
-__global__ void __launch_bounds__(128) k_bicg_xr_w(VecArgs va, void* x, const void* p, const void* sv, const void* t,
-                                                   void* r, const void* r0) {
+__global__ void __launch_bounds__(128) k_bicg_xrp_w(VecArgs va, FinArgs fin, void* x, void* p, const void* sv,
+                                                    const void* t, const void* v, void* r) {
   typedef Word<P> W;
   typedef typename W::R R;
-  LQ_WORD_PROLOGUE(P)
-  R red[3] = {0, 0, 0};
-  if (valid) {
-    const cx<R> al = c_of<R>(va.sc[s].alpha), om = c_of<R>(va.sc[s].omega);
-    cx<R> xv[W::NC], pv[W::NC], sv_[W::NC], tv[W::NC], w[W::NC];
-    W::get(wptr<P>(x, sd.off), i, xv);
-    W::get(wptr<P>(p, sd.off), i, pv);
-    W::get(wptr<P>(sv, sd.off), i, sv_);
-    W::get(wptr<P>(t, sd.off), i, tv);
-    W::get(wptr<P>(r0, sd.off), i, w);
+  int s, by;
+  grid_pos(va.nsys, s, by);
+  if (va.active && !va.active[s]) return;
+  const SysDesc sd = va.sys[s];
+  const int nw = sd.n * Prec<P>::NV;
+  constexpr int BW = 128 * XRP_WPT;  // words per block
+  if (by * BW >= nw) return;
+  const cx<R> al = c_of<R>(va.sc[s].alpha), om = c_of<R>(va.sc[s].omega), be = c_of<R>(va.sc[s].beta);
+  R red[1] = {0};
+  cx<R> xv[XRP_WPT][W::NC], pv[XRP_WPT][W::NC], sw[XRP_WPT][W::NC], tv[XRP_WPT][W::NC], vv[XRP_WPT][W::NC];
 #pragma unroll
-    for (int k = 0; k < W::NC; k++) {
-      xv[k] = xv[k] + al * pv[k] + om * sv_[k];
-      sv_[k] = sv_[k] - om * tv[k];
-    }
-    W::put(wptr_w<P>(x, sd.off), i, xv);
-    W::put(wptr_w<P>(r, sd.off), i, sv_);
-#pragma unroll
-    for (int k = 0; k < W::NC; k++) {
-      red[0] += w[k].re * sv_[k].re + w[k].im * sv_[k].im;
-      red[1] += w[k].re * sv_[k].im - w[k].im * sv_[k].re;
-      red[2] += sv_[k].re * sv_[k].re + sv_[k].im * sv_[k].im;
-    }
+  for (int u = 0; u < XRP_WPT; u++) {
+    const int i = by * BW + u * 128 + threadIdx.x;
+    if (i >= nw) continue;
+    W::get(wptr<P>(x, sd.off), i, xv[u]);
+    W::get(wptr<P>(p, sd.off), i, pv[u]);
+    W::get(wptr<P>(sv, sd.off), i, sw[u]);
+    W::get(wptr<P>(t, sd.off), i, tv[u]);
+    W::get(wptr<P>(v, sd.off), i, vv[u]);
   }
-  block_reduce_store<3, R>(red, va.partial + ((long long)s * va.pstride + by) * 4);
+#pragma unroll
+  for (int u = 0; u < XRP_WPT; u++) {
+    const int i = by * BW + u * 128 + threadIdx.x;
+    if (i >= nw) continue;
+#pragma unroll
+    for (int k = 0; k < W::NC; k++) {
+      xv[u][k] = xv[u][k] + al * pv[u][k] + om * sw[u][k];
+      sw[u][k] = sw[u][k] - om * tv[u][k];
+      pv[u][k] = sw[u][k] + be * (pv[u][k] - om * vv[u][k]);
+      red[0] += sw[u][k].re * sw[u][k].re + sw[u][k].im * sw[u][k].im;
+    }
+    W::put(wptr_w<P>(x, sd.off), i, xv[u]);
+    W::put(wptr_w<P>(r, sd.off), i, sw[u]);
+    W::put(wptr_w<P>(p, sd.off), i, pv[u]);
+  }
+  double* part = va.partial + (long long)s * va.pstride * 4;
+  block_reduce_store<1, R>(red, part + (long long)by * 4 + 2);
+  if (fin.mode != FIN_NONE) finish_last<1, 2, 4>(fin, part, (nw + BW - 1) / BW, s);
 }
 
-__global__ void __launch_bounds__(128) k_bicg_xr_h(VecArgs va, void* x, float* xn, const void* p, const float* pn,
-                                                   const void* sv, const float* svn, const void* t, const float* tn,
-                                                   void* r, float* rn, const void* r0, const float* r0n) {
+__global__ void __launch_bounds__(128) k_bicg_xrp_h(VecArgs va, FinArgs fin, void* x, float* xn, void* p, float* pn,
+                                                    const void* sv, const float* svn, const void* t, const float* tn,
+                                                    const void* v, const float* vn, void* r, float* rn) {
   LQ_SITE_PROLOGUE
-  float red[3] = {0.f, 0.f, 0.f};
+  float red[1] = {0.f};
   if (valid) {
-    const cx<float> al = c_of<float>(va.sc[s].alpha), om = c_of<float>(va.sc[s].omega);
-    cx<float> xv[12], pv[12], sv_[12], tv[12];
+    const cx<float> al = c_of<float>(va.sc[s].alpha), om = c_of<float>(va.sc[s].omega), be = c_of<float>(va.sc[s].beta);
+    cx<float> xv[12], pv[12], sw[12], tv[12];
     Prec<16>::load(xv, sys_ptr<16>(x, sd.off), nrm_ptr(xn, sd.off), sd.n, j);
     Prec<16>::load(pv, sys_ptr<16>(p, sd.off), nrm_ptr(pn, sd.off), sd.n, j);
-    Prec<16>::load(sv_, sys_ptr<16>(sv, sd.off), nrm_ptr(svn, sd.off), sd.n, j);
+    Prec<16>::load(sw, sys_ptr<16>(sv, sd.off), nrm_ptr(svn, sd.off), sd.n, j);
 #pragma unroll
-    for (int k = 0; k < 12; k++) xv[k] = xv[k] + al * pv[k] + om * sv_[k];
+    for (int k = 0; k < 12; k++) xv[k] = xv[k] + al * pv[k] + om * sw[k];
     Prec<16>::store(sys_ptr_w<16>(x, sd.off), nrm_ptr_w(xn, sd.off), sd.n, j, xv);
     Prec<16>::load(tv, sys_ptr<16>(t, sd.off), nrm_ptr(tn, sd.off), sd.n, j);
 #pragma unroll
-    for (int k = 0; k < 12; k++) sv_[k] = sv_[k] - om * tv[k];
-    Prec<16>::store(sys_ptr_w<16>(r, sd.off), nrm_ptr_w(rn, sd.off), sd.n, j, sv_);
-    Prec<16>::quantize(sv_);  // the values just stored
-    cx<float> w[12];
-    Prec<16>::load(w, sys_ptr<16>(r0, sd.off), nrm_ptr(r0n, sd.off), sd.n, j);
+    for (int k = 0; k < 12; k++) sw[k] = sw[k] - om * tv[k];
+    Prec<16>::store(sys_ptr_w<16>(r, sd.off), nrm_ptr_w(rn, sd.off), sd.n, j, sw);
+    Prec<16>::quantize(sw);  // the values just stored
+    Prec<16>::load(tv, sys_ptr<16>(v, sd.off), nrm_ptr(vn, sd.off), sd.n, j);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
-      red[0] += w[k].re * sv_[k].re + w[k].im * sv_[k].im;
-      red[1] += w[k].re * sv_[k].im - w[k].im * sv_[k].re;
-      red[2] += sv_[k].re * sv_[k].re + sv_[k].im * sv_[k].im;
+      pv[k] = sw[k] + be * (pv[k] - om * tv[k]);
+      red[0] += sw[k].re * sw[k].re + sw[k].im * sw[k].im;
     }
+    Prec<16>::store(sys_ptr_w<16>(p, sd.off), nrm_ptr_w(pn, sd.off), sd.n, j, pv);
   }
-  block_reduce_store<3, float>(red, va.partial + ((long long)s * va.pstride + by) * 4);
-}
-
-// ------------------------------------------------- p = r + beta (p - omega v)
-template <int P>
-__global__ void __launch_bounds__(128) k_bicg_p_w(VecArgs va, void* p, const void* r, const void* v) {
-  typedef Word<P> W;
-  typedef typename W::R R;
-  LQ_WORD_PROLOGUE(P)
-  if (!valid) return;
-  const cx<R> be = c_of<R>(va.sc[s].beta), om = c_of<R>(va.sc[s].omega);
-  cx<R> pv[W::NC], rv[W::NC], vv[W::NC];
-  W::get(wptr<P>(p, sd.off), i, pv);
-  W::get(wptr<P>(r, sd.off), i, rv);
-  W::get(wptr<P>(v, sd.off), i, vv);
-#pragma unroll
-  for (int k = 0; k < W::NC; k++) pv[k] = rv[k] + be * (pv[k] - om * vv[k]);
-  W::put(wptr_w<P>(p, sd.off), i, pv);
-}
-
-__global__ void __launch_bounds__(128) k_bicg_p_h(VecArgs va, void* p, float* pn, const void* r, const float* rn,
-                                                  const void* v, const float* vn) {
-  LQ_SITE_PROLOGUE
-  if (!valid) return;
-  const cx<float> be = c_of<float>(va.sc[s].beta), om = c_of<float>(va.sc[s].omega);
-  cx<float> pv[12], rv[12], vv[12];
-  Prec<16>::load(pv, sys_ptr<16>(p, sd.off), nrm_ptr(pn, sd.off), sd.n, j);
-  Prec<16>::load(rv, sys_ptr<16>(r, sd.off), nrm_ptr(rn, sd.off), sd.n, j);
-  Prec<16>::load(vv, sys_ptr<16>(v, sd.off), nrm_ptr(vn, sd.off), sd.n, j);
-#pragma unroll
-  for (int k = 0; k < 12; k++) pv[k] = rv[k] + be * (pv[k] - om * vv[k]);
-  Prec<16>::store(sys_ptr_w<16>(p, sd.off), nrm_ptr_w(pn, sd.off), sd.n, j, pv);
+  double* part = va.partial + (long long)s * va.pstride * 4;
+  block_reduce_store<1, float>(red, part + (long long)by * 4 + 2);
+  if (fin.mode != FIN_NONE) finish_last<1, 2, 4>(fin, part, (sd.n + 127) / 128, s);
 }
 
 // CG on the normal equations (the fallback for systems whose BiCGStab
@@ -378,154 +367,21 @@ __global__ void __launch_bounds__(128) k_convert(VecArgs va, const void* in, con
 }
 
 // ---------------------------------------------------------------- finalize
-// Sum of the block partials of system s = blockIdx.x, in a fixed order: each
-// thread of the block sums a strided subset, the warps reduce by shuffles and
-// warp 0 adds the warp sums in warp order.  Thread 0 receives the result.
+// One block per system: sum of its block partials (slots 0..2 of four) and its scalars, fin_update.
+// wps: words per site of the kernel that wrote the partials (1: one site per thread), so that the
+// system used ceil(n * wps / bdim) blocks.
 constexpr int FIN_THREADS = 512;
-LQ_DI void block_sum_partials(const double* partial, int pstride, int nb, int s, double out[3]) {
-  __shared__ double sh[FIN_THREADS / 32][3];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  double v[3] = {0.0, 0.0, 0.0};
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    const double* q = partial + ((long long)s * pstride + b) * 4;
-    v[0] += q[0];
-    v[1] += q[1];
-    v[2] += q[2];
-  }
-#pragma unroll
-  for (int q = 0; q < 3; q++) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-  }
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < 3; q++) sh[wid][q] = v[q];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    for (int q = 0; q < 3; q++) {
-      double t = 0.0;
-      for (int w = 0; w < nw; w++) t += sh[w][q];
-      out[q] = t;
-    }
-  }
-}
-
-LQ_DI double2 cdiv(double2 a, double2 b) {
-  double d = b.x * b.x + b.y * b.y;
-  return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
-}
-LQ_DI double2 cmul2(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-LQ_DI bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
-
-// One block per system: fold the block partials into the iteration scalars.
-//  FIN_INIT : rr = rho = |r|^2, rr0 = rr, iters = 0, target2 = max(tau2*rr, floor2)
-//  FIN_ALPHA: alpha = rho / <r0, v>
-//  FIN_OMEGA: omega = <t, s> / |t|^2
-//  FIN_BETA : rr = |r|^2, rho' = <r0, r>; stop the system when rr <= target2,
-//             on breakdown, NaN or divergence (rr > 1e8 rr0); else
-//             beta = (rho'/rho)(alpha/omega)
-//  FIN_NORM : rr = |r|^2 only
-//  CG on the normal equations (real scalars in .x):
-//  FIN_CG_RHO  : rho = |z|^2 (z = D^dag r), beta = 0 (the first direction is z)
-//  FIN_CG_ALPHA: alpha = rho / |v|^2 (v = D^ p); breakdown if |v|^2 is not positive
-//  FIN_CG_R    : rr = |r|^2; stop the system when rr <= target2, on NaN or divergence
-//  FIN_CG_BETA : beta = |z|^2 / rho, rho = |z|^2
-// tau2 / floor_rel2 are per call (FIN_INIT); floor_rel2 is relative to bb.
-// wps: words per site of the kernel that wrote the partials (1: one site per
-// thread), so that the system used ceil(n * wps / bdim) blocks.
 __global__ void k_finalize(int mode, int nsys, const SysDesc* sys, int* active, SolverScal* sc, const double* partial,
                            int pstride, int wps, int bdim, double tau2, double floor_rel2) {
   const int s = blockIdx.x;
   if (s >= nsys) return;
   if (active && !active[s]) return;  // uniform over the block
   const int nb = (sys[s].n * wps + bdim - 1) / bdim;
-  double v[3];
-  block_sum_partials(partial, pstride, nb, s, v);
+  double v[7] = {0.0};
+  block_sum_partials<3, 4>(partial + (long long)s * pstride * 4, nb, v);
   if (threadIdx.x != 0) return;
   SolverScal c = sc[s];
-  const double2 d = make_double2(v[0], v[1]);
-  switch (mode) {
-    case FIN_INIT:
-      c.rr = c.rr0 = v[2];
-      c.rho = make_double2(v[2], 0.0);
-      c.iters = 0;
-      c.status = 0;
-      c.target2 = fmax(tau2 * v[2], floor_rel2 * c.bb);
-      if (!(v[2] > c.target2)) active[s] = 0;
-      if (!isfinite(v[2])) {
-        c.status = 2;
-        active[s] = 0;
-      }
-      break;
-    case FIN_ALPHA:
-      if (!finite2(d) || (d.x == 0.0 && d.y == 0.0)) {
-        c.status = 1;
-        active[s] = 0;
-      } else {
-        c.alpha = cdiv(c.rho, d);
-      }
-      break;
-    case FIN_OMEGA:
-      if (!(v[2] > 0.0) || !isfinite(v[2])) {
-        c.omega = make_double2(0.0, 0.0);
-        c.status = 1;
-      } else {
-        c.omega = make_double2(d.x / v[2], d.y / v[2]);
-      }
-      break;
-    case FIN_BETA: {
-      c.iters += 1;
-      c.rr = v[2];
-      if (!isfinite(v[2]) || !finite2(d) || v[2] > 1e8 * c.rr0) {  // NaN or divergence
-        c.status = 2;
-        active[s] = 0;
-      } else if (v[2] <= c.target2) {
-        active[s] = 0;
-      } else if (c.status == 1 || (d.x == 0.0 && d.y == 0.0) || (c.omega.x == 0.0 && c.omega.y == 0.0)) {
-        c.status = 1;
-        active[s] = 0;
-      } else {
-        c.beta = cmul2(cdiv(d, c.rho), cdiv(c.alpha, c.omega));
-        c.rho = d;
-      }
-      break;
-    }
-    case FIN_NORM:
-      c.rr = v[2];
-      break;
-    case FIN_CG_RHO:
-      c.rho = make_double2(v[2], 0.0);
-      c.beta = make_double2(0.0, 0.0);
-      break;
-    case FIN_CG_ALPHA:
-      if (!(v[2] > 0.0) || !isfinite(v[2]) || !(c.rho.x > 0.0)) {
-        c.status = 1;
-        active[s] = 0;
-      } else {
-        c.alpha = make_double2(c.rho.x / v[2], 0.0);
-      }
-      break;
-    case FIN_CG_R:
-      c.iters += 1;
-      c.rr = v[2];
-      if (!isfinite(v[2]) || v[2] > 1e8 * c.rr0) {
-        c.status = 2;
-        active[s] = 0;
-      } else if (v[2] <= c.target2) {
-        active[s] = 0;
-      }
-      break;
-    case FIN_CG_BETA:
-      if (!(c.rho.x > 0.0) || !isfinite(v[2])) {
-        c.status = 1;
-        active[s] = 0;
-      } else {
-        c.beta = make_double2(v[2] / c.rho.x, 0.0);
-        c.rho = make_double2(v[2], 0.0);
-      }
-      break;
-  }
+  fin_update(mode, v, c, active + s, tau2, floor_rel2);
   sc[s] = c;
 }
 

@@ -14,7 +14,7 @@
 // is the whole lattice with periodic / antiperiodic BC.
 #pragma once
 
-#include "common.cuh"
+#include "finalize.cuh"
 
 namespace lq {
 
@@ -603,6 +603,7 @@ struct HopArgs {
   int nby;                          // site blocks per system in the grid
   int tile;                         // blocks per time tile of the grid order (0: systems fastest)
   int tblk;                         // 1: a block covers 32 sites x 4 time slices (site_of_block)
+  FinArgs fin;                      // what the last block does with the inner products (RED_DOT_W, RED_TSW)
 };
 
 // Epilogue terms present (compile time): D_hop x, A y, z.
@@ -657,35 +658,34 @@ int hop_lin_tuned(int cfg, bool clov, int red, int epi, dim3 gr, const HopArgs& 
 template <int P>
 int hop_clinv_tuned(int cfg, bool clov, int epi, dim3 gr, const HopArgs& a, cudaStream_t st);
 
-// Block reduction of NQ per-thread partial sums of type A (the kernel's own
-// precision: FP32 for the FP32 / FP16 solver, whose FP64 rate on this GPU is a
-// small fraction of its FP32 rate) through a warp-shuffle tree; the per-warp
-// sums are widened to FP64 and combined in FP64, and one partial per block is
-// stored.  The order is fixed, so results are deterministic.
-template <int NQ, typename A>
-LQ_DI void block_reduce_store(A v[NQ], double* dst) {
-  __shared__ double sh[32][NQ > 0 ? NQ : 1];
+// The fused inner products of a hop kernel over the stored values res: number of sums, and the sums of
+// one site (y: the epilogue's second input, w: the partner r0).
+//   RED_DOT_W: <w, out> (0, 1);  RED_TS: <out, y> (0, 1), |out|^2 (2);  RED_NORM: |out|^2 (2);
+//   RED_TSW: RED_TS with <w, out> (3, 4) and <w, y> (5, 6).
+constexpr int red_count(int red) { return red == RED_TSW ? 7 : 3; }
+template <int RED, int NC, typename R>
+LQ_DI void red_add(R* red, const cx<R>* res, const cx<R>* y, const cx<R>* w) {
 #pragma unroll
-  for (int q = 0; q < NQ; q++)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) sh[wid][q] = (double)v[q];
-  __syncthreads();
-  if (wid == 0) {
-    int nw = blockDim.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; q++) {
-      double t = lane < nw ? sh[lane][q] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      if (lane == 0) dst[q] = t;
+  for (int k = 0; k < NC; k++) {
+    if (RED == RED_DOT_W) {
+      red[0] += w[k].re * res[k].re + w[k].im * res[k].im;
+      red[1] += w[k].re * res[k].im - w[k].im * res[k].re;
+    } else {
+      if (RED != RED_NORM) {
+        red[0] += res[k].re * y[k].re + res[k].im * y[k].im;
+        red[1] += res[k].re * y[k].im - res[k].im * y[k].re;
+      }
+      red[2] += res[k].re * res[k].re + res[k].im * res[k].im;
+      if (RED == RED_TSW) {
+        red[3] += w[k].re * res[k].re + w[k].im * res[k].im;
+        red[4] += w[k].re * res[k].im - w[k].im * res[k].re;
+        red[5] += w[k].re * y[k].re + w[k].im * y[k].im;
+        red[6] += w[k].re * y[k].im - w[k].im * y[k].re;
+      }
     }
   }
 }
-
+// Stores the block's sums (4 doubles a block, 8 for RED_TSW) and finishes the system if asked to.
 template <int P>
 LQ_DI const void* sys_ptr(const void* pool, long long off) {
   return pool ? (const void*)((const char*)pool + off * (long long)Prec<P>::NV * 16) : nullptr;
@@ -697,11 +697,21 @@ LQ_DI void* sys_ptr_w(void* pool, long long off) {
 LQ_DI const float* nrm_ptr(const float* pool, long long off) { return pool ? pool + off : nullptr; }
 LQ_DI float* nrm_ptr_w(float* pool, long long off) { return pool ? pool + off : nullptr; }
 
+template <int RED, typename R>
+LQ_DI void red_store(R* red, const HopArgs& a, int s, int by, int nb) {
+  constexpr int PW = RED == RED_TSW ? 8 : 4;
+  double* part = a.partial + (long long)s * a.pstride * 4;
+  block_reduce_store<red_count(RED), R>(red, part + (long long)by * PW);
+  if constexpr (RED == RED_DOT_W) {
+    if (a.fin.mode != FIN_NONE) finish_last<2, 0, PW>(a.fin, part, nb, s);
+  } else if constexpr (RED == RED_TSW) {
+    if (a.fin.mode != FIN_NONE) finish_last<7, 0, PW>(a.fin, part, nb, s);
+  }
+}
+
 // out = beta * A(y) + alpha * D_hop x + gamma * z   on parity pout
 // (terms present per EPI; A = diag * 1 without clover), with an optional
-// fused per-system reduction over the stored values:
-//   RED_DOT_W: <w, out> (slots 0,1);  RED_TS: <out, y> (0,1) and |out|^2 (2);
-//   RED_NORM: |out|^2 (slot 2).
+// fused per-system reduction over the stored values (red_add).
 template <int P, bool DAG, bool CLOV, int RED, int EPI, int CFG = 0>
 __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_lin(HopArgs a) {
   typedef typename Prec<P>::R R;
@@ -713,7 +723,7 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_lin(HopArgs
   if (by * (int)blockDim.x >= sd.n) return;  // whole block beyond this system
   const int j = site_of_block(a.tblk, a.g.S3h, by, threadIdx.x);
   const FieldPtrs f = a.fields[sd.field];
-  R red[3] = {0, 0, 0};
+  R red[red_count(RED)] = {0};
   if (j < sd.n) {
     const int cb = sd.cb0 + j;
     cx<R> res[12];
@@ -730,7 +740,7 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_lin(HopArgs
       for (int k = 0; k < 12; k++) res[k] = {0, 0};
     }
     cx<R> yv[12];
-    if ((EPI & EPI_Y) || RED == RED_TS) Prec<P>::load(yv, sys_ptr<P>(a.y, sd.off), nrm_ptr(a.yn, sd.off), sd.n, j);
+    if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) Prec<P>::load(yv, sys_ptr<P>(a.y, sd.off), nrm_ptr(a.yn, sd.off), sd.n, j);
     if (EPI & EPI_Y) {
       cx<R> ay[12];
       if (CLOV) {
@@ -753,28 +763,12 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_lin(HopArgs
     Prec<P>::store(sys_ptr_w<P>(a.out, sd.off), nrm_ptr_w(a.outn, sd.off), sd.n, j, res);
     if (RED != RED_NONE) {
       Prec<P>::quantize(res);  // reduce over the stored (rounded) values
-      if (RED == RED_DOT_W) {
-        cx<R> wv[12];
-        Prec<P>::load(wv, sys_ptr<P>(a.w, sd.off), nrm_ptr(a.wn, sd.off), sd.n, j);
-#pragma unroll
-        for (int k = 0; k < 12; k++) {
-          red[0] += wv[k].re * res[k].re + wv[k].im * res[k].im;
-          red[1] += wv[k].re * res[k].im - wv[k].im * res[k].re;
-        }
-      } else if (RED == RED_TS) {
-#pragma unroll
-        for (int k = 0; k < 12; k++) {
-          red[0] += res[k].re * yv[k].re + res[k].im * yv[k].im;
-          red[1] += res[k].re * yv[k].im - res[k].im * yv[k].re;
-          red[2] += res[k].re * res[k].re + res[k].im * res[k].im;
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < 12; k++) red[2] += res[k].re * res[k].re + res[k].im * res[k].im;
-      }
+      cx<R> wv[12];
+      if (RED == RED_DOT_W || RED == RED_TSW) Prec<P>::load(wv, sys_ptr<P>(a.w, sd.off), nrm_ptr(a.wn, sd.off), sd.n, j);
+      red_add<RED, 12, R>(red, res, yv, wv);
     }
   }
-  if (RED != RED_NONE) block_reduce_store<3, R>(red, a.partial + ((long long)s * a.pstride + by) * 4);
+  if (RED != RED_NONE) red_store<RED, R>(red, a, s, by, (sd.n + 127) / 128);
 }
 
 // out = A^{-1} (alpha * D_hop x + beta * y) on even sites (pout = 0), terms
@@ -907,10 +901,10 @@ __global__ void __launch_bounds__(128, LQ_HOP2_MINB) k_hop2_lin(HopArgs a) {
 #pragma unroll
     for (int k = 0; k < 6; k++) res[k] = {0.f, 0.f};
   }
-  float red[3] = {0.f, 0.f, 0.f};
+  float red[red_count(RED)] = {0.f};
   if (valid) {
     cx<float> yv[6];
-    if ((EPI & EPI_Y) || RED == RED_TS) load_half32(yv, sys_ptr<32>(a.y, sd.off), sd.n, j, h);
+    if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) load_half32(yv, sys_ptr<32>(a.y, sd.off), sd.n, j, h);
     if (EPI & EPI_Y) {
       cx<float> ay[6];
       if (CLOV) {
@@ -931,27 +925,13 @@ __global__ void __launch_bounds__(128, LQ_HOP2_MINB) k_hop2_lin(HopArgs a) {
       for (int k = 0; k < 6; k++) res[k] = res[k] + ga * zv[k];
     }
     store_half32(sys_ptr_w<32>(a.out, sd.off), sd.n, j, h, res);
-    if (RED == RED_DOT_W) {
+    if (RED != RED_NONE) {
       cx<float> wv[6];
-      load_half32(wv, sys_ptr<32>(a.w, sd.off), sd.n, j, h);
-#pragma unroll
-      for (int k = 0; k < 6; k++) {
-        red[0] += wv[k].re * res[k].re + wv[k].im * res[k].im;
-        red[1] += wv[k].re * res[k].im - wv[k].im * res[k].re;
-      }
-    } else if (RED == RED_TS) {
-#pragma unroll
-      for (int k = 0; k < 6; k++) {
-        red[0] += res[k].re * yv[k].re + res[k].im * yv[k].im;
-        red[1] += res[k].re * yv[k].im - res[k].im * yv[k].re;
-        red[2] += res[k].re * res[k].re + res[k].im * res[k].im;
-      }
-    } else if (RED == RED_NORM) {
-#pragma unroll
-      for (int k = 0; k < 6; k++) red[2] += res[k].re * res[k].re + res[k].im * res[k].im;
+      if (RED == RED_DOT_W || RED == RED_TSW) load_half32(wv, sys_ptr<32>(a.w, sd.off), sd.n, j, h);
+      red_add<RED, 6, float>(red, res, yv, wv);
     }
   }
-  if (RED != RED_NONE) block_reduce_store<3, float>(red, a.partial + ((long long)s * a.pstride + by) * 4);
+  if (RED != RED_NONE) red_store<RED, float>(red, a, s, by, (sd.n + 63) / 64);
 }
 
 template <bool DAG, bool CLOV, int EPI>

@@ -17,6 +17,7 @@ int hop_lin_cfg(int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t st) {
   else if (red == RED_NONE && epi == XZ) k_hop_lin<P, false, CLOV, RED_NONE, XZ, CFG><<<gr, 128, 0, st>>>(a);
   else if (red == RED_DOT_W && epi == XY) k_hop_lin<P, false, CLOV, RED_DOT_W, XY, CFG><<<gr, 128, 0, st>>>(a);
   else if (red == RED_TS && epi == XY) k_hop_lin<P, false, CLOV, RED_TS, XY, CFG><<<gr, 128, 0, st>>>(a);
+  else if (red == RED_TSW && epi == XY) k_hop_lin<P, false, CLOV, RED_TSW, XY, CFG><<<gr, 128, 0, st>>>(a);
   else if (red == RED_NORM && epi == XYZ) k_hop_lin<P, false, CLOV, RED_NORM, XYZ, CFG><<<gr, 128, 0, st>>>(a);
   else return -1;
   return 0;

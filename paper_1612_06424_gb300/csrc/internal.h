@@ -37,6 +37,7 @@ struct Batch {
   int* active = nullptr;
   lq::SolverScal* sc = nullptr;
   double* partial = nullptr;
+  unsigned* count = nullptr;  // blocks that have arrived, per system (finish_last), zero between launches
 };
 
 constexpr int LQ_BLOCK = 128;
@@ -71,16 +72,19 @@ int lq_launch_pack_links(const lq::Geom& g, const double2* U, double2* U64, floa
 int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, double2* A64, double2* Ai64,
                      float4* A32, float4* Ai32, int* fail, cudaStream_t st);
 
-// out = beta*A(y) + alpha*D_hop x + gamma*z on parity pout (+ fused reduction)
+// out = beta*A(y) + alpha*D_hop x + gamma*z on parity pout (+ fused reduction; fin: what the kernel's last
+// block of a system does with the sums, FIN_ALPHA for RED_DOT_W, FIN_OMEGA_BETA for RED_TSW)
 int lq_hop_lin(int P, bool dag, bool clov, int red, const lqcd_lattice* L, const Batch& b, int pout, VecP x, VecP y,
-               VecP z, VecP w, VecP out, double alpha, double beta, double gamma, cudaStream_t st);
+               VecP z, VecP w, VecP out, double alpha, double beta, double gamma, cudaStream_t st,
+               int fin = lq::FIN_NONE);
 // out = A^{-1}(alpha*D_hop x + beta*y) on even sites
 int lq_hop_clinv(int P, bool dag, bool clov, const lqcd_lattice* L, const Batch& b, VecP x, VecP y, VecP out,
                  double alpha, double beta, cudaStream_t st);
 
 int lq_bicg_s(int P, const Batch& b, VecP r, VecP v, VecP s, cudaStream_t st);
-int lq_bicg_xr(int P, const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP r, VecP r0, cudaStream_t st);
-int lq_bicg_p(int P, const Batch& b, VecP p, VecP r, VecP v, cudaStream_t st);
+// x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2 (fin: FIN_STOP)
+int lq_bicg_xrp(int P, const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP v, VecP r, cudaStream_t st,
+                int fin = lq::FIN_NONE);
 int lq_inner_init(int P, const Batch& b, const double2* r64, VecP r, VecP r0, VecP p, VecP x, cudaStream_t st);
 // CG on the normal equations (P = 64 or 32): x += alpha p, r -= alpha v (|r|^2); p = z + beta p
 int lq_cg_xr(int P, const Batch& b, VecP x, VecP p, VecP r, VecP v, cudaStream_t st);

@@ -70,6 +70,8 @@ static void set_grid_order(HopArgs& a, const lqcd_lattice* L, const Batch& b, in
   a.tblk = sites_per_block == LQ_BLOCK ? tblk_of(b) : 0;
 }
 
+static FinArgs fin_args(const Batch& b, int mode) { return FinArgs{mode, b.active, b.sc, b.count}; }
+
 static HopArgs hop_args(const lqcd_lattice* L, const Batch& b, int pout) {
   HopArgs a{};
   a.g = L->g;
@@ -81,6 +83,7 @@ static HopArgs hop_args(const lqcd_lattice* L, const Batch& b, int pout) {
   a.pstride = b.pstride;
   a.nsys = b.nsys;
   a.diag = 1.0 / (2.0 * L->kappa);
+  a.fin.mode = FIN_NONE;
   set_grid_order(a, L, b, LQ_BLOCK);
   return a;
 }
@@ -119,6 +122,7 @@ static int launch_lin2(int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t
   else if (red == RED_NONE && epi == XZ) k_hop2_lin<DAG, CLOV, RED_NONE, XZ><<<gr, LQ_BLOCK, 0, st>>>(a);
   else if (red == RED_DOT_W && epi == XY) k_hop2_lin<DAG, CLOV, RED_DOT_W, XY><<<gr, LQ_BLOCK, 0, st>>>(a);
   else if (red == RED_TS && epi == XY) k_hop2_lin<DAG, CLOV, RED_TS, XY><<<gr, LQ_BLOCK, 0, st>>>(a);
+  else if (red == RED_TSW && epi == XY) k_hop2_lin<DAG, CLOV, RED_TSW, XY><<<gr, LQ_BLOCK, 0, st>>>(a);
   else if (red == RED_NORM && epi == XYZ) k_hop2_lin<DAG, CLOV, RED_NORM, XYZ><<<gr, LQ_BLOCK, 0, st>>>(a);
   else return -1;
   return 0;
@@ -146,6 +150,7 @@ static int launch_lin(int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t 
   else if (red == RED_NONE && epi == XZ) hop_go<P>(k_hop_lin<P, DAG, CLOV, RED_NONE, XZ>, gr, a, st);
   else if (red == RED_DOT_W && epi == XY) hop_go<P>(k_hop_lin<P, DAG, CLOV, RED_DOT_W, XY>, gr, a, st);
   else if (red == RED_TS && epi == XY) hop_go<P>(k_hop_lin<P, DAG, CLOV, RED_TS, XY>, gr, a, st);
+  else if (red == RED_TSW && epi == XY) hop_go<P>(k_hop_lin<P, DAG, CLOV, RED_TSW, XY>, gr, a, st);
   else if (red == RED_NORM && epi == XYZ) hop_go<P>(k_hop_lin<P, DAG, CLOV, RED_NORM, XYZ>, gr, a, st);
   else return -1;
   return 0;
@@ -158,8 +163,9 @@ static int launch_lin_p(bool dag, bool clov, int red, int epi, dim3 gr, const Ho
 }
 
 int lq_hop_lin(int P, bool dag, bool clov, int red, const lqcd_lattice* L, const Batch& b, int pout, VecP x, VecP y,
-               VecP z, VecP w, VecP out, double alpha, double beta, double gamma, cudaStream_t st) {
+               VecP z, VecP w, VecP out, double alpha, double beta, double gamma, cudaStream_t st, int fin) {
   HopArgs a = hop_args(L, b, pout);
+  a.fin = fin_args(b, fin);
   a.x = x.d; a.xn = x.nrm;
   a.y = y.d; a.yn = y.nrm;
   a.z = z.d; a.zn = z.nrm;
@@ -277,21 +283,16 @@ int lq_bicg_s(int P, const Batch& b, VecP r, VecP v, VecP s, cudaStream_t st) {
   return launched();
 }
 
-int lq_bicg_xr(int P, const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP r, VecP r0, cudaStream_t st) {
+int lq_bicg_xrp(int P, const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP v, VecP r, cudaStream_t st, int fin) {
   VecArgs va = vec_args(b);
-  if (P == 64) k_bicg_xr_w<64><<<grid_words(b, 64), LQ_BLOCK, 0, st>>>(va, x.d, p.d, s.d, t.d, r.d, r0.d);
-  else if (P == 32) k_bicg_xr_w<32><<<grid_words(b, 32), LQ_BLOCK, 0, st>>>(va, x.d, p.d, s.d, t.d, r.d, r0.d);
+  const FinArgs fa = fin_args(b, fin);
+  const long long nv = P == 64 ? 12 : 6, bw = LQ_BLOCK * XRP_WPT;
+  const dim3 gr = grid_lin(b, (b.max_n * nv + bw - 1) / bw);
+  if (P == 64) k_bicg_xrp_w<64><<<gr, LQ_BLOCK, 0, st>>>(va, fa, x.d, p.d, s.d, t.d, v.d, r.d);
+  else if (P == 32) k_bicg_xrp_w<32><<<gr, LQ_BLOCK, 0, st>>>(va, fa, x.d, p.d, s.d, t.d, v.d, r.d);
   else
-    k_bicg_xr_h<<<grid_of(b), LQ_BLOCK, 0, st>>>(va, x.d, x.nrm, p.d, p.nrm, s.d, s.nrm, t.d, t.nrm, r.d, r.nrm, r0.d,
-                                                 r0.nrm);
-  return launched();
-}
-
-int lq_bicg_p(int P, const Batch& b, VecP p, VecP r, VecP v, cudaStream_t st) {
-  VecArgs va = vec_args(b);
-  if (P == 64) k_bicg_p_w<64><<<grid_words(b, 64), LQ_BLOCK, 0, st>>>(va, p.d, r.d, v.d);
-  else if (P == 32) k_bicg_p_w<32><<<grid_words(b, 32), LQ_BLOCK, 0, st>>>(va, p.d, r.d, v.d);
-  else k_bicg_p_h<<<grid_of(b), LQ_BLOCK, 0, st>>>(va, p.d, p.nrm, r.d, r.nrm, v.d, v.nrm);
+    k_bicg_xrp_h<<<grid_of(b), LQ_BLOCK, 0, st>>>(va, fa, x.d, x.nrm, p.d, p.nrm, s.d, s.nrm, t.d, t.nrm, v.d, v.nrm,
+                                                  r.d, r.nrm);
   return launched();
 }
 
