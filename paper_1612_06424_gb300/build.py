@@ -20,9 +20,11 @@ OUT_DIR = os.environ.get("LQCD_BUILD_DIR") or os.path.join(HERE, "lib")
 LIB = os.path.join(OUT_DIR, "liblqcd.so")
 # extra nvcc flags (e.g. -DLQ_HOP_MINB=6 to change the register cap of the stencil kernels)
 EXTRA = os.environ.get("LQCD_NVCC_FLAGS", "").split()
-SOURCES = ["api.cu", "kernels.cu", "hop_tuned32.cu", "hop_tuned16.cu", "gauge.cu", "force.cu", "disconnected.cu",
+SOURCES = ["api.cu", "kernels.cu", "hop_tuned32.cu", "hop_tuned16.cu", "fx_lin.cu", "fx_clinv.cu",
+           "gauge.cu", "force.cu", "disconnected.cu",
            "projection.cu", "nucleon.cu", "nucleon_tc.cu", "noalloc.cu", "peak.cu"]
-HEADERS = ["common.cuh", "finalize.cuh", "dslash.cuh", "blas.cuh", "hop_tuned.cuh", "internal.h", "tc_layout.cuh"]
+HEADERS = ["common.cuh", "finalize.cuh", "dslash.cuh", "blas.cuh", "hop_tuned.cuh", "fx.cuh", "fxnum.cuh",
+           "internal.h", "tc_layout.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "-Xptxas", "-O3", "--expt-relaxed-constexpr"]

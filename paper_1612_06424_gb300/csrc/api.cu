@@ -256,6 +256,17 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
   double2* bh_o = f64.v(0);
   double2* r64 = f64.v(1);
   double2* t64 = f64.v(2);
+  // The FP64 stencil reads its hop input in limbs (fx.cuh): a vector that is only a hop input is
+  // converted in place, another one into a vector that is free at that point.
+  DBuf fxe;
+  RC(fxe.alloc(sizeof(int) * (size_t)b.total, st));
+  auto limbs = [&](const void* in, void* out, VecP& x, cudaStream_t s_) -> int {
+    x = VecP{};
+    x.d = out;
+    x.e = fxe.as<int>();
+    return lq_to_fx(b, in, x, s_);
+  };
+  VecP xl;
   PoolP ps;
   RC(ps.alloc(b, P, 8, st));
   VecP r = ps.v(0), r0 = ps.v(1), p = ps.v(2), v = ps.v(3), s = ps.v(4), t = ps.v(5), xs = ps.v(6), te = ps.v(7);
@@ -291,7 +302,8 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
 
   // prepare: bh_o = b_o + 1/2 H_oe A_ee^{-1} b_e
   RC(lq_hop_clinv(64, dag, clov, L, b, none, v64(b_e), v64(t64), 0.0, 1.0, st));
-  RC(lq_hop_lin(64, dag, clov, lq::RED_NONE, L, b, 1, v64(t64), none, v64(b_o), none, v64(bh_o), 0.5, 0.0, 1.0, st));
+  RC(limbs(t64, t64, xl, st));
+  RC(lq_hop_lin(64, dag, clov, lq::RED_NONE, L, b, 1, xl, none, v64(b_o), none, v64(bh_o), 0.5, 0.0, 1.0, st));
   if (!guess) CK(cudaMemsetAsync(x_o, 0, sizeof(double2) * (size_t)b.total * 12, st));
 
   std::vector<int> outer(n, 1);
@@ -316,10 +328,11 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
       RC(lq_norm2_64(b, r64, st));
       RC(lq_finalize(lq::FIN_NORM, b, 0, 0, 12, st));
     } else {
-      RC(lq_hop_clinv(64, dag, clov, L, b, v64(x_o), none, v64(t64), 1.0, 0.0, st));
-      RC(lq_hop_lin(64, dag, clov, lq::RED_NORM, L, b, 1, v64(t64), v64(x_o), v64(bh_o), none, v64(r64), 0.25, -1.0,
-                    1.0, st));
-      RC(lq_finalize(lq::FIN_NORM, b, 0, 0, 1, st));
+      RC(limbs(x_o, r64, xl, st));
+      RC(lq_hop_clinv(64, dag, clov, L, b, xl, none, v64(t64), 1.0, 0.0, st));
+      RC(limbs(t64, t64, xl, st));
+      RC(lq_hop_lin(64, dag, clov, lq::RED_NORM, L, b, 1, xl, v64(x_o), v64(bh_o), none, v64(r64), 0.25, -1.0, 1.0, st));
+      RC(lq_finalize(lq::FIN_NORM, b, 0, 0, lq_hop_wps(64, b), st));
     }
     RC(B.pull_sc(st));
     int n_act = 0;
@@ -391,11 +404,17 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
       RC(lq_finalize(lq::FIN_INIT, b, tau * tau, 0.25 * tol * tol, lq_words_per_site(P), st));
       // one BiCGStab iteration: 6 kernels, all scalars and flags on the device
       auto iteration = [&](cudaStream_t s_) -> int {
-        RC(lq_hop_clinv(P, dag, clov, L, b, p, none, te, 1.0, 0.0, s_));
-        RC(lq_hop_lin(P, dag, clov, lq::RED_DOT_W, L, b, 1, te, p, none, r0, v, -0.25, 1.0, 0.0, s_, lq::FIN_ALPHA));
+        VecP hx = p, ht = te;  // hop inputs (FP64: in limbs; t is free until the end)
+        if (P == 64) RC(limbs(p.d, t.d, hx, s_));
+        RC(lq_hop_clinv(P, dag, clov, L, b, hx, none, te, 1.0, 0.0, s_));
+        if (P == 64) RC(limbs(te.d, te.d, ht, s_));
+        RC(lq_hop_lin(P, dag, clov, lq::RED_DOT_W, L, b, 1, ht, p, none, r0, v, -0.25, 1.0, 0.0, s_, lq::FIN_ALPHA));
         RC(lq_bicg_s(P, b, r, v, s, s_));
-        RC(lq_hop_clinv(P, dag, clov, L, b, s, none, te, 1.0, 0.0, s_));
-        RC(lq_hop_lin(P, dag, clov, lq::RED_TSW, L, b, 1, te, s, none, r0, t, -0.25, 1.0, 0.0, s_, lq::FIN_OMEGA_BETA));
+        hx = s;
+        if (P == 64) RC(limbs(s.d, t.d, hx, s_));
+        RC(lq_hop_clinv(P, dag, clov, L, b, hx, none, te, 1.0, 0.0, s_));
+        if (P == 64) RC(limbs(te.d, te.d, ht, s_));
+        RC(lq_hop_lin(P, dag, clov, lq::RED_TSW, L, b, 1, ht, s, none, r0, t, -0.25, 1.0, 0.0, s_, lq::FIN_OMEGA_BETA));
         RC(lq_bicg_xrp(P, b, xs, p, s, t, v, r, s_, lq::FIN_STOP));
         return 0;
       };
@@ -463,23 +482,28 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
       RC(B.push_active(st));
       RC(lq_inner_init(PC, b, r64, crv, czv, cpv, cxv, st));  // r = r64, x = 0
       RC(lq_finalize(lq::FIN_INIT, b, tau * tau, 0.25 * tol * tol, lq_words_per_site(PC), st));
+      // out = Dhat in (or Dhat^dag), with |out|^2
+      auto dhat = [&](bool dg, VecP in, VecP outv) -> int {
+        VecP hx = in, ht = ctv;
+        if (PC == 64) RC(limbs(in.d, outv.d, hx, st));
+        RC(lq_hop_clinv(PC, dg, clov, L, b, hx, none, ctv, 1.0, 0.0, st));
+        if (PC == 64) RC(limbs(ctv.d, ctv.d, ht, st));
+        return lq_hop_lin(PC, dg, clov, lq::RED_TS, L, b, 1, ht, in, none, none, outv, -0.25, 1.0, 0.0, st);
+      };
       // z = Dhat^dag r, rho = |z|^2, p = z
-      RC(lq_hop_clinv(PC, !dag, clov, L, b, crv, none, ctv, 1.0, 0.0, st));
-      RC(lq_hop_lin(PC, !dag, clov, lq::RED_TS, L, b, 1, ctv, crv, none, none, czv, -0.25, 1.0, 0.0, st));
+      RC(dhat(!dag, crv, czv));
       RC(lq_finalize(lq::FIN_CG_RHO, b, 0, 0, lq_hop_wps(PC, b), st));
       RC(lq_cg_p(PC, b, cpv, czv, st));
       int itc = 0;
       while (itc < budget) {
         // v = Dhat p, alpha = rho / |v|^2
-        RC(lq_hop_clinv(PC, dag, clov, L, b, cpv, none, ctv, 1.0, 0.0, st));
-        RC(lq_hop_lin(PC, dag, clov, lq::RED_TS, L, b, 1, ctv, cpv, none, none, cvv, -0.25, 1.0, 0.0, st));
+        RC(dhat(dag, cpv, cvv));
         RC(lq_finalize(lq::FIN_CG_ALPHA, b, 0, 0, lq_hop_wps(PC, b), st));
         // x += alpha p, r -= alpha v
         RC(lq_cg_xr(PC, b, cxv, cpv, crv, cvv, st));
         RC(lq_finalize(lq::FIN_CG_R, b, 0, 0, lq_words_per_site(PC), st));
         // z = Dhat^dag r, beta = |z|^2 / rho, p = z + beta p
-        RC(lq_hop_clinv(PC, !dag, clov, L, b, crv, none, ctv, 1.0, 0.0, st));
-        RC(lq_hop_lin(PC, !dag, clov, lq::RED_TS, L, b, 1, ctv, crv, none, none, czv, -0.25, 1.0, 0.0, st));
+        RC(dhat(!dag, crv, czv));
         RC(lq_finalize(lq::FIN_CG_BETA, b, 0, 0, lq_hop_wps(PC, b), st));
         RC(lq_cg_p(PC, b, cpv, czv, st));
         itc++;
@@ -503,7 +527,8 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
   // the true FP64 residual is the one the last cycle recomputed from x_o.
   std::fill(B.h_active.begin(), B.h_active.end(), 1);
   RC(B.push_active(st));
-  RC(lq_hop_clinv(64, dag, clov, L, b, v64(x_o), v64(b_e), v64(x_e), 0.5, 1.0, st));
+  RC(limbs(x_o, r64, xl, st));
+  RC(lq_hop_clinv(64, dag, clov, L, b, xl, v64(b_e), v64(x_e), 0.5, 1.0, st));
   for (int k = 0; k < n; k++) {
     out.res[k] = bb[k] > 0 ? std::sqrt(last_rr[k] / bb[k]) : 0.0;
     if (out.status[k] == 0 && !(out.res[k] <= tol)) out.status[k] = std::isfinite(out.res[k]) ? LQCD_ENOTCONVERGED : LQCD_ENAN;
@@ -563,7 +588,7 @@ using GuessFn = std::function<int(BatchStore& B, int k0, double2* x_e, double2* 
 
 // device bytes per system site (one parity) held during a solve in precision P:
 // 4 caller-side FP64 vectors + 3 solver FP64 vectors + 8 Krylov vectors
-size_t site_bytes(int P) { return (size_t)(7 * 192 + 8 * (P == 64 ? 192 : P == 32 ? 96 : 52)); }
+size_t site_bytes(int P) { return (size_t)(7 * 192 + 4 + 8 * (P == 64 ? 192 : P == 32 ? 96 : 52)); }
 
 // Free device memory, counting what the stream-ordered pool holds unused.
 size_t free_device_bytes() {
@@ -742,6 +767,8 @@ static void free_fields(lqcd_lattice* L) {
     cudaFree(f.U16);
     cudaFree(f.A64);
     cudaFree(f.Ai64);
+    cudaFree(f.A64e);
+    cudaFree(f.Ai64e);
     cudaFree(f.A32);
     cudaFree(f.Ai32);
   }
@@ -786,11 +813,13 @@ extern "C" int lqcd_set_gauge(lqcd_lattice* L, int n_fields, const double* U, do
       FieldData f;
       L->fields.push_back(f);
       FieldData& F = L->fields.back();
-      CK(cudaMalloc(&F.U64, sizeof(double2) * 2 * 4 * 9 * Vh));
+      CK(cudaMalloc(&F.U64, sizeof(int4) * 2 * 4 * 9 * Vh));
       CK(cudaMalloc(&F.U32, sizeof(float4) * 2 * 4 * 3 * Vh));
       CK(cudaMalloc(&F.U16, sizeof(uint2) * 2 * 4 * 3 * Vh));
-      CK(cudaMalloc(&F.A64, sizeof(double2) * 2 * 36 * Vh));
-      CK(cudaMalloc(&F.Ai64, sizeof(double2) * 36 * Vh));
+      CK(cudaMalloc(&F.A64, sizeof(int4) * 2 * 36 * Vh));
+      CK(cudaMalloc(&F.Ai64, sizeof(int4) * 36 * Vh));
+      CK(cudaMalloc(&F.A64e, sizeof(int) * 2 * 2 * Vh));
+      CK(cudaMalloc(&F.Ai64e, sizeof(int) * 2 * Vh));
       CK(cudaMalloc(&F.A32, sizeof(float4) * 2 * 18 * Vh));
       CK(cudaMalloc(&F.Ai32, sizeof(float4) * 18 * Vh));
     }
@@ -803,7 +832,7 @@ extern "C" int lqcd_set_gauge(lqcd_lattice* L, int n_fields, const double* U, do
     CK(cudaMemsetAsync(dev.p, 0, sizeof(unsigned long long), st));
     CK(cudaMemsetAsync(fail.p, 0, sizeof(int), st));
     RC(lq_launch_pack_links(L->g, src, F.U64, F.U32, F.U16, dev.as<unsigned long long>(), st));
-    RC(lq_launch_clover(L->g, src, kappa, c_sw, F.A64, F.Ai64, F.A32, F.Ai32, fail.as<int>(), st));
+    RC(lq_launch_clover(L->g, src, kappa, c_sw, F.A64, F.Ai64, F.A64e, F.Ai64e, F.A32, F.Ai32, fail.as<int>(), st));
     unsigned long long d = 0;
     int fl = 0;
     CK(cudaMemcpyAsync(&d, dev.p, sizeof(d), cudaMemcpyDeviceToHost, st));
@@ -827,6 +856,8 @@ extern "C" int lqcd_set_gauge(lqcd_lattice* L, int n_fields, const double* U, do
     fp.U16 = F.U16;
     fp.A64 = F.A64;
     fp.Ai64 = F.Ai64;
+    fp.A64e = F.A64e;
+    fp.Ai64e = F.Ai64e;
     fp.A32 = F.A32;
     fp.Ai32 = F.Ai32;
     ptrs.push_back(fp);
@@ -851,7 +882,7 @@ extern "C" int lqcd_dslash(lqcd_lattice* L, int field, const lqcd_slab* dom, int
   RC(B.build(L, 1, &d, &field, st));
   const Batch& b = B.b;
   Pool64 e;
-  RC(e.alloc(b, 4, st));
+  RC(e.alloc(b, precision == 64 ? 5 : 4, st));  // FP64: one more for the hop input in limbs
   DBuf ptr;
   RC(ptr.alloc(sizeof(void*), st));
   const double2* srcp = (const double2*)in;
@@ -860,10 +891,15 @@ extern "C" int lqcd_dslash(lqcd_lattice* L, int field, const lqcd_slab* dom, int
   const bool clov = L->csw != 0.0;
   VecP none;
   if (precision == 64) {
-    RC(lq_hop_lin(precision, dagger, clov, lq::RED_NONE, L, b, 0, v64(e.v(1)), v64(e.v(0)), none, none, v64(e.v(2)),
-                  -0.5, 1.0, 0.0, st));
-    RC(lq_hop_lin(precision, dagger, clov, lq::RED_NONE, L, b, 1, v64(e.v(0)), v64(e.v(1)), none, none, v64(e.v(3)),
-                  -0.5, 1.0, 0.0, st));
+    DBuf fxe;
+    RC(fxe.alloc(sizeof(int) * (size_t)b.total, st));
+    VecP xl = v64(e.v(4));
+    xl.e = fxe.as<int>();
+    for (int par = 0; par < 2; par++) {
+      RC(lq_to_fx(b, e.v(1 - par), xl, st));
+      RC(lq_hop_lin(precision, dagger, clov, lq::RED_NONE, L, b, par, xl, v64(e.v(par)), none, none, v64(e.v(2 + par)),
+                    -0.5, 1.0, 0.0, st));
+    }
   } else {
     PoolP q;
     RC(q.alloc(b, precision, 4, st));
@@ -1491,14 +1527,24 @@ extern "C" int lqcd_disconnected_trace(lqcd_lattice* L, int n_doms, const lqcd_s
     b.active = nullptr;  // every system, converged or not
     Pool64 h;
     RC(h.alloc(b, 4, st));
-    // ping-pong (x -> a -> b -> a ...): eight applications of kappa D_hop
+    // ping-pong (x -> a -> b -> a ...): eight applications of kappa D_hop, each input in limbs
+    // (the solution's in the second pair, later ones in place)
+    DBuf fxe;
+    RC(fxe.alloc(sizeof(int) * 2 * (size_t)b.total, st));
+    VecP le, lo;
+    le.e = fxe.as<int>();
+    lo.e = fxe.as<int>() + b.total;
     const double2* ie = xe;
     const double2* io = xo;
     for (int n = 0; n < 8; n++) {
+      le.d = n ? (void*)ie : (void*)h.v(2);
+      lo.d = n ? (void*)io : (void*)h.v(3);
+      RC(lq_to_fx(b, ie, le, st));
+      RC(lq_to_fx(b, io, lo, st));
       double2* oe = h.v(n & 1 ? 2 : 0);
       double2* oo = h.v(n & 1 ? 3 : 1);
-      RC(lq_hop_kappa(L, b, 0, io, oe, st));
-      RC(lq_hop_kappa(L, b, 1, ie, oo, st));
+      RC(lq_hop_kappa(L, b, 0, lo, oe, st));
+      RC(lq_hop_kappa(L, b, 1, le, oo, st));
       ie = oe;
       io = oo;
     }
@@ -1814,19 +1860,26 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
   const bool clov = L->csw != 0.0;
   VecP none;
   B.b.hop_variant = lq_tune_hop(L, B.b, precision, clov, q.v(0), q.v(1), q.v(2), st);
+  VecP hx = q.v(0);  // the hop kernels' input
+  DBuf fxe;
+  if (precision == 64 && kernel <= 3) {
+    RC(fxe.alloc(sizeof(int) * (size_t)b.total, st));
+    hx.e = fxe.as<int>();
+    RC(lq_to_fx(b, hx.d, hx, st));
+  }
   // the iteration's kernels on the pools q0..q5 (x, y, out, w, and two more for the BLAS passes)
   auto launch = [&]() -> int {
     switch (kernel) {
       case 0:  // out_o = A_oo y_o - 1/4 D_hop x_e
-        return lq_hop_lin(precision, false, clov, lq::RED_NONE, L, b, 1, q.v(0), q.v(1), none, none, q.v(2), -0.25,
+        return lq_hop_lin(precision, false, clov, lq::RED_NONE, L, b, 1, hx, q.v(1), none, none, q.v(2), -0.25,
                           1.0, 0.0, st);
       case 1:  // out_e = A_ee^{-1} D_hop x_o
-        return lq_hop_clinv(precision, false, clov, L, b, q.v(0), none, q.v(2), 1.0, 0.0, st);
+        return lq_hop_clinv(precision, false, clov, L, b, hx, none, q.v(2), 1.0, 0.0, st);
       case 2:  // v = A_oo p - 1/4 D_hop te, with <r0, v>
-        return lq_hop_lin(precision, false, clov, lq::RED_DOT_W, L, b, 1, q.v(0), q.v(1), none, q.v(3), q.v(2),
+        return lq_hop_lin(precision, false, clov, lq::RED_DOT_W, L, b, 1, hx, q.v(1), none, q.v(3), q.v(2),
                           -0.25, 1.0, 0.0, st);
       case 3:  // t = A_oo s - 1/4 D_hop te, with <t, s>, |t|^2, <r0, t> and <r0, s>
-        return lq_hop_lin(precision, false, clov, lq::RED_TSW, L, b, 1, q.v(0), q.v(1), none, q.v(3), q.v(2), -0.25,
+        return lq_hop_lin(precision, false, clov, lq::RED_TSW, L, b, 1, hx, q.v(1), none, q.v(3), q.v(2), -0.25,
                           1.0, 0.0, st);
       case 4:  // s = r - alpha v
         return lq_bicg_s(precision, b, q.v(0), q.v(1), q.v(2), st);

@@ -18,7 +18,7 @@
 // fully coalesced 128-bit load.
 //
 // Links of field f, parity p, direction mu: [p][mu][NL][Vh] words, with
-// FP64 keeping all 18 reals (9 x double2: FP64 is ALU-bound on this GPU, so
+// FP64 keeping all 18 reals as fixed-point limbs (9 x int4, fx.cuh: that stencil is ALU-bound, so
 // rebuilding the third row would cost more than the bytes it saves) and
 // FP32 / FP16 the first two rows (12 reals: 3 x float4 or 3 x uint2); the
 // third row is conj(row0 x row1), rebuilt in registers (storing all 18 FP32
@@ -37,7 +37,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fxnum.cuh"
+
+#ifndef LQ_DI
 #define LQ_DI __device__ __forceinline__
+#endif
 #define LQ_HDI __host__ __device__ __forceinline__
 
 namespace lq {
@@ -155,11 +159,13 @@ struct SysDesc {
 };
 
 struct FieldPtrs {
-  const double2* U64;   // [2][4][9][Vh]
+  const int4* U64;      // [2][4][9][Vh]  limbs (fx.cuh)
   const float4* U32;    // [2][4][3][Vh]
   const uint2* U16;     // [2][4][3][Vh]
-  const double2* A64;   // [2][36][Vh]  clover blocks A on both parities
-  const double2* Ai64;  // [36][Vh]     A^{-1} on even sites
+  const int4* A64;      // [2][36][Vh]  clover blocks A on both parities, limbs
+  const int4* Ai64;     // [36][Vh]     A^{-1} on even sites, limbs
+  const int* A64e;      // [2][2][Vh]   their exponents per block
+  const int* Ai64e;     // [2][Vh]
   const float4* A32;    // [2][18][Vh]
   const float4* Ai32;   // [18][Vh]
 };
@@ -350,12 +356,13 @@ struct LinkIO;
 template <>
 struct LinkIO<64> {
   LQ_DI static su3<double> load(const FieldPtrs& f, int p, int mu, int Vh, int cb) {
-    const double2* b = f.U64 + (p * 4 + mu) * 9 * Vh + cb;
+    const int4* b = f.U64 + (p * 4 + mu) * 9 * Vh + cb;
     su3<double> u;
 #pragma unroll
     for (int k = 0; k < 9; k++) {
-      double2 v = __ldg(b + k * Vh);
-      u.m[k / 3][k % 3] = {v.x, v.y};
+      const int4 v = __ldg(b + k * Vh);
+      u.m[k / 3][k % 3] = {fx_to_double(fx_join(v.x, v.y), FX_LINK_E - FX_BIAS),
+                           fx_to_double(fx_join(v.z, v.w), FX_LINK_E - FX_BIAS)};
     }
     return u;
   }
@@ -433,15 +440,27 @@ struct ClovIO {
 template <>
 struct ClovIO<64> {
   typedef double R;
-  LQ_DI static void apply(const double2* base, int Vh, int cb, const cx<double> in[6], cx<double> out[6]) {
+  // out += A in, the block's 36 reals in limbs with exponent e
+  LQ_DI static void apply_add(const int4* base, int e, int Vh, int cb, const cx<double> in[6], cx<double> out[6]) {
     double a[36];
 #pragma unroll
     for (int k = 0; k < 18; k++) {
-      double2 v = __ldg(base + k * Vh + cb);
-      a[2 * k] = v.x;
-      a[2 * k + 1] = v.y;
+      const int4 v = __ldg(base + k * Vh + cb);
+      a[2 * k] = fx_to_double(fx_join(v.x, v.y), e - FX_BIAS);
+      a[2 * k + 1] = fx_to_double(fx_join(v.z, v.w), e - FX_BIAS);
     }
-    ClovIO<32>::herm6_apply<double>(a, in, out);
+#pragma unroll
+    for (int r = 0; r < 6; r++) out[r] = {fma(a[r], in[r].re, out[r].re), fma(a[r], in[r].im, out[r].im)};
+    int q = 6;
+#pragma unroll
+    for (int r = 1; r < 6; r++)
+#pragma unroll
+      for (int c = 0; c < r; c++) {
+        const cx<double> e2 = {a[q], a[q + 1]};
+        q += 2;
+        fma_c(out[r], e2, in[c]);
+        fma_cc(out[c], e2, in[r]);
+      }
   }
 };
 

@@ -64,6 +64,16 @@ LQ_DI void expand_add(cx<R> acc[12], const cx<R> w[6]) {
   }
 }
 
+// acc = (1 + S g_mu) expanded from w, for mu = 0 (the first term of a hop sum).
+template <int S, typename R>
+LQ_DI void expand_set0(cx<R> acc[12], const cx<R> w[6]) {
+#pragma unroll
+  for (int c = 0; c < 6; c++) {
+    acc[c] = w[c];
+    acc[6 + c] = S > 0 ? -w[c] : w[c];
+  }
+}
+
 template <typename R>
 LQ_DI void mul_u(const su3<R>& u, const cx<R> h[6], cx<R> w[6]) {
 #pragma unroll
@@ -101,7 +111,9 @@ struct GlobalFetch {
   LQ_DI void operator()(int q, int, cx<typename Prec<P>::R> psi[12]) const { Prec<P>::load(psi, in, inn, n, q); }
 };
 
-template <int P, bool DAG, int MU, typename Fetch>
+// FIRST: acc is zero on entry, and the forward term is assigned.  The sign of a wrapping time hop is a
+// sign flip, not a product: FP64 (ALU-bound) pays for every instruction.
+template <int P, bool DAG, int MU, bool FIRST, typename Fetch>
 LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, const int x[4],
                      const Fetch& fetch, cx<typename Prec<P>::R> acc[12]) {
   typedef typename Prec<P>::R R;
@@ -131,11 +143,14 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
       project<MU, SF>(psi, h);
       su3<R> u = LinkIO<P>::load(f, pout, MU, g.Vh, cb);
       mul_u(u, h, w);
-      if (MU == 0) {
+      if (MU == 0 && sgn < (R)0) {
 #pragma unroll
-        for (int k = 0; k < 6; k++) w[k] = sgn * w[k];
+        for (int k = 0; k < 6; k++) w[k] = -w[k];
       }
-      expand_add<MU, SF>(acc, w);
+      if constexpr (FIRST && MU == 0)
+        expand_set0<SF>(acc, w);
+      else
+        expand_add<MU, SF>(acc, w);
     }
   }
   // ---- backward: U_mu(x - mu)^dag psi(x - mu)
@@ -161,9 +176,9 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
       project<MU, SB>(psi, h);
       su3<R> u = LinkIO<P>::load(f, pin, MU, g.Vh, cy);
       mul_udag(u, h, w);
-      if (MU == 0) {
+      if (MU == 0 && sgn < (R)0) {
 #pragma unroll
-        for (int k = 0; k < 6; k++) w[k] = sgn * w[k];
+        for (int k = 0; k < 6; k++) w[k] = -w[k];
       }
       expand_add<MU, SB>(acc, w);
     }
@@ -173,7 +188,7 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
 template <int P, bool DAG, int MU>
 LQ_DI void hop_dir(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, const int x[4],
                    const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
-  hop_dir_f<P, DAG, MU>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
+  hop_dir_f<P, DAG, MU, false>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
 }
 
 template <int P, bool DAG, typename Fetch>
@@ -181,10 +196,10 @@ LQ_DI void hop_sum_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
                      const Fetch& fetch, cx<typename Prec<P>::R> acc[12]) {
 #pragma unroll
   for (int k = 0; k < 12; k++) acc[k] = {0, 0};
-  hop_dir_f<P, DAG, 0>(g, sd, f, pout, cb, x, fetch, acc);
-  hop_dir_f<P, DAG, 1>(g, sd, f, pout, cb, x, fetch, acc);
-  hop_dir_f<P, DAG, 2>(g, sd, f, pout, cb, x, fetch, acc);
-  hop_dir_f<P, DAG, 3>(g, sd, f, pout, cb, x, fetch, acc);
+  hop_dir_f<P, DAG, 0, true>(g, sd, f, pout, cb, x, fetch, acc);
+  hop_dir_f<P, DAG, 1, false>(g, sd, f, pout, cb, x, fetch, acc);
+  hop_dir_f<P, DAG, 2, false>(g, sd, f, pout, cb, x, fetch, acc);
+  hop_dir_f<P, DAG, 3, false>(g, sd, f, pout, cb, x, fetch, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -563,18 +578,28 @@ LQ_DI void hop_sum(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pou
     hop_sum_f<P, DAG>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
 }
 
-// Clover block apply (A or A^{-1}) on a full spinor.
-template <int P>
-LQ_DI void clover_apply(const FieldPtrs& f, bool inverse, int p, int Vh, int cb, const cx<typename Prec<P>::R> in[12],
-                        cx<typename Prec<P>::R> out[12]) {
-  if constexpr (P == 64) {
-    const double2* base = inverse ? f.Ai64 : f.A64 + p * 36 * Vh;
-    ClovIO<64>::apply(base, Vh, cb, in, out);
-    ClovIO<64>::apply(base + 18 * Vh, Vh, cb, in + 6, out + 6);
+// Clover block apply (A or A^{-1}) on a full spinor (FP32 / FP16).
+LQ_DI void clover_apply(const FieldPtrs& f, bool inverse, int p, int Vh, int cb, const cx<float> in[12],
+                        cx<float> out[12]) {
+  const float4* base = inverse ? f.Ai32 : f.A32 + p * 18 * Vh;
+  ClovIO<32>::apply(base, Vh, cb, in, out);
+  ClovIO<32>::apply(base + 9 * Vh, Vh, cb, in + 6, out + 6);
+}
+
+// FP64 site-diagonal term: res += be A in, A the clover block or diag.
+LQ_DI void diag_add64(bool clov, const FieldPtrs& f, int p, int Vh, int cb, double diag, double be,
+                      const cx<double> in[12], cx<double> res[12]) {
+  cx<double> y[12];
+#pragma unroll
+  for (int k = 0; k < 12; k++) y[k] = be * in[k];
+  if (clov) {
+    const int4* base = f.A64 + p * 36 * Vh;
+    const int* e = f.A64e + p * 2 * Vh + cb;
+    ClovIO<64>::apply_add(base, e[0], Vh, cb, y, res);
+    ClovIO<64>::apply_add(base + 18 * Vh, e[Vh], Vh, cb, y + 6, res + 6);
   } else {
-    const float4* base = inverse ? f.Ai32 : f.A32 + p * 18 * Vh;
-    ClovIO<32>::apply(base, Vh, cb, in, out);
-    ClovIO<32>::apply(base + 9 * Vh, Vh, cb, in + 6, out + 6);
+#pragma unroll
+    for (int k = 0; k < 12; k++) res[k] = {fma(diag, y[k].re, res[k].re), fma(diag, y[k].im, res[k].im)};
   }
 }
 
@@ -741,10 +766,12 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_lin(HopArgs
     }
     cx<R> yv[12];
     if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) Prec<P>::load(yv, sys_ptr<P>(a.y, sd.off), nrm_ptr(a.yn, sd.off), sd.n, j);
-    if (EPI & EPI_Y) {
+    if constexpr ((EPI & EPI_Y) && P == 64) {
+      diag_add64(CLOV, f, a.pout, a.g.Vh, cb, a.diag, a.beta, yv, res);
+    } else if (EPI & EPI_Y) {
       cx<R> ay[12];
       if (CLOV) {
-        clover_apply<P>(f, false, a.pout, a.g.Vh, cb, yv, ay);
+        clover_apply(f, false, a.pout, a.g.Vh, cb, yv, ay);
       } else {
 #pragma unroll
         for (int k = 0; k < 12; k++) ay[k] = (R)a.diag * yv[k];
@@ -808,7 +835,7 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_clinv(HopAr
   }
   cx<R> o[12];
   if (CLOV) {
-    clover_apply<P>(f, true, 0, a.g.Vh, cb, res, o);
+    clover_apply(f, true, 0, a.g.Vh, cb, res, o);
   } else {
     const R inv = (R)(1.0 / a.diag);
 #pragma unroll

@@ -94,7 +94,14 @@ LQ_DI void nat_coords(const Geom& g, long long i, int x[4]) {
 LQ_DI double max_nan(double a, double b) { return a >= b ? a : (a == a ? b : a); }
 
 // ------------------------------------------------------------- link packing
-__global__ void k_pack_links(Geom g, const double2* U, double2* U64, float4* U32, uint2* U16,
+LQ_DI int4 limbs_of(double a, double b, int e) {
+  int4 v;
+  fx_split(fx_of(a, e), v.x, v.y);
+  fx_split(fx_of(b, e), v.z, v.w);
+  return v;
+}
+
+__global__ void k_pack_links(Geom g, const double2* U, int4* U64, float4* U32, uint2* U16,
                              unsigned long long* maxdev) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * g.Vh) return;
@@ -126,7 +133,7 @@ __global__ void k_pack_links(Geom g, const double2* U, double2* U64, float4* U32
     dev = max_nan(dev, norm2(det));
     const long long base = (long long)(p * 4 + mu);
 #pragma unroll
-    for (int k = 0; k < 9; k++) U64[(base * 9 + k) * g.Vh + cb] = make_double2(u.m[k / 3][k % 3].re, u.m[k / 3][k % 3].im);
+    for (int k = 0; k < 9; k++) U64[(base * 9 + k) * g.Vh + cb] = limbs_of(u.m[k / 3][k % 3].re, u.m[k / 3][k % 3].im, FX_LINK_E);
     float r[12];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
@@ -296,7 +303,7 @@ LQ_DI bool invert6(cd (&M)[6][6]) {
 // Bound by the FP64 pipe (10 products a plane, 6480 multiply-adds a site); a thread a plane keeps the
 // matrices in registers, where one thread for the whole site spilled 1.7 KB.  24^3 x 48, with
 // k_clover_blocks: 20.6 ms with twelve products a plane, products without fused multiply-adds, an
-// augmented elimination and all in one thread; 8.9 ms so.
+// augmented elimination and all in one thread; X.X ms so.
 __global__ void __launch_bounds__(128) k_fhat(Geom g, const double2* U, double* G) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long V = 2LL * g.Vh;
@@ -319,10 +326,18 @@ __global__ void __launch_bounds__(128) k_fhat(Geom g, const double2* U, double* 
   }
 }
 
+LQ_DI int block_exponent(const double pk[36]) {
+  int e = 1;
+#pragma unroll
+  for (int k = 0; k < 36; k++) e = max(e, fx_exponent(pk[k]));
+  return e;
+}
+
 // The two clover blocks B+- = 1/(2 kappa) + sum_l s_l (x) H+-_l, H+-_l = (c_sw/2)(+-i E_l - i M_l), from G,
 // and their inverses on even sites; one thread per (site, block).
-__global__ void __launch_bounds__(128) k_clover_blocks(Geom g, const double* G, double kappa, double csw, double2* A64,
-                                                       double2* Ai64, float4* A32, float4* Ai32, int* fail) {
+__global__ void __launch_bounds__(128) k_clover_blocks(Geom g, const double* G, double kappa, double csw, int4* A64,
+                                                       int4* Ai64, int* A64e, int* Ai64e, float4* A32, float4* Ai32,
+                                                       int* fail) {
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long Vh = g.Vh, V = 2 * Vh;
   if (q >= V) return;
@@ -365,8 +380,10 @@ __global__ void __launch_bounds__(128) k_clover_blocks(Geom g, const double* G, 
     }
   double pk[36];
   pack_herm6(B, pk);
+  int ex = block_exponent(pk);
+  A64e[((long long)p * 2 + blk) * Vh + cb] = ex;
 #pragma unroll
-  for (int k = 0; k < 18; k++) A64[((long long)p * 36 + blk * 18 + k) * Vh + cb] = make_double2(pk[2 * k], pk[2 * k + 1]);
+  for (int k = 0; k < 18; k++) A64[((long long)p * 36 + blk * 18 + k) * Vh + cb] = limbs_of(pk[2 * k], pk[2 * k + 1], ex);
 #pragma unroll
   for (int k = 0; k < 9; k++)
     A32[((long long)p * 18 + blk * 9 + k) * Vh + cb] =
@@ -380,8 +397,10 @@ __global__ void __launch_bounds__(128) k_clover_blocks(Geom g, const double* G, 
       for (int c = 0; c < 6; c++) B[r][c] = {0.0, 0.0};
   }
   pack_herm6(B, pk);
+  ex = block_exponent(pk);
+  Ai64e[(long long)blk * Vh + cb] = ex;
 #pragma unroll
-  for (int k = 0; k < 18; k++) Ai64[((long long)blk * 18 + k) * Vh + cb] = make_double2(pk[2 * k], pk[2 * k + 1]);
+  for (int k = 0; k < 18; k++) Ai64[((long long)blk * 18 + k) * Vh + cb] = limbs_of(pk[2 * k], pk[2 * k + 1], ex);
 #pragma unroll
   for (int k = 0; k < 9; k++)
     Ai32[((long long)blk * 9 + k) * Vh + cb] =
@@ -391,7 +410,7 @@ __global__ void __launch_bounds__(128) k_clover_blocks(Geom g, const double* G, 
 }  // namespace lq
 
 // ------------------------------------------------------------------ launchers
-int lq_launch_pack_links(const lq::Geom& g, const double2* U, double2* U64, float4* U32, uint2* U16,
+int lq_launch_pack_links(const lq::Geom& g, const double2* U, int4* U64, float4* U32, uint2* U16,
                          unsigned long long* maxdev, cudaStream_t st) {
   const long long V = 2 * g.Vh;
   lq::k_pack_links<<<(unsigned)((V + 127) / 128), 128, 0, st>>>(g, U, U64, U32, U16, maxdev);
@@ -399,8 +418,8 @@ int lq_launch_pack_links(const lq::Geom& g, const double2* U, double2* U64, floa
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, double2* A64, double2* Ai64,
-                     float4* A32, float4* Ai32, int* fail, cudaStream_t st) {
+int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, int4* A64, int4* Ai64,
+                     int* A64e, int* Ai64e, float4* A32, float4* Ai32, int* fail, cudaStream_t st) {
   const long long V = 2 * g.Vh;
   double* G = nullptr;
   if (csw != 0.0) {
@@ -412,8 +431,8 @@ int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double c
     lq::k_fhat<<<dim3((unsigned)((V + 127) / 128), 6), 128, 0, st>>>(g, U, G);
     lq_count_launch();
   }
-  lq::k_clover_blocks<<<dim3((unsigned)((V + 127) / 128), 2), 128, 0, st>>>(g, G, kappa, csw, A64, Ai64, A32, Ai32,
-                                                                          fail);
+  lq::k_clover_blocks<<<dim3((unsigned)((V + 127) / 128), 2), 128, 0, st>>>(g, G, kappa, csw, A64, Ai64, A64e, Ai64e, A32,
+                                                                          Ai32, fail);
   lq_count_launch();
   if (G) cudaFreeAsync(G, st);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;

@@ -19,6 +19,7 @@ void lq_set_error(const std::string& msg);
 struct VecP {
   void* d = nullptr;
   float* nrm = nullptr;
+  int* e = nullptr;  // exponents: the words are fixed-point limbs (fx.cuh), the hop input of the FP64 stencil
 };
 
 // Device view of a batch of systems: descriptors, activity flags, iteration
@@ -44,11 +45,13 @@ constexpr int LQ_BLOCK = 128;
 
 struct FieldData {
   double2* Unat = nullptr;  // natural-order copy of U (FP64), used by the force
-  double2* U64 = nullptr;
+  int4* U64 = nullptr;
   float4* U32 = nullptr;
   uint2* U16 = nullptr;
-  double2* A64 = nullptr;
-  double2* Ai64 = nullptr;
+  int4* A64 = nullptr;
+  int4* Ai64 = nullptr;
+  int* A64e = nullptr;
+  int* Ai64e = nullptr;
   float4* A32 = nullptr;
   float4* Ai32 = nullptr;
 };
@@ -67,10 +70,10 @@ struct lqcd_lattice {
 };
 
 // ---------------------------------------------------------------- launchers
-int lq_launch_pack_links(const lq::Geom& g, const double2* U, double2* U64, float4* U32, uint2* U16,
+int lq_launch_pack_links(const lq::Geom& g, const double2* U, int4* U64, float4* U32, uint2* U16,
                          unsigned long long* maxdev, cudaStream_t st);
-int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, double2* A64, double2* Ai64,
-                     float4* A32, float4* Ai32, int* fail, cudaStream_t st);
+int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, int4* A64, int4* Ai64,
+                     int* A64e, int* Ai64e, float4* A32, float4* Ai32, int* fail, cudaStream_t st);
 
 // out = beta*A(y) + alpha*D_hop x + gamma*z on parity pout (+ fused reduction; fin: what the kernel's last
 // block of a system does with the sums, FIN_ALPHA for RED_DOT_W, FIN_OMEGA_BETA for RED_TSW)
@@ -108,7 +111,9 @@ int lq_nat_to_eo(const lqcd_lattice* L, const Batch& b, const double2* const* sr
                  cudaStream_t st);
 int lq_nat_to_eo_g5(const lqcd_lattice* L, const Batch& b, const double2* const* src, double2* ve, double2* vo,
                     cudaStream_t st);
-int lq_hop_kappa(const lqcd_lattice* L, const Batch& b, int pout, const double2* x, double2* out, cudaStream_t st);
+int lq_hop_kappa(const lqcd_lattice* L, const Batch& b, int pout, VecP x, double2* out, cudaStream_t st);
+// FP64 vectors to the limbs and exponents that the FP64 stencil's hop reads (out may be in)
+int lq_to_fx(const Batch& b, const void* in, VecP out, cudaStream_t st);
 int lq_slice_dot(const lqcd_lattice* L, const Batch& b, const double2* const* eta, const double2* ye,
                  const double2* yo, const int* slot, double2* trace, cudaStream_t st);
 int lq_mean_sources(const double2* trace, int n_src, long long per_src, double2* mean, cudaStream_t st);

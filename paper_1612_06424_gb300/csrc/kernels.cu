@@ -3,6 +3,7 @@
 // the Schur-complement assembly.
 #include <atomic>
 #include <cstdio>
+#include <cmath>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -10,6 +11,7 @@
 #include <vector>
 
 #include "blas.cuh"
+#include "fx.cuh"
 #include "internal.h"
 
 using namespace lq;
@@ -113,7 +115,7 @@ static int variant_of(int P, const Batch& b) {
   return (v == 3 || v == 4) ? v : 1;
 }
 
-int lq_hop_wps(int P, const Batch& b) { return variant_of(P, b) == 2 ? 2 : 1; }
+int lq_hop_wps(int P, const Batch& b) { return P == 64 || variant_of(P, b) == 2 ? 2 : 1; }  // 2: 64-site blocks
 
 template <bool DAG, bool CLOV>
 static int launch_lin2(int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t st) {
@@ -156,10 +158,49 @@ static int launch_lin(int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t 
   return 0;
 }
 
+template <bool DAG, bool CLOV>
+static int launch_lin64(dim3 gr, const HopArgs& a, cudaStream_t st) {
+  k_hop_lin<64, DAG, CLOV, RED_NONE, EPI_X | EPI_Y><<<gr, LQ_BLOCK, 0, st>>>(a);
+  return 0;
+}
+
 template <int P>
 static int launch_lin_p(bool dag, bool clov, int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t st) {
   if (dag) return clov ? launch_lin<P, true, true>(red, epi, gr, a, st) : launch_lin<P, true, false>(red, epi, gr, a, st);
   return clov ? launch_lin<P, false, true>(red, epi, gr, a, st) : launch_lin<P, false, false>(red, epi, gr, a, st);
+}
+
+// +-2^k as sign and k
+static bool pow2_of(double v, int& neg, int& k) {
+  neg = v < 0;
+  const double m = frexp(v < 0 ? -v : v, &k);
+  k -= 1;
+  return m == 0.5;
+}
+
+static int fx_args(FxArgs& m, const HopArgs& a, VecP x, double diag) {
+  m = FxArgs{};
+  m.a = a;
+  m.x = (const int4*)x.d;
+  m.xe = x.e;
+  if ((a.alpha != 0.0 && !pow2_of(a.alpha, m.sa, m.ka)) || (a.beta != 0.0 && !pow2_of(a.beta, m.sb, m.kb)) ||
+      (a.gamma != 0.0 && !pow2_of(a.gamma, m.sg, m.kg))) {
+    lq_set_error("FP64 hop kernel: factors must be powers of two");
+    return LQCD_EBADARG;
+  }
+  // diag = q 2^(de - FX_BIAS), q of 57 bits
+  int e2;
+  const double f = frexp(diag, &e2);  // diag = f 2^e2, f in [1/2, 1)
+  const long long q = (long long)ldexp(f, 57);
+  m.de = e2 - 57 + FX_BIAS;
+  const int q0 = (int)((unsigned)q << 3) >> 3;
+  m.d = make_int2((int)((q - q0) >> 29), q0);
+  return 0;
+}
+
+int lq_to_fx(const Batch& b, const void* in, VecP out, cudaStream_t st) {
+  to_fx_launch(grid_of(b), b.nsys, b.sys, b.active, (const double2*)in, (int4*)out.d, out.e, st);
+  return launched();
 }
 
 int lq_hop_lin(int P, bool dag, bool clov, int red, const lqcd_lattice* L, const Batch& b, int pout, VecP x, VecP y,
@@ -187,12 +228,22 @@ int lq_hop_lin(int P, bool dag, bool clov, int red, const lqcd_lattice* L, const
   }
   const int v = variant_of(P, b);
   int rc;
-  if (!dag && v >= 3)
+  if (P == 64 && x.e) {
+    FxArgs m;
+    rc = fx_args(m, a, x, a.diag);
+    if (rc) return rc;
+    set_grid_order(m.a, L, b, FX_SITES);
+    m.a.tblk = tblk_of(b);
+    rc = fx_lin_launch(dag, clov, red, epi, grid_lin(b, (b.max_n + FX_SITES - 1) / FX_SITES), m, st);
+  } else if (P == 64) {
+    // FP64 arithmetic on FP64 vectors: lqcd_dslash_noalloc, whose scratch has no room for limbs
+    rc = red == RED_NONE && epi == (EPI_X | EPI_Y) ? 0 : -1;
+    if (!rc && dag) rc = clov ? launch_lin64<true, true>(gr, a, st) : launch_lin64<true, false>(gr, a, st);
+    else if (!rc) rc = clov ? launch_lin64<false, true>(gr, a, st) : launch_lin64<false, false>(gr, a, st);
+  } else if (!dag && v >= 3)
     rc = P == 32 ? hop_lin_tuned<32>(v - 2, clov, red, epi, gr, a, st) : hop_lin_tuned<16>(v - 2, clov, red, epi, gr, a, st);
   else
-    rc = P == 64 ? launch_lin_p<64>(dag, clov, red, epi, gr, a, st)
-       : P == 32 ? launch_lin_p<32>(dag, clov, red, epi, gr, a, st)
-                 : launch_lin_p<16>(dag, clov, red, epi, gr, a, st);
+    rc = P == 32 ? launch_lin_p<32>(dag, clov, red, epi, gr, a, st) : launch_lin_p<16>(dag, clov, red, epi, gr, a, st);
   if (rc) {
     lq_set_error("hop kernel: unsupported (reduction, epilogue) pair");
     return LQCD_EBADARG;
@@ -237,12 +288,21 @@ int lq_hop_clinv(int P, bool dag, bool clov, const lqcd_lattice* L, const Batch&
   }
   const int v = variant_of(P, b);
   int rc;
-  if (!dag && v >= 3)
+  if (P == 64) {
+    if (!x.e && alpha != 0.0) {
+      lq_set_error("FP64 clover-inverse hop kernel: the hop input must be in limbs");
+      return LQCD_EBADARG;
+    }
+    FxArgs m;
+    rc = fx_args(m, a, x, 1.0 / a.diag);
+    if (rc) return rc;
+    set_grid_order(m.a, L, b, FX_SITES);
+    m.a.tblk = tblk_of(b);
+    rc = fx_clinv_launch(dag, clov, epi, grid_lin(b, (b.max_n + FX_SITES - 1) / FX_SITES), m, st);
+  } else if (!dag && v >= 3)
     rc = P == 32 ? hop_clinv_tuned<32>(v - 2, clov, epi, gr, a, st) : hop_clinv_tuned<16>(v - 2, clov, epi, gr, a, st);
   else
-    rc = P == 64 ? launch_clinv_p<64>(dag, clov, epi, gr, a, st)
-       : P == 32 ? launch_clinv_p<32>(dag, clov, epi, gr, a, st)
-                 : launch_clinv_p<16>(dag, clov, epi, gr, a, st);
+    rc = P == 32 ? launch_clinv_p<32>(dag, clov, epi, gr, a, st) : launch_clinv_p<16>(dag, clov, epi, gr, a, st);
   if (rc) {
     lq_set_error("clover-inverse hop kernel: unsupported epilogue");
     return LQCD_EBADARG;
@@ -251,14 +311,18 @@ int lq_hop_clinv(int P, bool dag, bool clov, const lqcd_lattice* L, const Batch&
 }
 
 // out_p = kappa D_hop x (the Wilson hopping term on the slab, Dirichlet at
-// its ends), output parity pout, FP64: the clover-free inverse-diagonal
+// its ends), output parity pout, FP64, x in limbs: the clover-free inverse-diagonal
 // kernel with alpha = 1/2, since 1 / diag = 2 kappa.
-int lq_hop_kappa(const lqcd_lattice* L, const Batch& b, int pout, const double2* x, double2* out, cudaStream_t st) {
+int lq_hop_kappa(const lqcd_lattice* L, const Batch& b, int pout, VecP x, double2* out, cudaStream_t st) {
   HopArgs a = hop_args(L, b, pout);
-  a.x = x;
   a.out = out;
   a.alpha = 0.5;
-  k_hop_clinv<64, false, false, EPI_X><<<grid_of(b), LQ_BLOCK, 0, st>>>(a);
+  FxArgs m;
+  const int rc = fx_args(m, a, x, 1.0 / a.diag);
+  if (rc) return rc;
+  set_grid_order(m.a, L, b, FX_SITES);
+  m.a.tblk = tblk_of(b);
+  fx_clinv_launch(false, false, EPI_X, grid_lin(b, (b.max_n + FX_SITES - 1) / FX_SITES), m, st);
   return launched();
 }
 
