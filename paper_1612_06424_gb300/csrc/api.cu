@@ -832,7 +832,7 @@ extern "C" int lqcd_set_gauge(lqcd_lattice* L, int n_fields, const double* U, do
     CK(cudaMemsetAsync(dev.p, 0, sizeof(unsigned long long), st));
     CK(cudaMemsetAsync(fail.p, 0, sizeof(int), st));
     RC(lq_launch_pack_links(L->g, src, F.U64, F.U32, F.U16, dev.as<unsigned long long>(), st));
-    RC(lq_launch_clover(L->g, src, kappa, c_sw, F.A64, F.Ai64, F.A64e, F.Ai64e, F.A32, F.Ai32, fail.as<int>(), st));
+    RC(lq_launch_clover(L->g, F.U64, kappa, c_sw, F.A64, F.Ai64, F.A64e, F.Ai64e, F.A32, F.Ai32, fail.as<int>(), st));
     unsigned long long d = 0;
     int fl = 0;
     CK(cudaMemcpyAsync(&d, dev.p, sizeof(d), cudaMemcpyDeviceToHost, st));

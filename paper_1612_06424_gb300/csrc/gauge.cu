@@ -31,52 +31,6 @@ LQ_DI su3<double> ld_nat(const double2* U, long long i, int mu) {
   return u;
 }
 
-LQ_DI su3<double> mm(const su3<double>& a, const su3<double>& b) {
-  su3<double> r;
-#pragma unroll
-  for (int i = 0; i < 3; i++)
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-      cd t = a.m[i][0] * b.m[0][j];
-      fma_c(t, a.m[i][1], b.m[1][j]);
-      fma_c(t, a.m[i][2], b.m[2][j]);
-      r.m[i][j] = t;
-    }
-  return r;
-}
-
-// a * b^dag
-LQ_DI su3<double> mmd(const su3<double>& a, const su3<double>& b) {
-  su3<double> r;
-#pragma unroll
-  for (int i = 0; i < 3; i++)
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-      cd t = {0, 0};
-#pragma unroll
-      for (int k = 0; k < 3; k++) fma_cc(t, b.m[j][k], a.m[i][k]);
-      r.m[i][j] = t;
-    }
-  return r;
-}
-
-// r - a^dag * b
-LQ_DI su3<double> sub_mdm(su3<double> r, const su3<double>& a, const su3<double>& b) {
-#pragma unroll
-  for (int i = 0; i < 3; i++)
-#pragma unroll
-    for (int j = 0; j < 3; j++)
-#pragma unroll
-      for (int k = 0; k < 3; k++) {  // r -= conj(a_ki) b_kj
-        cd& t = r.m[i][j];
-        t.re = fma(-a.m[k][i].re, b.m[k][j].re, t.re);
-        t.re = fma(-a.m[k][i].im, b.m[k][j].im, t.re);
-        t.im = fma(-a.m[k][i].re, b.m[k][j].im, t.im);
-        t.im = fma(a.m[k][i].im, b.m[k][j].re, t.im);
-      }
-  return r;
-}
-
 LQ_DI long long nat_index(const Geom& g, const int x[4]) {
   return (((long long)x[0] * g.L[1] + x[1]) * g.L[2] + x[2]) * g.L[3] + x[3];
 }
@@ -154,16 +108,80 @@ __global__ void k_pack_links(Geom g, const double2* U, int4* U64, float4* U32, u
 }
 
 // ------------------------------------------------------------------ clover
-LQ_DI su3<double> link_bc(const Geom& g, const double2* U, const int x[4], int mu) {
+// 3x3 complex matrices in fixed point (fxnum.cuh): entries q 2^-58 in limbs, as the links are stored.  A
+// product is 27 complex multiply-adds of 12 integer ones each, a tenth of the time of the FP64
+// product, and its entries are rounded at 2^-58 (FP64 rounds an entry of size 1 at 2^-53).
+struct mcl {
+  int4 m[3][3];  // (re1, re0, im1, im0)
+};
+
+LQ_DI mcl link_bc(const Geom& g, const int4* U, const int x[4], int mu) {
+  mcl u;
   if (g.bc_t == 0 && mu == 0 && x[0] == g.L[0] - 1) {
-    su3<double> z;
 #pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-      for (int b = 0; b < 3; b++) z.m[a][b] = {0, 0};
-    return z;
+    for (int k = 0; k < 9; k++) u.m[k / 3][k % 3] = make_int4(0, 0, 0, 0);
+    return u;
   }
-  return ld_nat(U, nat_index(g, x), mu);
+  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+  const int4* b = U + (long long)(p * 4 + mu) * 9 * g.Vh + eo_index(g, x);
+#pragma unroll
+  for (int k = 0; k < 9; k++) u.m[k / 3][k % 3] = __ldg(b + (long long)k * g.Vh);
+  return u;
+}
+
+LQ_DI void mc_mac(long long& hh, long long& cr, int a1, int a0, int b1, int b0) {
+  mad_wide(hh, a1, b1);
+  mad_wide(cr, a1, b0);
+  mad_wide(cr, a0, b1);
+}
+// entry of a product as 64-bit integers: sum over k of a_k b_k with the imaginary part of a (CA) or b (CB) negated
+template <bool CA, bool CB>
+LQ_DI longlong2 mc_dot(const int4 (&a)[3], const int4 (&b)[3]) {
+  long long hr = 0, cr = 1ll << 28, hi = 0, ci = 1ll << 28;  // (the halves round the shifts below)
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const int ai1 = CA ? -a[k].z : a[k].z, ai0 = CA ? -a[k].w : a[k].w;
+    const int bi1 = CB ? -b[k].z : b[k].z, bi0 = CB ? -b[k].w : b[k].w;
+    mc_mac(hr, cr, a[k].x, a[k].y, b[k].x, b[k].y);
+    mc_mac(hr, cr, -ai1, -ai0, bi1, bi0);
+    mc_mac(hi, ci, a[k].x, a[k].y, bi1, bi0);
+    mc_mac(hi, ci, ai1, ai0, b[k].x, b[k].y);
+  }
+  return make_longlong2(hr + (cr >> 29), hi + (ci >> 29));
+}
+LQ_DI int4 mc_limbs(longlong2 q) {
+  int4 v;
+  fx_split(q.x, v.x, v.y);
+  fx_split(q.y, v.z, v.w);
+  return v;
+}
+LQ_DI longlong2 mm_ij(const mcl& a, const mcl& b, int i, int j) {  // (a b)_ij
+  const int4 r[3] = {a.m[i][0], a.m[i][1], a.m[i][2]}, c[3] = {b.m[0][j], b.m[1][j], b.m[2][j]};
+  return mc_dot<false, false>(r, c);
+}
+LQ_DI longlong2 mmd_ij(const mcl& a, const mcl& b, int i, int j) {  // (a b^dag)_ij
+  const int4 r[3] = {a.m[i][0], a.m[i][1], a.m[i][2]}, c[3] = {b.m[j][0], b.m[j][1], b.m[j][2]};
+  return mc_dot<false, true>(r, c);
+}
+LQ_DI longlong2 mdm_ij(const mcl& a, const mcl& b, int i, int j) {  // (a^dag b)_ij
+  const int4 r[3] = {a.m[0][i], a.m[1][i], a.m[2][i]}, c[3] = {b.m[0][j], b.m[1][j], b.m[2][j]};
+  return mc_dot<true, false>(r, c);
+}
+LQ_DI mcl mc_mul(const mcl& a, const mcl& b) {
+  mcl r;
+#pragma unroll
+  for (int k = 0; k < 9; k++) r.m[k / 3][k % 3] = mc_limbs(mm_ij(a, b, k / 3, k % 3));
+  return r;
+}
+// a p^dag - q^dag b
+LQ_DI mcl mc_staple(const mcl& a, const mcl& p, const mcl& q, const mcl& b) {
+  mcl r;
+#pragma unroll
+  for (int k = 0; k < 9; k++) {
+    const longlong2 x = mmd_ij(a, p, k / 3, k % 3), y = mdm_ij(q, b, k / 3, k % 3);
+    r.m[k / 3][k % 3] = mc_limbs(make_longlong2(x.x - y.x, x.y - y.y));
+  }
+  return r;
 }
 
 LQ_DI void shift(const Geom& g, const int x[4], int mu, int d, int y[4]) {
@@ -185,7 +203,8 @@ LQ_DI void shift(const Geom& g, const int x[4], int mu, int d, int y[4]) {
 // common outer link: ten products a plane instead of twelve.
 //   M = U_mu(x) { U_nu(x+mu) [U_nu(x) U_mu(x+nu)]^dag - [U_mu(x-nu) U_nu(x-nu+mu)]^dag U_nu(x-nu) }
 //     + { U_nu(x) [U_nu(x-mu) U_mu(x-mu+nu)]^dag - [U_mu(x-mu-nu) U_nu(x-nu)]^dag U_nu(x-mu-nu) } U_mu(x-mu)
-LQ_DI su3<double> fhat(const Geom& g, const double2* U, const int x[4], int mu, int nu) {
+// The result is 8 Fhat in units of 2^-58 (anti-Hermitian; the entries (i, j), i >= j, are filled in).
+LQ_DI void fhat(const Geom& g, const int4* U, const int x[4], int mu, int nu, longlong2 (&f)[3][3]) {
   int xpm[4], xpn[4], xmm[4], xmn[4], xmmpn[4], xmmmn[4], xmnpm[4];
   shift(g, x, mu, 1, xpm);
   shift(g, x, nu, 1, xpn);
@@ -194,28 +213,30 @@ LQ_DI su3<double> fhat(const Geom& g, const double2* U, const int x[4], int mu, 
   shift(g, xmm, nu, 1, xmmpn);
   shift(g, xmm, nu, -1, xmmmn);
   shift(g, xmn, mu, 1, xmnpm);
-  su3<double> q;
+  const mcl un = link_bc(g, U, xmn, nu);
+  const mcl t1 = mc_staple(link_bc(g, U, xpm, nu), mc_mul(link_bc(g, U, x, nu), link_bc(g, U, xpn, mu)),
+                           mc_mul(link_bc(g, U, xmn, mu), link_bc(g, U, xmnpm, nu)), un);
+  longlong2 q[3][3];
   {
-    const su3<double> un = link_bc(g, U, xmn, nu);
-    su3<double> t = mmd(link_bc(g, U, xpm, nu), mm(link_bc(g, U, x, nu), link_bc(g, U, xpn, mu)));
-    t = sub_mdm(t, mm(link_bc(g, U, xmn, mu), link_bc(g, U, xmnpm, nu)), un);
-    q = mm(link_bc(g, U, x, mu), t);
-    t = mmd(link_bc(g, U, x, nu), mm(link_bc(g, U, xmm, nu), link_bc(g, U, xmmpn, mu)));
-    t = sub_mdm(t, mm(link_bc(g, U, xmmmn, mu), un), link_bc(g, U, xmmmn, nu));
-    const su3<double> um = link_bc(g, U, xmm, mu);
+    const mcl u = link_bc(g, U, x, mu);
 #pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-      for (int b = 0; b < 3; b++)
-#pragma unroll
-        for (int k = 0; k < 3; k++) fma_c(q.m[a][b], t.m[a][k], um.m[k][b]);
+    for (int k = 0; k < 9; k++) q[k / 3][k % 3] = mm_ij(u, t1, k / 3, k % 3);
   }
-  su3<double> f;
+  const mcl t2 = mc_staple(link_bc(g, U, x, nu), mc_mul(link_bc(g, U, xmm, nu), link_bc(g, U, xmmpn, mu)),
+                           mc_mul(link_bc(g, U, xmmmn, mu), un), link_bc(g, U, xmmmn, nu));
+  {
+    const mcl u = link_bc(g, U, xmm, mu);
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+      const longlong2 v = mm_ij(t2, u, k / 3, k % 3);
+      q[k / 3][k % 3].x += v.x;
+      q[k / 3][k % 3].y += v.y;
+    }
+  }
 #pragma unroll
   for (int a = 0; a < 3; a++)
 #pragma unroll
-    for (int b = 0; b < 3; b++) f.m[a][b] = 0.125 * (q.m[a][b] - conj(q.m[b][a]));
-  return f;
+    for (int b = 0; b <= a; b++) f[a][b] = make_longlong2(q[a][b].x - q[b][a].x, q[a][b].y + q[b][a].y);
 }
 
 // Pack the 6x6 Hermitian block B into 36 reals: 6 diagonal, then the 15
@@ -300,11 +321,12 @@ LQ_DI bool invert6(cd (&M)[6][6]) {
 // i Fhat of one plane per thread (Hermitian: 3 real diagonal entries, then the entries (1,0), (2,0),
 // (2,1)), planes 0-2 = (0,1) (0,2) (0,3), 3-5 = (2,3) (3,1) (1,2), into G[plane * 9 + k][site].
 //
-// Bound by the FP64 pipe (10 products a plane, 6480 multiply-adds a site); a thread a plane keeps the
-// matrices in registers, where one thread for the whole site spilled 1.7 KB.  24^3 x 48, with
-// k_clover_blocks: 20.6 ms with twelve products a plane, products without fused multiply-adds, an
-// augmented elimination and all in one thread; X.X ms so.
-__global__ void __launch_bounds__(128) k_fhat(Geom g, const double2* U, double* G) {
+// 10 products of 3 x 3 matrices a plane in fixed point (2160 complex products a site and 6 planes), on the integer pipe: links
+// have |U| <= 1 and need no exponent.  A thread a plane keeps the matrices in registers, where one thread for the whole
+// site spilled 1.7 KB.  24^3 x 48, with k_clover_blocks: 20.6 ms with twelve products a plane, products
+// without fused multiply-adds, an augmented elimination and all in one thread; 8.9 ms with the ten products in FP64, at
+// the FP64 pipe's rate; 5.1 ms so (3.1 ms this kernel).
+__global__ void __launch_bounds__(128) k_fhat(Geom g, const int4* U, double* G) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long V = 2LL * g.Vh;
   if (i >= V) return;
@@ -314,15 +336,17 @@ __global__ void __launch_bounds__(128) k_fhat(Geom g, const double2* U, double* 
   const int pl = blockIdx.y;
   const int mu = pl < 3 ? 0 : (pl == 3 ? 2 : pl == 4 ? 3 : 1);
   const int nu = pl < 3 ? pl + 1 : (pl == 3 ? 3 : pl == 4 ? 1 : 2);
-  const su3<double> f = fhat(g, U, x, mu, nu);
+  longlong2 f[3][3];
+  fhat(g, U, x, mu, nu, f);
+  constexpr int EX = FX_LINK_E - FX_BIAS - 3;
   double* out = G + (long long)pl * 9 * V + (long long)p * g.Vh + (i >> 1);
 #pragma unroll
-  for (int a = 0; a < 3; a++) out[a * V] = -f.m[a][a].im;
+  for (int a = 0; a < 3; a++) out[a * V] = -fx_to_double(f[a][a].y, EX);
   const int ra[3] = {1, 2, 2}, rb[3] = {0, 0, 1};
 #pragma unroll
   for (int k = 0; k < 3; k++) {  // i f
-    out[(3 + 2 * k) * V] = -f.m[ra[k]][rb[k]].im;
-    out[(4 + 2 * k) * V] = f.m[ra[k]][rb[k]].re;
+    out[(3 + 2 * k) * V] = -fx_to_double(f[ra[k]][rb[k]].y, EX);
+    out[(4 + 2 * k) * V] = fx_to_double(f[ra[k]][rb[k]].x, EX);
   }
 }
 
@@ -418,7 +442,7 @@ int lq_launch_pack_links(const lq::Geom& g, const double2* U, int4* U64, float4*
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, int4* A64, int4* Ai64,
+int lq_launch_clover(const lq::Geom& g, const int4* U, double kappa, double csw, int4* A64, int4* Ai64,
                      int* A64e, int* Ai64e, float4* A32, float4* Ai32, int* fail, cudaStream_t st) {
   const long long V = 2 * g.Vh;
   double* G = nullptr;

@@ -72,7 +72,8 @@ struct lqcd_lattice {
 // ---------------------------------------------------------------- launchers
 int lq_launch_pack_links(const lq::Geom& g, const double2* U, int4* U64, float4* U32, uint2* U16,
                          unsigned long long* maxdev, cudaStream_t st);
-int lq_launch_clover(const lq::Geom& g, const double2* U, double kappa, double csw, int4* A64, int4* Ai64,
+// U: the packed links in limbs
+int lq_launch_clover(const lq::Geom& g, const int4* U, double kappa, double csw, int4* A64, int4* Ai64,
                      int* A64e, int* Ai64e, float4* A32, float4* Ai32, int* fail, cudaStream_t st);
 
 // out = beta*A(y) + alpha*D_hop x + gamma*z on parity pout (+ fused reduction; fin: what the kernel's last
