@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256, 2) k_nucleon_block(int n, long long nsite
 // that the transposed rows B_xi[k][i][j0..] are read as runs of 1 KB too), and one read of B_xi serves
 // CT_NY sink slices.  Part p of pair (ix, iy) goes to part[((ix ny + iy) nsplit + p) 4]; k_contract_sum
 // adds the parts in a fixed order.  120 factors, 8 sink slices: 38.7 ms with one block per pair of
-// slices, 0.61 ms so.
+// slices, 0.6 ms so.
 constexpr int CT = 16;     // edge of a (j, k) tile
 constexpr int CT_NY = 4;   // sink slices per block
 
@@ -320,38 +320,81 @@ __global__ void __launch_bounds__(256) k_level_mean(long long size, int count, d
 // (a0, b0, c) cyclic: the terms with a, b and both mu -> nu(mu), a' <-> b' exchanged are equal in
 // pairs, which removes the factor 1/2 of M and half of the products.
 //
-// Bound by the FP64 pipe (one warp instruction in about 16 clocks and SM): 6600 multiply-adds a
-// site in this factored form, where the plain sums over all terms take 70000.  A block stages 16
-// sites of one slice in shared memory and spreads their 16 x 144 elements H and 16 x 36 elements T
-// over its 128 threads (consecutive threads take the 8 rows (mu, a) of one (c, g, c'), so their
-// reads of V and Z are broadcasts and those of S nearly free of conflicts); three blocks an SM
-// overlap one another's loads.  Up to four stages of a block share its final sums.  Propagator of 64 x 24^3:
-// 114.8 ms with the plain sums, one warp a site, and 11.4 ms so.
+// The products run in fixed point on the integer pipe (fxnum.cuh, 32 times the FP64 pipe's rate): a
+// site's 144 entries become 57-bit integers with one exponent, H and T are 64-bit sums, and each H Z and T U
+// is rounded to FP64 once and summed there.  1620 complex multiply-adds a site in the factored form, where the
+// plain sums over all terms take 17000.  A block stages 16 sites of one slice in shared memory and
+// spreads their 16 x 144 elements H and 16 x 36 elements T over its 128 threads (consecutive threads
+// take the 8 rows (mu, a) of one (c, g, c'), so their reads of V and Z are broadcasts and those of S nearly
+// free of conflicts); three blocks an SM overlap one another's loads.  Up to four stages of a block share its
+// final sums.  Propagator of 64 x 24^3: 114.8 ms with the plain FP64 sums, one warp a site; 11.4 ms factored in
+// FP64; 5.6 ms so (error against long double 1.4e-16, of the FP64 sums 3.1e-16).
 constexpr int NP_T = 128;        // threads
 constexpr int NP_SITES = 16;     // sites staged at a time
 constexpr int NP_GROUPS = 4;     // most stages per block
 constexpr int NP_WORDS = 144 + 72 + 72;  // S, V and Z of a site
 constexpr int NP_SMEM = NP_SITES * NP_WORDS * 16;
 
-LQ_DI void cfma_d(double2& t, double2 a, double2 b) {  // t += a b
-  t.x = fma(a.x, b.x, t.x);
-  t.x = fma(-a.y, b.y, t.x);
-  t.y = fma(a.x, b.y, t.y);
-  t.y = fma(a.y, b.x, t.y);
+struct np_acc {  // sum of products of limbs: hh 2^58 + cr 2^29
+  long long hr, cr, hi, ci;
+};
+// t += (NEG ? - : +) a b
+template <bool NEG>
+LQ_DI void np_mac(np_acc& t, int4 a, int4 b) {
+  const int r1 = NEG ? -a.x : a.x, r0 = NEG ? -a.y : a.y, i1 = NEG ? -a.z : a.z, i0 = NEG ? -a.w : a.w;
+  mad_wide(t.hr, r1, b.x);
+  mad_wide(t.cr, r1, b.y);
+  mad_wide(t.cr, r0, b.x);
+  mad_wide(t.hr, -i1, b.z);
+  mad_wide(t.cr, -i1, b.w);
+  mad_wide(t.cr, -i0, b.z);
+  mad_wide(t.hi, r1, b.z);
+  mad_wide(t.ci, r1, b.w);
+  mad_wide(t.ci, r0, b.z);
+  mad_wide(t.hi, i1, b.x);
+  mad_wide(t.ci, i1, b.y);
+  mad_wide(t.ci, i0, b.x);
 }
-LQ_DI void cfms_d(double2& t, double2 a, double2 b) {  // t -= a b
-  t.x = fma(-a.x, b.x, t.x);
-  t.x = fma(a.y, b.y, t.x);
-  t.y = fma(-a.x, b.y, t.y);
-  t.y = fma(-a.y, b.x, t.y);
+// The sum as limbs of 57 bits, 2^-c of it (c < 0: a multiple).
+LQ_DI int4 np_limbs(const np_acc& t, int& c) {
+  const long long re = t.hr + ((t.cr + (1ll << 28)) >> 29), im = t.hi + ((t.ci + (1ll << 28)) >> 29);
+  const unsigned long long mag = (unsigned long long)((re ^ (re >> 63)) | (im ^ (im >> 63)));
+  c = mag ? 7 - __clzll((long long)mag) : 0;
+  const long long half = c > 0 ? 1ll << (c - 1) : 0;
+  int4 q;
+  fx_split(c > 0 ? (re + half) >> c : re << -c, q.x, q.y);
+  fx_split(c > 0 ? (im + half) >> c : im << -c, q.z, q.w);
+  return q;
+}
+LQ_DI int4 np_add(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+LQ_DI int4 np_sub(int4 a, int4 b) { return make_int4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+// sum over mu' = 0..3 of cg(mu') (s[nu(mu') b'] r[mu' a'] - s[nu(mu') a'] r[mu' b']), nu = 1, 0, 3, 2 and cg = -, +, -, +;
+// element (mu, c) of s at (3 mu + c) ls, of r at (3 mu + c) lr
+LQ_DI np_acc np_pair(const int4* s, int ls, const int4* r, int lr, int ap, int bp) {
+  np_acc t = {0, 0, 0, 0};
+#pragma unroll
+  for (int m = 0; m < 4; m++) {
+    const int nm = m ^ 1;
+    const int4 s0 = s[(3 * nm + bp) * ls], r0 = r[(3 * m + ap) * lr];
+    const int4 s1 = s[(3 * nm + ap) * ls], r1 = r[(3 * m + bp) * lr];
+    if (m & 1) {
+      np_mac<false>(t, s0, r0);
+      np_mac<true>(t, s1, r1);
+    } else {
+      np_mac<true>(t, s0, r0);
+      np_mac<false>(t, s1, r1);
+    }
+  }
+  return t;
 }
 
 __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, long long V, const double2* prop,
                                                            long long prop_stride, int t0, double2* partial) {
-  extern __shared__ __align__(16) double2 np_sm[];
-  double2* S = np_sm;                          // [site][column 3 nu + b][row 3 mu + a]
-  double2* Vv = S + NP_SITES * 144;            // [site][c][g][column]
-  double2* Z = Vv + NP_SITES * 72;             // [site][g][c'][row]
+  extern __shared__ __align__(16) int4 np_sm[];
+  int4* S = np_sm;                         // [site][column 3 nu + b][row 3 mu + a]
+  int4* Vv = S + NP_SITES * 144;           // [site][c][g][column]
+  int4* Z = Vv + NP_SITES * 72;            // [site][g][c'][row]
+  __shared__ int ex[NP_SITES];             // exponents of the sites' entries
   const int slice = blockIdx.y;
   const double2* P = prop + (long long)blockIdx.z * prop_stride + (long long)(t0 + slice) * S3 * 12;
   double2 w1 = make_double2(0.0, 0.0), w2 = make_double2(0.0, 0.0);
@@ -360,83 +403,78 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
     const int ns = min(NP_SITES, S3 - y0);
     if (ns <= 0) break;
     if (grp) __syncthreads();
+    if (threadIdx.x < NP_SITES) ex[threadIdx.x] = 1;
+    __syncthreads();
+    double2* Sd = reinterpret_cast<double2*>(S);
     for (int q = threadIdx.x; q < ns * 144; q += NP_T) {
       const int col = q / (ns * 12), r = q - col * (ns * 12);
       const int site = r / 12;
-      S[site * 144 + col * 12 + (r - site * 12)] = __ldg(P + ((long long)col * V + y0) * 12 + r);
+      const double2 v = __ldg(P + ((long long)col * V + y0) * 12 + r);
+      Sd[site * 144 + col * 12 + (r - site * 12)] = v;
+      atomicMax(&ex[site], max(fx_exponent(v.x), fx_exponent(v.y)));
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < ns * 144; q += NP_T) {  // in place
+      const int E = ex[q / 144];
+      const double2 v = Sd[q];
+      int4 l;
+      fx_split(fx_of(v.x, E), l.x, l.y);
+      fx_split(fx_of(v.y, E), l.z, l.w);
+      S[q] = l;
     }
     __syncthreads();
     for (int q = threadIdx.x; q < ns * 72; q += NP_T) {
       const int site = q / 72, e = q - site * 72;
       {  // V: e = (c, g, column)
         const int c = e / 24, g = (e / 12) & 1, col = e % 12;
-        const double2 a = S[site * 144 + col * 12 + 3 * g + c], b = S[site * 144 + col * 12 + 3 * g + 6 + c];
-        Vv[q] = make_double2(a.x + b.x, a.y + b.y);
+        Vv[q] = np_add(S[site * 144 + col * 12 + 3 * g + c], S[site * 144 + col * 12 + 3 * g + 6 + c]);
       }
       {  // Z: e = (g, c', row)
         const int g = e / 36, cp = (e / 12) % 3, row = e % 12;
-        const double2 a = S[site * 144 + (3 * g + cp) * 12 + row], b = S[site * 144 + (3 * g + 6 + cp) * 12 + row];
-        Z[q] = make_double2(a.x - b.x, a.y - b.y);
+        Z[q] = np_sub(S[site * 144 + (3 * g + cp) * 12 + row], S[site * 144 + (3 * g + 6 + cp) * 12 + row]);
       }
     }
     __syncthreads();
+    // H and T in units of 2^58 2^(2 (E - FX_BIAS))
     for (int q = threadIdx.x; q < ns * 144; q += NP_T) {
       const int site = q / 144, e = q - site * 144;
       const int mu = (e & 7) >> 1, ai = e & 1, k = e >> 3;
       const int c = k / 6, g = (k / 3) & 1, cp = k % 3;
       const int a = (c + 1 + ai) % 3, b = (c + 2 - ai) % 3;
-      const int ap0 = (cp + 1) % 3, bp0 = (cp + 2) % 3;
-      const double2* s = S + site * 144 + 3 * mu + a;
-      const double2* v = Vv + site * 72 + (c * 2 + g) * 12;
-      double2 h = make_double2(0.0, 0.0);
-      // mu' = 0..3 with nu(mu') = 1, 0, 3, 2 and cg = -, +, -, +
-#pragma unroll
-      for (int m = 0; m < 4; m++) {
-        const int nm = m ^ 1;
-        const double2 s0 = s[(3 * nm + bp0) * 12], v0 = v[3 * m + ap0];
-        const double2 s1 = s[(3 * nm + ap0) * 12], v1 = v[3 * m + bp0];
-        if (m & 1) {
-          cfma_d(h, s0, v0);
-          cfms_d(h, s1, v1);
-        } else {
-          cfms_d(h, s0, v0);
-          cfma_d(h, s1, v1);
-        }
-      }
-      const double2 z = Z[site * 72 + (g * 3 + cp) * 12 + 3 * (mu ^ 1) + b];
-      if ((mu ^ ai) & 1)  // eps_{abc} cg(mu) = +1
-        cfma_d(w2, h, z);
-      else
-        cfms_d(w2, h, z);
+      const np_acc h = np_pair(S + site * 144 + 3 * mu + a, 12, Vv + site * 72 + (c * 2 + g) * 12, 1, (cp + 1) % 3,
+                               (cp + 2) % 3);
+      np_acc t = {0, 0, 0, 0};
+      int sh;
+      const int4 hl = np_limbs(h, sh);
+      np_mac<false>(t, hl, Z[site * 72 + (g * 3 + cp) * 12 + 3 * (mu ^ 1) + b]);
+      const int s = 3 * (ex[site] - FX_BIAS) + 2 * 58 + sh;
+      const double re = fx_sum<29>(t.hr, t.cr, s), im = fx_sum<29>(t.hi, t.ci, s);
+      const bool pos = (mu ^ ai) & 1;  // eps_{abc} cg(mu) = +1
+      w2.x += pos ? re : -re;
+      w2.y += pos ? im : -im;
+      if (ex[site] == 2047) w2.x = w2.y = w1.x = w1.y = nan("");  // a non-finite entry
     }
     for (int q = threadIdx.x; q < ns * 36; q += NP_T) {
       const int site = q / 36, e = q - site * 36;
       const int mu = e & 3, k = e >> 2;
       const int c = k / 3, cp = k % 3;
-      const int a0 = (c + 1) % 3, b0 = (c + 2) % 3, ap0 = (cp + 1) % 3, bp0 = (cp + 2) % 3;
-      const double2* s = S + site * 144 + 3 * mu + a0;
-      const double2* r = S + site * 144 + 3 * (mu ^ 1) + b0;
-      double2 t = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int m = 0; m < 4; m++) {
-        const int nm = m ^ 1;
-        const double2 s0 = s[(3 * nm + bp0) * 12], r0 = r[(3 * m + ap0) * 12];
-        const double2 s1 = s[(3 * nm + ap0) * 12], r1 = r[(3 * m + bp0) * 12];
-        if (m & 1) {
-          cfma_d(t, s0, r0);
-          cfms_d(t, s1, r1);
-        } else {
-          cfms_d(t, s0, r0);
-          cfma_d(t, s1, r1);
-        }
-      }
-      const double2* v = Vv + site * 72 + c * 24;
-      const double2 u0 = v[cp], u1 = v[6 + cp], u2 = v[12 + 3 + cp], u3 = v[12 + 9 + cp];
-      const double2 u = make_double2((u0.x - u1.x) + (u2.x - u3.x), (u0.y - u1.y) + (u2.y - u3.y));
-      if (mu & 1)
-        cfma_d(w1, t, u);
-      else
-        cfms_d(w1, t, u);
+      const int a0 = (c + 1) % 3, b0 = (c + 2) % 3;
+      const np_acc h = np_pair(S + site * 144 + 3 * mu + a0, 12, S + site * 144 + 3 * (mu ^ 1) + b0, 12, (cp + 1) % 3,
+                               (cp + 2) % 3);
+      // U, four entries of V: below 2^60, shifted by 3 into limbs
+      const int4* v = Vv + site * 72 + c * 24;
+      const int4 u0 = v[cp], u1 = v[6 + cp], u2 = v[12 + 3 + cp], u3 = v[12 + 9 + cp];
+      int4 u;
+      fx_split((fx_join(u0.x, u0.y) - fx_join(u1.x, u1.y) + fx_join(u2.x, u2.y) - fx_join(u3.x, u3.y) + 4) >> 3, u.x, u.y);
+      fx_split((fx_join(u0.z, u0.w) - fx_join(u1.z, u1.w) + fx_join(u2.z, u2.w) - fx_join(u3.z, u3.w) + 4) >> 3, u.z, u.w);
+      np_acc t = {0, 0, 0, 0};
+      int sh;
+      const int4 hl = np_limbs(h, sh);
+      np_mac<false>(t, hl, u);
+      const int s = 3 * (ex[site] - FX_BIAS) + 2 * 58 + sh + 3;
+      const double re = fx_sum<29>(t.hr, t.cr, s), im = fx_sum<29>(t.hi, t.ci, s);
+      w1.x += mu & 1 ? re : -re;
+      w1.y += mu & 1 ? im : -im;
     }
   }
   __shared__ double red[4][NP_T / 32];
@@ -456,20 +494,27 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
   }
 }
 
-// W[p][t] = sum over the blocks of (prop p, slice t), in block order.
-__global__ void k_nucleon_point_sum(int nblk, int n_t, int n_prop, const double2* partial, double2* W) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_t * n_prop) return;
-  double2 r1 = make_double2(0.0, 0.0), r2 = make_double2(0.0, 0.0);
+// W[p][t] = sum over the blocks of (prop p, slice t), one warp each, in a fixed order.
+__global__ void __launch_bounds__(128) k_nucleon_point_sum(int nblk, int n, const double2* partial, double2* W) {
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
   const double2* p = partial + (long long)i * nblk * 2;
-  for (int b = 0; b < nblk; b++) {
-    r1.x += p[2 * b].x;
-    r1.y += p[2 * b].y;
-    r2.x += p[2 * b + 1].x;
-    r2.y += p[2 * b + 1].y;
+  for (int b = lane; b < nblk; b += 32) {
+    const double2 x = p[2 * b], y = p[2 * b + 1];
+    v[0] += x.x;
+    v[1] += x.y;
+    v[2] += y.x;
+    v[3] += y.y;
   }
-  W[2 * i] = r1;
-  W[2 * i + 1] = r2;
+#pragma unroll
+  for (int q = 0; q < 4; q++)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+  if (lane == 0) {
+    W[2 * i] = make_double2(v[0], v[1]);
+    W[2 * i + 1] = make_double2(v[2], v[3]);
+  }
 }
 
 // The tensor-core block kernel (nucleon_tc.cu) unless LQCD_NUCLEON_TC=0 selects the FP32-FMA
@@ -503,7 +548,7 @@ int lq_nucleon_point(const lqcd_lattice* L, int n_prop, const double2* prop, int
   k_nucleon_point<<<dim3((unsigned)nblk, (unsigned)n_t, (unsigned)n_prop), NP_T, NP_SMEM, st>>>(
       S3, groups, L->V, prop, (long long)12 * L->V * 12, t0, partial);
   RC_LAUNCH();
-  k_nucleon_point_sum<<<(unsigned)((n_t * n_prop + 127) / 128), 128, 0, st>>>(nblk, n_t, n_prop, partial, W);
+  k_nucleon_point_sum<<<(unsigned)((n_t * n_prop + 3) / 4), 128, 0, st>>>(nblk, n_t * n_prop, partial, W);
   return launched_here();
 }
 
