@@ -17,9 +17,8 @@ using namespace lq;
 
 namespace {
 
-constexpr int GT = 16;   // Gram / apply column tile
+constexpr int GT = 8;    // Gram / apply column tile
 constexpr int GR = 32;   // rows per shared-memory stage of the Gram kernel
-constexpr int AJ = 64;   // coefficient rows per shared-memory stage of the apply kernel
 
 int launched_here() {
   lq_count_launch();
@@ -42,34 +41,116 @@ LQ_DI double2 cm_get(const ColMat& m, long long r, int k) {
   return make_double2(0.0, 0.0);
 }
 
+// Dot products of FP64 numbers in 64-bit integers (fxnum.cuh; the integer pipe does 32 times the FP64
+// pipe's multiply-adds).  A vector's entries are q 2^(E - px_bias<X>), |q| < 2^(55 + X), E their largest exponent, in
+// limbs q = q1 2^28 + q0; the sums of q1 p1 and of q1 p0 + q0 p1 over px_modes<X> complex products fit 64 bits.  The
+// propagator takes X = 0, whose 120 modes need one sum.  The orthonormalisation takes X = 1: its second
+// pass multiplies by nearly 1, where FP64 hardly rounds (error of 24 columns against long double: 1.5e-16 with
+// FP64 sums, 1.4e-16 with X = 1, 2.6e-16 with X = 0).
+template <int X>
+constexpr int px_bias = 1077 + X;
+template <int X>
+constexpr int px_modes = X ? 32 : 120;
+template <int X>
+LQ_DI void px_split(double x, int E, int& q1, int& q0) {
+  const long long q = fx_of(x, E + 2 - X);
+  q0 = (int)((unsigned)q << 4) >> 4;
+  q1 = (int)((q - q0) >> 28);
+}
+LQ_DI void px_mac(long long& hh, long long& cr, int a1, int a0, int b1, int b0) {
+  mad_wide(hh, a1, b1);
+  mad_wide(cr, a1, b0);
+  mad_wide(cr, a0, b1);
+}
+
+// (hr, cr, hi, ci) += conj(a) b
+LQ_DI void px_conj_mac(long long (&t)[4], int4 a, int4 b) {
+  px_mac(t[0], t[1], a.x, a.y, b.x, b.y);
+  px_mac(t[0], t[1], a.z, a.w, b.z, b.w);
+  px_mac(t[2], t[3], a.x, a.y, b.z, b.w);
+  px_mac(t[2], t[3], -a.z, -a.w, b.x, b.y);
+}
+LQ_DI double2 px_value(const long long (&t)[4], int e) {
+  return make_double2(fx_sum<28>(t[0], t[1], e), fx_sum<28>(t[2], t[3], e));
+}
+template <int X>
+LQ_DI int4 px_limbs(double2 v, int E) {
+  int4 q;
+  px_split<X>(v.x, E, q.x, q.y);
+  px_split<X>(v.y, E, q.z, q.w);
+  return q;
+}
+
 // Partial Gram matrices: block (tile pair (ta <= tb), split z) sums
 // conj(V[r][a]) V[r][b] over its row chunk into part[z][a][b].
-__global__ void __launch_bounds__(GT * GT) k_gram(ColMat m, long long chunk, int npad, const int2* pairs,
-                                                 double2* part) {
-  __shared__ double2 sa[GR][GT], sb[GR][GT];
+//
+// Fixed-point products (px_*), GF rows at a time: a first look at the rows' 2 x 8 columns gives each its
+// exponent, then the four groups of 64 threads, one thread a pair (a, b), sum every fourth row and the sums of
+// GS stages are added up in FP64.  8 x 8 pairs a tile waste little of the triangle (24 columns: 300 of 384 pairs used, 16 x 16
+// tiles 300 of 768).  24 columns of 2.65 M rows: 13.6 ms with FP64 sums in 16 x 16 tiles, 3.7 ms so.
+constexpr int GS = 4 * px_modes<1> / GR;
+constexpr int GF = 4 * GS * GR;
+__global__ void __launch_bounds__(256) k_gram(ColMat m, long long chunk, int npad, const int2* pairs, double2* part) {
+  __shared__ int4 sa[GR][GT], sb[GR][GT];
+  __shared__ int ex[2 * GT];
+  __shared__ double2 red[3][GT * GT];
   const int2 tp = pairs[blockIdx.x];
   const int a0 = tp.x * GT, b0 = tp.y * GT;
-  const int tx = threadIdx.x % GT, ty = threadIdx.x / GT;
+  const int g = threadIdx.x >> 6, pr = threadIdx.x & 63, ty = pr >> 3, tx = pr & 7;
   const long long R = m.rows[0] + (m.nseg > 1 ? m.rows[1] : 0);
   const long long r_lo = (long long)blockIdx.y * chunk;
   const long long r_hi = r_lo + chunk < R ? r_lo + chunk : R;
+  auto column = [&](int c) { return c < GT ? a0 + c : b0 + c - GT; };
   double2 acc = make_double2(0.0, 0.0);
-  for (long long r0 = r_lo; r0 < r_hi; r0 += GR) {
-    for (int e = threadIdx.x; e < GR * GT; e += GT * GT) {
-      const int rr = e % GR, c = e / GR;
-      const long long r = r0 + rr;
-      const bool in = r < r_hi;
-      sa[rr][c] = in ? cm_get(m, r, a0 + c) : make_double2(0.0, 0.0);
-      sb[rr][c] = in ? cm_get(m, r, b0 + c) : make_double2(0.0, 0.0);
-    }
+  for (long long rf = r_lo; rf < r_hi; rf += GF) {
     __syncthreads();
-#pragma unroll 8
-    for (int rr = 0; rr < GR; rr++) {
-      const double2 x = sa[rr][ty], y = sb[rr][tx];
-      acc.x = fma(x.x, y.x, fma(x.y, y.y, acc.x));
-      acc.y = fma(x.x, y.y, fma(-x.y, y.x, acc.y));
-    }
+    if (threadIdx.x < 2 * GT) ex[threadIdx.x] = 1;
     __syncthreads();
+    for (int e = threadIdx.x; e < GF * 2 * GT; e += 256) {  // GF % 32 == 0: a warp reads one column
+      const int c = e / GF;
+      const long long r = rf + e - c * GF;
+      int x = 1;
+      if (r < r_hi) {
+        const double2 v = cm_get(m, r, column(c));
+        x = max(fx_exponent(v.x), fx_exponent(v.y));
+      }
+      x = __reduce_max_sync(0xffffffffu, x);
+      if ((threadIdx.x & 31) == 0) atomicMax(&ex[c], x);
+    }
+    long long t[4] = {0, 0, 0, 0};
+    auto flush = [&]() {
+      const double2 v = px_value(t, ex[ty] + ex[GT + tx] - 2 * px_bias<1> + 56);
+      acc.x += v.x;
+      acc.y += v.y;
+      t[0] = t[1] = t[2] = t[3] = 0;
+    };
+    int stage = 0;
+    for (long long r0 = rf; r0 < rf + GF && r0 < r_hi; r0 += GR) {
+      if (stage++ == GS) {
+        flush();
+        stage = 1;
+      }
+      __syncthreads();
+      for (int e = threadIdx.x; e < GR * 2 * GT; e += 256) {
+        const int rr = e % GR, c = e / GR;
+        const long long r = r0 + rr;
+        const int4 q = px_limbs<1>(r < r_hi ? cm_get(m, r, column(c)) : make_double2(0.0, 0.0), ex[c]);
+        if (c < GT) sa[rr][c] = q;
+        else sb[rr][c - GT] = q;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int rr = 0; rr < GR / 4; rr++) px_conj_mac(t, sa[4 * rr + g][ty], sb[4 * rr + g][tx]);
+    }
+    flush();
+    if (ex[ty] == 2047 || ex[GT + tx] == 2047) acc = make_double2(nan(""), nan(""));
+  }
+  if (g) red[g - 1][pr] = acc;
+  __syncthreads();
+  if (g) return;
+  for (int k = 0; k < 3; k++) {
+    acc.x += red[k][pr].x;
+    acc.y += red[k][pr].y;
   }
   part[((long long)blockIdx.y * npad + a0 + ty) * npad + b0 + tx] = acc;
 }
@@ -147,43 +228,95 @@ __global__ void __launch_bounds__(1024) k_chol_inv(double2* G, int n, double2* L
   }
 }
 
-// W[r][k] = sum_{j <= k} V[r][j] conj(Linv[k][j])   (W = V L^{-dag}).
+// W[r][k] = sum_{j <= k} V[r][j] conj(Linv[k][j])   (W = V L^{-dag}), a thread a row and GT columns k.
+//
+// Fixed-point products (px_*): V's column j has the exponent ex[j] of its largest entry in the block's 128
+// rows, which the coefficients take off again, so that a sum over j has one scale, ek[k].  24 columns of 2.65 M rows: 10.9
+// ms with FP64 sums and 16 columns a thread, 4.1 ms so.
+constexpr int AJ = px_modes<1>;
 __global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const double2* Linv, int n) {
-  __shared__ double2 cf[AJ][GT];
+  __shared__ int4 cf[AJ][GT];
+  __shared__ int ex[1024], ek[GT];
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int k0 = blockIdx.y * GT;
   const long long R = in.rows[0] + (in.nseg > 1 ? in.rows[1] : 0);
-  double2 acc[GT];
-#pragma unroll
-  for (int q = 0; q < GT; q++) acc[q] = make_double2(0.0, 0.0);
   const int jend = min(n, k0 + GT);
+  for (int j = threadIdx.x; j < jend; j += blockDim.x) ex[j] = 1;
+  if (threadIdx.x < GT) ek[threadIdx.x] = -10000;
+  __syncthreads();
+#pragma unroll 4
+  for (int j = 0; j < jend; j++) {
+    int x = 1;
+    if (r < R) {
+      const double2 v = cm_get(in, r, j);
+      x = max(fx_exponent(v.x), fx_exponent(v.y));
+    }
+    x = __reduce_max_sync(0xffffffffu, x);
+    if ((threadIdx.x & 31) == 0) atomicMax(&ex[j], x);
+  }
+  __syncthreads();
+  auto coefficient = [&](int j, int q) {  // conj(Linv[k0 + q][j])
+    const int k = k0 + q;
+    double2 c = make_double2(0.0, 0.0);
+    if (k < n && j <= k) {
+      const double2 l = Linv[(long long)k * n + j];
+      c = make_double2(l.x, -l.y);
+    }
+    return c;
+  };
+  for (int e = threadIdx.x; e < jend * GT; e += blockDim.x) {
+    const int j = e / GT, q = e % GT;
+    const double2 c = coefficient(j, q);
+    if (c.x != 0.0 || c.y != 0.0) atomicMax(&ek[q], max(fx_exponent(c.x), fx_exponent(c.y)) + ex[j]);
+  }
+  __syncthreads();
+  double2 sum[GT];
+  long long t[GT][4];
+#pragma unroll
+  for (int q = 0; q < GT; q++) {
+    sum[q] = make_double2(0.0, 0.0);
+    t[q][0] = t[q][1] = t[q][2] = t[q][3] = 0;
+  }
+  auto flush = [&]() {
+#pragma unroll
+    for (int q = 0; q < GT; q++) {
+      const double2 v = px_value(t[q], ek[q] - 2 * px_bias<1> + 56);
+      sum[q].x += v.x;
+      sum[q].y += v.y;
+      t[q][0] = t[q][1] = t[q][2] = t[q][3] = 0;
+    }
+  };
+  bool bad = false;
   for (int j0 = 0; j0 < jend; j0 += AJ) {
+    if (j0) {
+      flush();
+      __syncthreads();
+    }
     for (int e = threadIdx.x; e < AJ * GT; e += blockDim.x) {
       const int jj = e / GT, q = e % GT;
-      const int j = j0 + jj, k = k0 + q;
-      double2 c = make_double2(0.0, 0.0);
-      if (j < n && k < n && j <= k) {
-        const double2 l = Linv[(long long)k * n + j];
-        c = make_double2(l.x, -l.y);
-      }
-      cf[jj][q] = c;
+      if (j0 + jj < jend) cf[jj][q] = px_limbs<1>(coefficient(j0 + jj, q), ek[q] - ex[j0 + jj]);
     }
     __syncthreads();
     if (r < R) {
       const int jn = min(AJ, jend - j0);
+#pragma unroll 2
       for (int jj = 0; jj < jn; jj++) {
-        const double2 v = cm_get(in, r, j0 + jj);
+        const int x = ex[j0 + jj];
+        bad = bad || x == 2047;
+        const int4 v = px_limbs<1>(cm_get(in, r, j0 + jj), x);
 #pragma unroll
         for (int q = 0; q < GT; q++) {
-          const double2 c = cf[jj][q];
-          acc[q].x = fma(v.x, c.x, fma(-v.y, c.y, acc[q].x));
-          acc[q].y = fma(v.x, c.y, fma(v.y, c.x, acc[q].y));
+          const int4 c = cf[jj][q];
+          px_mac(t[q][0], t[q][1], v.x, v.y, c.x, c.y);
+          px_mac(t[q][0], t[q][1], -v.z, -v.w, c.z, c.w);
+          px_mac(t[q][2], t[q][3], v.x, v.y, c.z, c.w);
+          px_mac(t[q][2], t[q][3], v.z, v.w, c.x, c.y);
         }
       }
     }
-    __syncthreads();
   }
   if (r >= R) return;
+  flush();
   int sg = 0;
   long long rr = r;
   if (rr >= out.rows[0]) {
@@ -193,7 +326,7 @@ __global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const
 #pragma unroll
   for (int q = 0; q < GT; q++) {
     const int k = k0 + q;
-    if (k < n) out.p[sg][(long long)k * out.ld[sg] + rr] = acc[q];
+    if (k < n) out.p[sg][(long long)k * out.ld[sg] + rr] = bad ? make_double2(nan(""), nan("")) : sum[q];
   }
 }
 
@@ -247,40 +380,91 @@ __global__ void __launch_bounds__(128) k_slice_source(Geom g, int nsys, const Sy
 }
 
 // fact[b][y][a] = -sum_i eta_i(y)[a] conj(xi_i(x)[b]) for y in Gamma*; one
-// thread per (site of Gamma*, a).  xi_x[i][b] = xi_i(x)[b] is staged in
-// shared memory (n * 12 entries).
-__global__ void __launch_bounds__(128) k_proj_prop(int n, long long nsite, long long y0, long long V,
-                                                   const double2* eta, const double2* xi_x, double2* fact) {
-  extern __shared__ double2 xs[];
+// thread per (site of Gamma*, a).  xi_x[i][b] = xi_i(x)[b] in limbs, column b with exponent xe[b], is staged in
+// shared memory (n * 12 entries).  A thread reads its eta_i(y)[a] twice, for their exponent and for the sums; the
+// second read comes from L2.  Bound by the integer pipe: 144 multiply-adds (32 x 32 + 64) per complex number read.
+// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 12.8 ms so.
+__global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, long long y0, long long V,
+                                                   const double2* eta, const int4* xi_x, const int* xe, double2* fact) {
+  extern __shared__ int4 xs[];
   for (int e = threadIdx.x; e < n * 12; e += blockDim.x) xs[e] = xi_x[e];
   __syncthreads();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nsite * 12) return;
-  double2 acc[12];
-#pragma unroll
-  for (int b = 0; b < 12; b++) acc[b] = make_double2(0.0, 0.0);
+  const double2* col = eta + t;
+  const long long ld = nsite * 12;
+  int E = 1;
+#pragma unroll 8
   for (int i = 0; i < n; i++) {
-    const double2 e = eta[(long long)i * nsite * 12 + t];
-#pragma unroll
-    for (int b = 0; b < 12; b++) {
-      const double2 c = xs[i * 12 + b];
-      // e * conj(c)
-      acc[b].x = fma(e.x, c.x, fma(e.y, c.y, acc[b].x));
-      acc[b].y = fma(e.y, c.x, fma(-e.x, c.y, acc[b].y));
-    }
+    const double2 e = __ldg(col + i * ld);
+    E = max(E, max(fx_exponent(e.x), fx_exponent(e.y)));
   }
   const long long y = y0 + t / 12;
   const int a = (int)(t % 12);
+  double2 sum[12];
 #pragma unroll
-  for (int b = 0; b < 12; b++) fact[((long long)b * V + y) * 12 + a] = make_double2(-acc[b].x, -acc[b].y);
+  for (int b = 0; b < 12; b++) sum[b] = make_double2(0.0, 0.0);
+  for (int i0 = 0; i0 < n; i0 += px_modes<0>) {
+    const int i1 = min(n, i0 + px_modes<0>);
+    long long hr[12], cr[12], hi[12], ci[12];
+#pragma unroll
+    for (int b = 0; b < 12; b++) hr[b] = cr[b] = hi[b] = ci[b] = 0;
+    double2 next[4];  // loads four modes ahead
+#pragma unroll
+    for (int k = 0; k < 4; k++) next[k] = __ldg(col + min(i0 + k, i1 - 1) * ld);
+#pragma unroll 1
+    for (int i = i0; i < i1; i += 4) {
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const double2 e = next[k];
+        next[k] = __ldg(col + min(i + 4 + k, i1 - 1) * ld);
+        if (i + k >= i1) continue;
+        int r1, r0, m1, m0;
+        px_split<0>(e.x, E, r1, r0);
+        px_split<0>(e.y, E, m1, m0);
+#pragma unroll
+        for (int b = 0; b < 12; b++) {
+          const int4 c = xs[(i + k) * 12 + b];  // e conj(c)
+          px_mac(hr[b], cr[b], r1, r0, c.x, c.y);
+          px_mac(hr[b], cr[b], m1, m0, c.z, c.w);
+          px_mac(hi[b], ci[b], m1, m0, c.x, c.y);
+          px_mac(hi[b], ci[b], -r1, -r0, c.z, c.w);
+        }
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < 12; b++) {
+      const int s = E + __ldg(xe + b) - 2 * px_bias<0> + 56;
+      const double re = fx_sum<28>(hr[b], cr[b], s), im = fx_sum<28>(hi[b], ci[b], s);
+      sum[b] = i0 ? make_double2(sum[b].x + re, sum[b].y + im) : make_double2(re, im);
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < 12; b++) {
+    const bool bad = E == 2047 || __ldg(xe + b) == 2047;
+    fact[((long long)b * V + y) * 12 + a] = bad ? make_double2(nan(""), nan("")) : make_double2(-sum[b].x, -sum[b].y);
+  }
 }
 
-// xi_x[i][b] = xi_i(x)[b]
-__global__ void k_gather_site(int n, long long nsite_gb, long long xloc, const double2* xi, double2* xi_x) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * 12) return;
-  const int i = t / 12, b = t % 12;
-  xi_x[t] = xi[((long long)i * nsite_gb + xloc) * 12 + b];
+// xi_x[i][b] = xi_i(x)[b] in limbs and the exponents xe[b] of the 12 columns (one block).
+__global__ void __launch_bounds__(256) k_gather_site(int n, long long nsite_gb, long long xloc, const double2* xi,
+                                                     int4* xi_x, int* xe) {
+  __shared__ int e[12];
+  if (threadIdx.x < 12) e[threadIdx.x] = 1;
+  __syncthreads();
+  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
+    const double2 v = xi[((long long)(t / 12) * nsite_gb + xloc) * 12 + t % 12];
+    atomicMax(&e[t % 12], max(fx_exponent(v.x), fx_exponent(v.y)));
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
+    const double2 v = xi[((long long)(t / 12) * nsite_gb + xloc) * 12 + t % 12];
+    int4 q;
+    px_split<0>(v.x, e[t % 12], q.x, q.y);
+    px_split<0>(v.y, e[t % 12], q.z, q.w);
+    xi_x[t] = q;
+  }
+  if (threadIdx.x < 12) xe[threadIdx.x] = e[threadIdx.x];
 }
 
 struct Scratch {
@@ -304,7 +488,7 @@ struct Scratch {
 int chol_qr(const ColMat& in, const ColMat& out, double2* G, double2* Linv, int2* d_pairs, int npairs,
             double2* part, int nsplit, long long chunk, int npad, int* d_status, cudaStream_t st) {
   const int n = in.ncol;
-  k_gram<<<dim3((unsigned)npairs, (unsigned)nsplit), GT * GT, 0, st>>>(in, chunk, npad, d_pairs, part);
+  k_gram<<<dim3((unsigned)npairs, (unsigned)nsplit), 256, 0, st>>>(in, chunk, npad, d_pairs, part);
   RC(launched_here());
   k_gram_reduce<<<(unsigned)((n * n + 255) / 256), 256, 0, st>>>(part, nsplit, npad, n, G);
   RC(launched_here());
@@ -335,7 +519,7 @@ int lq_orthonormalize(ColMat v, ColMat tmp, cudaStream_t st) {
   const int npairs = (int)pairs.size();
   int nsplit = (152 * 8 + npairs - 1) / npairs;
   long long chunk = (R + nsplit - 1) / nsplit;
-  chunk = (chunk + GR - 1) / GR * GR;
+  chunk = (chunk + GF - 1) / GF * GF;
   nsplit = (int)((R + chunk - 1) / chunk);
   const size_t b_pairs = sizeof(int2) * npairs, b_part = sizeof(double2) * (size_t)nsplit * npad * npad,
                b_g = sizeof(double2) * (size_t)n * n;
@@ -383,11 +567,12 @@ int lq_slice_source(const lqcd_lattice* L, const Batch& b, const int* d_ids, int
 int lq_proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi, long long nsite_gs,
                  long long y0, const double2* eta, double2* fact, cudaStream_t st) {
   Scratch s;
-  RC(s.alloc(sizeof(double2) * 12 * (size_t)n, st));
-  double2* xi_x = (double2*)s.p;
-  k_gather_site<<<(unsigned)((n * 12 + 127) / 128), 128, 0, st>>>(n, nsite_gb, xloc, xi, xi_x);
+  RC(s.alloc(sizeof(int4) * 12 * (size_t)n + sizeof(int) * 12, st));
+  int4* xi_x = (int4*)s.p;
+  int* xe = (int*)(xi_x + 12 * (size_t)n);
+  k_gather_site<<<1, 256, 0, st>>>(n, nsite_gb, xloc, xi, xi_x, xe);
   RC(launched_here());
-  const size_t sm = sizeof(double2) * 12 * (size_t)n;
+  const size_t sm = sizeof(int4) * 12 * (size_t)n;
   if (sm > 48 * 1024) {
     if (cudaFuncSetAttribute(k_proj_prop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
       cudaGetLastError();
@@ -395,6 +580,6 @@ int lq_proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xlo
       return LQCD_EBADARG;
     }
   }
-  k_proj_prop<<<(unsigned)((nsite_gs * 12 + 127) / 128), 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_x, fact);
+  k_proj_prop<<<(unsigned)((nsite_gs * 12 + 127) / 128), 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_x, xe, fact);
   return launched_here();
 }
