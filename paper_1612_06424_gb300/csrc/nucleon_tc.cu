@@ -26,12 +26,19 @@
 // One CTA per SM (512 threads, 16 warps): 128 rows (i, j) = 8 i x 16 j of one slice and 128
 // complex columns (32 k x 4 alpha) = 256 real columns, so the accumulator fills the 512 TMEM
 // columns (256 inner + 256 running sums).  Per chunk of 4 sites (24 real K values, three MMA
-// K-steps of 8) all threads stage the 56 spinors of the chunk (FP32, 16-byte loads prefetched
-// one chunk ahead) in shared memory; warps 0-7 build the split diquark operand A (128 rows) and
-// warps 8-15 the split operand Bt (256 rows) into one of two operand buffers in the canonical
+// K-steps of 8) the 56 spinors of the next chunk are on their way to shared memory (cp.async, two
+// staging buffers) while all warps build this chunk's split diquark operand A (128 rows, a thread one row
+// of one site) and then its split operand Bt (256 rows, a thread the two rows of a complex column, whose
+// values differ by sign and order only and are split once) into one of two operand buffers in the canonical
 // K-major layout without swizzle, and one thread issues 9 MMAs (3 K-steps x 3 products, each
 // M 128 x N 256 x K 8) and commits them to the buffer's mbarrier.  The building of chunk c+1
-// overlaps the MMAs of chunk c.
+// overlaps the MMAs of chunk c, also across the end of an inner group: the fold waits for the group's MMAs
+// only when the next chunk is built.
+//
+// Bound by that building, not by the MMAs: 370 instructions a thread and chunk at 52% of the issue slots, shared-memory
+// pipe 59%, tensor pipe 41% busy (a chunk takes 2830 clocks).  24^3 slices, 120 fields: 19.2 ms a slice with half of
+// the warps on each operand, every row of Bt split on its own and the staging through registers between two
+// barriers a chunk; 17.5 ms so.
 //
 // Operand layout (no swizzle, K-major): a core matrix is 8 rows x 16 bytes (4 TF32).  One
 // R-row x 8-value operand of one K-step is R/8 row groups x 2 core matrices:
@@ -70,9 +77,9 @@ constexpr int BUF = NSTEP * STEP;             // one chunk
 // warp's Bt rows on distinct banks)
 constexpr int SITE_STG = TC_SITE_STG;  // float2 per site
 constexpr int STG = XS * SITE_STG * 8;
-constexpr int SMEM = 2 * BUF + STG + 64;      // + 2 mbarriers, the TMEM address and a flag
+constexpr int SMEM = 2 * BUF + 2 * STG + 64;  // + 2 mbarriers, the TMEM address
 constexpr int TMEM_COLS = 512;                // inner accumulator (0..255) + running sums (256..511)
-constexpr int NPRE = 4;                       // 16-byte staging loads per thread and chunk
+constexpr int NPRE = 4;                       // 16-byte staging copies per thread and chunk
 
 // instruction descriptor of kind::tf32: D FP32 (bits 4-5 = 1), A and B TF32 (bits 7-9 and
 // 10-12 = 2), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28
@@ -164,17 +171,21 @@ LQ_DI float2 cg5_pair_tc(const float2* si, const float2* tj, int a, int b) {
   return r;
 }
 
-// store the hi / lo split of four consecutive K values of row r into K-block beta (0..5) of
-// the operand at byte offset `hi_off` of a step (lo at hi_off + mat)
-LQ_DI void put4(unsigned char* buf, int hi_off, int mat, int r, int beta, float4 v) {
-  float4 h, l;
-  split_tf32(v.x, h.x, l.x);
-  split_tf32(v.y, h.y, l.y);
-  split_tf32(v.z, h.z, l.z);
-  split_tf32(v.w, h.w, l.w);
-  const int off = (beta >> 1) * STEP + hi_off + tc_operand_offset(r, 4 * (beta & 1));
+// K-block beta (0..5, four consecutive K values) of row r of the operand at byte offset hi_off of a step
+LQ_DI int block_at(int hi_off, int r, int beta) {
+  return (beta >> 1) * STEP + hi_off + tc_operand_offset(r, 4 * (beta & 1));
+}
+// store hi / lo of four K values (lo at + mat)
+LQ_DI void put4(unsigned char* buf, int off, int mat, float4 h, float4 l) {
   *reinterpret_cast<float4*>(buf + off) = h;
   *reinterpret_cast<float4*>(buf + off + mat) = l;
+}
+
+// 16 bytes global -> shared, zeros when !on
+LQ_DI void copy16(uint32_t dst, const void* src, bool on) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(__cvta_generic_to_global(src)),
+               "r"(on ? 16 : 0)
+               : "memory");
 }
 
 // TMEM readout: warp w reads lanes 32 (w % 4) .. + 31 and real columns 64 (w / 4) .. + 63 of
@@ -221,10 +232,9 @@ __global__ void __launch_bounds__(NT, 1) k_nucleon_block_tc(int n, int S3p, cons
                                                              double2* B, int* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* buf0 = smem;
-  float2* stg = reinterpret_cast<float2*>(smem + 2 * BUF);  // [XS][SITE_STG]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * BUF + STG);
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + 2 * BUF + STG + 16);
-  int* fail = reinterpret_cast<int*>(smem + 2 * BUF + STG + 20);
+  float2* stg0 = reinterpret_cast<float2*>(smem + 2 * BUF);  // [2][XS][SITE_STG]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * BUF + 2 * STG);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + 2 * BUF + 2 * STG + 16);
 
   const int tid = threadIdx.x, warp = tid >> 5;
   const int ntj = (n + TJ - 1) / TJ;
@@ -239,7 +249,6 @@ __global__ void __launch_bounds__(NT, 1) k_nucleon_block_tc(int n, int S3p, cons
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar1) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    *fail = 0;
   }
   if (warp == 0) {
     const uint32_t h = (uint32_t)__cvta_generic_to_shared(tmem_holder);
@@ -252,10 +261,11 @@ __global__ void __launch_bounds__(NT, 1) k_nucleon_block_tc(int n, int S3p, cons
   fence_after();
   const uint32_t tmem = *tmem_holder;
 
-  // staging loads: thread t moves float4 q = t % 8 (two complex components; q < 6) of site
+  // staging copies: thread t moves float4 q = t % 8 (two complex components; q < 6) of site
   // x = (t / 8) % 4 of slots (t / 32) + 16 r, r < NPRE
   const int pq = tid & 7, px = (tid >> 3) & 3, pslot0 = tid >> 5;
   const float4* sf4 = reinterpret_cast<const float4*>(sf);
+  const uint32_t stg_s = (uint32_t)__cvta_generic_to_shared(stg0);
   long long gbase[NPRE];  // float4 index of (slot, site 0 of the slice), or -1
 #pragma unroll
   for (int r = 0; r < NPRE; r++) {
@@ -263,89 +273,104 @@ __global__ void __launch_bounds__(NT, 1) k_nucleon_block_tc(int n, int S3p, cons
     const int f = slot < TI ? i0 + slot : (slot < TI + TJ ? j0 + slot - TI : k0 + slot - TI - TJ);
     gbase[r] = (pq < 6 && slot < NSLOT && f < n) ? (((long long)ts * n + f) * S3p + px) * 6 + pq : -1;
   }
-  float4 pre[NPRE];
-  auto prefetch = [&](int x0) {
+  auto stage = [&](int c) {  // chunk c -> staging buffer c & 1
 #pragma unroll
-    for (int r = 0; r < NPRE; r++)
-      pre[r] = gbase[r] >= 0 ? sf4[gbase[r] + (long long)x0 * 6] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r = 0; r < NPRE; r++) {
+      const int slot = pslot0 + 16 * r;
+      if (pq < 6 && slot < NSLOT) {
+        const bool on = gbase[r] >= 0;
+        copy16(stg_s + (uint32_t)((c & 1) * STG + tc_stage_index(px, slot, 2 * pq) * 8),
+               sf4 + (on ? gbase[r] + (long long)c * XS * 6 : 0), on);
+      }
+    }
   };
   const int nchunk = S3p / XS;
-  prefetch(0);
+  // A: row am = 16 ii + jj, site ax
+  const int am = tid & 127, ax = tid >> 7;
+  stage(0);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
   bool ok = true;
   int issued = -1;  // last chunk whose MMAs were committed
   for (int c = 0; c < nchunk; c++) {
     const int b = c & 1;
     unsigned char* buf = buf0 + b * BUF;
-    // staging <- chunk c; then prefetch chunk c + 1
-#pragma unroll
-    for (int r = 0; r < NPRE; r++) {
-      const int slot = pslot0 + 16 * r;
-      if (pq < 6 && slot < NSLOT) {
-        *reinterpret_cast<float4*>(&stg[tc_stage_index(px, slot, 2 * pq)]) = pre[r];
-      }
-    }
-    if (c + 1 < nchunk) prefetch((c + 1) * XS);
+    const float2* stg = stg0 + b * (STG / 8);
+    if (c + 1 < nchunk) stage(c + 1);
     // the MMAs of chunk c - 2 read this operand buffer: wait for them
-    if (c >= 2 && !mbar_wait(b ? bar1 : bar0, (uint32_t)(((c - 2) >> 1) & 1))) *fail = 1;
-    __syncthreads();
-    if (*fail) {
-      ok = false;
-      break;
+    bool late = c >= 2 && !mbar_wait(b ? bar1 : bar0, (uint32_t)(((c - 2) >> 1) & 1));
+    {
+      // A: K values 6 ax .. 6 ax + 5
+      const float4* u = reinterpret_cast<const float4*>(&stg[tc_stage_index(ax, am >> 4, 0)]);
+      const float4* w = reinterpret_cast<const float4*>(&stg[tc_stage_index(ax, TI + (am & 15), 0)]);
+      float2 uu[12], ww[12];
+#pragma unroll
+      for (int e = 0; e < 6; e++) {
+        const float4 a4 = u[e], b4 = w[e];
+        uu[2 * e] = make_float2(a4.x, a4.y);
+        uu[2 * e + 1] = make_float2(a4.z, a4.w);
+        ww[2 * e] = make_float2(b4.x, b4.y);
+        ww[2 * e + 1] = make_float2(b4.z, b4.w);
+      }
+      float h[6], l[6];
+#pragma unroll
+      for (int cc = 0; cc < 3; cc++) {
+        const int a = (cc + 1) % 3, bb = (cc + 2) % 3;
+        const float2 p = cg5_pair_tc(uu, ww, a, bb), mm = cg5_pair_tc(uu, ww, bb, a);
+        split_tf32(p.x - mm.x, h[2 * cc], l[2 * cc]);
+        split_tf32(p.y - mm.y, h[2 * cc + 1], l[2 * cc + 1]);
+      }
+      // an even site's six values are a K-block and the first half of the next, an odd site's the second half and a
+      // K-block
+      const int odd = ax & 1, blk = (3 * ax) >> 1;
+      const int o4 = block_at(0, am, odd ? blk + 1 : blk), o2 = block_at(0, am, odd ? blk : blk + 1) + 8 * odd;
+      put4(buf, o4, MAT_A, odd ? make_float4(h[2], h[3], h[4], h[5]) : make_float4(h[0], h[1], h[2], h[3]),
+           odd ? make_float4(l[2], l[3], l[4], l[5]) : make_float4(l[0], l[1], l[2], l[3]));
+      *reinterpret_cast<float2*>(buf + o2) = odd ? make_float2(h[0], h[1]) : make_float2(h[4], h[5]);
+      *reinterpret_cast<float2*>(buf + o2 + MAT_A) = odd ? make_float2(l[0], l[1]) : make_float2(l[4], l[5]);
     }
-    if (warp < 8) {
-      // A: row m = 16 ii + jj, sites 2h, 2h + 1 (h = tid / 128): K values 12h .. 12h + 11
-      const int m = tid & 127, h = tid >> 7;
-      const int ii = m >> 4, jj = m & 15;
-      float v[12];
+    // Bt: rows 2 nc (Re S, -Im S) and 2 nc + 1 (Im S, Re S), nc = 4 kk + alpha; K-block beta holds the
+    // (x, c) pairs 2 beta and 2 beta + 1 (x = pair / 3, c = pair % 3).  The split of -v is minus that of v.
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+      const int e = tid + NT * r;
+      if (r && e >= 128 * 6) break;
+      const int nc = e & 127, beta = e >> 7;
+      const int kk = nc >> 2, al = nc & 3;
+      float h[4], l[4];
+#pragma unroll
+      for (int uu = 0; uu < 2; uu++) {
+        const int pr = 2 * beta + uu;
+        const int x = pr / 3, cc = pr % 3;
+        const float2 sv = stg[tc_stage_index(x, TI + TJ + kk, al * 3 + cc)];
+        split_tf32(sv.x, h[2 * uu], l[2 * uu]);
+        split_tf32(sv.y, h[2 * uu + 1], l[2 * uu + 1]);
+      }
+      // lanes 4-7, 12-15, ... store their odd row first: the 16-byte stores of a quarter warp then fall on distinct banks
+      const int sw = (nc >> 2) & 1;
 #pragma unroll
       for (int q = 0; q < 2; q++) {
-        const int x = 2 * h + q;
-        const float4* u = reinterpret_cast<const float4*>(&stg[tc_stage_index(x, ii, 0)]);
-        const float4* w = reinterpret_cast<const float4*>(&stg[tc_stage_index(x, TI + jj, 0)]);
-        float2 uu[12], ww[12];
-#pragma unroll
-        for (int e = 0; e < 6; e++) {
-          const float4 a4 = u[e], b4 = w[e];
-          uu[2 * e] = make_float2(a4.x, a4.y);
-          uu[2 * e + 1] = make_float2(a4.z, a4.w);
-          ww[2 * e] = make_float2(b4.x, b4.y);
-          ww[2 * e + 1] = make_float2(b4.z, b4.w);
-        }
-#pragma unroll
-        for (int cc = 0; cc < 3; cc++) {
-          const int a = (cc + 1) % 3, bb = (cc + 2) % 3;
-          const float2 p = cg5_pair_tc(uu, ww, a, bb), mm = cg5_pair_tc(uu, ww, bb, a);
-          v[6 * q + 2 * cc] = p.x - mm.x;
-          v[6 * q + 2 * cc + 1] = p.y - mm.y;
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 3; q++)
-        put4(buf, 0, MAT_A, m, 3 * h + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
-    } else {
-      // Bt: rows 2 nc (Re S, -Im S) and 2 nc + 1 (Im S, Re S), nc = 4 kk + alpha; K-block
-      // beta holds the (x, c) pairs 2 beta and 2 beta + 1 (x = pair / 3, c = pair % 3)
-      const int u0 = tid - 256;
-#pragma unroll
-      for (int r = 0; r < 6; r++) {
-        const int e = u0 + 256 * r;
-        const int row = e & 255, beta = e >> 8;
-        const int nc = row >> 1, q = row & 1;
-        const int kk = nc >> 2, al = nc & 3;
-        float vv[4];
-#pragma unroll
-        for (int uu = 0; uu < 2; uu++) {
-          const int pr = 2 * beta + uu;
-          const int x = pr / 3, cc = pr % 3;
-          const float2 sv = stg[tc_stage_index(x, TI + TJ + kk, al * 3 + cc)];
-          vv[2 * uu] = q ? sv.y : sv.x;
-          vv[2 * uu + 1] = q ? sv.x : -sv.y;
-        }
-        put4(buf, 2 * MAT_A, MAT_B, row, beta, make_float4(vv[0], vv[1], vv[2], vv[3]));
+        const bool im = q ^ sw;
+        put4(buf, block_at(2 * MAT_A, 2 * nc + (int)im, beta), MAT_B,
+             make_float4(im ? h[1] : h[0], im ? h[0] : -h[1], im ? h[3] : h[2], im ? h[2] : -h[3]),
+             make_float4(im ? l[1] : l[0], im ? l[0] : -l[1], im ? l[3] : l[2], im ? l[2] : -l[3]));
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // the end of an inner group: its MMAs (up to chunk c - 1), then the accumulator into the running sums
+    const bool fold = c > 0 && c % GROUP == 0;
+    if (fold && !late) late = !mbar_wait(b ? bar0 : bar1, (uint32_t)(((c - 1) >> 1) & 1));
+    if (__syncthreads_or(late)) {
+      ok = false;
+      break;
+    }
+    if (fold) {
+      fence_after();
+      fold_group(tmem, warp, c == GROUP);
+      fence_before();
+      __syncthreads();
+    }
     if (tid == 0) {
       fence_after();
       const uint32_t base = (uint32_t)__cvta_generic_to_shared(buf);
@@ -362,16 +387,14 @@ __global__ void __launch_bounds__(NT, 1) k_nucleon_block_tc(int n, int S3p, cons
       mma_commit(b ? bar1 : bar0);
     }
     issued = c;
-    // end of an inner group: wait for its MMAs, fold the accumulator into the running sums
-    if (c % GROUP == GROUP - 1 || c == nchunk - 1) {
-      if (!mbar_wait(b ? bar1 : bar0, (uint32_t)((c >> 1) & 1))) *fail = 1;
-      __syncthreads();
-      if (*fail) {
-        ok = false;
-        break;
-      }
+  }
+  if (ok) {  // the last group
+    const int c = nchunk - 1;
+    if (__syncthreads_or(!mbar_wait((c & 1) ? bar1 : bar0, (uint32_t)((c >> 1) & 1)))) {
+      ok = false;
+    } else {
       fence_after();
-      fold_group(tmem, warp, c < GROUP);
+      fold_group(tmem, warp, nchunk <= GROUP);
       fence_before();
       __syncthreads();
     }
