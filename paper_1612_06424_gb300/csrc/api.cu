@@ -79,11 +79,35 @@ struct DBuf {
   }
 };
 
+// A pinned host word for the poll of the active-system count.  The lattice keeps the words of finished solves (as many as
+// it had solves at a time): allocating and freeing one took longer, and synchronised the device, than a small
+// solve's other host work.
 struct PinnedInt {
+  const lqcd_lattice* L;
   int* h = nullptr;
-  PinnedInt() { cudaHostAlloc((void**)&h, sizeof(int) * 4, cudaHostAllocDefault); }
+  explicit PinnedInt(const lqcd_lattice* l) : L(l) {
+    {
+      std::lock_guard<std::mutex> lk(L->pinned_mu);
+      if (!L->pinned.empty()) {
+        h = L->pinned.back();
+        L->pinned.pop_back();
+      }
+    }
+    if (!h) cudaHostAlloc((void**)&h, sizeof(int) * 4, cudaHostAllocDefault);
+  }
+  PinnedInt(const PinnedInt&) = delete;
+  PinnedInt& operator=(const PinnedInt&) = delete;
   ~PinnedInt() {
-    if (h) cudaFreeHost(h);
+    if (!h) return;
+    std::lock_guard<std::mutex> lk(L->pinned_mu);
+    L->pinned.push_back(h);
+  }
+};
+
+struct GraphExec {
+  cudaGraphExec_t g = nullptr;
+  ~GraphExec() {
+    if (g) cudaGraphExecDestroy(g);
   }
 };
 
@@ -99,6 +123,28 @@ int check_lat(const lqcd_lattice* L) {
   return 0;
 }
 
+// Descriptor of the system on slab d of field f, its vectors at site offset off.
+int sys_desc(const lqcd_lattice* L, lqcd_slab d, int f, long long off, lq::SysDesc& s) {
+  if (d.t0 < 0 || d.t1 >= L->dims[0] || d.t0 > d.t1) {
+    lq_set_error("slab out of range: " + std::to_string(d.t0) + ".." + std::to_string(d.t1));
+    return LQCD_EBADARG;
+  }
+  if (f < 0 || f >= (int)L->fields.size()) {
+    lq_set_error("field index " + std::to_string(f) + " not loaded");
+    return LQCD_ENOFIELD;
+  }
+  s = lq::SysDesc{};
+  s.field = f;
+  s.t0 = d.t0;
+  s.t1 = d.t1;
+  s.wrap = (d.t0 == 0 && d.t1 == L->dims[0] - 1 && L->bc != LQCD_BC_OPEN) ? 1 : 0;
+  s.tsign = L->bc == LQCD_BC_ANTIPERIODIC ? -1.f : 1.f;
+  s.n = (int)((d.t1 - d.t0 + 1) * L->S3h);
+  s.cb0 = (int)(d.t0 * L->S3h);
+  s.off = off;
+  return 0;
+}
+
 // A batch with its own descriptor / flag / scalar / partial storage.
 struct BatchStore {
   Batch b;
@@ -111,24 +157,8 @@ struct BatchStore {
     h_sys.resize(n);
     long long off = 0, maxn = 0;  // maxn: sites per parity of the largest system
     for (int k = 0; k < n; k++) {
-      const lqcd_slab d = doms[k];
-      if (d.t0 < 0 || d.t1 >= L->dims[0] || d.t0 > d.t1) {
-        lq_set_error("slab out of range: " + std::to_string(d.t0) + ".." + std::to_string(d.t1));
-        return LQCD_EBADARG;
-      }
-      if (fields[k] < 0 || fields[k] >= (int)L->fields.size()) {
-        lq_set_error("field index " + std::to_string(fields[k]) + " not loaded");
-        return LQCD_ENOFIELD;
-      }
-      lq::SysDesc s{};
-      s.field = fields[k];
-      s.t0 = d.t0;
-      s.t1 = d.t1;
-      s.wrap = (d.t0 == 0 && d.t1 == L->dims[0] - 1 && L->bc != LQCD_BC_OPEN) ? 1 : 0;
-      s.tsign = L->bc == LQCD_BC_ANTIPERIODIC ? -1.f : 1.f;
-      s.n = (int)((d.t1 - d.t0 + 1) * L->S3h);
-      s.cb0 = (int)(d.t0 * L->S3h);
-      s.off = off;
+      lq::SysDesc s;
+      RC(sys_desc(L, doms[k], fields[k], off, s));
       off += s.n;
       maxn = std::max(maxn, (long long)s.n);
       h_sys[k] = s;
@@ -171,10 +201,6 @@ struct BatchStore {
   int pull_sc(cudaStream_t st) {
     CK(cudaMemcpyAsync(h_sc.data(), sc.p, sizeof(lq::SolverScal) * b.nsys, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    return 0;
-  }
-  int push_sc(cudaStream_t st) {
-    CK(cudaMemcpyAsync(sc.p, h_sc.data(), sizeof(lq::SolverScal) * b.nsys, cudaMemcpyHostToDevice, st));
     return 0;
   }
 };
@@ -270,7 +296,7 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
   PoolP ps;
   RC(ps.alloc(b, P, 8, st));
   VecP r = ps.v(0), r0 = ps.v(1), p = ps.v(2), v = ps.v(3), s = ps.v(4), t = ps.v(5), xs = ps.v(6), te = ps.v(7);
-  PinnedInt cnt;
+  PinnedInt cnt(L);
   DBuf dcnt;
   RC(dcnt.alloc(sizeof(int), st));
   VecP none;
@@ -286,19 +312,13 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
   RC(B.push_active(st));
   std::vector<double> bb(n);
   RC(lq_norm2_64(b, b_e, st));
-  RC(lq_finalize(lq::FIN_NORM, b, 0, 0, 12, st));
-  RC(B.pull_sc(st));
-  for (int k = 0; k < n; k++) bb[k] = B.h_sc[k].rr;
+  RC(lq_finalize(lq::FIN_BB, b, 0, 0, 12, st));
   RC(lq_norm2_64(b, b_o, st));
-  RC(lq_finalize(lq::FIN_NORM, b, 0, 0, 12, st));
+  RC(lq_finalize(lq::FIN_BB_ADD, b, 0, 0, 12, st));
   RC(B.pull_sc(st));
-  for (int k = 0; k < n; k++) {
-    bb[k] += B.h_sc[k].rr;
-    B.h_sc[k].bb = bb[k];
-  }
+  for (int k = 0; k < n; k++) bb[k] = B.h_sc[k].bb;
   if (verbose())
     for (int k = 0; k < n; k++) fprintf(stderr, "[lqcd] solve P=%d sys %d |eta|^2 = %.6e n=%d\n", P, k, bb[k], B.h_sys[k].n);
-  RC(B.push_sc(st));
 
   // prepare: bh_o = b_o + 1/2 H_oe A_ee^{-1} b_e
   RC(lq_hop_clinv(64, dag, clov, L, b, none, v64(b_e), v64(t64), 0.0, 1.0, st));
@@ -318,6 +338,8 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
   // Dhat, at the price of the squared condition number.
   static const bool force_cg = getenv("LQCD_KRYLOV") && std::string(getenv("LQCD_KRYLOV")) == "cgnr";
   std::vector<int> use_cg(n, force_cg ? 1 : 0);
+  GraphExec exec;  // check_every captured iterations, the same for every cycle
+  long long per_replay = 0;
   for (int cycle = 0;; cycle++) {
     // true residual of the preconditioned system: r64 = bh_o - Dhat x_o (FP64);
     // at the first cycle without a guess x_o = 0 and r64 = bh_o needs no operator
@@ -419,29 +441,30 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
         return 0;
       };
       if (use_graph && budget >= 2 * check_every) {
-        // check_every iterations captured once as a CUDA graph on a private
-        // stream, replayed between host convergence checks (retired systems
+        // check_every iterations captured once per solve as a CUDA graph on a
+        // private stream, replayed between host convergence checks (retired systems
         // skip every kernel, so iterations past convergence change nothing)
         cudaStream_t gs = L->graph_stream;
         CK(cudaEventRecord(L->graph_event, st));
         CK(cudaStreamWaitEvent(gs, L->graph_event, 0));
-        const long long c0 = lqcd_kernel_launches();
-        cudaGraph_t graph = nullptr;
-        CK(cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal));
-        int crc = 0;
-        for (int g = 0; g < check_every && !crc; g++) crc = iteration(gs);
-        cudaError_t ce = cudaStreamEndCapture(gs, &graph);
-        if (crc) return crc;
-        CK(ce);
-        const long long per_replay = lqcd_kernel_launches() - c0;
-        lq_count_launches(-per_replay);  // captured, not run
-        cudaGraphExec_t exec = nullptr;
-        cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(ie);
+        if (!exec.g) {
+          const long long c0 = lqcd_kernel_launches();
+          cudaGraph_t graph = nullptr;
+          CK(cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal));
+          int crc = 0;
+          for (int g = 0; g < check_every && !crc; g++) crc = iteration(gs);
+          cudaError_t ce = cudaStreamEndCapture(gs, &graph);
+          if (crc) return crc;
+          CK(ce);
+          per_replay = lqcd_kernel_launches() - c0;
+          lq_count_launches(-per_replay);  // captured, not run
+          cudaError_t ie = cudaGraphInstantiate(&exec.g, graph, 0);
+          cudaGraphDestroy(graph);
+          CK(ie);
+        }
         int grc = 0;
         while (it < budget) {
-          if (cudaGraphLaunch(exec, gs) != cudaSuccess) {
+          if (cudaGraphLaunch(exec.g, gs) != cudaSuccess) {
             lq_set_error("solve: CUDA graph launch failed");
             grc = LQCD_ECUDA;
             break;
@@ -451,7 +474,6 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
           if ((grc = poll(gs)) != 0) break;
           if (*cnt.h == 0) break;
         }
-        cudaGraphExecDestroy(exec);
         if (grc) return grc;
         CK(cudaEventRecord(L->graph_event, gs));
         CK(cudaStreamWaitEvent(st, L->graph_event, 0));
@@ -783,6 +805,7 @@ extern "C" int lqcd_destroy_lattice(lqcd_lattice* L) {
   free_fields(L);
   if (L->graph_stream) cudaStreamDestroy(L->graph_stream);
   if (L->graph_event) cudaEventDestroy(L->graph_event);
+  for (int* h : L->pinned) cudaFreeHost(h);
   delete L;
   return 0;
 }
@@ -878,29 +901,50 @@ extern "C" int lqcd_dslash(lqcd_lattice* L, int field, const lqcd_slab* dom, int
   }
   cudaStream_t st = (cudaStream_t)stream;
   lqcd_slab d = dom ? *dom : lqcd_slab{0, L->dims[0] - 1};
+  const bool clov = L->csw != 0.0;
+  VecP none;
+  if (precision == 64) {
+    // One allocation, and the descriptors travel as kernel arguments: a small lattice's call is all
+    // host work (4^4: 118 us with nine allocations and five copies, 59 us so).
+    lq::SysDesc s;
+    RC(sys_desc(L, d, field, 0, s));
+    Batch b;
+    b.nsys = 1;
+    b.max_n = b.total = s.n;
+    b.nby = (s.n + LQ_BLOCK - 1) / LQ_BLOCK;
+    b.tblk_ok = L->S3h % 32 == 0 && (d.t1 - d.t0 + 1) % 4 == 0;
+    const size_t vec = (size_t)s.n * 12 * sizeof(double2), exps = ((size_t)s.n * 2 * sizeof(int) + 255) / 256 * 256;
+    DBuf buf;
+    RC(buf.alloc(512 + exps + 6 * vec, st));
+    char* base = buf.as<char>();
+    b.sys = (lq::SysDesc*)base;
+    void** ptr = (void**)(base + 256);
+    double2* v[6];  // in, out (even, odd), in as limbs
+    for (int k = 0; k < 6; k++) v[k] = (double2*)(base + 512 + exps + k * vec);
+    VecP xl[2];
+    for (int k = 0; k < 2; k++) {
+      xl[k].d = v[4 + k];
+      xl[k].e = (int*)(base + 512) + (size_t)k * s.n;
+    }
+    RC(lq_dslash_in(L, s, (const double2*)in, out, (lq::SysDesc*)base, ptr, v[0], v[1], xl[0], xl[1], st));
+    for (int par = 0; par < 2; par++)
+      RC(lq_hop_lin(64, dagger, clov, lq::RED_NONE, L, b, par, xl[1 - par], v64(v[par]), none, none, v64(v[2 + par]),
+                    -0.5, 1.0, 0.0, st));
+    RC(lq_eo_to_nat(L, b, v[2], v[3], (double2* const*)ptr, 1.0, st));
+    CK(cudaStreamSynchronize(st));
+    return 0;
+  }
   BatchStore B;
   RC(B.build(L, 1, &d, &field, st));
   const Batch& b = B.b;
   Pool64 e;
-  RC(e.alloc(b, precision == 64 ? 5 : 4, st));  // FP64: one more for the hop input in limbs
+  RC(e.alloc(b, 4, st));
   DBuf ptr;
   RC(ptr.alloc(sizeof(void*), st));
   const double2* srcp = (const double2*)in;
   CK(cudaMemcpyAsync(ptr.p, &srcp, sizeof(void*), cudaMemcpyHostToDevice, st));
   RC(lq_nat_to_eo(L, b, ptr.as<const double2*>(), e.v(0), e.v(1), st));
-  const bool clov = L->csw != 0.0;
-  VecP none;
-  if (precision == 64) {
-    DBuf fxe;
-    RC(fxe.alloc(sizeof(int) * (size_t)b.total, st));
-    VecP xl = v64(e.v(4));
-    xl.e = fxe.as<int>();
-    for (int par = 0; par < 2; par++) {
-      RC(lq_to_fx(b, e.v(1 - par), xl, st));
-      RC(lq_hop_lin(precision, dagger, clov, lq::RED_NONE, L, b, par, xl, v64(e.v(par)), none, none, v64(e.v(2 + par)),
-                    -0.5, 1.0, 0.0, st));
-    }
-  } else {
+  {
     PoolP q;
     RC(q.alloc(b, precision, 4, st));
     RC(lq_convert(64, precision, b, v64(e.v(0)), q.v(0), st));

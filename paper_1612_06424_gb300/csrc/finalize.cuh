@@ -90,6 +90,7 @@ LQ_DI bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 //             r = s - omega t, beta = (rho'/rho)(alpha/omega)
 //  FIN_STOP : v[2] = |r|^2: stop the system when rr <= target2, on breakdown, NaN or divergence (rr > 1e8 rr0)
 //  FIN_NORM : rr = v[2] only
+//  FIN_BB, FIN_BB_ADD: bb = v[2], bb += v[2]
 //  CG on the normal equations (real scalars in .x), the sum in v[2]:
 //  FIN_CG_RHO  : rho = |z|^2 (z = D^dag r), beta = 0 (the first direction is z)
 //  FIN_CG_ALPHA: alpha = rho / |v|^2 (v = D^ p); breakdown if |v|^2 is not positive
@@ -151,6 +152,12 @@ LQ_DI void fin_update(int mode, const double* v, SolverScal& c, int* active, dou
       break;
     case FIN_NORM:
       c.rr = v[2];
+      break;
+    case FIN_BB:
+      c.bb = v[2];
+      break;
+    case FIN_BB_ADD:
+      c.bb += v[2];
       break;
     case FIN_CG_RHO:
       c.rho = make_double2(v[2], 0.0);

@@ -469,6 +469,8 @@ namespace lq {
 // FP64 vectors of a batch to limbs (out may be in) and exponents
 void to_fx_launch(dim3 gr, int nsys, const SysDesc* sys, const int* active, const double2* in, int4* out, int* oute,
                   cudaStream_t st);
+void dslash_in_launch(const Geom& g, const SysDesc& s, const double2* in, void* out, SysDesc* d_sys, void** d_ptr,
+                      double2* ve, double2* vo, int4* le, int4* lo, int* ee, int* eo, cudaStream_t st);
 int fx_lin_launch(bool dag, bool clov, int red, int epi, dim3 gr, const FxArgs& m, cudaStream_t st);
 int fx_clinv_launch(bool dag, bool clov, int epi, dim3 gr, const FxArgs& m, cudaStream_t st);
 }

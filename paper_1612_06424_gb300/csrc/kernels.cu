@@ -474,6 +474,12 @@ int lq_nat_to_eo(const lqcd_lattice* L, const Batch& b, const double2* const* sr
   return launched();
 }
 
+int lq_dslash_in(const lqcd_lattice* L, const SysDesc& s, const double2* in, void* out, SysDesc* d_sys, void** d_ptr,
+                 double2* ve, double2* vo, VecP le, VecP lo, cudaStream_t st) {
+  dslash_in_launch(L->g, s, in, out, d_sys, d_ptr, ve, vo, (int4*)le.d, (int4*)lo.d, le.e, lo.e, st);
+  return launched();
+}
+
 int lq_nat_to_eo_g5(const lqcd_lattice* L, const Batch& b, const double2* const* src, double2* ve, double2* vo,
                     cudaStream_t st) {
   k_nat_to_eo<true><<<grid_lin(b, b.nby, 2), LQ_BLOCK, 0, st>>>(L->g, b.nsys, b.sys, nullptr, src, ve, vo);
