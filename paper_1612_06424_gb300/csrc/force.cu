@@ -33,6 +33,8 @@
 // slab of 24^3 x 48 the plain form over all links took 47.6 ms, this one 5.3 ms.  Under open
 // time BC the link leaving the last time slice is absent (zero): every
 // product through it vanishes and its own force is zero.
+#include <algorithm>
+
 #include "dslash.cuh"
 #include "internal.h"
 
@@ -124,7 +126,9 @@ LQ_DI int plane_of(int mu, int nu) {
 // Slices whose links can have a force: one more than the slab on both sides, held in slots
 // 0 .. nsl-1 (the whole lattice in natural order when that covers it).
 struct ForceSlices {
-  int first, nsl, T;  // slot 0 holds slice `first`; slot k slice (first + k) mod T
+  int first, nsl, T;  // slot 0 is slice `first`; slot k slice (first + k) mod T
+  int base, held;     // the arrays hold the `held` slots from `base` on (mod T)
+  int out0, out1;     // the links of slots out0 .. out1 - 1 are computed
   long long s3;
 };
 LQ_DI int slot_of(const ForceSlices& fs, int t) {
@@ -133,8 +137,11 @@ LQ_DI int slot_of(const ForceSlices& fs, int t) {
 }
 // Index of site x in the arrays over the slots, -1 outside them.
 LQ_DI long long sidx(const Geom& g, const ForceSlices& fs, const int x[4]) {
-  const int k = slot_of(fs, x[0]);
+  int k = slot_of(fs, x[0]);
   if (k >= fs.nsl) return -1;
+  k -= fs.base;
+  if (k < 0) k += fs.T;
+  if (k >= fs.held) return -1;
   return k * fs.s3 + ((long long)x[1] * g.L[2] + x[2]) * g.L[3] + x[3];
 }
 
@@ -171,8 +178,8 @@ LQ_DI M3 load_B(const Geom& g, const ForceSlices& fs, const double2* B, const in
 __global__ void k_force_K(Geom g, ForceSlices fs, int t0, int t1, double csw, const double2* X, const double2* Y,
                           double2* K) {
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= fs.nsl * fs.s3) return;
-  const int t = (int)((fs.first + q / fs.s3) % fs.T);
+  if (q >= fs.held * fs.s3) return;
+  const int t = (int)((fs.first + fs.base + q / fs.s3) % fs.T);
   const long long i = t * fs.s3 + q % fs.s3;
   double2* out = K + q * 54;
   if (t < t0 || t > t1) {
@@ -293,12 +300,12 @@ LQ_DI M3 sub(const M3& a, const M3& b) {
 __global__ void __launch_bounds__(128) k_force_B(Geom g, ForceSlices fs, const FieldPtrs* fields, int field,
                                                  const double2* K, double2* B) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= 4 * fs.nsl * fs.s3) return;
+  if (gid >= 4 * fs.held * fs.s3) return;
   const long long q = gid >> 2;
   const int s = (int)(gid & 3);
   int x[4], y[4];
   ncoords(g, q % fs.s3, x);
-  x[0] = (int)((fs.first + q / fs.s3) % fs.T);
+  x[0] = (int)((fs.first + fs.base + q / fs.s3) % fs.T);
   shifted(g, x, s, 1, y);
   const M3 u = link(g, fields[field], x, s);
 #pragma unroll 1
@@ -351,7 +358,9 @@ __global__ void __launch_bounds__(128) k_force_link(Geom g, ForceSlices fs, cons
   int x[4];
   ncoords(g, i, x);
   const FieldPtrs f = fields[field];
-  if (slot_of(fs, x[0]) >= fs.nsl || (g.bc_t == 0 && rho == 0 && x[0] == g.L[0] - 1)) {
+  const int slot = slot_of(fs, x[0]);
+  if (slot < fs.nsl ? slot < fs.out0 || slot >= fs.out1 : fs.out0 > 0) return;  // another launch's
+  if (slot >= fs.nsl || (g.bc_t == 0 && rho == 0 && x[0] == g.L[0] - 1)) {
     for (int a = 0; a < 8; a++) out[a] = 0.0;
     return;
   }
@@ -411,23 +420,40 @@ int lq_force(const lqcd_lattice* L, int field, const lqcd_slab& dom, const doubl
   const int want = dom.t1 - dom.t0 + 3;
   fs.nsl = want >= fs.T ? fs.T : want;
   fs.first = want >= fs.T ? 0 : (dom.t0 + fs.T - 1) % fs.T;
-  const long long sites = fs.nsl * fs.s3;
+  // K and B take three times the K of all slices that the plain form held (54 complex numbers a site).  Where that is
+  // more than 2 GB, only as many slices at a time as keep within it: the links of a slice need B of the slices
+  // on either side, and that K of one more.  (24^3 x 48, whole lattice in runs of 13 slices of 48: 4% more work.)
+  constexpr int WORDS = 54 + 108;
+  const double room = std::max(54.0 * 16 * L->V, 2e9);
+  int run = fs.nsl;  // slots of links at a time
+  if (L->csw != 0.0 && (double)WORDS * 16 * fs.nsl * fs.s3 > room)
+    run = std::max(1, (int)(room / ((double)WORDS * 16 * fs.s3)) - 3);
+  if (run + 3 >= fs.nsl) run = fs.nsl;
   double2 *K = nullptr, *B = nullptr;
+  const long long room_sites = (run < fs.nsl ? run + 3 : fs.nsl) * fs.s3;
   if (L->csw != 0.0) {
-    if (cudaMallocAsync((void**)&K, sizeof(double2) * (54 + 108) * (size_t)sites, st) != cudaSuccess) {
+    if (cudaMallocAsync((void**)&K, sizeof(double2) * WORDS * (size_t)room_sites, st) != cudaSuccess) {
       cudaGetLastError();
       lq_set_error("link_force: allocation failed");
       return LQCD_ENOMEM;
     }
-    B = K + 54 * sites;
-    lq::k_force_K<<<(unsigned)((sites + 127) / 128), 128, 0, st>>>(L->g, fs, dom.t0, dom.t1, L->csw, X, Y, K);
-    lq_count_launch();
-    lq::k_force_B<<<(unsigned)((4 * sites + 127) / 128), 128, 0, st>>>(L->g, fs, L->d_fields, field, K, B);
+    B = K + 54 * room_sites;
+  }
+  for (fs.out0 = 0; fs.out0 < fs.nsl; fs.out0 += run) {
+    fs.out1 = std::min(fs.out0 + run, fs.nsl);
+    fs.base = run < fs.nsl ? (fs.out0 + fs.T - 1) % fs.T : 0;
+    fs.held = run < fs.nsl ? run + 3 : fs.nsl;
+    if (L->csw != 0.0) {
+      const long long sites = fs.held * fs.s3;
+      lq::k_force_K<<<(unsigned)((sites + 127) / 128), 128, 0, st>>>(L->g, fs, dom.t0, dom.t1, L->csw, X, Y, K);
+      lq_count_launch();
+      lq::k_force_B<<<(unsigned)((4 * sites + 127) / 128), 128, 0, st>>>(L->g, fs, L->d_fields, field, K, B);
+      lq_count_launch();
+    }
+    lq::k_force_link<<<(unsigned)((4 * L->V + 127) / 128), 128, 0, st>>>(L->g, fs, L->d_fields, field, dom.t0, dom.t1,
+                                                                          L->csw, X, Y, B, F);
     lq_count_launch();
   }
-  lq::k_force_link<<<(unsigned)((4 * L->V + 127) / 128), 128, 0, st>>>(L->g, fs, L->d_fields, field, dom.t0, dom.t1,
-                                                                        L->csw, X, Y, B, F);
-  lq_count_launch();
   if (K) cudaFreeAsync(K, st);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
