@@ -204,16 +204,14 @@ LQ_DI void hop_sum_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
 
 // ---------------------------------------------------------------------------
 // Software-pipelined hop sum (FP32 / FP16).  The eight hops are taken in a
-// fixed order k = 2*mu + (0 forward, 1 backward); the raw words of hop k+D
+// fixed order k = 2*mu + (0 forward, 1 backward); the raw words of later hops
 // (neighbour spinor and link, as stored) are loaded before hop k is
-// computed, so up to D hops' loads are in flight while the thread does
+// computed, so that loads are in flight while the thread does
 // arithmetic.  Loads are unconditional: a hop that leaves the slab (or
 // crosses the open time boundary) reads the thread's own in-range words and
 // is then weighted by 0, so the pipeline has no branches.
-#ifndef LQ_HOP_PIPE
-#define LQ_HOP_PIPE 1
-#endif
-
+//
+// FP32 keeps the words in flight in shared memory (hop_sum_ring), FP16 in registers (hop_sum_pipe).
 template <int P>
 struct HopRaw;
 template <>
@@ -228,30 +226,11 @@ struct HopRaw<16> {
   uint2 u[3];
 };
 
-// Pipeline depth per precision (hops whose loads are in flight while one is
-// computed): bounded by the register cap of the stencil kernels.  FP32 depth
-// 2 at 4 blocks per SM measured best on GB300 (depth 1: -3%; depth 2 or 3 at
-// 3 blocks per SM: -5% and -13%).
-#ifndef LQ_HOP_DEPTH32
-#define LQ_HOP_DEPTH32 2
-#endif
+// FP16: hops in flight while one is computed, bounded by the register cap of the stencil kernels.
 #ifndef LQ_HOP_DEPTH16
 #define LQ_HOP_DEPTH16 2
 #endif
-template <int P>
-struct HopDepth {
-  static constexpr int value = P == 16 ? LQ_HOP_DEPTH16 : LQ_HOP_DEPTH32;
-};
 
-LQ_DI void raw_load(HopRaw<32>& r, const void* in, const float*, int n, int q, const FieldPtrs& f, int p, int mu,
-                    int Vh, int cl) {
-  const float4* sp = (const float4*)in + q;
-#pragma unroll
-  for (int k = 0; k < 6; k++) r.s[k] = __ldg(sp + k * n);
-  const float4* b = f.U32 + (p * 4 + mu) * 3 * Vh + cl;
-#pragma unroll
-  for (int k = 0; k < 3; k++) r.u[k] = ld_once(b + k * Vh);
-}
 LQ_DI void raw_load(HopRaw<16>& r, const void* in, const float* inn, int n, int q, const FieldPtrs& f, int p, int mu,
                     int Vh, int cl) {
   const uint4* sp = (const uint4*)in + q;
@@ -379,15 +358,9 @@ LQ_DI f2_t f2_mul(f2_t a, f2_t b) {
   return d;
 }
 
-// LQ_HOP_PACK 1: the FP32 / FP16 hop sum transports and accumulates spin
-// pairs with f32x2 arithmetic (measured 2-6% faster on GB300 than scalar
-// FP32); 0: scalar.
-#ifndef LQ_HOP_PACK
-#define LQ_HOP_PACK 1
-#endif
 // Colour transport of the two spins of a half spinor with packed pairs: the
 // pair index is the spin, so one link element (broadcast to both halves)
-// multiplies both spins in one instruction.  w[sp][a] = sum_c U[a][c] h[sp][c]
+// multiplies both spins in one instruction (2-6% faster than scalar FP32).  w[sp][a] = sum_c U[a][c] h[sp][c]
 // (forward) or sum_c conj(U[c][a]) h[sp][c] (backward).
 template <bool FWD>
 LQ_DI void mul_u_pairs(const su3<float>& u, const cx<float> h[6], f2_t wr[3], f2_t wi[3]) {
@@ -476,33 +449,7 @@ LQ_DI void expand_add_p(AccP& A, const f2_t wr[3], const f2_t wi[3]) {
   }
 }
 
-// Hop k from its raw words: acc += weight * (1 -+ g_mu) U psi (forward) or
-// (1 +- g_mu) U^dag psi (backward).
-template <int P, bool DAG, int K>
-LQ_DI void hop_apply(const HopRaw<P>& r, float wgt, cx<float> (&acc)[12]) {
-  constexpr int MU = K >> 1;
-  constexpr bool FWD = (K & 1) == 0;
-  constexpr int SF = DAG ? +1 : -1;
-  constexpr int S = FWD ? SF : -SF;
-  cx<float> h[6], w[6];
-  {
-    cx<float> psi[12];
-    raw_spinor(r, psi);
-    project<MU, S>(psi, h);
-  }
-  const su3<float> u = raw_link(r);
-  if (FWD)
-    mul_u(u, h, w);
-  else
-    mul_udag(u, h, w);
-  if (MU == 0) {
-#pragma unroll
-    for (int k = 0; k < 6; k++) w[k] = wgt * w[k];
-  }
-  expand_add<MU, S>(acc, w);
-}
-
-// hop_apply with the packed accumulator.
+// Hop k from its raw words: A += weight * (1 -+ g_mu) U psi (forward) or (1 +- g_mu) U^dag psi (backward).
 template <int P, bool DAG, int K>
 LQ_DI void hop_apply(const HopRaw<P>& r, float wgt, AccP& A) {
   constexpr int MU = K >> 1;
@@ -531,29 +478,98 @@ LQ_DI void hop_apply(const HopRaw<P>& r, float wgt, AccP& A) {
 
 // One step of the pipeline: issue the loads of hop K + D, then compute hop K.
 // Only the time hops (K = 0, 1) carry a weight other than 1.
-template <int P, bool DAG, int K, int D, typename ACC>
+template <int P, bool DAG, int K, int D>
 LQ_DI void hop_pipe_step(HopRaw<P> (&buf)[D + 1], const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout,
                          int cb, int j, const int x[4], const void* in, const float* inn, float w0, float w1,
-                         ACC& acc) {
+                         AccP& acc) {
   if constexpr (K + D < 8) raw_fetch<P, K + D>(buf[(K + D) % (D + 1)], g, sd, f, pout, cb, j, x, in, inn);
   hop_apply<P, DAG, K>(buf[K % (D + 1)], K == 0 ? w0 : w1, acc);
   if constexpr (K + 1 < 8) hop_pipe_step<P, DAG, K + 1, D>(buf, g, sd, f, pout, cb, j, x, in, inn, w0, w1, acc);
 }
 
+// FP16: the ring of raw words in registers.
 template <int P, bool DAG, int D>
 LQ_DI void hop_sum_pipe(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j, const int x[4],
-                        const void* in, const float* inn, cx<float> acc[12]) {
+                        const void* in, const float* inn, AccP& A) {
   HopRaw<P> buf[D + 1];
   raw_fetch<P, 0>(buf[0], g, sd, f, pout, cb, j, x, in, inn);
   if constexpr (D > 1) raw_fetch<P, 1>(buf[1], g, sd, f, pout, cb, j, x, in, inn);
   if constexpr (D > 2) raw_fetch<P, 2>(buf[2], g, sd, f, pout, cb, j, x, in, inn);
   static_assert(D >= 1 && D <= 3, "pipeline depth");
   const float w0 = hop_target<0>(g, sd, pout, cb, j, x).w, w1 = hop_target<1>(g, sd, pout, cb, j, x).w;
-  if constexpr (LQ_HOP_PACK) {
+  hop_pipe_step<P, DAG, 0, D>(buf, g, sd, f, pout, cb, j, x, in, inn, w0, w1, A);
+}
+
+// FP32: every thread has two slots of its own in shared memory for a hop's nine 16-byte words, filled by cp.async
+// past L1 (.cg) two hops ahead; a slot is filled again once its words are used, and no thread reads another's, so there
+// is no barrier.
+//
+// The stencil is bound by the latency of its loads: the words in flight took a third of the registers, and 128
+// registers leave 16 warps an SM.  Without them 96 registers do, and 20 warps run (40 KB of shared memory a block).
+// Through L1 (.ca) the ring is slower than the registers were: a line that L1 keeps is written and read once more, and 200 KB
+// of slots leave little of it.  Clover, 48 systems of 8 x 32^3 on four slabs, registers -> ring: out = A y + D_hop x 557 -> 517 us,
+// A^-1 D_hop x 510 -> 475, with <r0, v> 663 -> 620, with <t, s>, |t|^2 and two with r0 686 -> 676; without clover, 24
+// systems of 16 x 24^3: 207 -> 197, 189 -> 178, 255 -> 226, 252 -> 246.  Links only in the ring, spinors in registers: 544 and more
+// for the first; a slot filled again before its hop is computed: 535; three slots: no room for more than 3 blocks.
+constexpr int RING = 2;                      // slots
+constexpr int RING_WORD = 128 * 16;          // bytes between a thread's words
+constexpr int RING_SLOT = 9 * RING_WORD;
+
+LQ_DI void ring_copy(uint32_t dst, const float4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(__cvta_generic_to_global(src)) : "memory");
+}
+template <int K>
+LQ_DI void ring_fetch(uint32_t base, const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j,
+                      const int x[4], const float4* in) {
+  if constexpr (K < 8) {
+    const uint32_t slot = base + (K % RING) * RING_SLOT;
+    const HopTgt t = hop_target<K>(g, sd, pout, cb, j, x);
+#pragma unroll
+    for (int k = 0; k < 6; k++) ring_copy(slot + k * RING_WORD, in + t.q + k * sd.n);
+    const float4* b = f.U32 + (t.pl * 4 + (K >> 1)) * 3 * g.Vh + t.cl;
+#pragma unroll
+    for (int k = 0; k < 3; k++) ring_copy(slot + (6 + k) * RING_WORD, b + k * g.Vh);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");  // one group a hop, empty past the last
+}
+template <bool DAG, int K>
+LQ_DI void ring_step(const float4 (*slots)[9][128], uint32_t base, const Geom& g, const SysDesc& sd, const FieldPtrs& f,
+                     int pout, int cb, int j, const int x[4], const float4* in, float w0, float w1, AccP& A) {
+  asm volatile("cp.async.wait_group %0;" ::"n"(RING - 1) : "memory");  // hop K's words are there
+  HopRaw<32> r;
+#pragma unroll
+  for (int k = 0; k < 6; k++) r.s[k] = slots[K % RING][k][threadIdx.x];
+#pragma unroll
+  for (int k = 0; k < 3; k++) r.u[k] = slots[K % RING][6 + k][threadIdx.x];
+  hop_apply<32, DAG, K>(r, K == 0 ? w0 : w1, A);
+  ring_fetch<K + RING>(base, g, sd, f, pout, cb, j, x, in);
+  if constexpr (K + 1 < 8) ring_step<DAG, K + 1>(slots, base, g, sd, f, pout, cb, j, x, in, w0, w1, A);
+}
+template <bool DAG>
+LQ_DI void hop_sum_ring(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j, const int x[4],
+                        const float4* in, AccP& A) {
+  __shared__ __align__(128) float4 slots[RING][9][128];
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(&slots[0][0][threadIdx.x]);
+  ring_fetch<0>(base, g, sd, f, pout, cb, j, x, in);
+  ring_fetch<1>(base, g, sd, f, pout, cb, j, x, in);
+  const float w0 = hop_target<0>(g, sd, pout, cb, j, x).w, w1 = hop_target<1>(g, sd, pout, cb, j, x).w;
+  ring_step<DAG, 0>(slots, base, g, sd, f, pout, cb, j, x, in, w0, w1, A);
+}
+
+// Sum of the eight hops at output site cb; D: pipeline depth (FP16).
+template <int P, bool DAG, int D>
+LQ_DI void hop_sum(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j, const int x[4],
+                   const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
+  if constexpr (P == 64) {
+    hop_sum_f<P, DAG>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
+  } else {
     AccP A;
 #pragma unroll
     for (int c = 0; c < 3; c++) A.ur[c] = A.ui[c] = A.lr[c] = A.li[c] = 0ull;
-    hop_pipe_step<P, DAG, 0, D>(buf, g, sd, f, pout, cb, j, x, in, inn, w0, w1, A);
+    if constexpr (P == 32)
+      hop_sum_ring<DAG>(g, sd, f, pout, cb, j, x, (const float4*)in, A);
+    else
+      hop_sum_pipe<P, DAG, D>(g, sd, f, pout, cb, j, x, in, inn, A);
 #pragma unroll
     for (int c = 0; c < 3; c++) {
       f2_unpack(A.ur[c], acc[c].re, acc[3 + c].re);
@@ -561,21 +577,7 @@ LQ_DI void hop_sum_pipe(const Geom& g, const SysDesc& sd, const FieldPtrs& f, in
       f2_unpack(A.lr[c], acc[6 + c].re, acc[9 + c].re);
       f2_unpack(A.li[c], acc[6 + c].im, acc[9 + c].im);
     }
-  } else {
-    cx<float>(&a12)[12] = *reinterpret_cast<cx<float>(*)[12]>(acc);
-#pragma unroll
-    for (int k = 0; k < 12; k++) a12[k] = {0.f, 0.f};
-    hop_pipe_step<P, DAG, 0, D>(buf, g, sd, f, pout, cb, j, x, in, inn, w0, w1, a12);
   }
-}
-
-template <int P, bool DAG, int D = HopDepth<P>::value>
-LQ_DI void hop_sum(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j, const int x[4],
-                   const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
-  if constexpr ((P == 32 || P == 16) && LQ_HOP_PIPE)
-    hop_sum_pipe<P, DAG, D>(g, sd, f, pout, cb, j, x, in, inn, acc);
-  else
-    hop_sum_f<P, DAG>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
 }
 
 // Clover block apply (A or A^{-1}) on a full spinor (FP32 / FP16).
@@ -634,44 +636,36 @@ struct HopArgs {
 // Epilogue terms present (compile time): D_hop x, A y, z.
 enum { EPI_X = 1, EPI_Y = 2, EPI_Z = 4 };
 
-// Registers are capped so that HopMinBlocks<P> blocks of 128 threads fit on
-// an SM: the FP32 / FP16 stencil is latency-bound, and occupancy together
-// with the hop pipeline is what hides its loads (with the depth-2 pipeline,
-// 4 blocks measured best for FP32 on GB300: 5 blocks spill and lose 10%;
-// LQ_HOP_MINB overrides both for experiments).  FP64 is ALU-bound and left
-// uncapped (a cap makes it spill).
-template <int P>
-struct HopMinBlocks {
-#ifdef LQ_HOP_MINB
-  static constexpr int value = P == 64 ? 1 : LQ_HOP_MINB;
-#else
-  static constexpr int value = P == 64 ? 1 : P == 32 ? 4 : 5;
-#endif
-};
-
 // Launch configurations of the one-thread-per-site stencil that the autotuner
-// chooses from (lq_tune_hop): CFG 0 is the default above; CFG 1 and 2 trade
-// blocks per SM (the register cap) against the depth of the hop pipeline.
-// FP64 has the default only.
-template <int P, int CFG>
+// chooses from (lq_tune_hop): the blocks of 128 threads per SM that the registers are capped for and, FP16, the
+// depth of the hop pipeline.  The FP32 / FP16 stencil is latency-bound, and occupancy together
+// with the pipeline is what hides its loads (LQ_HOP_MINB overrides the default's blocks for experiments).  FP32, CFG
+// 0: five blocks, 20 warps; with the seven sums and clover (WIDE) four, for five spill there (clover, 48 systems
+// of 8 x 32^3: 704 us instead of 676).  Six blocks (CFG 2) gain 4% without clover on 24 systems of 16 x 24^3 and lose 6%
+// with it.  FP64 is left uncapped (a cap makes it spill).
+template <int P, int CFG, bool WIDE = false>
 struct HopCfg {
-  static constexpr int minb = HopMinBlocks<P>::value;
-  static constexpr int depth = HopDepth<P>::value;
+#ifdef LQ_HOP_MINB
+  static constexpr int minb = P == 64 ? 1 : LQ_HOP_MINB;
+#else
+  static constexpr int minb = P == 64 ? 1 : P == 32 && WIDE ? 4 : 5;
+#endif
+  static constexpr int depth = LQ_HOP_DEPTH16;
 };
-template <>
-struct HopCfg<32, 1> {
-  static constexpr int minb = 3, depth = 3;
+template <bool WIDE>
+struct HopCfg<32, 1, WIDE> {
+  static constexpr int minb = 4, depth = 0;
 };
-template <>
-struct HopCfg<32, 2> {
-  static constexpr int minb = 5, depth = 1;
+template <bool WIDE>
+struct HopCfg<32, 2, WIDE> {
+  static constexpr int minb = WIDE ? 5 : 6, depth = 0;
 };
-template <>
-struct HopCfg<16, 1> {
+template <bool WIDE>
+struct HopCfg<16, 1, WIDE> {
   static constexpr int minb = 4, depth = 3;
 };
-template <>
-struct HopCfg<16, 2> {
+template <bool WIDE>
+struct HopCfg<16, 2, WIDE> {
   static constexpr int minb = 6, depth = 1;
 };
 constexpr int kHopCfgs = 3;
@@ -738,7 +732,7 @@ LQ_DI void red_store(R* red, const HopArgs& a, int s, int by, int nb) {
 // (terms present per EPI; A = diag * 1 without clover), with an optional
 // fused per-system reduction over the stored values (red_add).
 template <int P, bool DAG, bool CLOV, int RED, int EPI, int CFG = 0>
-__global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_lin(HopArgs a) {
+__global__ void __launch_bounds__(128, (HopCfg<P, CFG, (CLOV && RED == RED_TSW)>::minb)) k_hop_lin(HopArgs a) {
   typedef typename Prec<P>::R R;
   int s, by;
   grid_pos_tiled((int)blockIdx.x, a.nsys, a.nby, a.tile, s, by);

@@ -76,6 +76,27 @@ def test_stencil_over_a_wide_range(dims, dom, bc, csw, dag):
     lat.close()
 
 
+# 16 to 160 sites a parity against blocks of 128, slabs of one slice to all, every warp's slots of the ring
+@pytest.mark.parametrize("dims,dom", [((2, 2, 2, 4), None), ((4, 4, 4, 2), (3, 3)), ((4, 4, 4, 4), None),
+                                      ((10, 2, 4, 4), (1, 8)), ((6, 4, 2, 6), (0, 2))])
+@pytest.mark.parametrize("bc,csw,dag", [("open", 1.0, False), ("periodic", 0.0, True), ("antiperiodic", 1.0, True)])
+def test_fp32_stencil_edges(dims, dom, bc, csw, dag):
+    """2e-6 of the largest entry: 80 FP32 roundings of 6e-8 of terms below it, as for the larger lattice of the parity
+    tests."""
+    lqcd = _lq()
+    U = inputs.random_su3_field(dims, 0.4, 3)
+    lat = lqcd.Lattice(dims, bc)
+    lat.set_gauge(U, 0.13, csw)
+    op = oracle.Operator(dims, U, 0.13, csw, BCS[bc])
+    t0, t1 = dom or (0, dims[0] - 1)
+    sl = inputs.slab_sites(dims, t0, t1)
+    psi = op.masked(inputs.gaussian_spinor(dims, 4)[0], t0, t1)
+    ref = op.apply(psi, t0, t1, dagger=dag)[sl]
+    got = lat.dslash(_cuda(psi[sl]), 0, dom, dag, 32).cpu().numpy()
+    assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
+    lat.close()
+
+
 @pytest.mark.parametrize("n", [1, 4, 119, 120, 121, 241])
 def test_projected_propagator_sums(n):
     """One to three runs of 120 modes, whose sizes differ by twelve orders of magnitude."""
