@@ -422,7 +422,7 @@ int lq_force(const lqcd_lattice* L, int field, const lqcd_slab& dom, const doubl
   fs.first = want >= fs.T ? 0 : (dom.t0 + fs.T - 1) % fs.T;
   // K and B take three times the K of all slices that the plain form held (54 complex numbers a site).  Where that is
   // more than 2 GB, only as many slices at a time as keep within it: the links of a slice need B of the slices
-  // on either side, and that K of one more.  (24^3 x 48, whole lattice in runs of 13 slices of 48: 4% more work.)
+  // on either side, and that K of one more.
   constexpr int WORDS = 54 + 108;
   const double room = std::max(54.0 * 16 * L->V, 2e9);
   int run = fs.nsl;  // slots of links at a time
