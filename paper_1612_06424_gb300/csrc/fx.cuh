@@ -21,10 +21,11 @@
 // 2-norm, FP64 sums 2.1 to 2.7e-16.  Inputs keep denormals, a result below the normal range is zero; a non-finite
 // component makes its spinor and every result that it enters NaN.
 //
-// Bound by issue of integer instructions (three multiply-adds of 64 bits a product, then shifts, negations and
-// conversions) at 12 warps an SM.  32 x 16^3 with clover, 12 slabs of 14 slices: A y - D_hop x / 4 takes 683 us on the FP64 pipe, 260 us
-// so.  Four blocks an SM (126 registers, spilled) instead of three: 244 us there, but 1282 instead of 1203 us on
-// 16 x 24^3 with 24 systems; two: 246 and 1630 us.
+// Bound by latency at 12 warps an SM: issue slots 38% used (three multiply-adds of 64 bits a product, then shifts, negations
+// and conversions), waits for loads and for the multiply-adds' results in front.  32 x 16^3 with clover, 12 slabs of
+// 14 slices: A y - D_hop x / 4 takes 683 us on the FP64 pipe, 260 us so.  Four blocks an SM (126 registers, spilled)
+// instead of three: 244 us there, but 1282 instead of 1203 us on 16 x 24^3 with 24 systems; two: 246 and 1630 us.  The
+// hops' words through shared memory as in the FP32 stencil: 264 and 1355 us with four blocks, 235 and 1505 with mad_wide().
 #pragma once
 
 #include "dslash.cuh"

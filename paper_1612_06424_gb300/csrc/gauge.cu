@@ -44,67 +44,6 @@ LQ_DI void nat_coords(const Geom& g, long long i, int x[4]) {
 // max(a, b) that keeps a NaN of either
 LQ_DI double max_nan(double a, double b) { return a >= b ? a : (a == a ? b : a); }
 
-// ------------------------------------------------------------- link packing
-LQ_DI int4 limbs_of(double a, double b, int e) {
-  int4 v;
-  fx_split(fx_of(a, e), v.x, v.y);
-  fx_split(fx_of(b, e), v.z, v.w);
-  return v;
-}
-
-__global__ void k_pack_links(Geom g, const double2* U, int4* U64, float4* U32, uint2* U16,
-                             unsigned long long* maxdev) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2 * g.Vh) return;
-  int x[4];
-  nat_coords(g, i, x);
-  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-  const long long cb = i >> 1;
-  double dev = 0.0;
-  for (int mu = 0; mu < 4; mu++) {
-    su3<double> u = ld_nat(U, i, mu);
-    // unitarity: |U U^dag - 1| (Hermitian: the upper triangle), |det U - 1|; the largest of the
-    // squares, one root at the end
-#pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-      for (int b = a; b < 3; b++) {
-        cd e = {a == b ? -1.0 : 0.0, 0.0};
-#pragma unroll
-        for (int k = 0; k < 3; k++) fma_cc(e, u.m[b][k], u.m[a][k]);
-        dev = max_nan(dev, norm2(e));
-      }
-    cd det = {-1.0, 0.0};
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
-      const cd minor = u.m[1][k1] * u.m[2][k2] - u.m[1][k2] * u.m[2][k1];
-      fma_c(det, u.m[0][k], minor);
-    }
-    dev = max_nan(dev, norm2(det));
-    const long long base = (long long)(p * 4 + mu);
-#pragma unroll
-    for (int k = 0; k < 9; k++) U64[(base * 9 + k) * g.Vh + cb] = limbs_of(u.m[k / 3][k % 3].re, u.m[k / 3][k % 3].im, FX_LINK_E);
-    float r[12];
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      r[2 * k] = (float)u.m[k / 3][k % 3].re;
-      r[2 * k + 1] = (float)u.m[k / 3][k % 3].im;
-    }
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      U32[(base * 3 + k) * g.Vh + cb] = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
-      __half2 h0 = __floats2half2_rn(r[4 * k], r[4 * k + 1]);
-      __half2 h1 = __floats2half2_rn(r[4 * k + 2], r[4 * k + 3]);
-      U16[(base * 3 + k) * g.Vh + cb] = make_uint2(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1));
-    }
-  }
-  dev = sqrt(dev);
-  if (!(dev == dev)) dev = 1e300;  // NaN counts as non-unitary
-  atomicMax(maxdev, (unsigned long long)__double_as_longlong(dev));
-}
-
-// ------------------------------------------------------------------ clover
 // 3x3 complex matrices in fixed point (fxnum.cuh): entries q 2^-58 in limbs, as the links are stored.  A
 // product is 27 complex multiply-adds of 12 integer ones each, a tenth of the time of the FP64
 // product, and its entries are rounded at 2^-58 (FP64 rounds an entry of size 1 at 2^-53).
@@ -112,31 +51,17 @@ struct mcl {
   int4 m[3][3];  // (re1, re0, im1, im0)
 };
 
-LQ_DI mcl link_bc(const Geom& g, const int4* U, const int x[4], int mu) {
-  mcl u;
-  if (g.bc_t == 0 && mu == 0 && x[0] == g.L[0] - 1) {
-#pragma unroll
-    for (int k = 0; k < 9; k++) u.m[k / 3][k % 3] = make_int4(0, 0, 0, 0);
-    return u;
-  }
-  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-  const int4* b = U + (long long)(p * 4 + mu) * 9 * g.Vh + eo_index(g, x);
-#pragma unroll
-  for (int k = 0; k < 9; k++) u.m[k / 3][k % 3] = __ldg(b + (long long)k * g.Vh);
-  return u;
-}
-
 LQ_DI void mc_mac(long long& hh, long long& cr, int a1, int a0, int b1, int b0) {
   mad_wide(hh, a1, b1);
   mad_wide(cr, a1, b0);
   mad_wide(cr, a0, b1);
 }
 // entry of a product as 64-bit integers: sum over k of a_k b_k with the imaginary part of a (CA) or b (CB) negated
-template <bool CA, bool CB>
-LQ_DI longlong2 mc_dot(const int4 (&a)[3], const int4 (&b)[3]) {
+template <bool CA, bool CB, int N = 3>
+LQ_DI longlong2 mc_dot(const int4 (&a)[N], const int4 (&b)[N]) {
   long long hr = 0, cr = 1ll << 28, hi = 0, ci = 1ll << 28;  // (the halves round the shifts below)
 #pragma unroll
-  for (int k = 0; k < 3; k++) {
+  for (int k = 0; k < N; k++) {
     const int ai1 = CA ? -a[k].z : a[k].z, ai0 = CA ? -a[k].w : a[k].w;
     const int bi1 = CB ? -b[k].z : b[k].z, bi0 = CB ? -b[k].w : b[k].w;
     mc_mac(hr, cr, a[k].x, a[k].y, b[k].x, b[k].y);
@@ -152,6 +77,124 @@ LQ_DI int4 mc_limbs(longlong2 q) {
   fx_split(q.y, v.z, v.w);
   return v;
 }
+// ------------------------------------------------------------- link packing
+LQ_DI int4 limbs_of(double a, double b, int e) {
+  int4 v;
+  fx_split(fx_of(a, e), v.x, v.y);
+  fx_split(fx_of(b, e), v.z, v.w);
+  return v;
+}
+
+// Square of a link's deviation from SU(3): the largest entry of U U^dag - 1 (Hermitian: the upper triangle) and det U - 1.
+LQ_DI double su3_deviation(const su3<double>& u) {
+  double dev = 0.0;
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int b = a; b < 3; b++) {
+      cd e = {a == b ? -1.0 : 0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < 3; k++) fma_cc(e, u.m[b][k], u.m[a][k]);
+      dev = max_nan(dev, norm2(e));
+    }
+  cd det = {-1.0, 0.0};
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+    const cd minor = u.m[1][k1] * u.m[2][k2] - u.m[1][k2] * u.m[2][k1];
+    fma_c(det, u.m[0][k], minor);
+  }
+  return max_nan(dev, norm2(det));
+}
+// The same from the limbs (an eighth of the FP64 operations): false where the link is so far from SU(3), by 2^-10, that a
+// sum might not fit.
+LQ_DI bool su3_deviation(const int4 (&u)[3][3], double& dev) {
+  bool near = true;
+  auto add = [&](longlong2 v, bool one) {
+    if (one) v.x -= 1ll << 58;
+    near = near && llabs(v.x) < (1ll << 48) && llabs(v.y) < (1ll << 48);
+    const double re = fx_to_double(v.x, -58), im = fx_to_double(v.y, -58);
+    dev = fmax(dev, re * re + im * im);
+  };
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int b = a; b < 3; b++) add(mc_dot<false, true>(u[a], u[b]), a == b);
+  int4 m[3];
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+    const int4 n = u[1][k2];
+    const int4 l[2] = {u[1][k1], make_int4(-n.x, -n.y, -n.z, -n.w)}, r[2] = {u[2][k2], u[2][k1]};
+    m[k] = mc_limbs(mc_dot<false, false>(l, r));
+  }
+  add(mc_dot<false, false>(u[0], m), true);
+  return near;
+}
+
+// Natural to packed links in the three precisions and the largest deviation from SU(3), a thread a link (direction
+// blockIdx.y).  24^3 x 48: 0.75 ms with a thread a site, the deviation in FP64 and an atomic a thread; 0.36 ms so.
+__global__ void __launch_bounds__(128) k_pack_links(Geom g, const double2* U, int4* U64, float4* U32, uint2* U16,
+                                                    unsigned long long* maxdev) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned long long dv = 0;
+  if (i < 2 * g.Vh) {
+    const int mu = blockIdx.y;
+    int x[4];
+    nat_coords(g, i, x);
+    const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+    const long long cb = i >> 1;
+    const su3<double> u = ld_nat(U, i, mu);
+    int4 q[3][3];
+    int ex = 0;
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+      const cd e = u.m[k / 3][k % 3];
+      q[k / 3][k % 3] = limbs_of(e.re, e.im, FX_LINK_E);
+      ex = max(ex, max(fx_exponent(e.re), fx_exponent(e.im)));
+    }
+    double dev = 0.0;  // the largest of the squares, one root at the end
+    if (ex > 1023 || !su3_deviation(q, dev)) dev = su3_deviation(u);  // (entries of 2 and more: not limbs)
+    dev = sqrt(dev);
+    if (!(dev == dev)) dev = 1e300;  // NaN counts as non-unitary
+    dv = (unsigned long long)__double_as_longlong(dev);
+    const long long base = (long long)(p * 4 + mu);
+#pragma unroll
+    for (int k = 0; k < 9; k++) U64[(base * 9 + k) * g.Vh + cb] = q[k / 3][k % 3];
+    float r[12];
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      r[2 * k] = (float)u.m[k / 3][k % 3].re;
+      r[2 * k + 1] = (float)u.m[k / 3][k % 3].im;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      U32[(base * 3 + k) * g.Vh + cb] = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
+      __half2 h0 = __floats2half2_rn(r[4 * k], r[4 * k + 1]);
+      __half2 h1 = __floats2half2_rn(r[4 * k + 2], r[4 * k + 3]);
+      U16[(base * 3 + k) * g.Vh + cb] = make_uint2(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1));
+    }
+  }
+#pragma unroll
+  for (int k = 16; k; k >>= 1) dv = max(dv, __shfl_xor_sync(0xffffffffu, dv, k));
+  if ((threadIdx.x & 31) == 0 && dv) atomicMax(maxdev, dv);
+}
+
+// ------------------------------------------------------------------ clover
+LQ_DI mcl link_bc(const Geom& g, const int4* U, const int x[4], int mu) {
+  mcl u;
+  if (g.bc_t == 0 && mu == 0 && x[0] == g.L[0] - 1) {
+#pragma unroll
+    for (int k = 0; k < 9; k++) u.m[k / 3][k % 3] = make_int4(0, 0, 0, 0);
+    return u;
+  }
+  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+  const int4* b = U + (long long)(p * 4 + mu) * 9 * g.Vh + eo_index(g, x);
+#pragma unroll
+  for (int k = 0; k < 9; k++) u.m[k / 3][k % 3] = __ldg(b + (long long)k * g.Vh);
+  return u;
+}
+
 LQ_DI longlong2 mm_ij(const mcl& a, const mcl& b, int i, int j) {  // (a b)_ij
   const int4 r[3] = {a.m[i][0], a.m[i][1], a.m[i][2]}, c[3] = {b.m[0][j], b.m[1][j], b.m[2][j]};
   return mc_dot<false, false>(r, c);
@@ -436,7 +479,7 @@ __global__ void __launch_bounds__(128) k_clover_blocks(Geom g, long long c0, lon
 int lq_launch_pack_links(const lq::Geom& g, const double2* U, int4* U64, float4* U32, uint2* U16,
                          unsigned long long* maxdev, cudaStream_t st) {
   const long long V = 2 * g.Vh;
-  lq::k_pack_links<<<(unsigned)((V + 127) / 128), 128, 0, st>>>(g, U, U64, U32, U16, maxdev);
+  lq::k_pack_links<<<dim3((unsigned)((V + 127) / 128), 4), 128, 0, st>>>(g, U, U64, U32, U16, maxdev);
   lq_count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

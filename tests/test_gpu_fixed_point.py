@@ -76,6 +76,27 @@ def test_stencil_over_a_wide_range(dims, dom, bc, csw, dag):
     lat.close()
 
 
+# det(U) - 1 is 3 x of a scaled link and 3 i x of a turned one, U U^dag - 1 2 x and 0: 1e-10 lies between 3e-11 and 4e-11
+@pytest.mark.parametrize("change,good", [(lambda u: u * (1 + 3e-11), True), (lambda u: u * (1 - 4e-11), False),
+                                         (lambda u: u * np.exp(-3e-11j), True), (lambda u: u * np.exp(4e-11j), False),
+                                         (lambda u: u[[1, 0, 2]], False), (lambda u: 2 * u, False),
+                                         (lambda u: 1e-200 * u, False), (lambda u: 1e200 * u, False),
+                                         (lambda u: u * np.inf, False), (lambda u: u * np.nan, False)])
+def test_links_are_checked(change, good):
+    lqcd = _lq()
+    dims = (2, 2, 2, 4)
+    U = inputs.random_su3_field(dims, 0.4, 3).reshape(-1, 4, 3, 3).copy()
+    with np.errstate(invalid="ignore"):
+        U[17, 2] = change(U[17, 2])
+    lat = lqcd.Lattice(dims, "open")
+    if good:
+        lat.set_gauge(U, 0.13, 1.0)
+    else:
+        with pytest.raises(lqcd.LQCDError, match="not SU"):
+            lat.set_gauge(U, 0.13, 1.0)
+    lat.close()
+
+
 # 16 to 160 sites a parity against blocks of 128, slabs of one slice to all, every warp's slots of the ring
 @pytest.mark.parametrize("dims,dom", [((2, 2, 2, 4), None), ((4, 4, 4, 2), (3, 3)), ((4, 4, 4, 4), None),
                                       ((10, 2, 4, 4), (1, 8)), ((6, 4, 2, 6), (0, 2))])
