@@ -760,6 +760,7 @@ def run_headline(args):
     lat.set_gauge(Uf[0], wl["kappa"], wl["csw"])
     roofline, blas = _iteration_roofline(lat, [GS] * 12, [0] * 12, args.precision)
     fp64_peak = lqcd.fma_peak(64)
+    # (fixed-point sums: the fraction of the FP64 pipe's peak may pass 1)
     m64, _, f64 = lat.stencil_bench([GS] * 12, [0] * 12, 64, 0, 3)
     dslash64 = {"TFLOP/s": round(f64 / (m64 * 1e-3) / 1e12, 3), "ms": round(m64, 3), "bound": "alu",
                 "fp64_fma_peak_tflops_measured": round(fp64_peak, 3),

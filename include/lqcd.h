@@ -121,7 +121,7 @@ int lqcd_destroy_lattice(lqcd_lattice *lat);
 /* Load n_fields gauge fields U[n_fields][V][4][3][3] (complex128, natural
  * order; host memory if mem == LQCD_MEM_HOST, else device memory) with the
  * operator parameters kappa and c_sw (c_sw = 0: plain Wilson, Sec. 5).
- * Builds, per field, the even-odd packed links in FP64 / FP32 / FP16 (the
+ * Builds, per field, the even-odd packed links at FP64 (fixed-point limbs) / FP32 / FP16 (the
  * reduced copies keep the first two rows, the third is rebuilt as
  * conj(row0 x row1)), the clover blocks A(x) on every site and their
  * inverses on even sites.  Replaces any fields loaded before.
@@ -227,7 +227,7 @@ int lqcd_schur_solve(lqcd_lattice *lat, const lqcd_split *split, int n, const in
  * prop[p][3 s0 + c0][y][s][c], C = g0 g2, P_- = (1 - g0)/2; the correlator is
  * W1 - W2.  prop: device [n_prop][12][V][4][3] complex128 (e.g. fact or
  * fact + corr of lqcd_factorized_propagators); W: device [n_prop][n_t][2]
- * complex128.  FP64, one warp per site, block sums in a fixed order.
+ * complex128.  FP64 accuracy (products in fixed point), sums in a fixed order.
  * Stream-ordered.  Errors: LQCD_EBADARG, LQCD_ENOMEM, LQCD_ECUDA. */
 int lqcd_nucleon_point(lqcd_lattice *lat, int n_prop, const double *prop, int t0, int n_t, double *W, void *stream);
 
