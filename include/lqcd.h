@@ -300,7 +300,9 @@ int lqcd_projected_factors(lqcd_lattice *lat, const lqcd_split *split, int field
  *   fact[b](y)[a] = - sum_i eta_i(y)[a] conj(xi_i(x)[b]),  b = 3 s0 + c0,
  * from factors of lqcd_projected_factors (xi and eta may come from different
  * gauge fields: the n1^2 pairs of the two-level average).  fact: device
- * [12][V][4][3]; only the sites of Gamma* are written.  Synchronises.
+ * [12][V][4][3]; only the sites of Gamma* are written.  Each entry is off by
+ * a few 2^-53 of the sum of the magnitudes of its terms, whatever the modes'
+ * sizes; an entry with a term that is not finite is NaN.  Synchronises.
  * Errors: LQCD_EBADARG (1 <= n_modes <= 1024), LQCD_ECUDA. */
 int lqcd_projected_propagator(lqcd_lattice *lat, const lqcd_split *split, int n_modes, const double *xi,
                               const double *eta, const int x_src[4], double *fact, void *stream);

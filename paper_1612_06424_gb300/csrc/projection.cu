@@ -379,49 +379,140 @@ __global__ void __launch_bounds__(128) k_slice_source(Geom g, int nsys, const Sy
   }
 }
 
-// fact[b][y][a] = -sum_i eta_i(y)[a] conj(xi_i(x)[b]) for y in Gamma*; one
-// thread per (site of Gamma*, a).  xi_x[i][b] = xi_i(x)[b] in limbs, column b with exponent xe[b], is staged in
-// shared memory (n * 12 entries).  A thread reads its eta_i(y)[a] twice, for their exponent and for the sums; the
-// second read comes from L2.  Bound by the integer pipe: 144 multiply-adds (32 x 32 + 64) per complex number read.
-// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 12.8 ms so.
+// What k_proj_prop needs of a mode besides its limbs: the exponent r of its largest |xi_i(x)[b]|, and those of the twelve
+// entries relative to r and to the columns' scales, two to a word.
+struct __align__(16) ProjMode {
+  int r, pad;
+  unsigned d[6];
+};
+constexpr int PJ_NONE = -10000;  // exponent of a zero (two of them and an exponent of FP64 fit 16 bits)
+template <int X>
+constexpr int PJ_LOSS = 2 + X;
+
+LQ_DI int px_exponent(double2 v) { return max(max(fx_exponent(v.x), fx_exponent(v.y)), 1); }
+
+// The scales of a thread's sums: E, the largest exponent(eta_i) + md[i].r, and the columns that need one of their own (bit b; bit
+// 12: an eta_i is not finite), as E 2^13 + bits.
+template <int X>
+LQ_DI int pj_scan(int n, long long ld, const double2* col, const ProjMode* md) {
+  int E = PJ_NONE, emax = 1;
+  unsigned T[6];  // the largest exponent(eta_i) + exponent(xi_i[b]), relative to the columns' scales
+#pragma unroll
+  for (int k = 0; k < 6; k++) T[k] = 0x80008000u;
+  for (int i0 = 0; i0 < n; i0 += 8) {
+    double2 v[8];  // eight loads in flight (the last mode again past the end)
+#pragma unroll
+    for (int k = 0; k < 8; k++) v[k] = __ldg(col + min(i0 + k, n - 1) * ld);
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const int e = px_exponent(v[k]);
+      const int4* m = reinterpret_cast<const int4*>(md + min(i0 + k, n - 1));
+      const int4 m0 = __ldg(m), m1 = __ldg(m + 1);
+      const int s = e + m0.x;
+      emax = max(emax, e);
+      E = max(E, s);
+      const unsigned ss = __byte_perm((unsigned)s, 0, 0x1010);
+      const unsigned d[6] = {(unsigned)m0.z, (unsigned)m0.w, (unsigned)m1.x, (unsigned)m1.y, (unsigned)m1.z, (unsigned)m1.w};
+#pragma unroll
+      for (int q = 0; q < 6; q++) T[q] = __viaddmax_s16x2(d[q], ss, T[q]);
+    }
+  }
+  int w = E * 8192 + (emax == 2047 ? 4096 : 0);
+#pragma unroll
+  for (int b = 0; b < 12; b++)
+    if (E - (short)(T[b >> 1] >> (16 * (b & 1))) > PJ_LOSS<X>) w |= 1 << b;
+  return w;
+}
+template <int X>
+__global__ void __launch_bounds__(128) k_proj_scan(int n, long long ld, const double2* eta, const ProjMode* md, int* word) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < ld) word[t] = pj_scan<X>(n, ld, eta + t, md);
+}
+
+// sum_i eta_i conj(xi_i[b]), every term relative to 2^T, T the largest exponent(eta_i) + exponent(xi_i[b])
+template <int X>
+LQ_DI double2 px_column(int n, long long ld, const double2* col, const double2* xb) {
+  int T = 2;
+#pragma unroll 1
+  for (int i = 0; i < n; i++) {
+    const double2 x = __ldg(xb + 12 * i);
+    if (x.x != 0.0 || x.y != 0.0) T = max(T, px_exponent(x) + px_exponent(__ldg(col + i * ld)));
+  }
+  double2 sum = make_double2(0.0, 0.0);
+#pragma unroll 1
+  for (int i0 = 0; i0 < n; i0 += px_modes<X>) {
+    const int i1 = min(n, i0 + px_modes<X>);
+    long long t[4] = {0, 0, 0, 0};
+#pragma unroll 1
+    for (int i = i0; i < i1; i++) {
+      const double2 x = __ldg(xb + 12 * i);
+      if (x.x == 0.0 && x.y == 0.0) continue;
+      const int e = px_exponent(x);
+      px_conj_mac(t, px_limbs<X>(x, e), px_limbs<X>(__ldg(col + i * ld), T - e));
+    }
+    const double2 v = px_value(t, T - 2 * px_bias<X> + 56);
+    sum.x += v.x;
+    sum.y += v.y;
+  }
+  return sum;
+}
+
+// fact[b][y][a] = -sum_i eta_i(y)[a] conj(xi_i(x)[b]) for y in Gamma*; one thread per (site of Gamma*, a).
+//
+// Scales.  Modes may differ in size by any factor that their partners take off again, so mode i has an exponent, md[i].r, and
+// column b one, xe[b], of what is left of its entries; the limbs of xi_i(x)[b], staged in shared memory (n * 12 entries),
+// are relative to both, those of eta_i(y)[a] to E - r_i, E the largest exponent(eta_i) + r_i.  A sum is then off by a few
+// 2^-55 2^(E + xe[b]), which is what FP64 sums do as long as one of the terms of column b is not far below 2^(E + xe[b]).
+// pj_scan looks for such a term of each column, and where there is none within a factor of 2^PJ_LOSS the column is summed
+// again on a scale of its own (px_column).  Columns of modes of similar sizes seldom come there: of 120 normal modes 1e-6, of
+// 40 and of 4 1e-4.
+//
+// Bound by the integer pipe: 144 multiply-adds (32 x 32 + 64) per complex number read.  The scan is a kernel of its own
+// (SCANNED: word holds its results), bound by HBM, where there are more blocks than run at a time; next to the
+// sums it cost them 0.5 to 2 ms by the registers' and instructions' order alone.
+// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 13.1 ms so.
+template <int X, bool SCANNED>
 __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, long long y0, long long V,
-                                                   const double2* eta, const int4* xi_x, const int* xe, double2* fact) {
+                                                   const double2* eta, const int4* xi_l, const double2* xi_x,
+                                                   const ProjMode* md, const int4* r4, const int* xe, const int* word,
+                                                   double2* fact) {
   extern __shared__ int4 xs[];
-  for (int e = threadIdx.x; e < n * 12; e += blockDim.x) xs[e] = xi_x[e];
+  for (int e = threadIdx.x; e < n * 12; e += blockDim.x) xs[e] = xi_l[e];
   __syncthreads();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nsite * 12) return;
   const double2* col = eta + t;
   const long long ld = nsite * 12;
-  int E = 1;
-#pragma unroll 8
-  for (int i = 0; i < n; i++) {
-    const double2 e = __ldg(col + i * ld);
-    E = max(E, max(fx_exponent(e.x), fx_exponent(e.y)));
-  }
+  const int w = SCANNED ? __ldg(word + t) : pj_scan<X>(n, ld, col, md);
+  const int E = w >> 13;
   const long long y = y0 + t / 12;
   const int a = (int)(t % 12);
   double2 sum[12];
 #pragma unroll
   for (int b = 0; b < 12; b++) sum[b] = make_double2(0.0, 0.0);
-  for (int i0 = 0; i0 < n; i0 += px_modes<0>) {
-    const int i1 = min(n, i0 + px_modes<0>);
+  for (int i0 = 0; i0 < n; i0 += px_modes<X>) {
+    const int i1 = min(n, i0 + px_modes<X>);
     long long hr[12], cr[12], hi[12], ci[12];
 #pragma unroll
     for (int b = 0; b < 12; b++) hr[b] = cr[b] = hi[b] = ci[b] = 0;
     double2 next[4];  // loads four modes ahead
+    int4 rn = __ldg(r4 + i0 / 4);
 #pragma unroll
     for (int k = 0; k < 4; k++) next[k] = __ldg(col + min(i0 + k, i1 - 1) * ld);
+    const double2* ahead = col + (i0 + 4) * ld;
 #pragma unroll 1
     for (int i = i0; i < i1; i += 4) {
+      const int r[4] = {rn.x, rn.y, rn.z, rn.w};
+      rn = __ldg(r4 + min(i + 4, i1 - 1) / 4);
 #pragma unroll
       for (int k = 0; k < 4; k++) {
         const double2 e = next[k];
-        next[k] = __ldg(col + min(i + 4 + k, i1 - 1) * ld);
+        if (i + 4 + k < i1) next[k] = __ldg(ahead);
+        ahead += ld;
         if (i + k >= i1) continue;
         int r1, r0, m1, m0;
-        px_split<0>(e.x, E, r1, r0);
-        px_split<0>(e.y, E, m1, m0);
+        px_split<X>(e.x, E - r[k], r1, r0);
+        px_split<X>(e.y, E - r[k], m1, m0);
 #pragma unroll
         for (int b = 0; b < 12; b++) {
           const int4 c = xs[(i + k) * 12 + b];  // e conj(c)
@@ -434,37 +525,74 @@ __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, lo
     }
 #pragma unroll
     for (int b = 0; b < 12; b++) {
-      const int s = E + __ldg(xe + b) - 2 * px_bias<0> + 56;
+      const int s = E + __ldg(xe + b) - 2 * px_bias<X> + 56;
       const double re = fx_sum<28>(hr[b], cr[b], s), im = fx_sum<28>(hi[b], ci[b], s);
       sum[b] = i0 ? make_double2(sum[b].x + re, sum[b].y + im) : make_double2(re, im);
     }
   }
+  int redo = w & 4095;
 #pragma unroll
   for (int b = 0; b < 12; b++) {
-    const bool bad = E == 2047 || __ldg(xe + b) == 2047;
+    const bool bad = (w & 4096) || __ldg(xe + b) == 2047;
+    if (bad) redo &= ~(1 << b);
     fact[((long long)b * V + y) * 12 + a] = bad ? make_double2(nan(""), nan("")) : make_double2(-sum[b].x, -sum[b].y);
+  }
+#pragma unroll 1
+  while (redo) {
+    const int b = __ffs(redo) - 1;
+    redo &= redo - 1;
+    const double2 v = px_column<X>(n, ld, col, xi_x + b);
+    fact[((long long)b * V + y) * 12 + a] = make_double2(-v.x, -v.y);
   }
 }
 
-// xi_x[i][b] = xi_i(x)[b] in limbs and the exponents xe[b] of the 12 columns (one block).
+// xi_x[i][b] = xi_i(x)[b], the modes' and columns' exponents (xe[b] = 2047: column b has an entry that is not finite) and the
+// limbs (one block).
+template <int X>
 __global__ void __launch_bounds__(256) k_gather_site(int n, long long nsite_gb, long long xloc, const double2* xi,
-                                                     int4* xi_x, int* xe) {
-  __shared__ int e[12];
-  if (threadIdx.x < 12) e[threadIdx.x] = 1;
-  __syncthreads();
-  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
-    const double2 v = xi[((long long)(t / 12) * nsite_gb + xloc) * 12 + t % 12];
-    atomicMax(&e[t % 12], max(fx_exponent(v.x), fx_exponent(v.y)));
+                                                     int4* xi_l, double2* xi_x, ProjMode* md, int* r4, int* xe) {
+  __shared__ int ce[12], bad[12];
+  if (threadIdx.x < 12) {
+    ce[threadIdx.x] = PJ_NONE;
+    bad[threadIdx.x] = 0;
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
-    const double2 v = xi[((long long)(t / 12) * nsite_gb + xloc) * 12 + t % 12];
-    int4 q;
-    px_split<0>(v.x, e[t % 12], q.x, q.y);
-    px_split<0>(v.y, e[t % 12], q.z, q.w);
-    xi_x[t] = q;
+  auto exponent = [](double2 v) {  // of a number that counts: neither zero nor without a size
+    const int e = px_exponent(v);
+    return (v.x == 0.0 && v.y == 0.0) || e == 2047 ? PJ_NONE : e;
+  };
+  auto relative = [&](double2 v, int r) {
+    const int e = exponent(v);
+    return e == PJ_NONE ? PJ_NONE : e - r;
+  };
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    int r = PJ_NONE;
+#pragma unroll
+    for (int b = 0; b < 12; b++) {
+      const double2 v = xi[((long long)i * nsite_gb + xloc) * 12 + b];
+      xi_x[i * 12 + b] = v;
+      r = max(r, exponent(v));
+      if (px_exponent(v) == 2047) bad[b] = 1;
+    }
+#pragma unroll
+    for (int b = 0; b < 12; b++) atomicMax(&ce[b], relative(xi_x[i * 12 + b], r));
+    md[i].r = r4[i] = r;
   }
-  if (threadIdx.x < 12) xe[threadIdx.x] = e[threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const int r = md[i].r;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      const int d0 = relative(xi_x[i * 12 + 2 * k], r) - ce[2 * k], d1 = relative(xi_x[i * 12 + 2 * k + 1], r) - ce[2 * k + 1];
+      md[i].d[k] = ((unsigned)d0 & 0xffffu) | ((unsigned)d1 << 16);
+    }
+  }
+  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
+    double2 v = xi_x[t];
+    if (exponent(v) == PJ_NONE) v = make_double2(0.0, 0.0);
+    xi_l[t] = px_limbs<X>(v, max(md[t / 12].r + ce[t % 12], 1));
+  }
+  if (threadIdx.x < 12) xe[threadIdx.x] = bad[threadIdx.x] ? 2047 : ce[threadIdx.x];
 }
 
 struct Scratch {
@@ -564,22 +692,48 @@ int lq_slice_source(const lqcd_lattice* L, const Batch& b, const int* d_ids, int
   return launched_here();
 }
 
-int lq_proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi, long long nsite_gs,
-                 long long y0, const double2* eta, double2* fact, cudaStream_t st) {
+template <int X, bool SCANNED>
+static int proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi,
+                     long long nsite_gs, long long y0, const double2* eta, double2* fact, cudaStream_t st) {
   Scratch s;
-  RC(s.alloc(sizeof(int4) * 12 * (size_t)n + sizeof(int) * 12, st));
-  int4* xi_x = (int4*)s.p;
-  int* xe = (int*)(xi_x + 12 * (size_t)n);
-  k_gather_site<<<1, 256, 0, st>>>(n, nsite_gb, xloc, xi, xi_x, xe);
+  const size_t n4 = ((size_t)n + 3) / 4 * 4;
+  const long long nt = nsite_gs * 12;
+  RC(s.alloc((sizeof(int4) + sizeof(double2)) * 12 * n + (sizeof(ProjMode) + sizeof(int)) * n4 + sizeof(int) * 12 +
+                 (SCANNED ? sizeof(int) * (size_t)nt : 0),
+             st));
+  int4* xi_l = (int4*)s.p;
+  double2* xi_x = (double2*)(xi_l + 12 * (size_t)n);
+  ProjMode* md = (ProjMode*)(xi_x + 12 * (size_t)n);
+  int* r4 = (int*)(md + n4);
+  int* xe = r4 + n4;
+  int* word = xe + 12;
+  k_gather_site<X><<<1, 256, 0, st>>>(n, nsite_gb, xloc, xi, xi_l, xi_x, md, r4, xe);
   RC(launched_here());
   const size_t sm = sizeof(int4) * 12 * (size_t)n;
   if (sm > 48 * 1024) {
-    if (cudaFuncSetAttribute(k_proj_prop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_proj_prop<X, SCANNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
+        cudaSuccess) {
       cudaGetLastError();
       lq_set_error("projected propagator: too many modes for shared memory");
       return LQCD_EBADARG;
     }
   }
-  k_proj_prop<<<(unsigned)((nsite_gs * 12 + 127) / 128), 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_x, xe, fact);
+  const unsigned blocks = (unsigned)((nt + 127) / 128);
+  if (SCANNED) {
+    k_proj_scan<X><<<blocks, 128, 0, st>>>(n, nt, eta, md, word);
+    RC(launched_here());
+  }
+  k_proj_prop<X, SCANNED><<<blocks, 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_l, xi_x, md, (const int4*)r4, xe, word, fact);
   return launched_here();
+}
+
+// Up to 32 modes fit one sum with a bit more.
+int lq_proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi, long long nsite_gs,
+                 long long y0, const double2* eta, double2* fact, cudaStream_t st) {
+  const bool scan = nsite_gs * 12 > 152 * 2 * 128;
+  if (n <= px_modes<1>)
+    return scan ? proj_prop<1, true>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st)
+                : proj_prop<1, false>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+  return scan ? proj_prop<0, true>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st)
+              : proj_prop<0, false>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
 }
