@@ -227,7 +227,9 @@ int lqcd_schur_solve(lqcd_lattice *lat, const lqcd_split *split, int n, const in
  * prop[p][3 s0 + c0][y][s][c], C = g0 g2, P_- = (1 - g0)/2; the correlator is
  * W1 - W2.  prop: device [n_prop][12][V][4][3] complex128 (e.g. fact or
  * fact + corr of lqcd_factorized_propagators); W: device [n_prop][n_t][2]
- * complex128.  FP64 accuracy (products in fixed point), sums in a fixed order.
+ * complex128.  FP64 accuracy (products in fixed point; a site's share is off by
+ * a multiple of 2^-53 of the sum of the magnitudes of its terms, whatever the
+ * entries' sizes), sums in a fixed order.
  * Stream-ordered.  Errors: LQCD_EBADARG, LQCD_ENOMEM, LQCD_ECUDA. */
 int lqcd_nucleon_point(lqcd_lattice *lat, int n_prop, const double *prop, int t0, int n_t, double *W, void *stream);
 

@@ -321,14 +321,23 @@ __global__ void __launch_bounds__(256) k_level_mean(long long size, int count, d
 // pairs, which removes the factor 1/2 of M and half of the products.
 //
 // The products run in fixed point on the integer pipe (fxnum.cuh, 32 times the FP64 pipe's rate): a
-// site's 144 entries become 57-bit integers with one exponent, H and T are 64-bit sums, and each H Z and T U
+// site's 144 entries become 57-bit integers, H and T are 64-bit sums, and each H Z and T U
 // is rounded to FP64 once and summed there.  1620 complex multiply-adds a site in the factored form, where the
 // plain sums over all terms take 17000.  A block stages 16 sites of one slice in shared memory and
 // spreads their 16 x 144 elements H and 16 x 36 elements T over its 128 threads (consecutive threads
 // take the 8 rows (mu, a) of one (c, g, c'), so their reads of V and Z are broadcasts and those of S nearly
 // free of conflicts); three blocks an SM overlap one another's loads.  Up to four stages of a block share its
-// final sums.  Propagator of 64 x 24^3: 114.8 ms with the plain FP64 sums, one warp a site; 11.4 ms factored in
-// FP64; 5.6 ms so (error against long double 1.4e-16, of the FP64 sums 3.1e-16).
+// final sums.
+//
+// Scales.  Every term has each sink colour and each source colour once, so each of these has an exponent of its own (rho_a,
+// kappa_b; S_{(mu a),(nu b)} is stored relative to 2^(rho_a + kappa_b)) and all terms share their sum.  What is left can differ
+// by spins or by pairs of colours.  The error of a site, 0.7 2^-53 of the product of the scales, is then one of its terms only
+// if one of them is about that large: np_large_terms looks for a term of W1 and one of W2 whose three entries all lie
+// within a factor of four of their scales, and a site without them is summed in FP64 (6600 multiply-adds on a pipe a 32nd as
+// fast, which takes 2.7 times as long).
+//
+// Propagator of 64 x 24^3: 114.8 ms with the plain FP64 sums, one warp a site; 11.4 ms factored in
+// FP64; 5.8 ms so, 0.14 of them for the scales (error against long double 1.4e-16, of the FP64 sums 3.1e-16).
 constexpr int NP_T = 128;        // threads
 constexpr int NP_SITES = 16;     // sites staged at a time
 constexpr int NP_GROUPS = 4;     // most stages per block
@@ -388,13 +397,94 @@ LQ_DI np_acc np_pair(const int4* s, int ls, const int4* r, int lr, int ap, int b
   return t;
 }
 
+// The sets of large entries as bits 3 nu + b of a word for each row 3 mu + a.  Colours c' for which some mu' and {a', b', c'} have
+// (nu(mu'), b') in x and (mu', a') in y.
+LQ_DI int np_third_colour(int x, int y) {
+  x = ((x & 0x1c7) << 3) | ((x >> 3) & 0x1c7);                             // bit (mu', b')
+  const int x1 = ((x >> 1) & 0x6db) | ((x & 0x249) << 2), y1 = ((y >> 1) & 0x6db) | ((y & 0x249) << 2);  // colour c' + 1
+  const int x2 = ((x >> 2) & 0x249) | ((x << 1) & 0xdb6), y2 = ((y >> 2) & 0x249) | ((y << 1) & 0xdb6);  // c' + 2
+  const int p = (x1 & y2) | (x2 & y1);
+  return (p | p >> 3 | p >> 6 | p >> 9) & 7;
+}
+// colours of the sources of spin g and g + 2
+LQ_DI int np_source_colour(int z, int g) { return (z >> (3 * g) | z >> (3 * g + 6)) & 7; }
+// Bit 0: W1 has a term of three large entries, bit 1: W2 has; the eighth j of all terms.
+LQ_DI int np_large_terms(const int* row, int j) {
+  int found = 0;
+  for (int m = j; m < 48; m += 8) {  // H Z: (mu, g) and the order of a, b, c
+    const int mu = m & 3, g = (m >> 2) & 1, o = m >> 3;
+    const int a = o >> 1, b = (a + 1 + (o & 1)) % 3, c = 3 - a - b;
+    if (np_third_colour(row[3 * mu + a], row[3 * g + c] | row[3 * g + 6 + c]) &
+        np_source_colour(row[3 * (mu ^ 1) + b], g))
+      found |= 2;
+  }
+  for (int m = j; m < 12; m += 8) {  // T U: mu and c
+    const int mu = m & 3, c = m >> 2;
+    const int u = np_source_colour(row[c] | row[6 + c], 0) | np_source_colour(row[3 + c] | row[9 + c], 1);
+    if (np_third_colour(row[3 * mu + (c + 1) % 3], row[3 * (mu ^ 1) + (c + 2) % 3]) & u) found |= 1;
+  }
+  return found;
+}
+
+LQ_DI void np_fma(double2& t, double2 a, double2 b, double sg) {  // t += sg a b
+  const double x = sg * a.x, y = sg * a.y;
+  t.x = fma(x, b.x, fma(-y, b.y, t.x));
+  t.y = fma(x, b.y, fma(y, b.x, t.y));
+}
+// np_pair in FP64
+LQ_DI double2 np_pair64(const double2* s, int ls, const double2* r, int lr, int ap, int bp) {
+  double2 t = make_double2(0.0, 0.0);
+  for (int m = 0; m < 4; m++) {
+    const double sg = m & 1 ? 1.0 : -1.0;
+    const int nm = m ^ 1;
+    np_fma(t, s[(3 * nm + bp) * ls], r[(3 * m + ap) * lr], sg);
+    np_fma(t, s[(3 * nm + ap) * ls], r[(3 * m + bp) * lr], -sg);
+  }
+  return t;
+}
+// One site in FP64 by the whole block: its entries S (as staged), room for V and Z; adds this thread's part to w1, w2.
+LQ_DI void np_site64(const double2* S, double2* Vv, double2* Z, double2& w1, double2& w2) {
+  __syncthreads();
+  for (int e = threadIdx.x; e < 72; e += NP_T) {
+    const int c = e / 24, g = (e / 12) & 1, col = e % 12;
+    const double2 a = S[col * 12 + 3 * g + c], b = S[col * 12 + 3 * g + 6 + c];
+    Vv[e] = make_double2(a.x + b.x, a.y + b.y);
+    const int gz = e / 36, cp = (e / 12) % 3, row = e % 12;
+    const double2 u = S[(3 * gz + cp) * 12 + row], v = S[(3 * gz + 6 + cp) * 12 + row];
+    Z[e] = make_double2(u.x - v.x, u.y - v.y);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 144 + 36; e += NP_T) {
+    if (e < 144) {
+      const int mu = (e & 7) >> 1, ai = e & 1, k = e >> 3;
+      const int c = k / 6, g = (k / 3) & 1, cp = k % 3;
+      const int a = (c + 1 + ai) % 3, b = (c + 2 - ai) % 3;
+      const double2 h = np_pair64(S + 3 * mu + a, 12, Vv + (c * 2 + g) * 12, 1, (cp + 1) % 3, (cp + 2) % 3);
+      np_fma(w2, h, Z[(g * 3 + cp) * 12 + 3 * (mu ^ 1) + b], (mu ^ ai) & 1 ? 1.0 : -1.0);
+    } else {
+      const int mu = e & 3, k = (e - 144) >> 2;
+      const int c = k / 3, cp = k % 3;
+      const double2 h = np_pair64(S + 3 * mu + (c + 1) % 3, 12, S + 3 * (mu ^ 1) + (c + 2) % 3, 12, (cp + 1) % 3, (cp + 2) % 3);
+      const double2* v = Vv + c * 24;
+      const double2 u0 = v[cp], u1 = v[6 + cp], u2 = v[12 + 3 + cp], u3 = v[12 + 9 + cp];
+      np_fma(w1, h, make_double2(u0.x - u1.x + (u2.x - u3.x), u0.y - u1.y + (u2.y - u3.y)), mu & 1 ? 1.0 : -1.0);
+    }
+  }
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, long long V, const double2* prop,
                                                            long long prop_stride, int t0, double2* partial) {
   extern __shared__ __align__(16) int4 np_sm[];
   int4* S = np_sm;                         // [site][column 3 nu + b][row 3 mu + a]
   int4* Vv = S + NP_SITES * 144;           // [site][c][g][column]
   int4* Z = Vv + NP_SITES * 72;            // [site][g][c'][row]
-  __shared__ int ex[NP_SITES];             // exponents of the sites' entries
+  __shared__ int blk[NP_SITES][9];         // largest exponent of the entries of colours (a, b)
+  __shared__ int scale[NP_SITES][7];       // rho_a, kappa_b and their sum
+  __shared__ int large[NP_SITES][12];      // rows' large entries
+  __shared__ int found[NP_SITES];          // np_large_terms; 0 for a site that is not summed in fixed point
+  enum { FIXED, ZERO, NONFINITE };
+  __shared__ int kind[NP_SITES];
   const int slice = blockIdx.y;
   const double2* P = prop + (long long)blockIdx.z * prop_stride + (long long)(t0 + slice) * S3 * 12;
   double2 w1 = make_double2(0.0, 0.0), w2 = make_double2(0.0, 0.0);
@@ -403,24 +493,53 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
     const int ns = min(NP_SITES, S3 - y0);
     if (ns <= 0) break;
     if (grp) __syncthreads();
-    if (threadIdx.x < NP_SITES) ex[threadIdx.x] = 1;
+    for (int q = threadIdx.x; q < NP_SITES * 12; q += NP_T) {
+      large[q / 12][q % 12] = 0;
+      if (q < NP_SITES * 9) blk[q / 9][q % 9] = 1;
+      if (q < NP_SITES) found[q] = 0;
+    }
     __syncthreads();
     double2* Sd = reinterpret_cast<double2*>(S);
     for (int q = threadIdx.x; q < ns * 144; q += NP_T) {
       const int col = q / (ns * 12), r = q - col * (ns * 12);
-      const int site = r / 12;
+      const int site = r / 12, row = r - site * 12;
       const double2 v = __ldg(P + ((long long)col * V + y0) * 12 + r);
-      Sd[site * 144 + col * 12 + (r - site * 12)] = v;
-      atomicMax(&ex[site], max(fx_exponent(v.x), fx_exponent(v.y)));
+      Sd[site * 144 + col * 12 + row] = v;
+      atomicMax(&blk[site][3 * (row % 3) + col % 3], max(fx_exponent(v.x), fx_exponent(v.y)));
+    }
+    __syncthreads();
+    if (threadIdx.x < ns) {
+      const int* e = blk[threadIdx.x];
+      int* sc = scale[threadIdx.x];
+      int rho[3], kap[3], top = 1;
+#pragma unroll
+      for (int b = 0; b < 3; b++) kap[b] = max(max(e[b], e[3 + b]), e[6 + b]);
+#pragma unroll
+      for (int a = 0; a < 3; a++) rho[a] = max(max(e[3 * a] - kap[0], e[3 * a + 1] - kap[1]), e[3 * a + 2] - kap[2]);
+#pragma unroll
+      for (int b = 0; b < 3; b++) {
+        top = max(top, kap[b]);
+        kap[b] = max(max(e[b] - rho[0], e[3 + b] - rho[1]), e[6 + b] - rho[2]);
+      }
+      sc[6] = 0;
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        sc[k] = rho[k];
+        sc[3 + k] = kap[k];
+        sc[6] += rho[k] + kap[k];
+      }
+      kind[threadIdx.x] = top == 2047 ? NONFINITE : top == 1 ? ZERO : FIXED;  // (top 1: a product of three is zero)
     }
     __syncthreads();
     for (int q = threadIdx.x; q < ns * 144; q += NP_T) {  // in place
-      const int E = ex[q / 144];
+      const int site = q / 144, e = q - site * 144, col = e / 12, row = e - col * 12;
+      const int E = scale[site][row % 3] + scale[site][3 + col % 3];
       const double2 v = Sd[q];
       int4 l;
       fx_split(fx_of(v.x, E), l.x, l.y);
       fx_split(fx_of(v.y, E), l.z, l.w);
       S[q] = l;
+      if (max(fx_exponent(v.x), fx_exponent(v.y)) >= E - 1) atomicOr(&large[site][row], 1 << col);
     }
     __syncthreads();
     for (int q = threadIdx.x; q < ns * 72; q += NP_T) {
@@ -434,10 +553,17 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
         Z[q] = np_sub(S[site * 144 + (3 * g + cp) * 12 + row], S[site * 144 + (3 * g + 6 + cp) * 12 + row]);
       }
     }
+    if (threadIdx.x < 8 * ns) {
+      static_assert(NP_T == 8 * NP_SITES, "eight threads a site");
+      const int site = threadIdx.x >> 3;
+      const int f = kind[site] == FIXED ? np_large_terms(large[site], threadIdx.x & 7) : 0;
+      if (f) atomicOr(&found[site], f);
+    }
     __syncthreads();
-    // H and T in units of 2^58 2^(2 (E - FX_BIAS))
+    // H and T in units of 2^58 2^(the scales of their entries - 2 FX_BIAS)
     for (int q = threadIdx.x; q < ns * 144; q += NP_T) {
       const int site = q / 144, e = q - site * 144;
+      if (found[site] != 3) continue;
       const int mu = (e & 7) >> 1, ai = e & 1, k = e >> 3;
       const int c = k / 6, g = (k / 3) & 1, cp = k % 3;
       const int a = (c + 1 + ai) % 3, b = (c + 2 - ai) % 3;
@@ -447,15 +573,15 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
       int sh;
       const int4 hl = np_limbs(h, sh);
       np_mac<false>(t, hl, Z[site * 72 + (g * 3 + cp) * 12 + 3 * (mu ^ 1) + b]);
-      const int s = 3 * (ex[site] - FX_BIAS) + 2 * 58 + sh;
+      const int s = scale[site][6] - 3 * FX_BIAS + 2 * 58 + sh;
       const double re = fx_sum<29>(t.hr, t.cr, s), im = fx_sum<29>(t.hi, t.ci, s);
       const bool pos = (mu ^ ai) & 1;  // eps_{abc} cg(mu) = +1
       w2.x += pos ? re : -re;
       w2.y += pos ? im : -im;
-      if (ex[site] == 2047) w2.x = w2.y = w1.x = w1.y = nan("");  // a non-finite entry
     }
     for (int q = threadIdx.x; q < ns * 36; q += NP_T) {
       const int site = q / 36, e = q - site * 36;
+      if (found[site] != 3) continue;
       const int mu = e & 3, k = e >> 2;
       const int c = k / 3, cp = k % 3;
       const int a0 = (c + 1) % 3, b0 = (c + 2) % 3;
@@ -471,10 +597,22 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
       int sh;
       const int4 hl = np_limbs(h, sh);
       np_mac<false>(t, hl, u);
-      const int s = 3 * (ex[site] - FX_BIAS) + 2 * 58 + sh + 3;
+      const int s = scale[site][6] - 3 * FX_BIAS + 2 * 58 + sh + 3;
       const double re = fx_sum<29>(t.hr, t.cr, s), im = fx_sum<29>(t.hi, t.ci, s);
       w1.x += mu & 1 ? re : -re;
       w1.y += mu & 1 ? im : -im;
+    }
+    // the other sites, one at a time
+    for (int site = 0; site < ns; site++) {
+      if (found[site] == 3 || kind[site] == ZERO) continue;
+      if (kind[site] == NONFINITE) {
+        if (threadIdx.x == 0) w2.x = w2.y = w1.x = w1.y = nan("");
+        continue;
+      }
+      __syncthreads();  // the site's limbs are read no more
+      for (int q = threadIdx.x; q < 144; q += NP_T)
+        Sd[q] = __ldg(P + ((long long)(q / 12) * V + y0 + site) * 12 + q % 12);
+      np_site64(Sd, reinterpret_cast<double2*>(Vv), reinterpret_cast<double2*>(Z), w1, w2);
     }
   }
   __shared__ double red[4][NP_T / 32];

@@ -7,6 +7,8 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
+
 pytestmark = pytest.mark.gpu
 
 U64 = 2.0 ** -53
@@ -61,4 +63,51 @@ def test_projected_propagator_keeps_small_terms(n, scales):
     got, e, s = got[:, y], _long(eta.reshape(n, S, 12)[:, y]), _long(xi[:, np.ravel_multi_index(x, dims)].reshape(n, 12))
     ref, M = -np.einsum("nya,nb->bya", e, s.conj()), np.einsum("nya,nb->bya", abs(e), abs(s))
     assert np.all(np.abs(got - ref) <= 16 * n * U64 * M)
+    lat.close()
+
+
+def _nucleon_point(p, T, real):
+    """oracle.nucleon_point_correlator in long double, or (real) with every factor of every term replaced by its magnitude."""
+    e, cg5 = oracle.EPS3, oracle.charge_conjugation() @ oracle.gamma(4)
+    m = oracle.gamma(4) @ (0.5 * (np.eye(4) - oracle.gamma(0)))
+    P = _long(p).reshape(4, 3, -1, 4, 3).transpose(2, 3, 4, 0, 1)
+    if real:
+        e, cg5, m, P = abs(e), abs(cg5), abs(m), abs(P)
+    words = ("abc,ABC,mn,MN,gd,ymaNB,ynbMA,ydcgC->", "abc,ABC,mn,MN,gd,ymaNB,ynbgC,ydcMA->")
+    return np.array([[np.einsum(w, e, e, cg5, cg5, m, Pt, Pt, Pt, optimize="optimal") for w in words]
+                     for Pt in np.split(P, T)])
+
+
+# slices of 8 (half a stage) and 80 sites
+@pytest.mark.parametrize("dims", [(3, 2, 2, 2), (2, 4, 2, 10)])
+@pytest.mark.parametrize("scales", ["plain", "colours", "spins", "entries", "sites", "cancelling", "diagonal", "zeros"])
+def test_nucleon_point_keeps_small_terms(dims, scales):
+    """Sites summed in fixed point have a term of at least 2^-6 of the product of the scales, whose error of 0.7 u is then 45 u of
+    that term, with 4 standard deviations 180 u; FP64 sums of a few thousand terms keep less: 256 u of the sum of the terms."""
+    lqcd = _lq()
+    lat = lqcd.Lattice((4,) + dims[1:], "open")
+    r, c = _rng(22, *dims)
+    V, T = int(np.prod(dims)), dims[0]
+    p = c(12, V, 4, 3)
+    ten = lambda w, *s: 10.0 ** r.uniform(-w, w, s)  # noqa: E731
+    if scales == "colours":
+        p = p * np.tile([1e6, 1, 1e-6], 4).reshape(12, 1, 1, 1) * np.array([1e-5, 1, 1e5]) * ten(30, 1, V, 1, 1)
+    if scales == "spins":
+        p = p * np.repeat([1e8, 1e-8, 1e8, 1e-8], 3).reshape(12, 1, 1, 1) * np.array([1e-4, 1e4, 1, 1]).reshape(4, 1)
+    if scales == "entries":
+        p = p * ten(8, 12, V, 4, 3)
+    if scales == "sites":
+        p = p * ten(90, 1, V, 1, 1)
+    if scales == "cancelling":
+        p[:, :, 2:] = -p[:, :, :2] * (1 + 1e-9)
+    if scales == "diagonal":
+        p = p * (1e-12 + ((np.arange(12) % 3)[:, None, None, None] == np.arange(3)))
+    if scales == "zeros":
+        p[:, 1], p[3], p[:, 2:4, 1] = 0, 0, 0
+        p[6:, 4] = 0
+        p[np.arange(12) % 3 == 1, 5] = 0
+    full = np.zeros((12, lat.V, 4, 3), complex)
+    full[:, :V] = p
+    got = lat.nucleon_point(_cuda(full), 0, T).cpu().numpy()[0]
+    assert np.all(np.abs(got - _nucleon_point(p, T, False)) <= 256 * U64 * _nucleon_point(p, T, True))
     lat.close()
