@@ -174,12 +174,15 @@ __global__ void k_gram_reduce(const double2* part, int nsplit, int npad, int n, 
 // One block: G = L L^dag in place (lower triangle), then Linv = L^{-1}.
 // status = 1 when a pivot falls below 1e-14 of its column's squared norm
 // (the column's part orthogonal to the previous ones is below 1e-7 of its
-// norm: linearly dependent at FP64 precision for Cholesky QR).  n <= 1024.
-__global__ void __launch_bounds__(1024) k_chol_inv(double2* G, int n, double2* Linv, int* status) {
+// norm: linearly dependent at FP64 precision for Cholesky QR).  cexp: the exponents of the columns' norms.  n <= 1024.
+__global__ void __launch_bounds__(1024) k_chol_inv(double2* G, int n, double2* Linv, int* cexp, int* status) {
   __shared__ int bad;
   __shared__ double diag0[1024];
   if (threadIdx.x == 0) bad = 0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) diag0[k] = G[(long long)k * n + k].x;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    diag0[k] = G[(long long)k * n + k].x;
+    cexp[k] = fx_exponent(sqrt(diag0[k]));
+  }
   __syncthreads();
   for (int k = 0; k < n; k++) {
     if (threadIdx.x == 0) {
@@ -230,31 +233,33 @@ __global__ void __launch_bounds__(1024) k_chol_inv(double2* G, int n, double2* L
 
 // W[r][k] = sum_{j <= k} V[r][j] conj(Linv[k][j])   (W = V L^{-dag}), a thread a row and GT columns k.
 //
-// Fixed-point products (px_*): V's column j has the exponent ex[j] of its largest entry in the block's 128
-// rows, which the coefficients take off again, so that a sum over j has one scale, ek[k].  24 columns of 2.65 M rows: 10.9
+// Fixed-point products (px_*): column j of V has the exponent cx[j] of its norm, which the coefficients take off again, so
+// that a sum over j has one scale, ek[k]; the row has the exponent er of its largest entry relative to the columns', so a small
+// row keeps as many digits as a large one.  (A single W[r][k] far below its row's others does not: the coefficients'
+// own errors, 2^-53 of the norms, are worth as much in it.)  24 columns of 2.65 M rows: 10.9
 // ms with FP64 sums and 16 columns a thread, 4.1 ms so.
 constexpr int AJ = px_modes<1>;
-__global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const double2* Linv, int n) {
+__global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const double2* Linv, const int* cexp, int n) {
   __shared__ int4 cf[AJ][GT];
-  __shared__ int ex[1024], ek[GT];
+  __shared__ int cx[1024], ek[GT];
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int k0 = blockIdx.y * GT;
   const long long R = in.rows[0] + (in.nseg > 1 ? in.rows[1] : 0);
   const int jend = min(n, k0 + GT);
-  for (int j = threadIdx.x; j < jend; j += blockDim.x) ex[j] = 1;
+  for (int j = threadIdx.x; j < jend; j += blockDim.x) cx[j] = cexp[j];
   if (threadIdx.x < GT) ek[threadIdx.x] = -10000;
   __syncthreads();
+  int er = -10000;
+  bool bad = false;
+  if (r < R) {
 #pragma unroll 4
-  for (int j = 0; j < jend; j++) {
-    int x = 1;
-    if (r < R) {
+    for (int j = 0; j < jend; j++) {
       const double2 v = cm_get(in, r, j);
-      x = max(fx_exponent(v.x), fx_exponent(v.y));
+      const int x = max(max(fx_exponent(v.x), fx_exponent(v.y)), 1);
+      er = max(er, x - cx[j]);
+      bad = bad || x == 2047;
     }
-    x = __reduce_max_sync(0xffffffffu, x);
-    if ((threadIdx.x & 31) == 0) atomicMax(&ex[j], x);
   }
-  __syncthreads();
   auto coefficient = [&](int j, int q) {  // conj(Linv[k0 + q][j])
     const int k = k0 + q;
     double2 c = make_double2(0.0, 0.0);
@@ -267,7 +272,7 @@ __global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const
   for (int e = threadIdx.x; e < jend * GT; e += blockDim.x) {
     const int j = e / GT, q = e % GT;
     const double2 c = coefficient(j, q);
-    if (c.x != 0.0 || c.y != 0.0) atomicMax(&ek[q], max(fx_exponent(c.x), fx_exponent(c.y)) + ex[j]);
+    if (c.x != 0.0 || c.y != 0.0) atomicMax(&ek[q], max(fx_exponent(c.x), fx_exponent(c.y)) + cx[j]);
   }
   __syncthreads();
   double2 sum[GT];
@@ -280,13 +285,12 @@ __global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const
   auto flush = [&]() {
 #pragma unroll
     for (int q = 0; q < GT; q++) {
-      const double2 v = px_value(t[q], ek[q] - 2 * px_bias<1> + 56);
+      const double2 v = px_value(t[q], ek[q] + er - 2 * px_bias<1> + 56);
       sum[q].x += v.x;
       sum[q].y += v.y;
       t[q][0] = t[q][1] = t[q][2] = t[q][3] = 0;
     }
   };
-  bool bad = false;
   for (int j0 = 0; j0 < jend; j0 += AJ) {
     if (j0) {
       flush();
@@ -294,16 +298,14 @@ __global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const
     }
     for (int e = threadIdx.x; e < AJ * GT; e += blockDim.x) {
       const int jj = e / GT, q = e % GT;
-      if (j0 + jj < jend) cf[jj][q] = px_limbs<1>(coefficient(j0 + jj, q), ek[q] - ex[j0 + jj]);
+      if (j0 + jj < jend) cf[jj][q] = px_limbs<1>(coefficient(j0 + jj, q), ek[q] - cx[j0 + jj]);
     }
     __syncthreads();
     if (r < R) {
       const int jn = min(AJ, jend - j0);
 #pragma unroll 2
       for (int jj = 0; jj < jn; jj++) {
-        const int x = ex[j0 + jj];
-        bad = bad || x == 2047;
-        const int4 v = px_limbs<1>(cm_get(in, r, j0 + jj), x);
+        const int4 v = px_limbs<1>(cm_get(in, r, j0 + jj), er + cx[j0 + jj]);
 #pragma unroll
         for (int q = 0; q < GT; q++) {
           const int4 c = cf[jj][q];
@@ -613,17 +615,17 @@ struct Scratch {
 };
 
 // One Cholesky-QR pass: out = in R^{-1}, in = out R.
-int chol_qr(const ColMat& in, const ColMat& out, double2* G, double2* Linv, int2* d_pairs, int npairs,
+int chol_qr(const ColMat& in, const ColMat& out, double2* G, double2* Linv, int* cexp, int2* d_pairs, int npairs,
             double2* part, int nsplit, long long chunk, int npad, int* d_status, cudaStream_t st) {
   const int n = in.ncol;
   k_gram<<<dim3((unsigned)npairs, (unsigned)nsplit), 256, 0, st>>>(in, chunk, npad, d_pairs, part);
   RC(launched_here());
   k_gram_reduce<<<(unsigned)((n * n + 255) / 256), 256, 0, st>>>(part, nsplit, npad, n, G);
   RC(launched_here());
-  k_chol_inv<<<1, 1024, 0, st>>>(G, n, Linv, d_status);
+  k_chol_inv<<<1, 1024, 0, st>>>(G, n, Linv, cexp, d_status);
   RC(launched_here());
   const long long R = in.rows[0] + (in.nseg > 1 ? in.rows[1] : 0);
-  k_apply_rinv<<<dim3((unsigned)((R + 127) / 128), (unsigned)((n + GT - 1) / GT)), 128, 0, st>>>(in, out, Linv, n);
+  k_apply_rinv<<<dim3((unsigned)((R + 127) / 128), (unsigned)((n + GT - 1) / GT)), 128, 0, st>>>(in, out, Linv, cexp, n);
   return launched_here();
 }
 
@@ -652,20 +654,21 @@ int lq_orthonormalize(ColMat v, ColMat tmp, cudaStream_t st) {
   const size_t b_pairs = sizeof(int2) * npairs, b_part = sizeof(double2) * (size_t)nsplit * npad * npad,
                b_g = sizeof(double2) * (size_t)n * n;
   Scratch s;
-  RC(s.alloc(b_pairs + b_part + 2 * b_g + 256 + 64, st));
+  RC(s.alloc(b_pairs + b_part + 2 * b_g + 256 + 64 + sizeof(int) * n, st));
   char* base = (char*)s.p;
   int2* d_pairs = (int2*)base;
   double2* part = (double2*)(base + ((b_pairs + 255) / 256) * 256);
   double2* G = (double2*)((char*)part + b_part);
   double2* Linv = (double2*)((char*)G + b_g);
   int* d_status = (int*)((char*)Linv + b_g);
+  int* cexp = d_status + 16;
   if (cudaMemcpyAsync(d_pairs, pairs.data(), b_pairs, cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemsetAsync(d_status, 0, sizeof(int), st) != cudaSuccess) {
     lq_set_error("orthonormalisation: copy failed");
     return LQCD_ECUDA;
   }
-  RC(chol_qr(v, tmp, G, Linv, d_pairs, npairs, part, nsplit, chunk, npad, d_status, st));
-  RC(chol_qr(tmp, v, G, Linv, d_pairs, npairs, part, nsplit, chunk, npad, d_status, st));
+  RC(chol_qr(v, tmp, G, Linv, cexp, d_pairs, npairs, part, nsplit, chunk, npad, d_status, st));
+  RC(chol_qr(tmp, v, G, Linv, cexp, d_pairs, npairs, part, nsplit, chunk, npad, d_status, st));
   int h_status = 0;
   if (cudaMemcpyAsync(&h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess) {

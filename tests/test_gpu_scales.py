@@ -8,6 +8,7 @@ import pytest
 import torch
 
 import oracle
+from paper_1612_06424_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -110,4 +111,34 @@ def test_nucleon_point_keeps_small_terms(dims, scales):
     full[:, :V] = p
     got = lat.nucleon_point(_cuda(full), 0, T).cpu().numpy()[0]
     assert np.all(np.abs(got - _nucleon_point(p, T, False)) <= 256 * U64 * _nucleon_point(p, T, True))
+    lat.close()
+
+
+# tiles of 8 columns, runs of 32 coefficients
+@pytest.mark.parametrize("n", [1, 8, 9, 33])
+def test_orthonormal_columns_keep_small_rows(n):
+    """Every row of the result is off by n u times the condition number (below 10) of its own size: 1e-13 sqrt(n) of the row's largest
+    entry relative to the columns' norms."""
+    lqcd = _lq()
+    dims = (4, 4, 6, 6)
+    lat = lqcd.Lattice(dims, "open")
+    lat.set_gauge(inputs.unit_field(dims), 0.12, 0.0)
+    r, c = _rng(23, n)
+    S3 = int(np.prod(dims[1:]))
+    v = c(n, 3 * S3, 4, 3) * 10.0 ** r.uniform(-4, 4, (n, 1, 1, 1)) * 10.0 ** np.minimum(r.uniform(-12, 8, (3 * S3, 4, 3)), 0)
+    v[:, :, 2:] = 0
+    phi, _ = lat.boundary_modes(_cuda(v), (0, 2), 1, 0, 0, lqcd.SolverParams(tol=1e-12, precision=64))
+    A = _long(v[:, S3:2 * S3, :2].reshape(n, -1).T) / 2  # its negative below
+    G = 2 * A.conj().T @ A
+    s = np.sqrt(np.diag(G).real)
+    L = np.zeros((n, n), np.clongdouble)  # G = L L^dag, W = A L^-dag column by column
+    W = np.zeros_like(A)
+    for k in range(n):
+        L[k, k] = np.sqrt(G[k, k] - (abs(L[k, :k]) ** 2).sum())
+        L[k + 1:, k] = (G[k + 1:, k] - L[k + 1:, :k] @ L[k, :k].conj()) / L[k, k]
+        W[:, k] = (A[:, k] - W[:, :k] @ L[k, :k].conj()) / L[k, k]
+    got = phi.cpu().numpy().reshape(n, S3, 2, 2, 3)
+    for sign, half in ((1, got[:, :, 0]), (-1, got[:, :, 1])):
+        err = np.abs(sign * half.reshape(n, -1).T - W)
+        assert np.all(err.max(1) <= 1e-13 * n ** 0.5 * np.abs(A / s).max(1))
     lat.close()
