@@ -361,8 +361,8 @@ struct LinkIO<64> {
 #pragma unroll
     for (int k = 0; k < 9; k++) {
       const int4 v = __ldg(b + k * Vh);
-      u.m[k / 3][k % 3] = {fx_to_double(fx_join(v.x, v.y), FX_LINK_E - FX_BIAS),
-                           fx_to_double(fx_join(v.z, v.w), FX_LINK_E - FX_BIAS)};
+      u.m[k / 3][k % 3] = {fx_to_double<false>(fx_join(v.x, v.y), FX_LINK_E - FX_BIAS),
+                           fx_to_double<false>(fx_join(v.z, v.w), FX_LINK_E - FX_BIAS)};
     }
     return u;
   }

@@ -18,7 +18,7 @@
 //     of the eight neighbours, and the result is rounded to FP64 once.
 //
 // Error against long double over random fields, D, open and periodic, with and without clover: 1.9 to 2.2e-16 of the
-// 2-norm, FP64 sums 2.1 to 2.7e-16.  Inputs keep denormals, a result below the normal range is zero; a non-finite
+// 2-norm, FP64 sums 2.1 to 2.7e-16.  Inputs and results keep denormals; a non-finite
 // component makes its spinor and every result that it enters NaN.
 //
 // Bound by latency at 12 warps an SM: issue slots 38% used (three multiply-adds of 64 bits a product, then shifts, negations

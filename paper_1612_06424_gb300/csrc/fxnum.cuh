@@ -38,26 +38,30 @@ LQ_DI void fx_split(long long q, int& q1, int& q0) {
 }
 LQ_DI long long fx_join(int q1, int q0) { return ((long long)q1 << 29) + q0; }
 
-// v 2^e rounded to nearest; zero below the normal range.
+// v 2^e rounded to nearest.  DEN: also below the normal range, else zero there.
+template <bool DEN = true>
 LQ_DI double fx_to_double(long long v, int e) {
   if (v == 0) return 0.0;
   unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
   const int c = __clzll((long long)m);
   m <<= c;
   const int ex = 1086 - c + e;  // biased exponent of the leading bit
-  const long long b = ((long long)(ex - 1) << 52) + (long long)(m >> 11) + (long long)((m >> 10) & 1);
-  if (ex <= 0) return 0.0;
-  const long long bits = ex >= 2047 ? 0x7ff0000000000000ll : b;
+  long long bits = ((long long)(ex - 1) << 52) + (long long)(m >> 11) + (long long)((m >> 10) & 1);
+  if (ex <= 0) {  // below the normal range: m 2^(ex - 12) units of the last place
+    const int s = 12 - ex;
+    bits = !DEN ? 0 : s < 64 ? (long long)(m >> s) + (long long)((m >> (s - 1)) & 1) : s == 64 ? (long long)(m >> 63) : 0;
+  }
+  if (ex >= 2047) bits = 0x7ff0000000000000ll;
   return __longlong_as_double(v < 0 ? bits | (long long)0x8000000000000000ull : bits);
 }
 
 // (hh 2^L + cr) 2^(e - L) rounded once: the two partial sums of a product in limbs of L bits, cr joined at the
 // precision that hh leaves free
-template <int L>
+template <int L, bool DEN>
 LQ_DI double fx_sum(long long hh, long long cr, int e) {
   const int k = min(max(__clzll(hh < 0 ? ~hh : hh) - 2, 0), L);
   const int s = L - k;
-  return fx_to_double((hh << k) + (s ? (cr + (1ll << (s - 1))) >> s : cr), e - k);
+  return fx_to_double<DEN>((hh << k) + (s ? (cr + (1ll << (s - 1))) >> s : cr), e - k);
 }
 
 // exponent of the links' fixed scale: value q 2^-58

@@ -113,7 +113,7 @@ LQ_DI bool su3_deviation(const int4 (&u)[3][3], double& dev) {
   auto add = [&](longlong2 v, bool one) {
     if (one) v.x -= 1ll << 58;
     near = near && llabs(v.x) < (1ll << 48) && llabs(v.y) < (1ll << 48);
-    const double re = fx_to_double(v.x, -58), im = fx_to_double(v.y, -58);
+    const double re = fx_to_double<false>(v.x, -58), im = fx_to_double<false>(v.y, -58);
     dev = fmax(dev, re * re + im * im);
   };
 #pragma unroll
@@ -383,12 +383,12 @@ __global__ void __launch_bounds__(128) k_fhat(Geom g, const int4* U, long long c
   const long long nc = 2 * h;
   double* out = G + pl * 9 * nc + p * h + (i >> 1);
 #pragma unroll
-  for (int a = 0; a < 3; a++) out[a * nc] = -fx_to_double(f[a][a].y, EX);
+  for (int a = 0; a < 3; a++) out[a * nc] = -fx_to_double<false>(f[a][a].y, EX);
   const int ra[3] = {1, 2, 2}, rb[3] = {0, 0, 1};
 #pragma unroll
   for (int k = 0; k < 3; k++) {  // i f
-    out[(3 + 2 * k) * nc] = -fx_to_double(f[ra[k]][rb[k]].y, EX);
-    out[(4 + 2 * k) * nc] = fx_to_double(f[ra[k]][rb[k]].x, EX);
+    out[(3 + 2 * k) * nc] = -fx_to_double<false>(f[ra[k]][rb[k]].y, EX);
+    out[(4 + 2 * k) * nc] = fx_to_double<false>(f[ra[k]][rb[k]].x, EX);
   }
 }
 

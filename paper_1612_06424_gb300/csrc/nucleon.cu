@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
   __shared__ int scale[NP_SITES][7];       // rho_a, kappa_b and their sum
   __shared__ int large[NP_SITES][12];      // rows' large entries
   __shared__ int found[NP_SITES];          // np_large_terms; 0 for a site that is not summed in fixed point
-  enum { FIXED, ZERO, NONFINITE };
+  enum { FIXED, ZERO, NONFINITE, TINY };
   __shared__ int kind[NP_SITES];
   const int slice = blockIdx.y;
   const double2* P = prop + (long long)blockIdx.z * prop_stride + (long long)(t0 + slice) * S3 * 12;
@@ -528,7 +528,8 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
         sc[3 + k] = kap[k];
         sc[6] += rho[k] + kap[k];
       }
-      kind[threadIdx.x] = top == 2047 ? NONFINITE : top == 1 ? ZERO : FIXED;  // (top 1: a product of three is zero)
+      // (top 1: a product of three is zero; TINY: a term's last places may be denormals, which FP64 keeps)
+      kind[threadIdx.x] = top == 2047 ? NONFINITE : top == 1 ? ZERO : sc[6] < 3 * 1023 - 900 ? TINY : FIXED;
     }
     __syncthreads();
     for (int q = threadIdx.x; q < ns * 144; q += NP_T) {  // in place
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
       const int4 hl = np_limbs(h, sh);
       np_mac<false>(t, hl, Z[site * 72 + (g * 3 + cp) * 12 + 3 * (mu ^ 1) + b]);
       const int s = scale[site][6] - 3 * FX_BIAS + 2 * 58 + sh;
-      const double re = fx_sum<29>(t.hr, t.cr, s), im = fx_sum<29>(t.hi, t.ci, s);
+      const double re = fx_sum<29, false>(t.hr, t.cr, s), im = fx_sum<29, false>(t.hi, t.ci, s);
       const bool pos = (mu ^ ai) & 1;  // eps_{abc} cg(mu) = +1
       w2.x += pos ? re : -re;
       w2.y += pos ? im : -im;
@@ -598,7 +599,7 @@ __global__ void __launch_bounds__(NP_T, 3) k_nucleon_point(int S3, int groups, l
       const int4 hl = np_limbs(h, sh);
       np_mac<false>(t, hl, u);
       const int s = scale[site][6] - 3 * FX_BIAS + 2 * 58 + sh + 3;
-      const double re = fx_sum<29>(t.hr, t.cr, s), im = fx_sum<29>(t.hi, t.ci, s);
+      const double re = fx_sum<29, false>(t.hr, t.cr, s), im = fx_sum<29, false>(t.hi, t.ci, s);
       w1.x += mu & 1 ? re : -re;
       w1.y += mu & 1 ? im : -im;
     }

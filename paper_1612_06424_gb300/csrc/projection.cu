@@ -70,8 +70,9 @@ LQ_DI void px_conj_mac(long long (&t)[4], int4 a, int4 b) {
   px_mac(t[2], t[3], a.x, a.y, b.z, b.w);
   px_mac(t[2], t[3], -a.z, -a.w, b.x, b.y);
 }
+template <bool DEN>
 LQ_DI double2 px_value(const long long (&t)[4], int e) {
-  return make_double2(fx_sum<28>(t[0], t[1], e), fx_sum<28>(t[2], t[3], e));
+  return make_double2(fx_sum<28, DEN>(t[0], t[1], e), fx_sum<28, DEN>(t[2], t[3], e));
 }
 template <int X>
 LQ_DI int4 px_limbs(double2 v, int E) {
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(256) k_gram(ColMat m, long long chunk, int npa
     }
     long long t[4] = {0, 0, 0, 0};
     auto flush = [&]() {
-      const double2 v = px_value(t, ex[ty] + ex[GT + tx] - 2 * px_bias<1> + 56);
+      const double2 v = px_value<false>(t, ex[ty] + ex[GT + tx] - 2 * px_bias<1> + 56);
       acc.x += v.x;
       acc.y += v.y;
       t[0] = t[1] = t[2] = t[3] = 0;
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(128) k_apply_rinv(ColMat in, ColMat out, const
   auto flush = [&]() {
 #pragma unroll
     for (int q = 0; q < GT; q++) {
-      const double2 v = px_value(t[q], ek[q] + er - 2 * px_bias<1> + 56);
+      const double2 v = px_value<true>(t[q], ek[q] + er - 2 * px_bias<1> + 56);
       sum[q].x += v.x;
       sum[q].y += v.y;
       t[q][0] = t[q][1] = t[q][2] = t[q][3] = 0;
@@ -393,10 +394,10 @@ constexpr int PJ_LOSS = 2 + X;
 
 LQ_DI int px_exponent(double2 v) { return max(max(fx_exponent(v.x), fx_exponent(v.y)), 1); }
 
-// The scales of a thread's sums: E, the largest exponent(eta_i) + md[i].r, and the columns that need one of their own (bit b; bit
-// 12: an eta_i is not finite), as E 2^13 + bits.
+// The scales of a thread's sums: E, the largest exponent(eta_i) + md[i].r, and the columns that need one of their own (bit b; also
+// where the result may be a denormal number; bit 12: an eta_i is not finite), as E 2^13 + bits.
 template <int X>
-LQ_DI int pj_scan(int n, long long ld, const double2* col, const ProjMode* md) {
+LQ_DI int pj_scan(int n, long long ld, const double2* col, const ProjMode* md, const int* xe) {
   int E = PJ_NONE, emax = 1;
   unsigned T[6];  // the largest exponent(eta_i) + exponent(xi_i[b]), relative to the columns' scales
 #pragma unroll
@@ -422,13 +423,14 @@ LQ_DI int pj_scan(int n, long long ld, const double2* col, const ProjMode* md) {
   int w = E * 8192 + (emax == 2047 ? 4096 : 0);
 #pragma unroll
   for (int b = 0; b < 12; b++)
-    if (E - (short)(T[b >> 1] >> (16 * (b & 1))) > PJ_LOSS<X>) w |= 1 << b;
+    if (E - (short)(T[b >> 1] >> (16 * (b & 1))) > PJ_LOSS<X> || E + __ldg(xe + b) < 2 * 1023 - 900) w |= 1 << b;
   return w;
 }
 template <int X>
-__global__ void __launch_bounds__(128) k_proj_scan(int n, long long ld, const double2* eta, const ProjMode* md, int* word) {
+__global__ void __launch_bounds__(128) k_proj_scan(int n, long long ld, const double2* eta, const ProjMode* md,
+                                                   const int* xe, int* word) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < ld) word[t] = pj_scan<X>(n, ld, eta + t, md);
+  if (t < ld) word[t] = pj_scan<X>(n, ld, eta + t, md, xe);
 }
 
 // sum_i eta_i conj(xi_i[b]), every term relative to 2^T, T the largest exponent(eta_i) + exponent(xi_i[b])
@@ -452,7 +454,7 @@ LQ_DI double2 px_column(int n, long long ld, const double2* col, const double2* 
       const int e = px_exponent(x);
       px_conj_mac(t, px_limbs<X>(x, e), px_limbs<X>(__ldg(col + i * ld), T - e));
     }
-    const double2 v = px_value(t, T - 2 * px_bias<X> + 56);
+    const double2 v = px_value<true>(t, T - 2 * px_bias<X> + 56);
     sum.x += v.x;
     sum.y += v.y;
   }
@@ -472,7 +474,7 @@ LQ_DI double2 px_column(int n, long long ld, const double2* col, const double2* 
 // Bound by the integer pipe: 144 multiply-adds (32 x 32 + 64) per complex number read.  The scan is a kernel of its own
 // (SCANNED: word holds its results), bound by HBM, where there are more blocks than run at a time; next to the
 // sums it cost them 0.5 to 2 ms by the registers' and instructions' order alone.
-// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 13.1 ms so.
+// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 13.0 ms so.
 template <int X, bool SCANNED>
 __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, long long y0, long long V,
                                                    const double2* eta, const int4* xi_l, const double2* xi_x,
@@ -485,7 +487,7 @@ __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, lo
   if (t >= nsite * 12) return;
   const double2* col = eta + t;
   const long long ld = nsite * 12;
-  const int w = SCANNED ? __ldg(word + t) : pj_scan<X>(n, ld, col, md);
+  const int w = SCANNED ? __ldg(word + t) : pj_scan<X>(n, ld, col, md, xe);
   const int E = w >> 13;
   const long long y = y0 + t / 12;
   const int a = (int)(t % 12);
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, lo
 #pragma unroll
     for (int b = 0; b < 12; b++) {
       const int s = E + __ldg(xe + b) - 2 * px_bias<X> + 56;
-      const double re = fx_sum<28>(hr[b], cr[b], s), im = fx_sum<28>(hi[b], ci[b], s);
+      const double re = fx_sum<28, false>(hr[b], cr[b], s), im = fx_sum<28, false>(hi[b], ci[b], s);
       sum[b] = i0 ? make_double2(sum[b].x + re, sum[b].y + im) : make_double2(re, im);
     }
   }
@@ -723,7 +725,7 @@ static int proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long
   }
   const unsigned blocks = (unsigned)((nt + 127) / 128);
   if (SCANNED) {
-    k_proj_scan<X><<<blocks, 128, 0, st>>>(n, nt, eta, md, word);
+    k_proj_scan<X><<<blocks, 128, 0, st>>>(n, nt, eta, md, xe, word);
     RC(launched_here());
   }
   k_proj_prop<X, SCANNED><<<blocks, 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_l, xi_x, md, (const int4*)r4, xe, word, fact);

@@ -142,3 +142,34 @@ def test_orthonormal_columns_keep_small_rows(n):
         err = np.abs(sign * half.reshape(n, -1).T - W)
         assert np.all(err.max(1) <= 1e-13 * n ** 0.5 * np.abs(A / s).max(1))
     lat.close()
+
+
+@pytest.mark.parametrize("csw", [0.0, 1.0])
+def test_operator_below_the_normal_range(csw):
+    """Inputs of 20 bits, scaled by 2^-1040 without rounding: the result is that of the unscaled input, rounded once more."""
+    lqcd = _lq()
+    dims = (4, 2, 4, 2)
+    lat = lqcd.Lattice(dims, "open")
+    lat.set_gauge(inputs.random_su3_field(dims, 0.4, 3), 0.13, csw)
+    _, c = _rng(24)
+    z = np.round(c(lat.V, 4, 3).view(float) * 2 ** 17) / 2 ** 20
+    want = lat.dslash(_cuda(z.view(complex)), 0, None, False, 64).cpu().numpy().view(float)
+    got = lat.dslash(_cuda(np.ldexp(z, -1040).view(complex)), 0, None, False, 64).cpu().numpy().view(float)
+    assert np.all(np.abs(got - np.ldexp(want, -1040)) <= 2.0 ** -1074) and np.abs(got).max() > 0
+    lat.close()
+
+
+def test_sums_below_the_normal_range():
+    """Products near 2^-1050 of numbers of 20 bits: half a unit of the last place for each addition of FP64 numbers there."""
+    lqcd = _lq()
+    dims, x, n = (4, 2, 2, 2), (0, 1, 0, 1), 5
+    lat = lqcd.Lattice(dims, "open")
+    _, c = _rng(25)
+    xi, eta = (np.round(c(n, 16, 4, 3).view(float) * 2 ** 17).view(complex) / 2 ** 20 for _ in range(2))
+    sums = lambda k: lat.projected_propagator(_cuda(xi * 2.0 ** k), _cuda(eta * 2.0 ** k), (0, 1), (2, 3), x)  # noqa: E731
+    got, want = (sums(k).cpu().numpy()[:, 16:].copy().view(float) for k in (-525, 0))
+    assert np.all(np.abs(got - np.ldexp(want, -1050)) <= 2 * n * 2.0 ** -1074) and np.abs(got).max() > 0
+    p = np.round(c(12, lat.V, 4, 3).view(float) * 2 ** 17).view(complex) / 2 ** 20
+    got, want = (lat.nucleon_point(_cuda(p * 2.0 ** k)).cpu().numpy().view(float) for k in (-350, 0))
+    assert np.all(np.abs(got - np.ldexp(want, -1050)) <= 8 * 4608 * 2.0 ** -1074) and np.abs(got).max() > 2.0 ** -1055
+    lat.close()
