@@ -915,22 +915,13 @@ extern "C" int lqcd_dslash(lqcd_lattice* L, int field, const lqcd_slab* dom, int
     b.tblk_ok = L->S3h % 32 == 0 && (d.t1 - d.t0 + 1) % 4 == 0;
     const size_t vec = (size_t)s.n * 12 * sizeof(double2), exps = ((size_t)s.n * 2 * sizeof(int) + 255) / 256 * 256;
     DBuf buf;
-    RC(buf.alloc(512 + exps + 6 * vec, st));
+    RC(buf.alloc(512 + exps + 4 * vec, st));
     char* base = buf.as<char>();
     b.sys = (lq::SysDesc*)base;
     void** ptr = (void**)(base + 256);
-    double2* v[6];  // in, out (even, odd), in as limbs
-    for (int k = 0; k < 6; k++) v[k] = (double2*)(base + 512 + exps + k * vec);
-    VecP xl[2];
-    for (int k = 0; k < 2; k++) {
-      xl[k].d = v[4 + k];
-      xl[k].e = (int*)(base + 512) + (size_t)k * s.n;
-    }
-    RC(lq_dslash_in(L, s, (const double2*)in, out, (lq::SysDesc*)base, ptr, v[0], v[1], xl[0], xl[1], st));
-    for (int par = 0; par < 2; par++)
-      RC(lq_hop_lin(64, dagger, clov, lq::RED_NONE, L, b, par, xl[1 - par], v64(v[par]), none, none, v64(v[2 + par]),
-                    -0.5, 1.0, 0.0, st));
-    RC(lq_eo_to_nat(L, b, v[2], v[3], (double2* const*)ptr, 1.0, st));
+    double2* v[4];  // in, then out in its place (even, odd); in as limbs
+    for (int k = 0; k < 4; k++) v[k] = (double2*)(base + 512 + exps + k * vec);
+    RC(lq_dslash_fx(L, b, s, dagger, clov, (const double2*)in, out, ptr, v, (int*)(base + 512), (int*)(base + 512) + s.n, st));
     CK(cudaStreamSynchronize(st));
     return 0;
   }

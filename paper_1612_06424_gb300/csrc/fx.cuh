@@ -270,12 +270,13 @@ struct FxArgs {
   int de;
 };
 
-// Chirality block sp of a system's FP64 vector at site j.
+// Chirality block sp of a system's FP64 vector at site j.  NC: the kernel does not write the vector.
+template <bool NC = true>
 LQ_DI void fx_load6(cx<double> v[6], const void* pool, const SysDesc& sd, int j, int sp) {
   const double2* p = (const double2*)pool + sd.off * 12 + (long long)6 * sp * sd.n + j;
 #pragma unroll
   for (int k = 0; k < 6; k++) {
-    const double2 w = __ldg(p + k * sd.n);
+    const double2 w = NC ? __ldg(p + k * sd.n) : p[k * sd.n];
     v[k] = {w.x, w.y};
   }
 }
@@ -296,7 +297,7 @@ LQ_DI int fx_site(const HopArgs& a, int by) {
   return site_of_block(a.tblk, a.g.S3h, by >> 1, (by & 1) * FX_SITES + (int)(threadIdx.x >> 1));
 }
 
-// out = beta A(y) + alpha D_hop x + gamma z with k_hop_lin's reductions, y, z, w, out in FP64.
+// out = beta A(y) + alpha D_hop x + gamma z with k_hop_lin's reductions, y, z, w, out in FP64; out may be y.
 template <bool DAG, bool CLOV, int RED, int EPI>
 __global__ void __launch_bounds__(128, FX_BLOCKS) k_fx_lin(FxArgs m) {
   const HopArgs& a = m.a;
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(128, FX_BLOCKS) k_fx_lin(FxArgs m) {
   int et = e1 + 3, e2 = 0, e3 = 0;
   cx<double> yv[6], zv[6];
   int ey = 1, ez = 1;
-  if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) fx_load6(yv, a.y, sd, j, sp);
+  if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) fx_load6<false>(yv, a.y, sd, j, sp);
   if (EPI & EPI_Z) fx_load6(zv, a.z, sd, j, sp);
   if (EPI & EPI_Y) {
     ey = fx_max_exponent<6>(yv);

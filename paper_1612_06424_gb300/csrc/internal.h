@@ -113,10 +113,10 @@ int lq_convert(int Pin, int Pout, const Batch& b, VecP in, VecP out, cudaStream_
 // layout conversion: natural complex128 slab vectors <-> even-odd FP64 pools
 int lq_nat_to_eo(const lqcd_lattice* L, const Batch& b, const double2* const* src, double2* ve, double2* vo,
                  cudaStream_t st);
-// the input half of lqcd_dslash in FP64: descriptor and output pointer to the device, the natural vector
-// `in` to even / odd FP64 vectors and to limbs
-int lq_dslash_in(const lqcd_lattice* L, const lq::SysDesc& s, const double2* in, void* out, lq::SysDesc* d_sys,
-                 void** d_ptr, double2* ve, double2* vo, VecP le, VecP lo, cudaStream_t st);
+// D or D^dag of the natural vector `in` of the one system s of b at FP64 accuracy, into out.  Scratch: b.sys, d_ptr (a
+// pointer), four vectors of the system's parities and their exponents ee, eo.
+int lq_dslash_fx(const lqcd_lattice* L, const Batch& b, const lq::SysDesc& s, bool dagger, bool clov, const double2* in,
+                 void* out, void** d_ptr, double2* const v[4], int* ee, int* eo, cudaStream_t st);
 int lq_nat_to_eo_g5(const lqcd_lattice* L, const Batch& b, const double2* const* src, double2* ve, double2* vo,
                     cudaStream_t st);
 int lq_hop_kappa(const lqcd_lattice* L, const Batch& b, int pout, VecP x, double2* out, cudaStream_t st);

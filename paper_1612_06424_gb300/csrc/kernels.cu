@@ -474,10 +474,18 @@ int lq_nat_to_eo(const lqcd_lattice* L, const Batch& b, const double2* const* sr
   return launched();
 }
 
-int lq_dslash_in(const lqcd_lattice* L, const SysDesc& s, const double2* in, void* out, SysDesc* d_sys, void** d_ptr,
-                 double2* ve, double2* vo, VecP le, VecP lo, cudaStream_t st) {
-  dslash_in_launch(L->g, s, in, out, d_sys, d_ptr, ve, vo, (int4*)le.d, (int4*)lo.d, le.e, lo.e, st);
-  return launched();
+int lq_dslash_fx(const lqcd_lattice* L, const Batch& b, const SysDesc& s, bool dagger, bool clov, const double2* in,
+                 void* out, void** d_ptr, double2* const v[4], int* ee, int* eo, cudaStream_t st) {
+  dslash_in_launch(L->g, s, in, out, const_cast<SysDesc*>(b.sys), d_ptr, v[0], v[1], (int4*)v[2], (int4*)v[3], ee, eo, st);
+  int rc = launched();
+  for (int par = 0; par < 2 && !rc; par++) {  // each parity's result takes the place of its input
+    VecP x, y;
+    x.d = v[3 - par];
+    x.e = par ? ee : eo;
+    y.d = v[par];
+    rc = lq_hop_lin(64, dagger, clov, RED_NONE, L, b, par, x, y, VecP{}, VecP{}, y, -0.5, 1.0, 0.0, st);
+  }
+  return rc ? rc : lq_eo_to_nat(L, b, v[0], v[1], (double2* const*)d_ptr, 1.0, st);
 }
 
 int lq_nat_to_eo_g5(const lqcd_lattice* L, const Batch& b, const double2* const* src, double2* ve, double2* vo,

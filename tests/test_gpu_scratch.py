@@ -1,0 +1,50 @@
+"""What the FP64 operator takes of the device's memory, and the form that takes none."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+from paper_1612_06424_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _lq():
+    from paper_1612_06424_gb300 import build, lqcd
+
+    build.build()
+    return lqcd
+
+
+class _Pool:
+    """The default stream-ordered memory pool's mark of the most memory in use (CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH)."""
+
+    def __init__(self):
+        self.cu, self.h = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+        assert self.cu.cuDeviceGetDefaultMemPool(ctypes.byref(self.h), torch.cuda.current_device()) == 0
+
+    def used(self, attr):
+        v = ctypes.c_uint64()
+        assert self.cu.cuMemPoolGetAttribute(self.h, attr, ctypes.byref(v)) == 0
+        return v.value
+
+    def peak_of(self, call):
+        torch.cuda.synchronize()
+        zero, before = ctypes.c_uint64(0), self.used(7)
+        assert self.cu.cuMemPoolSetAttribute(self.h, 8, ctypes.byref(zero)) == 0
+        call()
+        return self.used(8) - before
+
+
+@pytest.mark.parametrize("dom", [None, (2, 5)])
+def test_dslash_takes_four_vectors_of_a_parity(dom):
+    lqcd = _lq()
+    dims = (8, 12, 8, 12)
+    lat = lqcd.Lattice(dims, "periodic")
+    lat.set_gauge(inputs.unit_field(dims), 0.13, 0.0)
+    n = lat.slab_len(*(dom or (0, 7)))
+    psi = torch.randn((n, 4, 3), dtype=torch.complex128, device="cuda")
+    peak = _Pool().peak_of(lambda: lat.dslash(psi, 0, dom, False, 64))
+    assert 0 < peak <= 4 * 192 * (n // 2) + 8 * (n // 2) + 4096
+    lat.close()
