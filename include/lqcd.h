@@ -428,18 +428,19 @@ int lqcd_fma_peak(int bits, double *tflops, void *stream);
  * application whose own allocator owns the GPU's memory, or a latency-
  * critical path where an allocation's cost or failure is not acceptable --
  * it calls no cudaMalloc / cudaFree or allocating library routine: its
- * scratch (even / odd copies of in and out, the system descriptor, a
- * pointer table) lives in one file-scope device array of
- * LQCD_NOALLOC_SCRATCH_BYTES that every GPU loading the library holds until
+ * scratch (even / odd copies of in, replaced by out, and their fixed-point
+ * form, the system descriptor, the output pointer) lives in a file-scope
+ * device array of LQCD_NOALLOC_SCRATCH_BYTES, and one of 170 KB for
+ * exponents, that every GPU loading the library holds until
  * the process exits.  The caller still owns and passes in / out (device).
  * Limit: the scratch needs 512 + 768 n bytes for a slab of n sites per
  * parity, so the slab may hold at most 2 floor((LQCD_NOALLOC_SCRATCH_BYTES -
  * 512) / 768) = 43 688 sites (e.g. a 16^3 x 10 slab); larger slabs return
- * LQCD_EBADARG.  The descriptor and the in / out pointers reach the scratch
- * array as kernel arguments of a one-thread set-up kernel.
+ * LQCD_EBADARG.  The descriptor and the output pointer reach the scratch
+ * array as arguments of the first kernel.
  * The first call on a device looks up the array's device address (with that
- * device current) and caches it.  All calls share the one array and it
- * keeps the last call's contents (every word a call reads is written by
+ * device current) and caches it.  All calls share the arrays, which
+ * keep the last call's contents (every word a call reads is written by
  * that call first): calls that overlap on the GPU -- on different streams
  * or host threads without ordering between them -- race and must not be
  * issued.  Stream-ordered; does not synchronise.  Errors: LQCD_EBADARG, LQCD_ENOFIELD, LQCD_ECUDA. */

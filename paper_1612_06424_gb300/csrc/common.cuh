@@ -403,7 +403,7 @@ struct LinkIO<16> {
   }
 };
 
-// Clover block access: FP64 for P = 64, FP32 otherwise.
+// Clover block access (FP32 blocks).
 template <int P>
 struct ClovIO {
   typedef float R;
@@ -433,33 +433,6 @@ struct ClovIO {
         q += 2;
         fma_c(out[r], e, in[c]);
         fma_cc(out[c], e, in[r]);
-      }
-  }
-};
-
-template <>
-struct ClovIO<64> {
-  typedef double R;
-  // out += A in, the block's 36 reals in limbs with exponent e
-  LQ_DI static void apply_add(const int4* base, int e, int Vh, int cb, const cx<double> in[6], cx<double> out[6]) {
-    double a[36];
-#pragma unroll
-    for (int k = 0; k < 18; k++) {
-      const int4 v = __ldg(base + k * Vh + cb);
-      a[2 * k] = fx_to_double(fx_join(v.x, v.y), e - FX_BIAS);
-      a[2 * k + 1] = fx_to_double(fx_join(v.z, v.w), e - FX_BIAS);
-    }
-#pragma unroll
-    for (int r = 0; r < 6; r++) out[r] = {fma(a[r], in[r].re, out[r].re), fma(a[r], in[r].im, out[r].im)};
-    int q = 6;
-#pragma unroll
-    for (int r = 1; r < 6; r++)
-#pragma unroll
-      for (int c = 0; c < r; c++) {
-        const cx<double> e2 = {a[q], a[q + 1]};
-        q += 2;
-        fma_c(out[r], e2, in[c]);
-        fma_cc(out[c], e2, in[r]);
       }
   }
 };

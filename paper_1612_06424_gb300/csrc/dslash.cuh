@@ -64,16 +64,6 @@ LQ_DI void expand_add(cx<R> acc[12], const cx<R> w[6]) {
   }
 }
 
-// acc = (1 + S g_mu) expanded from w, for mu = 0 (the first term of a hop sum).
-template <int S, typename R>
-LQ_DI void expand_set0(cx<R> acc[12], const cx<R> w[6]) {
-#pragma unroll
-  for (int c = 0; c < 6; c++) {
-    acc[c] = w[c];
-    acc[6 + c] = S > 0 ? -w[c] : w[c];
-  }
-}
-
 template <typename R>
 LQ_DI void mul_u(const su3<R>& u, const cx<R> h[6], cx<R> w[6]) {
 #pragma unroll
@@ -100,22 +90,10 @@ LQ_DI void mul_udag(const su3<R>& u, const cx<R> h[6], cx<R> w[6]) {
     }
 }
 
-// Neighbour spinor fetch of the stencil: (local index, window hint) -> psi.
-// Window hints: 0 the site's own row (x2, x3 hops), 1 / 2 the rows at
-// x1 -+ 1, 3 / 4 the rows at x0 -+ 1.
-template <int P>
-struct GlobalFetch {
-  const void* in;
-  const float* inn;
-  int n;
-  LQ_DI void operator()(int q, int, cx<typename Prec<P>::R> psi[12]) const { Prec<P>::load(psi, in, inn, n, q); }
-};
-
-// FIRST: acc is zero on entry, and the forward term is assigned.  The sign of a wrapping time hop is a
-// sign flip, not a product: FP64 (ALU-bound) pays for every instruction.
-template <int P, bool DAG, int MU, bool FIRST, typename Fetch>
-LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, const int x[4],
-                     const Fetch& fetch, cx<typename Prec<P>::R> acc[12]) {
+// The two hops of direction MU, without a pipeline.
+template <int P, bool DAG, int MU>
+LQ_DI void hop_dir(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, const int x[4],
+                   const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
   typedef typename Prec<P>::R R;
   constexpr int SF = DAG ? +1 : -1;  // forward projector (1 + SF g_mu)
   constexpr int SB = -SF;           // backward projector
@@ -139,7 +117,7 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
     if (ok) {
       const int cy = eo_index(g, y);
       cx<R> psi[12], h[6], w[6];
-      fetch(cy - sd.cb0, MU == 0 ? 4 : MU == 1 ? 2 : 0, psi);
+      Prec<P>::load(psi, in, inn, sd.n, cy - sd.cb0);
       project<MU, SF>(psi, h);
       su3<R> u = LinkIO<P>::load(f, pout, MU, g.Vh, cb);
       mul_u(u, h, w);
@@ -147,10 +125,7 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
 #pragma unroll
         for (int k = 0; k < 6; k++) w[k] = -w[k];
       }
-      if constexpr (FIRST && MU == 0)
-        expand_set0<SF>(acc, w);
-      else
-        expand_add<MU, SF>(acc, w);
+      expand_add<MU, SF>(acc, w);
     }
   }
   // ---- backward: U_mu(x - mu)^dag psi(x - mu)
@@ -172,7 +147,7 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
     if (ok) {
       const int cy = eo_index(g, y);
       cx<R> psi[12], h[6], w[6];
-      fetch(cy - sd.cb0, MU == 0 ? 3 : MU == 1 ? 1 : 0, psi);
+      Prec<P>::load(psi, in, inn, sd.n, cy - sd.cb0);
       project<MU, SB>(psi, h);
       su3<R> u = LinkIO<P>::load(f, pin, MU, g.Vh, cy);
       mul_udag(u, h, w);
@@ -183,23 +158,6 @@ LQ_DI void hop_dir_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int p
       expand_add<MU, SB>(acc, w);
     }
   }
-}
-
-template <int P, bool DAG, int MU>
-LQ_DI void hop_dir(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, const int x[4],
-                   const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
-  hop_dir_f<P, DAG, MU, false>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
-}
-
-template <int P, bool DAG, typename Fetch>
-LQ_DI void hop_sum_f(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, const int x[4],
-                     const Fetch& fetch, cx<typename Prec<P>::R> acc[12]) {
-#pragma unroll
-  for (int k = 0; k < 12; k++) acc[k] = {0, 0};
-  hop_dir_f<P, DAG, 0, true>(g, sd, f, pout, cb, x, fetch, acc);
-  hop_dir_f<P, DAG, 1, false>(g, sd, f, pout, cb, x, fetch, acc);
-  hop_dir_f<P, DAG, 2, false>(g, sd, f, pout, cb, x, fetch, acc);
-  hop_dir_f<P, DAG, 3, false>(g, sd, f, pout, cb, x, fetch, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -560,23 +518,19 @@ LQ_DI void hop_sum_ring(const Geom& g, const SysDesc& sd, const FieldPtrs& f, in
 template <int P, bool DAG, int D>
 LQ_DI void hop_sum(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j, const int x[4],
                    const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
-  if constexpr (P == 64) {
-    hop_sum_f<P, DAG>(g, sd, f, pout, cb, x, GlobalFetch<P>{in, inn, sd.n}, acc);
-  } else {
-    AccP A;
+  AccP A;
 #pragma unroll
-    for (int c = 0; c < 3; c++) A.ur[c] = A.ui[c] = A.lr[c] = A.li[c] = 0ull;
-    if constexpr (P == 32)
-      hop_sum_ring<DAG>(g, sd, f, pout, cb, j, x, (const float4*)in, A);
-    else
-      hop_sum_pipe<P, DAG, D>(g, sd, f, pout, cb, j, x, in, inn, A);
+  for (int c = 0; c < 3; c++) A.ur[c] = A.ui[c] = A.lr[c] = A.li[c] = 0ull;
+  if constexpr (P == 32)
+    hop_sum_ring<DAG>(g, sd, f, pout, cb, j, x, (const float4*)in, A);
+  else
+    hop_sum_pipe<P, DAG, D>(g, sd, f, pout, cb, j, x, in, inn, A);
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
-      f2_unpack(A.ur[c], acc[c].re, acc[3 + c].re);
-      f2_unpack(A.ui[c], acc[c].im, acc[3 + c].im);
-      f2_unpack(A.lr[c], acc[6 + c].re, acc[9 + c].re);
-      f2_unpack(A.li[c], acc[6 + c].im, acc[9 + c].im);
-    }
+  for (int c = 0; c < 3; c++) {
+    f2_unpack(A.ur[c], acc[c].re, acc[3 + c].re);
+    f2_unpack(A.ui[c], acc[c].im, acc[3 + c].im);
+    f2_unpack(A.lr[c], acc[6 + c].re, acc[9 + c].re);
+    f2_unpack(A.li[c], acc[6 + c].im, acc[9 + c].im);
   }
 }
 
@@ -586,23 +540,6 @@ LQ_DI void clover_apply(const FieldPtrs& f, bool inverse, int p, int Vh, int cb,
   const float4* base = inverse ? f.Ai32 : f.A32 + p * 18 * Vh;
   ClovIO<32>::apply(base, Vh, cb, in, out);
   ClovIO<32>::apply(base + 9 * Vh, Vh, cb, in + 6, out + 6);
-}
-
-// FP64 site-diagonal term: res += be A in, A the clover block or diag.
-LQ_DI void diag_add64(bool clov, const FieldPtrs& f, int p, int Vh, int cb, double diag, double be,
-                      const cx<double> in[12], cx<double> res[12]) {
-  cx<double> y[12];
-#pragma unroll
-  for (int k = 0; k < 12; k++) y[k] = be * in[k];
-  if (clov) {
-    const int4* base = f.A64 + p * 36 * Vh;
-    const int* e = f.A64e + p * 2 * Vh + cb;
-    ClovIO<64>::apply_add(base, e[0], Vh, cb, y, res);
-    ClovIO<64>::apply_add(base + 18 * Vh, e[Vh], Vh, cb, y + 6, res + 6);
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; k++) res[k] = {fma(diag, y[k].re, res[k].re), fma(diag, y[k].im, res[k].im)};
-  }
 }
 
 // Arguments of the hop kernels.  Vector pointers are pool bases; system s
@@ -642,13 +579,13 @@ enum { EPI_X = 1, EPI_Y = 2, EPI_Z = 4 };
 // with the pipeline is what hides its loads (LQ_HOP_MINB overrides the default's blocks for experiments).  FP32, CFG
 // 0: five blocks, 20 warps; with the seven sums and clover (WIDE) four, for five spill there (clover, 48 systems
 // of 8 x 32^3: 704 us instead of 676).  Six blocks (CFG 2) gain 4% without clover on 24 systems of 16 x 24^3 and lose 6%
-// with it.  FP64 is left uncapped (a cap makes it spill).
+// with it.
 template <int P, int CFG, bool WIDE = false>
 struct HopCfg {
 #ifdef LQ_HOP_MINB
-  static constexpr int minb = P == 64 ? 1 : LQ_HOP_MINB;
+  static constexpr int minb = LQ_HOP_MINB;
 #else
-  static constexpr int minb = P == 64 ? 1 : P == 32 && WIDE ? 4 : 5;
+  static constexpr int minb = P == 32 && WIDE ? 4 : 5;
 #endif
   static constexpr int depth = LQ_HOP_DEPTH16;
 };
@@ -760,9 +697,7 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG, (CLOV && RED == RED_TSW)>
     }
     cx<R> yv[12];
     if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) Prec<P>::load(yv, sys_ptr<P>(a.y, sd.off), nrm_ptr(a.yn, sd.off), sd.n, j);
-    if constexpr ((EPI & EPI_Y) && P == 64) {
-      diag_add64(CLOV, f, a.pout, a.g.Vh, cb, a.diag, a.beta, yv, res);
-    } else if (EPI & EPI_Y) {
+    if (EPI & EPI_Y) {
       cx<R> ay[12];
       if (CLOV) {
         clover_apply(f, false, a.pout, a.g.Vh, cb, yv, ay);

@@ -158,12 +158,6 @@ static int launch_lin(int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t 
   return 0;
 }
 
-template <bool DAG, bool CLOV>
-static int launch_lin64(dim3 gr, const HopArgs& a, cudaStream_t st) {
-  k_hop_lin<64, DAG, CLOV, RED_NONE, EPI_X | EPI_Y><<<gr, LQ_BLOCK, 0, st>>>(a);
-  return 0;
-}
-
 template <int P>
 static int launch_lin_p(bool dag, bool clov, int red, int epi, dim3 gr, const HopArgs& a, cudaStream_t st) {
   if (dag) return clov ? launch_lin<P, true, true>(red, epi, gr, a, st) : launch_lin<P, true, false>(red, epi, gr, a, st);
@@ -228,18 +222,17 @@ int lq_hop_lin(int P, bool dag, bool clov, int red, const lqcd_lattice* L, const
   }
   const int v = variant_of(P, b);
   int rc;
-  if (P == 64 && x.e) {
+  if (P == 64) {
+    if (!x.e) {
+      lq_set_error("FP64 hop kernel: the hop input must be in limbs");
+      return LQCD_EBADARG;
+    }
     FxArgs m;
     rc = fx_args(m, a, x, a.diag);
     if (rc) return rc;
     set_grid_order(m.a, L, b, FX_SITES);
     m.a.tblk = tblk_of(b);
     rc = fx_lin_launch(dag, clov, red, epi, grid_lin(b, (b.max_n + FX_SITES - 1) / FX_SITES), m, st);
-  } else if (P == 64) {
-    // FP64 arithmetic on FP64 vectors: lqcd_dslash_noalloc, whose scratch has no room for limbs
-    rc = red == RED_NONE && epi == (EPI_X | EPI_Y) ? 0 : -1;
-    if (!rc && dag) rc = clov ? launch_lin64<true, true>(gr, a, st) : launch_lin64<true, false>(gr, a, st);
-    else if (!rc) rc = clov ? launch_lin64<false, true>(gr, a, st) : launch_lin64<false, false>(gr, a, st);
   } else if (!dag && v >= 3)
     rc = P == 32 ? hop_lin_tuned<32>(v - 2, clov, red, epi, gr, a, st) : hop_lin_tuned<16>(v - 2, clov, red, epi, gr, a, st);
   else

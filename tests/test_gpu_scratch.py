@@ -48,3 +48,36 @@ def test_dslash_takes_four_vectors_of_a_parity(dom):
     peak = _Pool().peak_of(lambda: lat.dslash(psi, 0, dom, False, 64))
     assert 0 < peak <= 4 * 192 * (n // 2) + 8 * (n // 2) + 4096
     lat.close()
+
+
+# 2 x 21840 sites are four sites a parity below the limit of the scratch
+@pytest.mark.parametrize("dims,dom,bc", [((2, 2, 2, 4), None, "periodic"), ((6, 4, 2, 10), (1, 4), "open"),
+                                         ((4, 2, 2, 2730), None, "antiperiodic"), ((4, 8, 8, 4), None, "open")])
+@pytest.mark.parametrize("csw,dag", [(0.0, 0), (1.0, 1)])
+def test_noalloc_dslash_is_dslash(dims, dom, bc, csw, dag):
+    """The same kernels in the same order, also replayed from a captured graph."""
+    lqcd = _lq()
+    lat = lqcd.Lattice(dims, bc)
+    lat.set_gauge(inputs.random_su3_field(dims, 0.4, 91), 0.13, csw)
+    n = lat.slab_len(*(dom or (0, dims[0] - 1)))
+    psi = torch.from_numpy(inputs.gaussian_spinor(dims, 92)[0][:n] * 10.0 ** np.arange(-6, 6).reshape(4, 3)).cuda()
+    out = torch.full_like(psi, float("nan"))
+    L = lqcd.lib()
+    L.lqcd_dslash_noalloc.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(lqcd.Slab), ctypes.c_int,
+                                      ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+
+    def call():
+        rc = L.lqcd_dslash_noalloc(lat._h, 0, ctypes.byref(lqcd.Slab(*dom)) if dom else None, dag, psi.data_ptr(),
+                                   out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert rc == 0, L.lqcd_last_error()
+
+    peak = _Pool().peak_of(call)
+    assert peak == 0
+    assert torch.equal(out, lat.dslash(psi, 0, dom, bool(dag), 64))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    psi.mul_(0.5)
+    graph.replay()
+    assert torch.equal(out, lat.dslash(psi, 0, dom, bool(dag), 64))
+    lat.close()
