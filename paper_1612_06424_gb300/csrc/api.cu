@@ -1871,8 +1871,8 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
                                   double* bytes_per_launch, double* flops_per_launch, void* stream) {
   RC(check_lat(L));
   if (n_sys < 1 || !doms || !field_ids || reps < 1 || (precision != 64 && precision != 32 && precision != 16) ||
-      kernel < 0 || kernel > 6) {
-    lq_set_error("stencil_bench: bad arguments");
+      kernel < 0 || kernel > 5) {
+    lq_set_error("stencil_bench: bad arguments (kernels 0 to 5)");
     return LQCD_EBADARG;
   }
   cudaStream_t st = (cudaStream_t)stream;
@@ -1940,7 +1940,7 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
   const double S = precision == 64 ? 192.0 : precision == 32 ? 96.0 : 52.0;
   const double Lk = precision == 64 ? 144.0 : precision == 32 ? 48.0 : 24.0;
   const double C = clov ? (precision == 64 ? 576.0 : 288.0) : 0.0;
-  static const double passes[7] = {3, 2, 4, 4, 3, 8, 8};
+  static const double passes[6] = {3, 2, 4, 4, 3, 8};
   double bytes = 0.0, sites = 0.0;
   std::vector<std::vector<char>> used(L->fields.size(), std::vector<char>(L->dims[0], 0));
   for (int k = 0; k < n_sys; k++) {
@@ -1954,8 +1954,8 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
         if (c) bytes += (8.0 * Lk + C) * (double)L->S3h;
   // flop per system site: hop 1320, site-diagonal block 504 (clover) or 24, epilogue and reductions
   const double diag = clov ? 504.0 : 24.0;
-  const double flop[7] = {1320.0 + diag + 72.0, 1320.0 + diag + 24.0, 1320.0 + diag + 72.0 + 96.0,
-                          1320.0 + diag + 72.0 + 336.0, 96.0, 528.0, 528.0};
+  const double flop[6] = {1320.0 + diag + 72.0, 1320.0 + diag + 24.0, 1320.0 + diag + 72.0 + 96.0,
+                          1320.0 + diag + 72.0 + 336.0, 96.0, 528.0};
   const double fl = sites * flop[kernel];
   if (ms_per_launch) *ms_per_launch = ms / reps;
   if (bytes_per_launch) *bytes_per_launch = bytes;

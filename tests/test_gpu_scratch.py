@@ -1,4 +1,4 @@
-"""What the FP64 operator takes of the device's memory, and the form that takes none."""
+"""What the FP64 operator takes of the device's memory, the form that takes none, and the timing hook."""
 import ctypes
 
 import numpy as np
@@ -80,4 +80,18 @@ def test_noalloc_dslash_is_dslash(dims, dom, bc, csw, dag):
     psi.mul_(0.5)
     graph.replay()
     assert torch.equal(out, lat.dslash(psi, 0, dom, bool(dag), 64))
+    lat.close()
+
+
+def test_stencil_bench_knows_its_kernels():
+    """Six kernels, each under one number: an iteration's sum over all numbers counts none twice."""
+    lqcd = _lq()
+    lat = lqcd.Lattice((4, 4, 4, 4), "open")
+    lat.set_gauge(inputs.unit_field((4, 4, 4, 4)), 0.13, 1.0)
+    for kernel in range(6):
+        for precision in (64, 32, 16):
+            assert lat.stencil_bench([(0, 3)] * 2, [0] * 2, precision, kernel, 1)[0] > 0
+    for kernel in (-1, 6):
+        with pytest.raises(lqcd.LQCDError, match="bad arguments"):
+            lat.stencil_bench([(0, 3)], [0], 32, kernel, 1)
     lat.close()
