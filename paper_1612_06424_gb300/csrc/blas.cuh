@@ -378,7 +378,7 @@ __global__ void k_finalize(int mode, int nsys, const SysDesc* sys, int* active, 
   if (active && !active[s]) return;  // uniform over the block
   const int nb = (sys[s].n * wps + bdim - 1) / bdim;
   double v[7] = {0.0};
-  block_sum_partials<3, 4>(partial + (long long)s * pstride * 4, nb, v);
+  block_sum_partials<3, 4, FIN_THREADS / 32>(partial + (long long)s * pstride * 4, nb, v);
   if (threadIdx.x != 0) return;
   SolverScal c = sc[s];
   fin_update(mode, v, c, active + s, tau2, floor_rel2);

@@ -514,8 +514,11 @@ LQ_DI void hop_sum_ring(const Geom& g, const SysDesc& sd, const FieldPtrs& f, in
   ring_step<DAG, 0>(slots, base, g, sd, f, pout, cb, j, x, in, w0, w1, A);
 }
 
-// Sum of the eight hops at output site cb; D: pipeline depth (FP16).
-template <int P, bool DAG, int D>
+template <int P, int CFG, bool WIDE = false>
+struct HopCfg;
+
+// Sum of the eight hops at output site cb.
+template <int P, bool DAG, int CFG>
 LQ_DI void hop_sum(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pout, int cb, int j, const int x[4],
                    const void* in, const float* inn, cx<typename Prec<P>::R> acc[12]) {
   AccP A;
@@ -524,7 +527,7 @@ LQ_DI void hop_sum(const Geom& g, const SysDesc& sd, const FieldPtrs& f, int pou
   if constexpr (P == 32)
     hop_sum_ring<DAG>(g, sd, f, pout, cb, j, x, (const float4*)in, A);
   else
-    hop_sum_pipe<P, DAG, D>(g, sd, f, pout, cb, j, x, in, inn, A);
+    hop_sum_pipe<P, DAG, HopCfg<P, CFG>::depth>(g, sd, f, pout, cb, j, x, in, inn, A);
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     f2_unpack(A.ur[c], acc[c].re, acc[3 + c].re);
@@ -577,10 +580,10 @@ enum { EPI_X = 1, EPI_Y = 2, EPI_Z = 4 };
 // chooses from (lq_tune_hop): the blocks of 128 threads per SM that the registers are capped for and, FP16, the
 // depth of the hop pipeline.  The FP32 / FP16 stencil is latency-bound, and occupancy together
 // with the pipeline is what hides its loads (LQ_HOP_MINB overrides the default's blocks for experiments).  FP32, CFG
-// 0: five blocks, 20 warps; with the seven sums and clover (WIDE) four, for five spill there (clover, 48 systems
-// of 8 x 32^3: 704 us instead of 676).  Six blocks (CFG 2) gain 4% without clover on 24 systems of 16 x 24^3 and lose 6%
-// with it.
-template <int P, int CFG, bool WIDE = false>
+// 0: five blocks, 20 warps; with the seven sums and clover (WIDE) four: five spill there and measure the same (clover, 48
+// systems of 8 x 32^3: 662 and 664 us).  Six blocks (CFG 2) gain 4% without clover and sums on 24 systems of 16 x 24^3 and 1%
+// with <t, s>, |t|^2 and two with r0, lose 2% with <r0, v> and 4 to 10% with clover.
+template <int P, int CFG, bool WIDE>
 struct HopCfg {
 #ifdef LQ_HOP_MINB
   static constexpr int minb = LQ_HOP_MINB;
@@ -591,11 +594,11 @@ struct HopCfg {
 };
 template <bool WIDE>
 struct HopCfg<32, 1, WIDE> {
-  static constexpr int minb = 4, depth = 0;
+  static constexpr int minb = 4;
 };
 template <bool WIDE>
 struct HopCfg<32, 2, WIDE> {
-  static constexpr int minb = WIDE ? 5 : 6, depth = 0;
+  static constexpr int minb = WIDE ? 5 : 6;
 };
 template <bool WIDE>
 struct HopCfg<16, 1, WIDE> {
@@ -641,7 +644,6 @@ LQ_DI void red_add(R* red, const cx<R>* res, const cx<R>* y, const cx<R>* w) {
     }
   }
 }
-// Stores the block's sums (4 doubles a block, 8 for RED_TSW) and finishes the system if asked to.
 template <int P>
 LQ_DI const void* sys_ptr(const void* pool, long long off) {
   return pool ? (const void*)((const char*)pool + off * (long long)Prec<P>::NV * 16) : nullptr;
@@ -653,6 +655,7 @@ LQ_DI void* sys_ptr_w(void* pool, long long off) {
 LQ_DI const float* nrm_ptr(const float* pool, long long off) { return pool ? pool + off : nullptr; }
 LQ_DI float* nrm_ptr_w(float* pool, long long off) { return pool ? pool + off : nullptr; }
 
+// Stores the block's sums (4 doubles a block, 8 for RED_TSW) and finishes the system if asked to.
 template <int RED, typename R>
 LQ_DI void red_store(R* red, const HopArgs& a, int s, int by, int nb) {
   constexpr int PW = RED == RED_TSW ? 8 : 4;
@@ -671,6 +674,11 @@ LQ_DI void red_store(R* red, const HopArgs& a, int s, int by, int nb) {
 template <int P, bool DAG, bool CLOV, int RED, int EPI, int CFG = 0>
 __global__ void __launch_bounds__(128, (HopCfg<P, CFG, (CLOV && RED == RED_TSW)>::minb)) k_hop_lin(HopArgs a) {
   typedef typename Prec<P>::R R;
+  // the blocks that the registers are capped for also fit the shared memory of an SM (228 KB, 1 KB of it a block's)
+  static_assert(P != 32 || HopCfg<P, CFG, (CLOV && RED == RED_TSW)>::minb *
+                                   (RING * RING_SLOT + (RED == RED_NONE ? 0 : red_smem(red_count(RED))) + 1024) <=
+                               228 * 1024,
+                "blocks per SM");
   int s, by;
   grid_pos_tiled((int)blockIdx.x, a.nsys, a.nby, a.tile, s, by);
   if (s >= a.nsys) return;
@@ -686,7 +694,7 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG, (CLOV && RED == RED_TSW)>
     if (EPI & EPI_X) {
       int x[4];
       eo_coords(a.g, cb, a.pout, x);
-      hop_sum<P, DAG, HopCfg<P, CFG>::depth>(a.g, sd, f, a.pout, cb, j, x, sys_ptr<P>(a.x, sd.off),
+      hop_sum<P, DAG, CFG>(a.g, sd, f, a.pout, cb, j, x, sys_ptr<P>(a.x, sd.off),
                                              nrm_ptr(a.xn, sd.off), res);
       const R al = (R)a.alpha;
 #pragma unroll
@@ -746,7 +754,7 @@ __global__ void __launch_bounds__(128, (HopCfg<P, CFG>::minb)) k_hop_clinv(HopAr
   if (EPI & EPI_X) {
     int x[4];
     eo_coords(a.g, cb, a.pout, x);
-    hop_sum<P, DAG, HopCfg<P, CFG>::depth>(a.g, sd, f, a.pout, cb, j, x, sys_ptr<P>(a.x, sd.off),
+    hop_sum<P, DAG, CFG>(a.g, sd, f, a.pout, cb, j, x, sys_ptr<P>(a.x, sd.off),
                                            nrm_ptr(a.xn, sd.off), res);
     const R al = (R)a.alpha;
 #pragma unroll

@@ -19,9 +19,12 @@ namespace lq {
 // sums are widened to FP64 and combined in FP64, one thread per sum in warp order (a shuffle tree
 // of FP64 sums held a block back by about 1400 clocks: 35 FP64 steps for 7 sums), and one
 // partial per block is stored.  The order is fixed, so results are deterministic.
+constexpr int RED_WARPS = 4;  // warps of a block (k_finalize has more)
+constexpr int red_smem(int nq) { return 2 * RED_WARPS * nq * 8 + 16; }  // block_reduce_store and finish_last
+
 template <int NQ, typename A>
 LQ_DI void block_reduce_store(A v[NQ], double* dst) {
-  __shared__ double sh[32][NQ > 0 ? NQ : 1];
+  __shared__ double sh[RED_WARPS][NQ];
 #pragma unroll
   for (int q = 0; q < NQ; q++)
 #pragma unroll
@@ -32,9 +35,8 @@ LQ_DI void block_reduce_store(A v[NQ], double* dst) {
     for (int q = 0; q < NQ; q++) sh[wid][q] = (double)v[q];
   __syncthreads();
   if (threadIdx.x < NQ) {
-    const int nw = blockDim.x >> 5;
     double t = sh[0][threadIdx.x];
-    for (int w = 1; w < nw; w++) t += sh[w][threadIdx.x];
+    for (int w = 1; w < RED_WARPS; w++) t += sh[w][threadIdx.x];
     dst[threadIdx.x] = t;
   }
 }
@@ -42,9 +44,9 @@ LQ_DI void block_reduce_store(A v[NQ], double* dst) {
 // Sum of nb block partials of NQ values (PW doubles apart), in a fixed order: each thread of the block
 // sums a strided subset, the warps reduce by shuffles and thread 0 adds the warp sums in warp order
 // and receives the result.  Partials are read past L1 (other blocks of this launch wrote them).
-template <int NQ, int PW>
+template <int NQ, int PW, int WARPS = RED_WARPS>
 LQ_DI void block_sum_partials(const double* partial, int nb, double* out) {
-  __shared__ double sh[32][NQ];
+  __shared__ double sh[WARPS][NQ];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double v[NQ];
 #pragma unroll
@@ -65,11 +67,10 @@ LQ_DI void block_sum_partials(const double* partial, int nb, double* out) {
     for (int q = 0; q < NQ; q++) sh[wid][q] = v[q];
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
 #pragma unroll
     for (int q = 0; q < NQ; q++) {
       double t = 0.0;
-      for (int w = 0; w < nw; w++) t += sh[w][q];
+      for (int w = 0; w < WARPS; w++) t += sh[w][q];
       out[q] = t;
     }
   }
