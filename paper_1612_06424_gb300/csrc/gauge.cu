@@ -490,12 +490,17 @@ constexpr long long CLOVER_CHUNK = 1 << 19;
 
 int lq_launch_clover(const lq::Geom& g, const int4* U, double kappa, double csw, int4* A64, int4* Ai64,
                      int* A64e, int* Ai64e, float4* A32, float4* Ai32, int* fail, cudaStream_t st) {
-  const long long Vh = g.Vh, chunk = std::min(Vh, CLOVER_CHUNK);
+  const long long Vh = g.Vh;
+  long long chunk = std::min(Vh, CLOVER_CHUNK);
   double* G = nullptr;
-  if (csw != 0.0 && cudaMallocAsync((void**)&G, sizeof(double) * 108 * chunk, st) != cudaSuccess) {
+  while (csw != 0.0 && cudaMallocAsync((void**)&G, sizeof(double) * 108 * chunk, st) != cudaSuccess) {
     cudaGetLastError();
-    lq_set_error("set_gauge: device allocation of the clover scratch failed");
-    return LQCD_ENOMEM;
+    G = nullptr;
+    if (chunk <= 1024) {
+      lq_set_error("set_gauge: device allocation of the clover scratch failed");
+      return LQCD_ENOMEM;
+    }
+    chunk = (chunk + 7) / 8;  // a nearly full device: shorter runs
   }
   for (long long c0 = 0; c0 < Vh; c0 += chunk) {
     const long long h = std::min(chunk, Vh - c0);

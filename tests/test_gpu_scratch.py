@@ -29,6 +29,10 @@ class _Pool:
         assert self.cu.cuMemPoolGetAttribute(self.h, attr, ctypes.byref(v)) == 0
         return v.value
 
+    def trim(self):
+        torch.cuda.synchronize()
+        assert self.cu.cuMemPoolTrimTo(self.h, ctypes.c_size_t(0)) == 0
+
     def peak_of(self, call):
         torch.cuda.synchronize()
         zero, before = ctypes.c_uint64(0), self.used(7)
@@ -94,4 +98,25 @@ def test_stencil_bench_knows_its_kernels():
     for kernel in (-1, 6):
         with pytest.raises(lqcd.LQCDError, match="bad arguments"):
             lat.stencil_bench([(0, 3)], [0], 32, kernel, 1)
+    lat.close()
+
+
+def test_set_gauge_on_a_nearly_full_device():
+    """A field is loaded again (its storage stays) with 200 MB left, half of what runs of 2^19 sites take for the clover planes."""
+    lqcd = _lq()
+    dims = (24, 24, 24, 80)
+    lat = lqcd.Lattice(dims, "open")
+    U = inputs.random_su3_field_device(dims, 0.4, 3, rng="device").contiguous()
+    psi = torch.randn((lat.V, 4, 3), dtype=torch.complex128, device="cuda")
+    lat.set_gauge(U, 0.13, 1.0)
+    want = lat.dslash(psi, 0, None, False, 64)
+    lat.set_gauge(U, 0.13, 0.0)
+    torch.cuda.empty_cache()
+    pool = _Pool()
+    pool.trim()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (200 << 20), dtype=torch.uint8, device="cuda")
+    lat.set_gauge(U, 0.13, 1.0)
+    del fill
+    torch.cuda.empty_cache()
+    assert torch.equal(lat.dslash(psi, 0, None, False, 64), want)
     lat.close()
