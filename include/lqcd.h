@@ -398,14 +398,17 @@ int lqcd_dslash_bench(lqcd_lattice *lat, int n_sys, const lqcd_slab *doms, const
  *   0  out_o = A_oo y_o - 1/4 D_hop x_e            (3 spinor passes)
  *   1  out_e = A_ee^{-1} D_hop x_o                 (2 passes; first half of D^)
  *   2  kernel 0 with the reduction <r0, out>       (4 passes)
- *   3  kernel 0 with <out, y>, |out|^2, <r0, out> and <r0, y>   (4 passes)
+ *   3  kernel 0 with <out, y>, |out|^2, <r0, out> and <r0, y>   (4 passes; in
+ *      FP64 with <out, y> and |out|^2, 3 passes)
  *   4  s = r - alpha v                             (3 passes)
- *   5  x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2   (8 passes)
+ *   5  x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2   (8 passes; in
+ *      FP64 x, r, <r0, r> and |r|^2, 7 passes)
+ *   6  FP64 only: p = r + beta (p - omega v)       (4 passes)
  * bytes_per_launch: algorithmic bytes = passes x spinor bytes per system
  * site, plus (8 links + 1 clover block) per distinct field site of the
  * slabs for kernels 0-3.  flops_per_launch: per system site, hop 1320 +
  * site-diagonal block (504 with clover, else 24) + epilogue / reductions
- * (kernels 0-3), or the vector arithmetic (kernels 4, 5).  Errors:
+ * (kernels 0-3), or the vector arithmetic (kernels 4-6).  Errors:
  * LQCD_EBADARG, LQCD_ENOFIELD, LQCD_ENOMEM, LQCD_ECUDA. */
 int lqcd_stencil_bench(lqcd_lattice *lat, int n_sys, const lqcd_slab *doms, const int *field_ids, int precision,
                        int kernel, int reps, double *ms_per_launch, double *bytes_per_launch,

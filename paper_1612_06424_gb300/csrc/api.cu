@@ -424,7 +424,7 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
       // check that follows decides (0.5 tol measured 2.8% faster than 0.3 tol on the 48^3 x 96
       // factorized propagator, worst final residual 8.5e-11)
       RC(lq_finalize(lq::FIN_INIT, b, tau * tau, 0.25 * tol * tol, lq_words_per_site(P), st));
-      // one BiCGStab iteration: 6 kernels, all scalars and flags on the device
+      // one BiCGStab iteration: 6 kernels (FP64: 7, and 4 conversions), all scalars and flags on the device
       auto iteration = [&](cudaStream_t s_) -> int {
         VecP hx = p, ht = te;  // hop inputs (FP64: in limbs; t is free until the end)
         if (P == 64) RC(limbs(p.d, t.d, hx, s_));
@@ -435,10 +435,14 @@ int solve_core(lqcd_lattice* L, BatchStore& B, bool dag, const lqcd_solver_param
         hx = s;
         if (P == 64) RC(limbs(s.d, t.d, hx, s_));
         RC(lq_hop_clinv(P, dag, clov, L, b, hx, none, te, 1.0, 0.0, s_));
-        if (P == 64) RC(limbs(te.d, te.d, ht, s_));
+        if (P == 64) {
+          RC(limbs(te.d, te.d, ht, s_));
+          RC(lq_hop_lin(64, dag, clov, lq::RED_TS, L, b, 1, ht, s, none, none, t, -0.25, 1.0, 0.0, s_, lq::FIN_OMEGA));
+          RC(lq_bicg_xr64(b, xs, p, s, t, r, r0, s_, lq::FIN_BETA));
+          return lq_bicg_p64(b, p, r, v, s_);
+        }
         RC(lq_hop_lin(P, dag, clov, lq::RED_TSW, L, b, 1, ht, s, none, r0, t, -0.25, 1.0, 0.0, s_, lq::FIN_OMEGA_BETA));
-        RC(lq_bicg_xrp(P, b, xs, p, s, t, v, r, s_, lq::FIN_STOP));
-        return 0;
+        return lq_bicg_xrp(P, b, xs, p, s, t, v, r, s_, lq::FIN_STOP);
       };
       if (use_graph && budget >= 2 * check_every) {
         // check_every iterations captured once per solve as a CUDA graph on a
@@ -1871,8 +1875,8 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
                                   double* bytes_per_launch, double* flops_per_launch, void* stream) {
   RC(check_lat(L));
   if (n_sys < 1 || !doms || !field_ids || reps < 1 || (precision != 64 && precision != 32 && precision != 16) ||
-      kernel < 0 || kernel > 5) {
-    lq_set_error("stencil_bench: bad arguments (kernels 0 to 5)");
+      kernel < 0 || kernel > (precision == 64 ? 6 : 5)) {
+    lq_set_error("stencil_bench: bad arguments (kernels 0 to 5, in FP64 0 to 6)");
     return LQCD_EBADARG;
   }
   cudaStream_t st = (cudaStream_t)stream;
@@ -1913,12 +1917,15 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
       case 2:  // v = A_oo p - 1/4 D_hop te, with <r0, v>
         return lq_hop_lin(precision, false, clov, lq::RED_DOT_W, L, b, 1, hx, q.v(1), none, q.v(3), q.v(2),
                           -0.25, 1.0, 0.0, st);
-      case 3:  // t = A_oo s - 1/4 D_hop te, with <t, s>, |t|^2, <r0, t> and <r0, s>
-        return lq_hop_lin(precision, false, clov, lq::RED_TSW, L, b, 1, hx, q.v(1), none, q.v(3), q.v(2), -0.25,
-                          1.0, 0.0, st);
+      case 3:  // t = A_oo s - 1/4 D_hop te, with <t, s>, |t|^2, and (not in FP64) <r0, t> and <r0, s>
+        return lq_hop_lin(precision, false, clov, precision == 64 ? lq::RED_TS : lq::RED_TSW, L, b, 1, hx, q.v(1), none,
+                          q.v(3), q.v(2), -0.25, 1.0, 0.0, st);
       case 4:  // s = r - alpha v
         return lq_bicg_s(precision, b, q.v(0), q.v(1), q.v(2), st);
-      default:  // x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2
+      case 6:  // p = r + beta (p - omega v)
+        return lq_bicg_p64(b, q.v(2), q.v(0), q.v(1), st);
+      default:  // x += alpha p + omega s, r = s - omega t, and <r0, r>, |r|^2 or p = r + beta (p - omega v), |r|^2
+        if (precision == 64) return lq_bicg_xr64(b, q.v(2), q.v(0), q.v(1), q.v(4), q.v(5), q.v(3), st);
         return lq_bicg_xrp(precision, b, q.v(2), q.v(0), q.v(1), q.v(4), q.v(3), q.v(5), st);
     }
   };
@@ -1940,11 +1947,11 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
   const double S = precision == 64 ? 192.0 : precision == 32 ? 96.0 : 52.0;
   const double Lk = precision == 64 ? 144.0 : precision == 32 ? 48.0 : 24.0;
   const double C = clov ? (precision == 64 ? 576.0 : 288.0) : 0.0;
-  static const double passes[6] = {3, 2, 4, 4, 3, 8};
+  static const double passes[2][7] = {{3, 2, 4, 4, 3, 8}, {3, 2, 4, 3, 3, 7, 4}};
   double bytes = 0.0, sites = 0.0;
   std::vector<std::vector<char>> used(L->fields.size(), std::vector<char>(L->dims[0], 0));
   for (int k = 0; k < n_sys; k++) {
-    bytes += passes[kernel] * S * (double)B.h_sys[k].n;
+    bytes += passes[precision == 64][kernel] * S * (double)B.h_sys[k].n;
     sites += (double)B.h_sys[k].n;
     for (int t = doms[k].t0; t <= doms[k].t1; t++) used[field_ids[k]][t] = 1;
   }
@@ -1954,9 +1961,11 @@ extern "C" int lqcd_stencil_bench(lqcd_lattice* L, int n_sys, const lqcd_slab* d
         if (c) bytes += (8.0 * Lk + C) * (double)L->S3h;
   // flop per system site: hop 1320, site-diagonal block 504 (clover) or 24, epilogue and reductions
   const double diag = clov ? 504.0 : 24.0;
-  const double flop[6] = {1320.0 + diag + 72.0, 1320.0 + diag + 24.0, 1320.0 + diag + 72.0 + 96.0,
-                          1320.0 + diag + 72.0 + 336.0, 96.0, 528.0};
-  const double fl = sites * flop[kernel];
+  const double flop[2][7] = {{1320.0 + diag + 72.0, 1320.0 + diag + 24.0, 1320.0 + diag + 72.0 + 96.0,
+                              1320.0 + diag + 72.0 + 336.0, 96.0, 528.0},
+                             {1320.0 + diag + 72.0, 1320.0 + diag + 24.0, 1320.0 + diag + 72.0 + 96.0,
+                              1320.0 + diag + 72.0 + 144.0, 96.0, 432.0, 192.0}};
+  const double fl = sites * flop[precision == 64][kernel];
   if (ms_per_launch) *ms_per_launch = ms / reps;
   if (bytes_per_launch) *bytes_per_launch = bytes;
   if (flops_per_launch) *flops_per_launch = fl;

@@ -118,7 +118,42 @@ __global__ void __launch_bounds__(128) k_bicg_s_h(VecArgs va, const void* r, con
   Prec<16>::store(sys_ptr_w<16>(so, sd.off), nrm_ptr_w(son, sd.off), sd.n, j, a);
 }
 
-// ------- x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v) ; |r|^2
+// ------- FP64: x += alpha p + omega s ; r = s - omega t ; <r0, r>, |r|^2, and p = r + beta (p - omega v)
+// Two passes over the vectors, since beta comes from the stored r.  The recurrence that k_bicg_xrp_w goes by saves three of
+// eleven vector passes, 3% of an iteration here, but an FP64 solve has no outer cycles that restart it: on nearly
+// singular matrices it took 17000 to 60000 iterations, or never ended, where these kernels take 7000.
+__global__ void __launch_bounds__(128) k_bicg_xr_64(VecArgs va, FinArgs fin, double2* x, const double2* p,
+                                                    const double2* sv, const double2* t, double2* r, const double2* r0) {
+  LQ_WORD_PROLOGUE(64)
+  double red[3] = {0.0, 0.0, 0.0};
+  if (valid) {
+    const long long q = sd.off * 12 + i;
+    const cx<double> al = c_of<double>(va.sc[s].alpha), om = c_of<double>(va.sc[s].omega);
+    const double2 xv = x[q], pv = __ldg(p + q), s2 = __ldg(sv + q), tv = __ldg(t + q), wv = __ldg(r0 + q);
+    const cx<double> s1 = {s2.x, s2.y}, w = {wv.x, wv.y};
+    const cx<double> xn = cx<double>{xv.x, xv.y} + al * cx<double>{pv.x, pv.y} + om * s1;
+    const cx<double> rn = s1 - om * cx<double>{tv.x, tv.y};
+    x[q] = make_double2(xn.re, xn.im);
+    r[q] = make_double2(rn.re, rn.im);
+    red[0] = w.re * rn.re + w.im * rn.im;
+    red[1] = w.re * rn.im - w.im * rn.re;
+    red[2] = rn.re * rn.re + rn.im * rn.im;
+  }
+  double* part = va.partial + (long long)s * va.pstride * 4;
+  block_reduce_store<3, double>(red, part + (long long)by * 4);
+  if (fin.mode != FIN_NONE) finish_last<3, 0, 4>(fin, part, (sd.n * 12 + 127) / 128, s);
+}
+__global__ void __launch_bounds__(128) k_bicg_p_64(VecArgs va, double2* p, const double2* r, const double2* v) {
+  LQ_WORD_PROLOGUE(64)
+  if (!valid) return;
+  const long long q = sd.off * 12 + i;
+  const cx<double> be = c_of<double>(va.sc[s].beta), om = c_of<double>(va.sc[s].omega);
+  const double2 pv = p[q], rv = __ldg(r + q), vv = __ldg(v + q);
+  const cx<double> n = cx<double>{rv.x, rv.y} + be * (cx<double>{pv.x, pv.y} - om * cx<double>{vv.x, vv.y});
+  p[q] = make_double2(n.re, n.im);
+}
+
+// ------- FP32 and FP16: x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v) ; |r|^2
 // One pass over the five vectors: beta is known beforehand (FIN_OMEGA_BETA takes <r0, r> from <r0, s>
 // and <r0, t>).  8 vector passes against 11 for an x, r update followed by a p update, for one more
 // (r0) in the stencil before it.

@@ -184,7 +184,8 @@ struct SolverScal {
 // Fused reductions of the hop kernels and modes of the scalar finalize.
 enum { RED_NONE = 0, RED_DOT_W = 1, RED_TS = 2, RED_NORM = 3, RED_TSW = 4 };
 enum { FIN_NONE = -1, FIN_ALPHA = 0, FIN_OMEGA_BETA = 1, FIN_STOP = 2, FIN_INIT = 3, FIN_NORM = 4,
-       FIN_CG_RHO = 5, FIN_CG_ALPHA = 6, FIN_CG_R = 7, FIN_CG_BETA = 8, FIN_BB = 9, FIN_BB_ADD = 10 };
+       FIN_CG_RHO = 5, FIN_CG_ALPHA = 6, FIN_CG_R = 7, FIN_CG_BETA = 8, FIN_BB = 9, FIN_BB_ADD = 10,
+       FIN_OMEGA = 11, FIN_BETA = 12 };
 
 // ------------------------------------------------------------ precision I/O
 template <int P>

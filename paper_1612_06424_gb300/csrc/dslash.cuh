@@ -663,6 +663,8 @@ LQ_DI void red_store(R* red, const HopArgs& a, int s, int by, int nb) {
   block_reduce_store<red_count(RED), R>(red, part + (long long)by * PW);
   if constexpr (RED == RED_DOT_W) {
     if (a.fin.mode != FIN_NONE) finish_last<2, 0, PW>(a.fin, part, nb, s);
+  } else if constexpr (RED == RED_TS) {
+    if (a.fin.mode != FIN_NONE) finish_last<3, 0, PW>(a.fin, part, nb, s);
   } else if constexpr (RED == RED_TSW) {
     if (a.fin.mode != FIN_NONE) finish_last<7, 0, PW>(a.fin, part, nb, s);
   }

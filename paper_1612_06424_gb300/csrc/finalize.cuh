@@ -89,6 +89,8 @@ LQ_DI bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 //  FIN_OMEGA_BETA: v[0..1] = <t, s>, v[2] = |t|^2, v[3..4] = <r0, t>, v[5..6] = <r0, s>:
 //             omega = <t, s> / |t|^2, rho' = <r0, r> = <r0, s> - omega <r0, t> for the coming
 //             r = s - omega t, beta = (rho'/rho)(alpha/omega)
+//  FIN_OMEGA: v[0..1] = <t, s>, v[2] = |t|^2: omega
+//  FIN_BETA : v[0..1] = <r0, r>, v[2] = |r|^2: beta from omega and rho' = <r0, r>, and FIN_STOP
 //  FIN_STOP : v[2] = |r|^2: stop the system when rr <= target2, on breakdown, NaN or divergence (rr > 1e8 rr0)
 //  FIN_NORM : rr = v[2] only
 //  FIN_BB, FIN_BB_ADD: bb = v[2], bb += v[2]
@@ -98,6 +100,16 @@ LQ_DI bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 //  FIN_CG_R    : rr = |r|^2; stop the system when rr <= target2, on NaN or divergence
 //  FIN_CG_BETA : beta = |z|^2 / rho, rho = |z|^2
 // status: 1 breakdown, 2 NaN or divergence.
+LQ_DI void next_direction(SolverScal& c, double2 rho) {  // rho' = <r0, r> and beta = (rho'/rho)(alpha/omega)
+  if (!finite2(rho)) {
+    c.status = 2;
+  } else if ((rho.x == 0.0 && rho.y == 0.0) || (c.omega.x == 0.0 && c.omega.y == 0.0)) {
+    c.status = 1;
+  } else {
+    c.beta = cmul2(cdiv(rho, c.rho), cdiv(c.alpha, c.omega));
+    c.rho = rho;
+  }
+}
 LQ_DI void fin_update(int mode, const double* v, SolverScal& c, int* active, double tau2, double floor_rel2) {
   const double2 d = make_double2(v[0], v[1]);
   switch (mode) {
@@ -121,7 +133,8 @@ LQ_DI void fin_update(int mode, const double* v, SolverScal& c, int* active, dou
         c.alpha = cdiv(c.rho, d);
       }
       break;
-    case FIN_OMEGA_BETA: {
+    case FIN_OMEGA:
+    case FIN_OMEGA_BETA:
       c.beta = make_double2(0.0, 0.0);
       if (!(v[2] > 0.0) || !isfinite(v[2])) {
         c.omega = make_double2(0.0, 0.0);
@@ -129,18 +142,14 @@ LQ_DI void fin_update(int mode, const double* v, SolverScal& c, int* active, dou
         break;
       }
       c.omega = make_double2(d.x / v[2], d.y / v[2]);
-      const double2 w = cmul2(c.omega, make_double2(v[3], v[4]));
-      const double2 rho = make_double2(v[5] - w.x, v[6] - w.y);
-      if (!finite2(rho)) {
-        c.status = 2;
-      } else if ((rho.x == 0.0 && rho.y == 0.0) || (c.omega.x == 0.0 && c.omega.y == 0.0)) {
-        c.status = 1;
-      } else {
-        c.beta = cmul2(cdiv(rho, c.rho), cdiv(c.alpha, c.omega));
-        c.rho = rho;
+      if (mode == FIN_OMEGA_BETA) {
+        const double2 w = cmul2(c.omega, make_double2(v[3], v[4]));
+        next_direction(c, make_double2(v[5] - w.x, v[6] - w.y));
       }
       break;
-    }
+    case FIN_BETA:
+      if (c.status == 0) next_direction(c, d);
+      // fall through
     case FIN_STOP:
       c.iters += 1;
       c.rr = v[2];

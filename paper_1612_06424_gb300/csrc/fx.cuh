@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(128, FX_BLOCKS) k_fx_lin(FxArgs m) {
   int et = e1 + 3, e2 = 0, e3 = 0;
   cx<double> yv[6], zv[6];
   int ey = 1, ez = 1;
-  if ((EPI & EPI_Y) || RED == RED_TS || RED == RED_TSW) fx_load6<false>(yv, a.y, sd, j, sp);
+  if ((EPI & EPI_Y) || RED == RED_TS) fx_load6<false>(yv, a.y, sd, j, sp);
   if (EPI & EPI_Z) fx_load6(zv, a.z, sd, j, sp);
   if (EPI & EPI_Y) {
     ey = fx_max_exponent<6>(yv);
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(128, FX_BLOCKS) k_fx_lin(FxArgs m) {
     fx_store6(a.out, sd, j, sp, res);
     if (RED != RED_NONE) {
       cx<double> wv[6];
-      if (RED == RED_DOT_W || RED == RED_TSW) fx_load6(wv, a.w, sd, j, sp);
+      if (RED == RED_DOT_W) fx_load6(wv, a.w, sd, j, sp);
       red_add<RED, 6, double>(red, res, yv, wv);
     }
   }

@@ -71,7 +71,6 @@ static int pick(int red, int epi, dim3 gr, const FxArgs& m, cudaStream_t st) {
   else if (red == RED_NONE && epi == XZ) k_fx_lin<DAG, CLOV, RED_NONE, XZ><<<gr, 128, 0, st>>>(m);
   else if (red == RED_DOT_W && epi == XY) k_fx_lin<DAG, CLOV, RED_DOT_W, XY><<<gr, 128, 0, st>>>(m);
   else if (red == RED_TS && epi == XY) k_fx_lin<DAG, CLOV, RED_TS, XY><<<gr, 128, 0, st>>>(m);
-  else if (red == RED_TSW && epi == XY) k_fx_lin<DAG, CLOV, RED_TSW, XY><<<gr, 128, 0, st>>>(m);
   else if (red == RED_NORM && epi == XYZ) k_fx_lin<DAG, CLOV, RED_NORM, XYZ><<<gr, 128, 0, st>>>(m);
   else return -1;
   return 0;

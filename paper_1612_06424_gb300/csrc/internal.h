@@ -80,7 +80,7 @@ int lq_launch_clover(const lq::Geom& g, const int4* U, double kappa, double csw,
                      int* A64e, int* Ai64e, float4* A32, float4* Ai32, int* fail, cudaStream_t st);
 
 // out = beta*A(y) + alpha*D_hop x + gamma*z on parity pout (+ fused reduction; fin: what the kernel's last
-// block of a system does with the sums, FIN_ALPHA for RED_DOT_W, FIN_OMEGA_BETA for RED_TSW)
+// block of a system does with the sums, FIN_ALPHA for RED_DOT_W, FIN_OMEGA for RED_TS, FIN_OMEGA_BETA for RED_TSW)
 int lq_hop_lin(int P, bool dag, bool clov, int red, const lqcd_lattice* L, const Batch& b, int pout, VecP x, VecP y,
                VecP z, VecP w, VecP out, double alpha, double beta, double gamma, cudaStream_t st,
                int fin = lq::FIN_NONE);
@@ -89,7 +89,10 @@ int lq_hop_clinv(int P, bool dag, bool clov, const lqcd_lattice* L, const Batch&
                  double alpha, double beta, cudaStream_t st);
 
 int lq_bicg_s(int P, const Batch& b, VecP r, VecP v, VecP s, cudaStream_t st);
-// x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2 (fin: FIN_STOP)
+// FP64: x += alpha p + omega s, r = s - omega t, <r0, r>, |r|^2 (fin: FIN_BETA); p = r + beta (p - omega v)
+int lq_bicg_xr64(const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP r, VecP r0, cudaStream_t st, int fin = lq::FIN_NONE);
+int lq_bicg_p64(const Batch& b, VecP p, VecP r, VecP v, cudaStream_t st);
+// FP32, FP16: x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), |r|^2 (fin: FIN_STOP)
 int lq_bicg_xrp(int P, const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP v, VecP r, cudaStream_t st,
                 int fin = lq::FIN_NONE);
 int lq_inner_init(int P, const Batch& b, const double2* r64, VecP r, VecP r0, VecP p, VecP x, cudaStream_t st);

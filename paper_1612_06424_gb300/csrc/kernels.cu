@@ -340,16 +340,28 @@ int lq_bicg_s(int P, const Batch& b, VecP r, VecP v, VecP s, cudaStream_t st) {
   return launched();
 }
 
+int lq_bicg_xr64(const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP r, VecP r0, cudaStream_t st, int fin) {
+  k_bicg_xr_64<<<grid_words(b, 64), LQ_BLOCK, 0, st>>>(vec_args(b), fin_args(b, fin), (double2*)x.d, (const double2*)p.d,
+                                                       (const double2*)s.d, (const double2*)t.d, (double2*)r.d,
+                                                       (const double2*)r0.d);
+  return launched();
+}
+
+int lq_bicg_p64(const Batch& b, VecP p, VecP r, VecP v, cudaStream_t st) {
+  k_bicg_p_64<<<grid_words(b, 64), LQ_BLOCK, 0, st>>>(vec_args(b), (double2*)p.d, (const double2*)r.d, (const double2*)v.d);
+  return launched();
+}
+
 int lq_bicg_xrp(int P, const Batch& b, VecP x, VecP p, VecP s, VecP t, VecP v, VecP r, cudaStream_t st, int fin) {
   VecArgs va = vec_args(b);
   const FinArgs fa = fin_args(b, fin);
-  const long long nv = P == 64 ? 12 : 6, bw = LQ_BLOCK * XRP_WPT;
-  const dim3 gr = grid_lin(b, (b.max_n * nv + bw - 1) / bw);
-  if (P == 64) k_bicg_xrp_w<64><<<gr, LQ_BLOCK, 0, st>>>(va, fa, x.d, p.d, s.d, t.d, v.d, r.d);
-  else if (P == 32) k_bicg_xrp_w<32><<<gr, LQ_BLOCK, 0, st>>>(va, fa, x.d, p.d, s.d, t.d, v.d, r.d);
-  else
+  if (P == 32) {
+    const long long bw = LQ_BLOCK * XRP_WPT;
+    k_bicg_xrp_w<32><<<grid_lin(b, (b.max_n * 6 + bw - 1) / bw), LQ_BLOCK, 0, st>>>(va, fa, x.d, p.d, s.d, t.d, v.d, r.d);
+  } else {
     k_bicg_xrp_h<<<grid_of(b), LQ_BLOCK, 0, st>>>(va, fa, x.d, x.nrm, p.d, p.nrm, s.d, s.nrm, t.d, t.nrm, v.d, v.nrm,
                                                   r.d, r.nrm);
+  }
   return launched();
 }
 

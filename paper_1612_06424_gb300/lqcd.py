@@ -341,7 +341,7 @@ class Lattice:
 
     def stencil_bench(self, doms, field_ids, precision: int = 32, kernel: int = 0, reps: int = 20, stream=None):
         """(ms per launch, algorithmic bytes, flops) of one kernel of the solver's iteration
-        (0-3: hop kernels, 4, 5: vector updates; see lqcd_stencil_bench in include/lqcd.h)."""
+        (0-3: hop kernels, 4, 5, in FP64 6: vector updates; see lqcd_stencil_bench in include/lqcd.h)."""
         n = len(doms)
         sl = (Slab * n)(*[Slab(*d) for d in doms])
         fi = (ctypes.c_int * n)(*field_ids)

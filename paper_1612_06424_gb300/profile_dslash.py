@@ -8,7 +8,7 @@ Prints ms per launch, algorithmic GB/s and TFLOP/s.  Each launch is one
 kernel of the solver's BiCGStab iteration over every system of the batch
 (--kernels, numbered as lqcd_stencil_bench: 0 plain second half of D^,
 1 clover-inverse first half, 2 / 3 second half with the fused reductions,
-4, 5 the vector updates); the default is 0 (k_hop_lin, out_o = A_oo y_o -
+4, 5 and in FP64 6 the vector updates); the default is 0 (k_hop_lin, out_o = A_oo y_o -
 1/4 D_hop x_e).
 With --factorized it instead runs one 12-source factorized propagator with
 correction on the 16^3x32 workload (Gamma 0..13, DeltaGamma 14..17, Gamma*
