@@ -732,13 +732,19 @@ static int proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long
   return launched_here();
 }
 
+template <int X>
+static int proj_prop_x(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi,
+                       long long nsite_gs, long long y0, const double2* eta, double2* fact, cudaStream_t st) {
+  if (nsite_gs * 12 > 152 * 2 * 128) {
+    const int rc = proj_prop<X, true>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+    if (rc != LQCD_ENOMEM) return rc;  // no room for the scan's words: the form without
+  }
+  return proj_prop<X, false>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+}
+
 // Up to 32 modes fit one sum with a bit more.
 int lq_proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi, long long nsite_gs,
                  long long y0, const double2* eta, double2* fact, cudaStream_t st) {
-  const bool scan = nsite_gs * 12 > 152 * 2 * 128;
-  if (n <= px_modes<1>)
-    return scan ? proj_prop<1, true>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st)
-                : proj_prop<1, false>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
-  return scan ? proj_prop<0, true>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st)
-              : proj_prop<0, false>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+  return n <= px_modes<1> ? proj_prop_x<1>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st)
+                          : proj_prop_x<0>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
 }
