@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_1612_06424_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -120,3 +121,21 @@ def test_set_gauge_on_a_nearly_full_device():
     torch.cuda.empty_cache()
     assert torch.equal(lat.dslash(psi, 0, None, False, 64), want)
     lat.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(608, 1), (304, 5), (607, 1)])
+def test_contraction_without_parts(nx, ny):
+    """As many pairs as fill the GPU take one part each and no scratch: summed in place.  16 products a sum."""
+    lqcd = _lq()
+    r = np.random.default_rng(94)
+    c = lambda *s: r.standard_normal(s) + 1j * r.standard_normal(s)  # noqa: E731
+    bx, by = c(nx, 2, 2, 2, 4), c(ny, 2, 2, 2, 4)
+    gx, gy = torch.from_numpy(bx).cuda(), torch.from_numpy(by).cuda()
+    W = []
+    peak = _Pool().peak_of(lambda: W.append(lqcd.nucleon_contract(gx, gy).cpu().numpy()))
+    assert (peak == 0) == (nx != 607)
+    z = np.einsum("gd,yijkd->yijkg", oracle.gamma(4) @ (0.5 * (np.eye(4) - oracle.gamma(0))), by)
+    for q, axes in enumerate("jik kij".split()):
+        ref = -np.einsum("x%sg,yijkg->xy" % axes, bx, z)
+        M = np.einsum("x%sg,yijkg->xy" % axes, np.abs(bx), np.abs(z))
+        assert np.all(np.abs(W[0][:, :, q] - ref) <= 4 * 2 ** 0.5 * 16 * 2.0 ** -53 * M)
