@@ -759,12 +759,15 @@ def run_headline(args):
     # roofline of the stencil as the solver launches it, on the Gamma* batch of a step
     lat.set_gauge(Uf[0], wl["kappa"], wl["csw"])
     roofline, blas = _iteration_roofline(lat, [GS] * 12, [0] * 12, args.precision)
-    fp64_peak = lqcd.fma_peak(64)
-    # (fixed-point sums: the fraction of the FP64 pipe's peak may pass 1)
+    # the FP64 stencil runs on the integer pipe: three multiply-adds of 32 x 32 + 64 bits for each of FP64, 64 of them a
+    # clock and SM (measured) at the highest clock
     m64, _, f64 = lat.stencil_bench([GS] * 12, [0] * 12, 64, 0, 3)
-    dslash64 = {"TFLOP/s": round(f64 / (m64 * 1e-3) / 1e12, 3), "ms": round(m64, 3), "bound": "alu",
-                "fp64_fma_peak_tflops_measured": round(fp64_peak, 3),
-                "alu_frac": round(f64 / (m64 * 1e-3) / 1e12 / fp64_peak, 3)}
+    n64 = 12 * lat.slab_len(*GS) / 2 * 3 * (8 * 2 * 9 * 4 + (2 * (6 * 2 + 15 * 8) if wl["csw"] else 24))
+    int_peak = torch.cuda.get_device_properties(0).multi_processor_count * 64 * (clocks.get("sm_max_mhz") or 2070.0) * 1e6
+    dslash64 = {"TFLOP/s": round(f64 / (m64 * 1e-3) / 1e12, 3), "ms": round(m64, 3), "bound": "integer pipe, latency",
+                "fp64_fma_peak_tflops_measured": round(lqcd.fma_peak(64), 3),
+                "int_mad_T/s": round(n64 / (m64 * 1e-3) / 1e12, 3), "int_mad_peak_T/s": round(int_peak / 1e12, 3),
+                "alu_frac": round(n64 / (m64 * 1e-3) / int_peak, 3)}
     s3 = dims[1] * dims[2] * dims[3]
     U_sample = Uf[0][:SAMPLE_SLICES * s3].cpu().numpy() if want_cpu else None
     lat.close()
