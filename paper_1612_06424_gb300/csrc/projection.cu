@@ -44,7 +44,7 @@ LQ_DI double2 cm_get(const ColMat& m, long long r, int k) {
 // Dot products of FP64 numbers in 64-bit integers (fxnum.cuh; the integer pipe does 32 times the FP64
 // pipe's multiply-adds).  A vector's entries are q 2^(E - px_bias<X>), |q| < 2^(55 + X), E their largest exponent, in
 // limbs q = q1 2^28 + q0; the sums of q1 p1 and of q1 p0 + q0 p1 over px_modes<X> complex products fit 64 bits.  The
-// propagator takes X = 0, whose 120 modes need one sum.  The orthonormalisation takes X = 1: its second
+// propagator takes X = 0, whose 120 modes need one sum, or more for fewer modes.  The orthonormalisation takes X = 1: its second
 // pass multiplies by nearly 1, where FP64 hardly rounds (error of 24 columns against long double: 1.5e-16 with
 // FP64 sums, 1.4e-16 with X = 1, 2.6e-16 with X = 0).
 template <int X>
@@ -383,14 +383,16 @@ __global__ void __launch_bounds__(128) k_slice_source(Geom g, int nsys, const Sy
 }
 
 // What k_proj_prop needs of a mode besides its limbs: the exponent r of its largest |xi_i(x)[b]|, and those of the twelve
-// entries relative to r and to the columns' scales, two to a word.
+// entries relative to r and to the columns' scales.
 struct __align__(16) ProjMode {
   int r, pad;
-  unsigned d[6];
+  short d[12];
 };
 constexpr int PJ_NONE = -10000;  // exponent of a zero (two of them and an exponent of FP64 fit 16 bits)
 template <int X>
 constexpr int PJ_LOSS = 2 + X;
+template <int X>
+constexpr int PJ_MODES = X == 2 ? 15 : X == 1 ? 60 : 120;  // products whose 64-bit sums fit (below 16, 64 and 128)
 
 LQ_DI int px_exponent(double2 v) { return max(max(fx_exponent(v.x), fx_exponent(v.y)), 1); }
 
@@ -402,23 +404,31 @@ LQ_DI int pj_scan(int n, long long ld, const double2* col, const ProjMode* md, c
   unsigned T[6];  // the largest exponent(eta_i) + exponent(xi_i[b]), relative to the columns' scales
 #pragma unroll
   for (int k = 0; k < 6; k++) T[k] = 0x80008000u;
-  for (int i0 = 0; i0 < n; i0 += 8) {
-    double2 v[8];  // eight loads in flight (the last mode again past the end)
+  auto add = [&](double2 v, int i) {
+    const int e = px_exponent(v);
+    const int4* m = reinterpret_cast<const int4*>(md + i);
+    const int4 m0 = __ldg(m), m1 = __ldg(m + 1);
+    const int s = e + m0.x;
+    emax = max(emax, e);
+    E = max(E, s);
+    const unsigned ss = __byte_perm((unsigned)s, 0, 0x1010);
+    const unsigned d[6] = {(unsigned)m0.z, (unsigned)m0.w, (unsigned)m1.x, (unsigned)m1.y, (unsigned)m1.z, (unsigned)m1.w};
 #pragma unroll
-    for (int k = 0; k < 8; k++) v[k] = __ldg(col + min(i0 + k, n - 1) * ld);
+    for (int q = 0; q < 6; q++) T[q] = __viaddmax_s16x2(d[q], ss, T[q]);
+  };
+  int i0 = 0;
+  for (; i0 + 8 <= n; i0 += 8) {
+    double2 v[8];  // eight loads in flight
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const int e = px_exponent(v[k]);
-      const int4* m = reinterpret_cast<const int4*>(md + min(i0 + k, n - 1));
-      const int4 m0 = __ldg(m), m1 = __ldg(m + 1);
-      const int s = e + m0.x;
-      emax = max(emax, e);
-      E = max(E, s);
-      const unsigned ss = __byte_perm((unsigned)s, 0, 0x1010);
-      const unsigned d[6] = {(unsigned)m0.z, (unsigned)m0.w, (unsigned)m1.x, (unsigned)m1.y, (unsigned)m1.z, (unsigned)m1.w};
+    for (int k = 0; k < 8; k++) v[k] = __ldg(col + (i0 + k) * ld);
 #pragma unroll
-      for (int q = 0; q < 6; q++) T[q] = __viaddmax_s16x2(d[q], ss, T[q]);
-    }
+    for (int k = 0; k < 8; k++) add(v[k], i0 + k);
+  }
+  for (; i0 < n; i0 += 2) {  // the last one of an odd number twice
+    const int i1 = min(i0 + 1, n - 1);
+    const double2 u = __ldg(col + i0 * ld), v = __ldg(col + i1 * ld);
+    add(u, i0);
+    add(v, i1);
   }
   int w = E * 8192 + (emax == 2047 ? 4096 : 0);
 #pragma unroll
@@ -433,26 +443,34 @@ __global__ void __launch_bounds__(128) k_proj_scan(int n, long long ld, const do
   if (t < ld) word[t] = pj_scan<X>(n, ld, eta + t, md, xe);
 }
 
-// sum_i eta_i conj(xi_i[b]), every term relative to 2^T, T the largest exponent(eta_i) + exponent(xi_i[b])
+// sum_i eta_i conj(xi_i[b]) by a warp, a lane a mode, every term relative to 2^T, T the largest exponent(eta_i) + exponent(xi_i[b]).
+// (By one thread the loads' latency in a row, 0.6 us a mode, set the time of small calls.)
 template <int X>
 LQ_DI double2 px_column(int n, long long ld, const double2* col, const double2* xb) {
+  const int lane = threadIdx.x & 31;
   int T = 2;
 #pragma unroll 1
-  for (int i = 0; i < n; i++) {
+  for (int i = lane; i < n; i += 32) {
     const double2 x = __ldg(xb + 12 * i);
     if (x.x != 0.0 || x.y != 0.0) T = max(T, px_exponent(x) + px_exponent(__ldg(col + i * ld)));
   }
+  T = __reduce_max_sync(0xffffffffu, T);
   double2 sum = make_double2(0.0, 0.0);
 #pragma unroll 1
-  for (int i0 = 0; i0 < n; i0 += px_modes<X>) {
-    const int i1 = min(n, i0 + px_modes<X>);
+  for (int i0 = 0; i0 < n; i0 += PJ_MODES<X>) {
+    const int i1 = min(n, i0 + PJ_MODES<X>);
     long long t[4] = {0, 0, 0, 0};
 #pragma unroll 1
-    for (int i = i0; i < i1; i++) {
+    for (int i = i0 + lane; i < i1; i += 32) {
       const double2 x = __ldg(xb + 12 * i);
       if (x.x == 0.0 && x.y == 0.0) continue;
       const int e = px_exponent(x);
       px_conj_mac(t, px_limbs<X>(x, e), px_limbs<X>(__ldg(col + i * ld), T - e));
+    }
+#pragma unroll 1
+    for (int o = 16; o; o >>= 1) {
+#pragma unroll
+      for (int k = 0; k < 4; k++) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
     }
     const double2 v = px_value<true>(t, T - 2 * px_bias<X> + 56);
     sum.x += v.x;
@@ -469,13 +487,13 @@ LQ_DI double2 px_column(int n, long long ld, const double2* col, const double2* 
 // 2^-55 2^(E + xe[b]), which is what FP64 sums do as long as one of the terms of column b is not far below 2^(E + xe[b]).
 // pj_scan looks for such a term of each column, and where there is none within a factor of 2^PJ_LOSS the column is summed
 // again on a scale of its own (px_column).  Columns of modes of similar sizes seldom come there: of 120 normal modes 1e-6, of
-// 40 and of 4 1e-4.
+// 2 2e-5.
 //
-// Bound by the integer pipe: 144 multiply-adds (32 x 32 + 64) per complex number read.  The scan is a kernel of its own
-// (SCANNED: word holds its results), bound by HBM, where there are more blocks than run at a time; next to the
-// sums it cost them 0.5 to 2 ms by the registers' and instructions' order alone.
-// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 13.0 ms so.
-template <int X, bool SCANNED>
+// Bound by the integer pipe: 144 multiply-adds (32 x 32 + 64) per complex number read.  For many modes (X = 0) the scan is a
+// kernel of its own, bound by HBM, whose results are in word; next to the sums it cost them 4 to 20% by the order of
+// registers and instructions alone.  For fewer a kernel more is what costs.
+// 120 modes on 24 slices of 24^3: 37.0 ms with FP64 sums (at the FP64 pipe's peak), 12.7 ms so; 24 modes 3.2 ms.
+template <int X>
 __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, long long y0, long long V,
                                                    const double2* eta, const int4* xi_l, const double2* xi_x,
                                                    const ProjMode* md, const int4* r4, const int* xe, const int* word,
@@ -483,19 +501,19 @@ __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, lo
   extern __shared__ int4 xs[];
   for (int e = threadIdx.x; e < n * 12; e += blockDim.x) xs[e] = xi_l[e];
   __syncthreads();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nsite * 12) return;
+  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, ld = nsite * 12;
+  const bool valid = t0 < ld;
+  const long long t = valid ? t0 : ld - 1;  // in range; nothing is stored for it
   const double2* col = eta + t;
-  const long long ld = nsite * 12;
-  const int w = SCANNED ? __ldg(word + t) : pj_scan<X>(n, ld, col, md, xe);
+  const int w = X == 0 ? __ldg(word + t) : pj_scan<X>(n, ld, col, md, xe);
   const int E = w >> 13;
   const long long y = y0 + t / 12;
   const int a = (int)(t % 12);
   double2 sum[12];
 #pragma unroll
   for (int b = 0; b < 12; b++) sum[b] = make_double2(0.0, 0.0);
-  for (int i0 = 0; i0 < n; i0 += px_modes<X>) {
-    const int i1 = min(n, i0 + px_modes<X>);
+  for (int i0 = 0; i0 < n; i0 += PJ_MODES<X>) {
+    const int i1 = min(n, i0 + PJ_MODES<X>);
     long long hr[12], cr[12], hi[12], ci[12];
 #pragma unroll
     for (int b = 0; b < 12; b++) hr[b] = cr[b] = hi[b] = ci[b] = 0;
@@ -534,67 +552,61 @@ __global__ void __launch_bounds__(128, 2) k_proj_prop(int n, long long nsite, lo
       sum[b] = i0 ? make_double2(sum[b].x + re, sum[b].y + im) : make_double2(re, im);
     }
   }
-  int redo = w & 4095;
+  int redo = valid ? w & 4095 : 0;
 #pragma unroll
   for (int b = 0; b < 12; b++) {
     const bool bad = (w & 4096) || __ldg(xe + b) == 2047;
     if (bad) redo &= ~(1 << b);
-    fact[((long long)b * V + y) * 12 + a] = bad ? make_double2(nan(""), nan("")) : make_double2(-sum[b].x, -sum[b].y);
+    if (valid)
+      fact[((long long)b * V + y) * 12 + a] = bad ? make_double2(nan(""), nan("")) : make_double2(-sum[b].x, -sum[b].y);
   }
+  const int lane = threadIdx.x & 31;
 #pragma unroll 1
-  while (redo) {
-    const int b = __ffs(redo) - 1;
-    redo &= redo - 1;
-    const double2 v = px_column<X>(n, ld, col, xi_x + b);
-    fact[((long long)b * V + y) * 12 + a] = make_double2(-v.x, -v.y);
+  for (unsigned lanes = __ballot_sync(0xffffffffu, redo != 0); lanes; lanes &= lanes - 1) {
+    const int l = __ffs(lanes) - 1;
+#pragma unroll 1
+    for (int cols = __shfl_sync(0xffffffffu, redo, l); cols; cols &= cols - 1) {
+      const int b = __ffs(cols) - 1;
+      const double2 v = px_column<X>(n, ld, eta + (t0 - lane + l), xi_x + b);
+      if (lane == l) fact[((long long)b * V + y) * 12 + a] = make_double2(-v.x, -v.y);
+    }
   }
 }
 
 // xi_x[i][b] = xi_i(x)[b], the modes' and columns' exponents (xe[b] = 2047: column b has an entry that is not finite) and the
-// limbs (one block).
+// limbs: one block, a thread an entry.
 template <int X>
-__global__ void __launch_bounds__(256) k_gather_site(int n, long long nsite_gb, long long xloc, const double2* xi,
-                                                     int4* xi_l, double2* xi_x, ProjMode* md, int* r4, int* xe) {
-  __shared__ int ce[12], bad[12];
+__global__ void __launch_bounds__(1024) k_gather_site(int n, long long nsite_gb, long long xloc, const double2* xi,
+                                                      int4* xi_l, double2* xi_x, ProjMode* md, int* r4, int* xe) {
+  __shared__ int r[1024], ce[12], bad[12];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) r[i] = PJ_NONE;
   if (threadIdx.x < 12) {
     ce[threadIdx.x] = PJ_NONE;
     bad[threadIdx.x] = 0;
   }
   __syncthreads();
+  auto entry = [&](int t) { return __ldg(xi + ((long long)(t / 12) * nsite_gb + xloc) * 12 + t % 12); };
   auto exponent = [](double2 v) {  // of a number that counts: neither zero nor without a size
     const int e = px_exponent(v);
     return (v.x == 0.0 && v.y == 0.0) || e == 2047 ? PJ_NONE : e;
   };
-  auto relative = [&](double2 v, int r) {
+  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) atomicMax(&r[t / 12], exponent(entry(t)));
+  __syncthreads();
+  for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
+    const double2 v = entry(t);
     const int e = exponent(v);
-    return e == PJ_NONE ? PJ_NONE : e - r;
-  };
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    int r = PJ_NONE;
-#pragma unroll
-    for (int b = 0; b < 12; b++) {
-      const double2 v = xi[((long long)i * nsite_gb + xloc) * 12 + b];
-      xi_x[i * 12 + b] = v;
-      r = max(r, exponent(v));
-      if (px_exponent(v) == 2047) bad[b] = 1;
-    }
-#pragma unroll
-    for (int b = 0; b < 12; b++) atomicMax(&ce[b], relative(xi_x[i * 12 + b], r));
-    md[i].r = r4[i] = r;
+    if (e != PJ_NONE) atomicMax(&ce[t % 12], e - r[t / 12]);
+    if (px_exponent(v) == 2047) bad[t % 12] = 1;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int r = md[i].r;
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      const int d0 = relative(xi_x[i * 12 + 2 * k], r) - ce[2 * k], d1 = relative(xi_x[i * 12 + 2 * k + 1], r) - ce[2 * k + 1];
-      md[i].d[k] = ((unsigned)d0 & 0xffffu) | ((unsigned)d1 << 16);
-    }
-  }
   for (int t = threadIdx.x; t < n * 12; t += blockDim.x) {
-    double2 v = xi_x[t];
-    if (exponent(v) == PJ_NONE) v = make_double2(0.0, 0.0);
-    xi_l[t] = px_limbs<X>(v, max(md[t / 12].r + ce[t % 12], 1));
+    const int i = t / 12, b = t % 12;
+    const double2 v = entry(t);
+    const int e = exponent(v);
+    xi_x[t] = v;
+    xi_l[t] = px_limbs<X>(e == PJ_NONE ? make_double2(0.0, 0.0) : v, max(r[i] + ce[b], 1));
+    md[i].d[b] = (short)((e == PJ_NONE ? PJ_NONE : e - r[i]) - ce[b]);
+    if (b == 0) md[i].r = r4[i] = r[i];
   }
   if (threadIdx.x < 12) xe[threadIdx.x] = bad[threadIdx.x] ? 2047 : ce[threadIdx.x];
 }
@@ -697,14 +709,14 @@ int lq_slice_source(const lqcd_lattice* L, const Batch& b, const int* d_ids, int
   return launched_here();
 }
 
-template <int X, bool SCANNED>
+template <int X>
 static int proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi,
                      long long nsite_gs, long long y0, const double2* eta, double2* fact, cudaStream_t st) {
   Scratch s;
   const size_t n4 = ((size_t)n + 3) / 4 * 4;
   const long long nt = nsite_gs * 12;
   RC(s.alloc((sizeof(int4) + sizeof(double2)) * 12 * n + (sizeof(ProjMode) + sizeof(int)) * n4 + sizeof(int) * 12 +
-                 (SCANNED ? sizeof(int) * (size_t)nt : 0),
+                 (X == 0 ? sizeof(int) * (size_t)nt : 0),
              st));
   int4* xi_l = (int4*)s.p;
   double2* xi_x = (double2*)(xi_l + 12 * (size_t)n);
@@ -712,39 +724,34 @@ static int proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long
   int* r4 = (int*)(md + n4);
   int* xe = r4 + n4;
   int* word = xe + 12;
-  k_gather_site<X><<<1, 256, 0, st>>>(n, nsite_gb, xloc, xi, xi_l, xi_x, md, r4, xe);
+  k_gather_site<X><<<1, 1024, 0, st>>>(n, nsite_gb, xloc, xi, xi_l, xi_x, md, r4, xe);
   RC(launched_here());
   const size_t sm = sizeof(int4) * 12 * (size_t)n;
   if (sm > 48 * 1024) {
-    if (cudaFuncSetAttribute(k_proj_prop<X, SCANNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-        cudaSuccess) {
+    if (cudaFuncSetAttribute(k_proj_prop<X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
       cudaGetLastError();
       lq_set_error("projected propagator: too many modes for shared memory");
       return LQCD_EBADARG;
     }
   }
   const unsigned blocks = (unsigned)((nt + 127) / 128);
-  if (SCANNED) {
+  if (X == 0) {
     k_proj_scan<X><<<blocks, 128, 0, st>>>(n, nt, eta, md, xe, word);
     RC(launched_here());
   }
-  k_proj_prop<X, SCANNED><<<blocks, 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_l, xi_x, md, (const int4*)r4, xe, word, fact);
+  k_proj_prop<X><<<blocks, 128, sm, st>>>(n, nsite_gs, y0, L->V, eta, xi_l, xi_x, md, (const int4*)r4, xe, word, fact);
   return launched_here();
 }
 
-template <int X>
-static int proj_prop_x(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi,
-                       long long nsite_gs, long long y0, const double2* eta, double2* fact, cudaStream_t st) {
-  if (nsite_gs * 12 > 152 * 2 * 128) {
-    const int rc = proj_prop<X, true>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
-    if (rc != LQCD_ENOMEM) return rc;  // no room for the scan's words: the form without
-  }
-  return proj_prop<X, false>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
-}
-
-// Up to 32 modes fit one sum with a bit more.
+// The widest limbs whose sums hold all modes: the more bits, the seldomer a column needs a second sum.  Above 60 modes
+// the scan's words take 4 bytes a component of eta; without room for them, and where all blocks run at a time and another kernel
+// is the larger cost (120 modes on three slices of 4 x 4 x 8: 158 us, 143 in runs), runs of 60.
 int lq_proj_prop(const lqcd_lattice* L, int n, long long nsite_gb, long long xloc, const double2* xi, long long nsite_gs,
                  long long y0, const double2* eta, double2* fact, cudaStream_t st) {
-  return n <= px_modes<1> ? proj_prop_x<1>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st)
-                          : proj_prop_x<0>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+  if (n <= PJ_MODES<2>) return proj_prop<2>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+  if (n > PJ_MODES<1> && nsite_gs * 12 > 152 * 2 * 128) {
+    const int rc = proj_prop<0>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
+    if (rc != LQCD_ENOMEM) return rc;
+  }
+  return proj_prop<1>(L, n, nsite_gb, xloc, xi, nsite_gs, y0, eta, fact, st);
 }

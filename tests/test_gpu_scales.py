@@ -35,8 +35,8 @@ def _long(a):
     return a.astype(np.clongdouble)
 
 
-# one run of 32 modes (the wider limbs) and past it, one to three runs of 120
-@pytest.mark.parametrize("n", [1, 2, 5, 32, 33, 120, 121, 241])
+# up to 15 and up to 60 modes (wider limbs), one to three runs of 120
+@pytest.mark.parametrize("n", [1, 2, 5, 15, 16, 32, 33, 60, 61, 120, 121, 122, 241])
 @pytest.mark.parametrize("scales", ["reciprocal", "columns", "modes", "all", "zeros"])
 def test_projected_propagator_keeps_small_terms(n, scales):
     """Two entries, each rounded at 2^-54 of its scale, times the other below twice its scale, and the low parts' product: at
