@@ -133,6 +133,9 @@ int lqcd_set_gauge(lqcd_lattice *lat, int n_fields, const double *U, double kapp
 /* out = D_L in (dagger = 0) or D_L^dag in (dagger = 1) for the slab dom
  * (NULL: the whole lattice, with the lattice's time BC) on field `field`,
  * evaluated in `precision` (64, 32 or 16) through the even-odd packed data.
+ * Precision 64 sums products in fixed point with a scale per site: each
+ * component of out is off by a few 2^-53 of the largest component of in at
+ * the site and its neighbours; one that is not finite makes them NaN.
  * in / out: device slab vectors (see "slab" above) in complex128.
  * Sec. 3 eq. block_inverse: D_L is the sub-block of D on the slab's sites. */
 int lqcd_dslash(lqcd_lattice *lat, int field, const lqcd_slab *dom, int dagger, int precision, const double *in,

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(256) k_level_mean(long long size, int count, d
 // fast, which takes 2.7 times as long).
 //
 // Propagator of 64 x 24^3: 114.8 ms with the plain FP64 sums, one warp a site; 11.4 ms factored in
-// FP64; 5.8 ms so, 0.14 of them for the scales (error against long double 1.4e-16, of the FP64 sums 3.1e-16).
+// FP64; 5.8 ms so, 0.1 of them for the scales (error against long double over six propagators 2.3e-16 rms, of the FP64 sums 4.1e-16).
 constexpr int NP_T = 128;        // threads
 constexpr int NP_SITES = 16;     // sites staged at a time
 constexpr int NP_GROUPS = 4;     // most stages per block
