@@ -334,10 +334,10 @@ __global__ void __launch_bounds__(256) k_level_mean(long long size, int count, d
 // by spins or by pairs of colours.  The error of a site, 0.7 2^-53 of the product of the scales, is then one of its terms only
 // if one of them is about that large: np_large_terms looks for a term of W1 and one of W2 whose three entries all lie
 // within a factor of four of their scales, and a site without them is summed in FP64 (6600 multiply-adds on a pipe a 32nd as
-// fast, which takes 2.7 times as long).
+// fast: 64 x 24^3 takes 13.7 ms if all sites do, as with entries spread over 16 decades).
 //
 // Propagator of 64 x 24^3: 114.8 ms with the plain FP64 sums, one warp a site; 11.4 ms factored in
-// FP64; 5.8 ms so, 0.1 of them for the scales (error against long double over six propagators 2.3e-16 rms, of the FP64 sums 4.1e-16).
+// FP64; 5.7 ms so, 0.1 of them for the scales (error against long double over six propagators 2.3e-16 rms, of the FP64 sums 4.1e-16).
 constexpr int NP_T = 128;        // threads
 constexpr int NP_SITES = 16;     // sites staged at a time
 constexpr int NP_GROUPS = 4;     // most stages per block
